@@ -77,8 +77,8 @@ int ecc_limbs(ecc_curve_t curve);
  * multiplication; inputs are converted into Montgomery form and back).
  * field: ECC_FIELD_BASE (q = p) or ECC_FIELD_SCALAR (q = group order n).
  * a, b, out: n rows of L limbs (L = ecc_limbs() for the base field, 8 for the
- * scalar field); inputs must be canonical.  On the P-256 and secp256k1 base
- * fields these unit operations reduce with the special form of the prime
+ * scalar field); inputs must be canonical.  On the P-256, secp256k1
+ * and SM2 base fields the library reduces with the special form of the prime
  * (Section 4.2); the results are the same integers. */
 int ecc_fp_mul(ecc_curve_t curve, int field, size_t n, const uint32_t* a, const uint32_t* b,
                uint32_t* out, void* stream);
@@ -340,11 +340,10 @@ int ecc_bench_imad(size_t threads, int iters, uint32_t* sink, void* stream);
 
 /* Montgomery multiplications in registers: each thread runs `iters` rounds of
  * 4 independent mont_mul chains of the curve's base field.  reduction 0 = the
- * generic Montgomery reduction (Algorithm 2, as in every fused kernel);
- * 1 = the special-form reduction of Section 4.2 (P-256: u = T_0 and u q by
- * additions; secp256k1: u q = u 2^256 - u (2^32 + 977), one product per row;
- * ECC_EUNSUPPORTED on the other curves; the ecc_fp_* unit operations on these
- * two base fields use it).
+ * generic Montgomery reduction (Algorithm 2, as in the kernels on BN254,
+ * BLS12-381 and the scalar fields); 1 = the special-form reduction of Section
+ * 4.2 that the kernels on P-256 and secp256k1 use (P-256: additions only;
+ * secp256k1: one row of products by 977; ECC_EUNSUPPORTED on the other curves).
  * sink as above. */
 int ecc_bench_modmul(ecc_curve_t curve, int reduction, size_t threads, int iters, uint32_t* sink,
                      void* stream);

@@ -11,6 +11,31 @@ struct Secp256k1Fp {
   static constexpr int N = 8;
   static constexpr int BITS = 256;
   static constexpr uint32_t QINV = 0xd2253531u;
+  static constexpr int FORM = 2;
+  static constexpr uint64_t QINV62 = 0x27c7f6e22ddacacfull;  // q^-1 mod 2^62
+  ECC_DEV static constexpr uint32_t qinv() { return QINV; }
+  ECC_DEV static constexpr uint64_t qinv62() { return QINV62; }
+  ECC_DEV static constexpr uint32_t p(int i) {
+    switch (i) { case 0: return 0xfffffc2fu; case 1: return 0xfffffffeu; case 2: return 0xffffffffu; case 3: return 0xffffffffu; case 4: return 0xffffffffu; case 5: return 0xffffffffu; case 6: return 0xffffffffu; case 7: return 0xffffffffu; default: return 0u; }
+  }
+  ECC_DEV static constexpr uint32_t r2(int i) {
+    switch (i) { case 0: return 0x00000001u; case 1: return 0x00000000u; case 2: return 0x00000000u; case 3: return 0x00000000u; case 4: return 0x00000000u; case 5: return 0x00000000u; case 6: return 0x00000000u; case 7: return 0x00000000u; default: return 0u; }
+  }
+  ECC_DEV static constexpr uint32_t one(int i) {
+    switch (i) { case 0: return 0x00000001u; case 1: return 0x00000000u; case 2: return 0x00000000u; case 3: return 0x00000000u; case 4: return 0x00000000u; case 5: return 0x00000000u; case 6: return 0x00000000u; case 7: return 0x00000000u; default: return 0u; }
+  }
+  ECC_DEV static constexpr uint32_t pm2(int i) {
+    switch (i) { case 0: return 0xfffffc2du; case 1: return 0xfffffffeu; case 2: return 0xffffffffu; case 3: return 0xffffffffu; case 4: return 0xffffffffu; case 5: return 0xffffffffu; case 6: return 0xffffffffu; case 7: return 0xffffffffu; default: return 0u; }
+  }
+  ECC_DEV static constexpr uint32_t r3(int i) {
+    switch (i) { case 0: return 0x00000001u; case 1: return 0x00000000u; case 2: return 0x00000000u; case 3: return 0x00000000u; case 4: return 0x00000000u; case 5: return 0x00000000u; case 6: return 0x00000000u; case 7: return 0x00000000u; default: return 0u; }
+  }
+};
+
+struct Secp256k1FpMont {
+  static constexpr int N = 8;
+  static constexpr int BITS = 256;
+  static constexpr uint32_t QINV = 0xd2253531u;
   static constexpr int FORM = 0;
   static constexpr uint64_t QINV62 = 0x27c7f6e22ddacacfull;  // q^-1 mod 2^62
   ECC_DEV static constexpr uint32_t qinv() { return QINV; }
@@ -30,10 +55,6 @@ struct Secp256k1Fp {
   ECC_DEV static constexpr uint32_t r3(int i) {
     switch (i) { case 0: return 0x3795f671u; case 1: return 0x002bb1e3u; case 2: return 0x00000b73u; case 3: return 0x00000001u; case 4: return 0x00000000u; case 5: return 0x00000000u; case 6: return 0x00000000u; case 7: return 0x00000000u; default: return 0u; }
   }
-};
-
-struct Secp256k1FpSpecial : Secp256k1Fp {
-  static constexpr int FORM = 2;
 };
 
 struct Secp256k1Fn {
@@ -69,7 +90,7 @@ struct Secp256k1 {
     switch (i) { case 0: return 0x00000000u; case 1: return 0x00000000u; case 2: return 0x00000000u; case 3: return 0x00000000u; case 4: return 0x00000000u; case 5: return 0x00000000u; case 6: return 0x00000000u; case 7: return 0x00000000u; default: return 0u; }
   }
   ECC_DEV static constexpr uint32_t b(int i) {
-    switch (i) { case 0: return 0x00001ab7u; case 1: return 0x00000007u; case 2: return 0x00000000u; case 3: return 0x00000000u; case 4: return 0x00000000u; case 5: return 0x00000000u; case 6: return 0x00000000u; case 7: return 0x00000000u; default: return 0u; }
+    switch (i) { case 0: return 0x00000007u; case 1: return 0x00000000u; case 2: return 0x00000000u; case 3: return 0x00000000u; case 4: return 0x00000000u; case 5: return 0x00000000u; case 6: return 0x00000000u; case 7: return 0x00000000u; default: return 0u; }
   }
   ECC_DEV static constexpr uint32_t gx(int i) {
     switch (i) { case 0: return 0x16f81798u; case 1: return 0x59f2815bu; case 2: return 0x2dce28d9u; case 3: return 0x029bfcdbu; case 4: return 0xce870b07u; case 5: return 0x55a06295u; case 6: return 0xf9dcbbacu; case 7: return 0x79be667eu; default: return 0u; }
@@ -87,7 +108,7 @@ struct P256Fp {
   static constexpr int N = 8;
   static constexpr int BITS = 256;
   static constexpr uint32_t QINV = 0x00000001u;
-  static constexpr int FORM = 0;
+  static constexpr int FORM = 1;
   static constexpr uint64_t QINV62 = 0x3fffffffffffffffull;  // q^-1 mod 2^62
   ECC_DEV static constexpr uint32_t qinv() { return QINV; }
   ECC_DEV static constexpr uint64_t qinv62() { return QINV62; }
@@ -108,8 +129,8 @@ struct P256Fp {
   }
 };
 
-struct P256FpSpecial : P256Fp {
-  static constexpr int FORM = 1;
+struct P256FpMont : P256Fp {
+  static constexpr int FORM = 0;
 };
 
 struct P256Fn {
@@ -307,7 +328,7 @@ struct SM2Fp {
   static constexpr int N = 8;
   static constexpr int BITS = 256;
   static constexpr uint32_t QINV = 0x00000001u;
-  static constexpr int FORM = 0;
+  static constexpr int FORM = 3;
   static constexpr uint64_t QINV62 = 0x3fffffffffffffffull;  // q^-1 mod 2^62
   ECC_DEV static constexpr uint32_t qinv() { return QINV; }
   ECC_DEV static constexpr uint64_t qinv62() { return QINV62; }
@@ -326,6 +347,10 @@ struct SM2Fp {
   ECC_DEV static constexpr uint32_t r3(int i) {
     switch (i) { case 0: return 0x00000016u; case 1: return 0x00000012u; case 2: return 0xfffffff8u; case 3: return 0x0000000eu; case 4: return 0x0000000cu; case 5: return 0x0000000au; case 6: return 0x00000009u; case 7: return 0x0000001bu; default: return 0u; }
   }
+};
+
+struct SM2FpMont : SM2Fp {
+  static constexpr int FORM = 0;
 };
 
 struct SM2Fn {

@@ -1,13 +1,24 @@
 // Prime-field arithmetic on 32-bit limbs (modular arithmetic layer, Section 4).
 //
 // Elements are N little-endian 32-bit limbs (N even: 8 for 254/256-bit fields,
-// 12 for the 381-bit field) held in registers, in Montgomery form a*R mod q with
-// R = 2^(32N), canonical in [0, q).  A field is a traits class F with
-//   N, qinv() = -q^-1 mod 2^32, qinv62() = q^-1 mod 2^62, FORM (0 generic,
-//   1 the P-256 prime, 2 the secp256k1 prime), p(i),
-//   r2(i) = R^2 mod q, one(i) = R mod q, pm2(i) = q - 2.
+// 12 for the 381-bit field) held in registers, in Montgomery form a*R mod q,
+// canonical in [0, q), with R = 2^(32N), except that the secp256k1 base field
+// (FORM 2) is held as plain integers (R = 1).  A field is a traits class F with
+//   N, qinv() = -q^-1 mod 2^32, qinv62() = q^-1 mod 2^62, FORM (0 generic, 1 the
+//   P-256 prime, 2 the secp256k1 prime, 3 the SM2 prime), p(i),
+//   r2(i) = R^2 mod q, r3(i) = R^3 mod q, one(i) = R mod q, pm2(i) = q - 2.
 //
-// mont_mul is Montgomery multiplication (Algorithm 2) with the operand-scanning
+// FORM 1-3 multiply as a full 512-bit product (mul_wide8, sqr_wide8) followed by
+// a reduction that uses the shape of the prime (Section 4.2): additions only for
+// P-256 and SM2, one row of 977 h_i products for secp256k1.  The multiply-add
+// pipe takes one warp instruction per 4 cycles, so the 64 (73) wide multiply-adds
+// instead of 136 set the time, and the additions run on the other integer pipe
+// beside them.  GB300, 16 warps per SM, G modmul/s against the generic product:
+// P-256 113 against 68, secp256k1 110 against 68, SM2 107 against 68; squarings
+// (36 products instead of 64) 136, 143 and 132; one warp alone takes 245 ns
+// instead of 420 (178 for a squaring).
+//
+// The generic mont_mul is Montgomery multiplication (Algorithm 2) with the operand-scanning
 // order interleaved row by row.  Each row A*b_i is split into an "even" chain
 // (a_j b_i, j even) and an "odd" chain (a_j b_i, j odd), the mad_n carry chains
 // of Section 4.1: within one chain the 64-bit products sit on disjoint word
@@ -132,61 +143,289 @@ ECC_DEV void fe_neg(uint32_t* r, const uint32_t* a) {
   fe_sub<F>(r, z, a);
 }
 
-// Reduction row of mont_mul for q = 2^256 - 2^224 + 2^192 + 2^96 - 1 (NIST
-// P-256), the special-form reduction of Section 4.2 done our way: -q^-1 mod
-// 2^32 is 1, so u = T_0, and every limb of q is 0, 1 or 2^32 - 1, so
-// u q_j needs no multiplication: u (2^32 - 1) = hu 2^32 + nu with nu = -u mod
-// 2^32 and hu = u - [u != 0].  The even chain adds u (q_0 + q_2 2^64 + q_6 2^192)
-// to c (q_4 = 0): word 0 becomes u + nu, which is 0 with carry [u != 0], and
-// that carry plus hu makes u at word 1.  The odd chain adds
-// u (q_1 + q_7 2^192) to d (q_3 = q_5 = 0).  Both chains are additions: the
-// row costs no multiply-adds instead of 2N + 2.
-ECC_DEV void p256_reduce_row(uint32_t* c, uint32_t* d) {
-  const uint32_t u = c[0];
-  const uint32_t nu = 0u - u;
-  const uint32_t hu = u - (u != 0u ? 1u : 0u);
-  c[1] = ptx::add_cc(c[1], u);
-  c[2] = ptx::addc_cc(c[2], nu);
-  c[3] = ptx::addc_cc(c[3], hu);
-  c[4] = ptx::addc_cc(c[4], 0);
-  c[5] = ptx::addc_cc(c[5], 0);
-  c[6] = ptx::addc_cc(c[6], u);
-  c[7] = ptx::addc_cc(c[7], 0);
-  c[8] = ptx::addc(c[8], 0);
-  d[0] = ptx::add_cc(d[0], nu);
-  d[1] = ptx::addc_cc(d[1], hu);
-  d[2] = ptx::addc_cc(d[2], 0);
-  d[3] = ptx::addc_cc(d[3], 0);
-  d[4] = ptx::addc_cc(d[4], 0);
-  d[5] = ptx::addc_cc(d[5], 0);
-  d[6] = ptx::addc_cc(d[6], nu);
-  d[7] = ptx::addc_cc(d[7], hu);
-  d[8] = ptx::addc(d[8], 0);
+// T = a * b, 16 words.  Products on even words go to E, on odd words to O (the
+// mad_n chains of Section 4.1), so each row is one 4-product chain per array; a
+// row's carry out either meets a fresh word pair, where product plus carry
+// cannot overflow, or is caught in ec / oc and enters the next row's fresh pair.
+ECC_DEV void mul_wide8(uint32_t* T, const uint32_t* a, const uint32_t* b) {
+  uint32_t E[16], O[16];
+#pragma unroll
+  for (int j = 0; j < 8; j += 2) {
+    const uint64_t e = (uint64_t)a[j] * b[0], o = (uint64_t)a[j + 1] * b[0];
+    E[j] = (uint32_t)e;
+    E[j + 1] = (uint32_t)(e >> 32);
+    O[j + 1] = (uint32_t)o;
+    O[j + 2] = (uint32_t)(o >> 32);
+  }
+  uint32_t ec = 0, oc = 0;
+#pragma unroll
+  for (int i = 1; i < 8; ++i) {
+    uint32_t* const F = (i & 1) ? E : O;  // takes a_1, a_3, a_5, a_7 (top pair fresh)
+    uint32_t* const H = (i & 1) ? O : E;  // takes a_0, a_2, a_4, a_6 (carry out to come)
+    F[i + 1] = ptx::mad_lo_cc(a[1], b[i], F[i + 1]);
+    F[i + 2] = ptx::madc_hi_cc(a[1], b[i], F[i + 2]);
+    F[i + 3] = ptx::madc_lo_cc(a[3], b[i], F[i + 3]);
+    F[i + 4] = ptx::madc_hi_cc(a[3], b[i], F[i + 4]);
+    F[i + 5] = ptx::madc_lo_cc(a[5], b[i], F[i + 5]);
+    F[i + 6] = ptx::madc_hi_cc(a[5], b[i], F[i + 6]);
+    F[i + 7] = ptx::madc_lo_cc(a[7], b[i], (i & 1) ? ec : oc);
+    F[i + 8] = ptx::madc_hi(a[7], b[i], 0);
+    H[i] = ptx::mad_lo_cc(a[0], b[i], H[i]);
+    H[i + 1] = ptx::madc_hi_cc(a[0], b[i], H[i + 1]);
+    H[i + 2] = ptx::madc_lo_cc(a[2], b[i], H[i + 2]);
+    H[i + 3] = ptx::madc_hi_cc(a[2], b[i], H[i + 3]);
+    H[i + 4] = ptx::madc_lo_cc(a[4], b[i], H[i + 4]);
+    H[i + 5] = ptx::madc_hi_cc(a[4], b[i], H[i + 5]);
+    H[i + 6] = ptx::madc_lo_cc(a[6], b[i], H[i + 6]);
+    H[i + 7] = ptx::madc_hi_cc(a[6], b[i], H[i + 7]);
+    ((i & 1) ? oc : ec) = ptx::addc(0, 0);
+  }
+  // E holds words 0..15, O words 1..14 and its last carry at word 15
+  T[0] = E[0];
+  T[1] = ptx::add_cc(E[1], O[1]);
+#pragma unroll
+  for (int k = 2; k < 15; ++k) T[k] = ptx::addc_cc(E[k], O[k]);
+  T[15] = ptx::addc(E[15], oc);
 }
 
-// Reduction row of mont_mul for q = 2^256 - 2^32 - 977 (secp256k1), the
-// special-form idea of Section 4.2 applied to this prime: u q = u 2^256 -
-// u (2^32 + 977), so the row needs one 32 x 32 -> 64 product (977 u) instead
-// of N.  -q^-1 mod 2^32 is not 1 for this prime, so u = T_0 QINV stays a
-// multiplication.  Word 0 of T + u q is exactly 0 with no carry (u makes
-// T_0 = 977 u mod 2^32), and the words above it receive
-// A = u 2^224 - (u + floor(977 u / 2^32)) in the frame of d (d[k] is word
-// k + 1): A is a non-negative 256-bit value (0 when u = 0), added with one
-// carry chain whose carry lands in d's top word.
-ECC_DEV void secp256k1_reduce_row(uint32_t* c, uint32_t* d, uint32_t qinv) {
-  const uint32_t u = c[0] * qinv;
-  const uint32_t s1 = ptx::add_cc(__umulhi(u, 977u), u);
-  const uint32_t s2 = ptx::addc(0, 0);
-  uint32_t A[8];
-  A[0] = ptx::sub_cc(0, s1);
-  A[1] = ptx::subc_cc(0, s2);
+// T = a^2, 16 words: the 28 products a_i a_j, i < j, once (E and O as above),
+// doubled by a shift, plus the 8 squares as one chain.
+ECC_DEV void sqr_wide8(uint32_t* T, const uint32_t* a) {
+  uint32_t E[16], O[16];
 #pragma unroll
-  for (int k = 2; k < 7; ++k) A[k] = ptx::subc_cc(0, 0);
-  A[7] = ptx::subc(u, 0);
-  d[0] = ptx::add_cc(d[0], A[0]);
+  for (int j = 1; j < 8; ++j) {  // row 0: a_0 a_j at word j
+    const uint64_t w = (uint64_t)a[0] * a[j];
+    uint32_t* const A = (j & 1) ? O : E;
+    A[j] = (uint32_t)w;
+    A[j + 1] = (uint32_t)(w >> 32);
+  }
+  E[8] = 0;
+  O[9] = 0;
 #pragma unroll
-  for (int k = 1; k < 8; ++k) d[k] = ptx::addc_cc(d[k], A[k]);
-  d[8] = ptx::addc(d[8], 0);
+  for (int i = 1; i < 7; ++i) {
+    // a_i a_j at words i + j: first j = i + 1, i + 3, .. (odd words), then
+    // j = i + 2, i + 4, .. (even words).  The chain that ends with a_7 meets a
+    // fresh top pair (its low word may hold the other row's caught carry).
+#pragma unroll
+    for (int par = 1; par <= 2; ++par) {
+      uint32_t* const A = par == 1 ? O : E;
+      const int last = ((7 - i - par) & 1) ? 6 : 7;
+      if (last < i + par) continue;
+#pragma unroll
+      for (int j = i + par; j <= last; j += 2) {
+        const int w = i + j;
+        A[w] = j == i + par ? ptx::mad_lo_cc(a[i], a[j], A[w]) : ptx::madc_lo_cc(a[i], a[j], A[w]);
+        A[w + 1] = j == 7 ? ptx::madc_hi(a[i], a[j], 0) : ptx::madc_hi_cc(a[i], a[j], A[w + 1]);
+      }
+      if (last == 6) A[i + 8] = ptx::addc(0, 0);
+    }
+  }
+  uint32_t D[16];
+  D[1] = O[1];
+  D[2] = ptx::add_cc(E[2], O[2]);
+#pragma unroll
+  for (int k = 3; k < 14; ++k) D[k] = ptx::addc_cc(E[k], O[k]);
+  D[14] = ptx::addc_cc(O[14], 0);
+  D[15] = ptx::addc(0, 0);
+  uint32_t S[16];
+  S[0] = 0;
+  S[1] = D[1] << 1;
+#pragma unroll
+  for (int k = 2; k < 16; ++k) S[k] = __funnelshift_l(D[k - 1], D[k], 1);
+  T[0] = ptx::mad_lo_cc(a[0], a[0], S[0]);
+  T[1] = ptx::madc_hi_cc(a[0], a[0], S[1]);
+#pragma unroll
+  for (int k = 1; k < 7; ++k) {
+    T[2 * k] = ptx::madc_lo_cc(a[k], a[k], S[2 * k]);
+    T[2 * k + 1] = ptx::madc_hi_cc(a[k], a[k], S[2 * k + 1]);
+  }
+  T[14] = ptx::madc_lo_cc(a[7], a[7], S[14]);
+  T[15] = ptx::madc_hi(a[7], a[7], S[15]);
+}
+
+// r = t mod q for t < 2q (t: N + 1 words)
+template <class F>
+ECC_DEV void fe_sub_once(uint32_t* r, const uint32_t* t) {
+  constexpr int N = F::N;
+  uint32_t s[N];
+  s[0] = ptx::sub_cc(t[0], F::p(0));
+#pragma unroll
+  for (int k = 1; k < N; ++k) s[k] = ptx::subc_cc(t[k], F::p(k));
+  const uint32_t top = ptx::subc(t[N], 0);  // 0xffffffff iff t < q
+#pragma unroll
+  for (int k = 0; k < N; ++k) r[k] = top == 0xffffffffu ? t[k] : s[k];
+}
+
+// T R^-1 mod p for p = 2^256 - 2^224 + 2^192 + 2^96 - 1 (NIST P-256), T < p 2^256,
+// destroying T.  p = -1 mod 2^96, so u = T mod 2^96 clears 96 bits at a time:
+// (T + u p) / 2^96 = (T >> 96) + u + 2^96 W with W = u (1 - 2^32 + 2^64), five
+// words that follow u's three without overlap, so a step is W (7 additions) and
+// one 8-word chain; a chain's carry has the weight of the next step's third word
+// of W and enters there.  Two 96-bit steps and one of 64 bits: 43 additions.
+template <class F>
+ECC_DEV void redc_p256(uint32_t* r, uint32_t* T) {
+  uint32_t W1, W2, W3, W4, x2, x3, x4;
+#pragma unroll
+  for (int k = 0; k < 6; k += 3) {
+    const uint32_t u0 = T[k], u1 = T[k + 1], u2 = T[k + 2];
+    x2 = k == 0 ? ptx::add_cc(u2, u0) : ptx::addc_cc(u2, u0);  // carry of the first step
+    x3 = ptx::addc_cc(u1, 0);
+    x4 = ptx::addc(u2, 0);
+    W1 = ptx::sub_cc(u1, u0);
+    W2 = ptx::subc_cc(x2, u1);
+    W3 = ptx::subc_cc(x3, u2);
+    W4 = ptx::subc(x4, 0);
+    T[k + 3] = ptx::add_cc(T[k + 3], u0);
+    T[k + 4] = ptx::addc_cc(T[k + 4], u1);
+    T[k + 5] = ptx::addc_cc(T[k + 5], u2);
+    T[k + 6] = ptx::addc_cc(T[k + 6], u0);
+    T[k + 7] = ptx::addc_cc(T[k + 7], W1);
+    T[k + 8] = ptx::addc_cc(T[k + 8], W2);
+    T[k + 9] = ptx::addc_cc(T[k + 9], W3);
+    T[k + 10] = ptx::addc_cc(T[k + 10], W4);
+  }
+  // u = T mod 2^64: T >> 64 plus 2^32 u + 2^128 u (1 - 2^32 + 2^64)
+  const uint32_t u0 = T[6], u1 = T[7];
+  x2 = ptx::addc_cc(u0, 0);  // carry of the second step
+  x3 = ptx::addc(u1, 0);
+  W1 = ptx::sub_cc(u1, u0);
+  W2 = ptx::subc_cc(x2, u1);
+  W3 = ptx::subc(x3, 0);
+  uint32_t t[9];
+  t[0] = T[8];
+  t[1] = ptx::add_cc(T[9], u0);
+  t[2] = ptx::addc_cc(T[10], u1);
+  t[3] = ptx::addc_cc(T[11], 0);
+  t[4] = ptx::addc_cc(T[12], u0);
+  t[5] = ptx::addc_cc(T[13], W1);
+  t[6] = ptx::addc_cc(T[14], W2);
+  t[7] = ptx::addc_cc(T[15], W3);
+  t[8] = ptx::addc(0, 0);
+  fe_sub_once<F>(r, t);
+}
+
+// T mod p for p = 2^256 - 2^32 - 977 (secp256k1), any 512-bit T.  With
+// T = lo + 2^256 hi the value is lo + 977 hi + 2^32 hi mod p: the products
+// 977 h_i for even i go onto lo, those for odd i onto 2^32 hi (each product pair
+// on words that the array already holds), so the fold is 8 wide multiply-adds
+// and one merge.  The words above 2^256 (below 2^34) fold once more.
+template <class F>
+ECC_DEV void red_secp256k1(uint32_t* r, const uint32_t* T) {
+  const uint32_t* h = T + 8;
+  constexpr uint32_t C = 977u;
+  uint32_t e[9], o[10];
+  e[0] = ptx::mad_lo_cc(h[0], C, T[0]);
+  e[1] = ptx::madc_hi_cc(h[0], C, T[1]);
+#pragma unroll
+  for (int k = 2; k < 8; k += 2) {
+    e[k] = ptx::madc_lo_cc(h[k], C, T[k]);
+    e[k + 1] = ptx::madc_hi_cc(h[k], C, T[k + 1]);
+  }
+  e[8] = ptx::addc(0, 0);
+  o[1] = ptx::mad_lo_cc(h[1], C, h[0]);
+  o[2] = ptx::madc_hi_cc(h[1], C, h[1]);
+#pragma unroll
+  for (int k = 3; k < 9; k += 2) {
+    o[k] = ptx::madc_lo_cc(h[k], C, h[k - 1]);
+    o[k + 1] = ptx::madc_hi_cc(h[k], C, h[k]);
+  }
+  o[9] = ptx::addc(0, 0);
+  e[1] = ptx::add_cc(e[1], o[1]);
+#pragma unroll
+  for (int k = 2; k < 9; ++k) e[k] = ptx::addc_cc(e[k], o[k]);
+  const uint32_t g = ptx::addc(o[9], 0);
+  // (e_8 + 2^32 g)(2^32 + 977), g <= 1
+  const uint64_t w = (uint64_t)e[8] * C;
+  uint32_t x1 = ptx::add_cc((uint32_t)(w >> 32), e[8]);
+  uint32_t x2 = ptx::addc(g, 0);
+  x1 = ptx::add_cc(x1, g * C);
+  x2 = ptx::addc(x2, 0);
+  uint32_t t[8], s[8];
+  t[0] = ptx::add_cc(e[0], (uint32_t)w);
+  t[1] = ptx::addc_cc(e[1], x1);
+  t[2] = ptx::addc_cc(e[2], x2);
+#pragma unroll
+  for (int k = 3; k < 8; ++k) t[k] = ptx::addc_cc(e[k], 0);
+  uint32_t over = ptx::addc(0, 0);
+  // t + 2^256 over < 2p: t + 2^32 + 977 carries, or over is set, iff it is >= p
+  s[0] = ptx::add_cc(t[0], C);
+  s[1] = ptx::addc_cc(t[1], 1u);
+#pragma unroll
+  for (int k = 2; k < 8; ++k) s[k] = ptx::addc_cc(t[k], 0);
+  over = ptx::addc(over, 0);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) r[k] = over ? s[k] : t[k];
+}
+
+// T R^-1 mod p for p = 2^256 - 2^224 - 2^96 + 2^64 - 1 (SM2), T < p 2^256.  With
+// m = T_lo (-p^-1) mod 2^256 the result is (T + m p) / 2^256, and both parts are
+// additions of shifted m:
+//   m = T_lo + (m << 64) - (m << 96) - (m << 224) mod 2^256 (word by word; the
+//       carry of the sum and the two borrows are the low part's carry),
+//   r = T_hi + m + (m >> 192) - (m >> 160) - (m >> 32) + carry - borrows.
+// 55 additions, against 88 for four 64-bit steps (107 against 75-85 G modmul/s).
+template <class F>
+ECC_DEV void redc_sm2(uint32_t* r, const uint32_t* T) {
+  uint32_t m[8], A[8], c, b;
+  m[0] = T[0];
+  m[1] = T[1];
+  m[2] = ptx::add_cc(T[2], m[0]);
+  A[3] = ptx::addc_cc(T[3], m[1]);
+  A[4] = ptx::addc_cc(T[4], m[2]);
+  c = ptx::addc(0, 0);
+  m[3] = ptx::sub_cc(A[3], m[0]);
+  m[4] = ptx::subc_cc(A[4], m[1]);
+  b = ptx::subc(0, 0);
+  ptx::add_cc(c, 0xffffffffu);  // restores the carry (a borrow: 0 - b below)
+  A[5] = ptx::addc_cc(T[5], m[3]);
+  A[6] = ptx::addc_cc(T[6], m[4]);
+  c = ptx::addc(0, 0);
+  ptx::sub_cc(0, b);
+  m[5] = ptx::subc_cc(A[5], m[2]);
+  m[6] = ptx::subc_cc(A[6], m[3]);
+  b = ptx::subc(0, 0);
+  ptx::add_cc(c, 0xffffffffu);
+  A[7] = ptx::addc_cc(T[7], m[5]);
+  c = ptx::addc(0, 0);  // carry of the low part
+  ptx::sub_cc(0, b);
+  m[7] = ptx::subc_cc(A[7], m[4]);
+  b = ptx::subc(0, 0);  // its first borrow
+  m[7] = ptx::sub_cc(m[7], m[0]);
+  const uint32_t b2 = ptx::subc(0, 0);  // its second borrow
+  // S = (m >> 32) + (m >> 160) - (m >> 192) + second borrow
+  uint32_t S[8], t[9];
+  const uint32_t d0 = ptx::sub_cc(m[5], m[6]);
+  const uint32_t d1 = ptx::subc_cc(m[6], m[7]);
+  const uint32_t d2 = ptx::subc(m[7], 0);
+  ptx::add_cc(b2, 1u);  // carries iff b2 is all ones
+  S[0] = ptx::addc_cc(m[1], d0);
+  S[1] = ptx::addc_cc(m[2], d1);
+  S[2] = ptx::addc_cc(m[3], d2);
+#pragma unroll
+  for (int k = 3; k < 7; ++k) S[k] = ptx::addc_cc(m[k + 1], 0);
+  S[7] = ptx::addc(0, 0);
+  ptx::add_cc(c, 0xffffffffu);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) t[k] = ptx::addc_cc(T[8 + k], m[k]);
+  t[8] = ptx::addc(0, 0);
+  ptx::sub_cc(0, b);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) t[k] = ptx::subc_cc(t[k], S[k]);
+  t[8] = ptx::subc(t[8], 0);
+  fe_sub_once<F>(r, t);
+}
+
+// The reduction of a 512-bit product for FORM 1-3 (T is destroyed).
+template <class F>
+ECC_DEV void reduce_wide(uint32_t* r, uint32_t* T) {
+  static_assert(F::FORM >= 1 && F::FORM <= 3 && F::N == 8, "special-form primes");
+  if constexpr (F::FORM == 1) {
+    redc_p256<F>(r, T);
+  } else if constexpr (F::FORM == 2) {
+    red_secp256k1<F>(r, T);
+  } else {
+    redc_sm2<F>(r, T);
+  }
 }
 
 // Montgomery product r = a * b * R^-1 mod q (r may alias a or b).
@@ -194,6 +433,12 @@ template <class F>
 ECC_DEV void mont_mul(uint32_t* r, const uint32_t* a, const uint32_t* b) {
   constexpr int N = F::N;
   static_assert(N % 2 == 0, "even limb count");
+  if constexpr (F::FORM != 0) {
+    uint32_t T[16];
+    mul_wide8(T, a, b);
+    reduce_wide<F>(r, T);
+    return;
+  }
   uint32_t c[N + 1], d[N + 1];
 #pragma unroll
   for (int i = 0; i < N + 1; ++i) {
@@ -239,14 +484,6 @@ ECC_DEV void mont_mul(uint32_t* r, const uint32_t* a, const uint32_t* b) {
       c[j + 1] = ptx::madc_hi_cc(a[j], bi, c[j + 1]);
     }
     c[N] = ptx::addc(c[N], 0);
-    if constexpr (F::FORM == 1) {
-      p256_reduce_row(c, d);
-      continue;
-    }
-    if constexpr (F::FORM == 2) {
-      secp256k1_reduce_row(c, d, F::qinv());
-      continue;
-    }
     // reduction row: u = T_0 * QINV, T += u * q (even and odd chains)
     const uint32_t u = c[0] * F::qinv();
     c[0] = ptx::mad_lo_cc(u, F::p(0), c[0]);
@@ -272,23 +509,27 @@ ECC_DEV void mont_mul(uint32_t* r, const uint32_t* a, const uint32_t* b) {
 #pragma unroll
   for (int k = 1; k < N; ++k) t[k] = ptx::addc_cc(d[k], c[k + 1]);
   t[N] = ptx::addc(d[N], 0);
-  uint32_t s[N];
-  s[0] = ptx::sub_cc(t[0], F::p(0));
-#pragma unroll
-  for (int k = 1; k < N; ++k) s[k] = ptx::subc_cc(t[k], F::p(k));
-  const uint32_t top = ptx::subc(t[N], 0);  // 0xffffffff iff t < q
-#pragma unroll
-  for (int k = 0; k < N; ++k) r[k] = top == 0xffffffffu ? t[k] : s[k];
+  fe_sub_once<F>(r, t);
 }
 
 template <class F>
 ECC_DEV void mont_sqr(uint32_t* r, const uint32_t* a) {
-  mont_mul<F>(r, a, a);
+  if constexpr (F::FORM != 0) {
+    uint32_t T[16];
+    sqr_wide8(T, a);
+    reduce_wide<F>(r, T);
+  } else {
+    mont_mul<F>(r, a, a);
+  }
 }
 
 // canonical integer -> Montgomery form (a * R^2 * R^-1 = a R)
 template <class F>
 ECC_DEV void to_mont(uint32_t* r, const uint32_t* a) {
+  if constexpr (F::FORM == 2) {  // held as plain integers
+    fe_copy<F>(r, a);
+    return;
+  }
   uint32_t r2[F::N];
 #pragma unroll
   for (int i = 0; i < F::N; ++i) r2[i] = F::r2(i);
@@ -298,6 +539,10 @@ ECC_DEV void to_mont(uint32_t* r, const uint32_t* a) {
 // Montgomery form -> canonical integer
 template <class F>
 ECC_DEV void from_mont(uint32_t* r, const uint32_t* a) {
+  if constexpr (F::FORM == 2) {
+    fe_copy<F>(r, a);
+    return;
+  }
   uint32_t one[F::N];
 #pragma unroll
   for (int i = 0; i < F::N; ++i) one[i] = i == 0 ? 1u : 0u;

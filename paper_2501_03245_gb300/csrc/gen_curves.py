@@ -42,14 +42,15 @@ CURVES = [
 ]
 
 
-# Moduli that also get a second traits class with a reduction of their own
-# (fp.cuh, mont_mul): FORM 1 is the NIST P-256 prime 2^256 - 2^224 + 2^192 +
-# 2^96 - 1, whose -q^-1 mod 2^32 is 1 and whose limbs are 0, 1 and 2^32 - 1
-# only; FORM 2 is the secp256k1 prime 2^256 - 2^32 - 977.  The main traits
-# classes are FORM 0 (the generic Montgomery reduction).
-SPECIAL = {
-    0xFFFFFFFF00000001000000000000000000000000FFFFFFFFFFFFFFFFFFFFFFFF: ("P256FpSpecial", 1),
-    (1 << 256) - (1 << 32) - 977: ("Secp256k1FpSpecial", 2),
+# Moduli whose multiplication uses the shape of the prime (fp.cuh): FORM 1 is the
+# NIST P-256 prime 2^256 - 2^224 + 2^192 + 2^96 - 1, FORM 2 the secp256k1 prime
+# 2^256 - 2^32 - 977 (elements held as plain integers: R = 1), FORM 3 the SM2
+# prime 2^256 - 2^224 - 2^96 + 2^64 - 1.  Each also gets a class <name>Mont with
+# the generic Montgomery multiplication, which the probes compare with.
+FORMS = {
+    0xFFFFFFFF00000001000000000000000000000000FFFFFFFFFFFFFFFFFFFFFFFF: 1,
+    (1 << 256) - (1 << 32) - 977: 2,
+    (1 << 256) - (1 << 224) - (1 << 96) + (1 << 64) - 1: 3,
 }
 
 
@@ -64,25 +65,32 @@ def arr(name, v, n):
             f"    switch (i) {{ {cases} default: return 0u; }}\n  }}\n")
 
 
-def field(name, q):
+def traits(name, q, form):
     n = (q.bit_length() + 31) // 32
     n += n % 2  # even limb count for the even/odd carry chains
-    R = 1 << (32 * n)
+    R = 1 if form == 2 else 1 << (32 * n)
     qinv = (-pow(q, -1, 1 << 32)) % (1 << 32)
     s = f"struct {name} {{\n"
     s += f"  static constexpr int N = {n};\n"
     s += f"  static constexpr int BITS = {q.bit_length()};\n"
     s += f"  static constexpr uint32_t QINV = 0x{qinv:08x}u;\n"
-    s += "  static constexpr int FORM = 0;\n"
+    s += f"  static constexpr int FORM = {form};\n"
     s += f"  static constexpr uint64_t QINV62 = 0x{pow(q, -1, 1 << 62):016x}ull;  // q^-1 mod 2^62\n"
     s += "  ECC_DEV static constexpr uint32_t qinv() { return QINV; }\n"
     s += "  ECC_DEV static constexpr uint64_t qinv62() { return QINV62; }\n"
     s += arr("p", q, n) + arr("r2", R * R % q, n) + arr("one", R % q, n) + arr("pm2", q - 2, n)
     s += arr("r3", R * R * R % q, n)
     s += "};\n\n"
-    if q in SPECIAL:
-        sname, form = SPECIAL[q]
-        s += f"struct {sname} : {name} {{\n  static constexpr int FORM = {form};\n}};\n\n"
+    return s, n, R
+
+
+def field(name, q):
+    form = FORMS.get(q, 0)
+    s, n, R = traits(name, q, form)
+    if form == 2:
+        s += traits(name + "Mont", q, 0)[0]
+    elif form:
+        s += f"struct {name}Mont : {name} {{\n  static constexpr int FORM = 0;\n}};\n\n"
     return s, n, R
 
 

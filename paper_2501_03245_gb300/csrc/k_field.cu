@@ -184,9 +184,9 @@ int field_limbs(int curve, int field) {
 
 #define ECC_FIELD_DISPATCH(curve, field, CALL)          \
   switch ((curve) * 2 + (field)) {                      \
-    case 0: { using F = Secp256k1FpSpecial; return CALL; } \
+    case 0: { using F = Secp256k1Fp; return CALL; }     \
     case 1: { using F = Secp256k1Fn; return CALL; }     \
-    case 2: { using F = P256FpSpecial; return CALL; }   \
+    case 2: { using F = P256Fp; return CALL; }          \
     case 3: { using F = P256Fn; return CALL; }          \
     case 4: { using F = BN254Fp; return CALL; }         \
     case 5: { using F = BN254Fn; return CALL; }         \
@@ -235,7 +235,7 @@ cudaError_t launch_bench_inv(int curve, int method, size_t threads, int iters, u
   const unsigned t = (unsigned)(threads < 128 ? threads : 128);
   const unsigned b = (unsigned)((threads + t - 1) / t);
   switch (curve) {
-    case 0: k_bench_inv<Secp256k1Fp><<<b, t, 0, st>>>(method, iters, sink); break;
+    case 0: k_bench_inv<Secp256k1FpMont><<<b, t, 0, st>>>(method, iters, sink); break;
     case 1: k_bench_inv<P256Fp><<<b, t, 0, st>>>(method, iters, sink); break;
     case 2: k_bench_inv<BN254Fp><<<b, t, 0, st>>>(method, iters, sink); break;
     case 3: k_bench_inv<BLS12_381Fp><<<b, t, 0, st>>>(method, iters, sink); break;
@@ -250,20 +250,20 @@ cudaError_t launch_bench_modmul(int curve, int reduction, size_t threads, int it
   const unsigned b = (unsigned)((threads + 255) / 256);
   if (reduction == 1) {
     if (curve == 1) {
-      k_bench_modmul<P256FpSpecial><<<b, 256, 0, st>>>(iters, sink);
+      k_bench_modmul<P256Fp><<<b, 256, 0, st>>>(iters, sink);
     } else if (curve == 0) {
-      k_bench_modmul<Secp256k1FpSpecial><<<b, 256, 0, st>>>(iters, sink);
+      k_bench_modmul<Secp256k1Fp><<<b, 256, 0, st>>>(iters, sink);
     } else {
       return cudaErrorNotSupported;
     }
     return cudaGetLastError();
   }
   switch (curve) {
-    case 0: k_bench_modmul<Secp256k1Fp><<<b, 256, 0, st>>>(iters, sink); break;
-    case 1: k_bench_modmul<P256Fp><<<b, 256, 0, st>>>(iters, sink); break;
+    case 0: k_bench_modmul<Secp256k1FpMont><<<b, 256, 0, st>>>(iters, sink); break;
+    case 1: k_bench_modmul<P256FpMont><<<b, 256, 0, st>>>(iters, sink); break;
     case 2: k_bench_modmul<BN254Fp><<<b, 256, 0, st>>>(iters, sink); break;
     case 3: k_bench_modmul<BLS12_381Fp><<<b, 256, 0, st>>>(iters, sink); break;
-    case 4: k_bench_modmul<SM2Fp><<<b, 256, 0, st>>>(iters, sink); break;
+    case 4: k_bench_modmul<SM2FpMont><<<b, 256, 0, st>>>(iters, sink); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
