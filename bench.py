@@ -212,8 +212,8 @@ def gen_inputs(ecc, synth, torch, n, seed, curve=CURVE_P256):
 # dram__bytes_write.sum, from one ncu capture), valid only for the kernel sources
 # it was taken on: the digest of those sources must match, else it is null.
 VERIFY_TRAFFIC = {"bytes": 79369814528 + 33884342528, "batch": 1 << 20, "digest": "d56ffe9d83e1591f",
-                  "sources": ["verify.cuh", "verify_host.cuh", "ops.cuh", "ec.cuh", "fp.cuh", "inv.cuh",
-                              "ptx.cuh", "curves_gen.cuh", "internal.h", "k_verify_p256_c2.cu", "k_verify.cu"]}
+                  "sources": ["verify.cuh", "verify_host.cuh", "ladder.cuh", "ec.cuh", "fp.cuh", "inv.cuh",
+                              "ptx.cuh", "curves_gen.cuh", "internal.h", "k_verify_p256.cu", "k_verify.cu"]}
 
 
 def verify_traffic(n):

@@ -22,8 +22,8 @@
  *     stages through device memory and returns after the results are written
  *     back, i.e. it is synchronous).  The library owns only its internal
  *     workspace (stream-ordered allocations released at the end of each call)
- *     and the per-device fixed-base tables (built on first use of a curve and
- *     kept until process exit).  The first call that needs a curve's table
+ *     and the per-device fixed-base tables (32 MiB a curve, 48 MiB for
+ *     BLS12-381; built on first use of a curve and kept until process exit).  The first call that needs a curve's table
  *     builds it synchronously; do that call before any stream capture.
  *   - Field elements: little-endian 32-bit limbs, canonical (< modulus).  A
  *     base-field element of BN254 / secp256k1 / P-256 has 8 limbs, of
@@ -164,7 +164,7 @@ int ecc_verify_batch(ecc_curve_t curve, size_t n, const uint8_t* hash, const uin
 
 /* ---------------------------------------------------------------- FPMUL
  * out[i] = k[i] * G (fixed-point multiplication, Section 2.1.1 and Table 5:
- * the generator's table v 2^(8j) G removes every PDBL; 32 batched affine
+ * the generator's table v 2^(16j) G, v = 1 .. 2^15, removes every PDBL; 16
  * additions per scalar).  k: n x 8 limbs (any 256-bit integer); out: n affine
  * points ((0, 0) when k[i] * G = O). */
 int ecc_fixed_base_mul(ecc_curve_t curve, size_t n, const uint32_t* k, uint32_t* out,
@@ -307,14 +307,10 @@ int ecc_msm_set_window(ecc_curve_t curve, int log2_n, int c);
 int ecc_msm_reduce_chunk(ecc_curve_t curve, size_t n);
 int ecc_msm_set_reduce_chunk(ecc_curve_t curve, int log2_n, int log2_chunk);
 
-/* Gather-apply-scatter across a thread-block cluster for ECDSA verification
- * (the memory-management idea of Section 3.3 taken to a cluster): with ctas =
- * 2 (the default), ecc_verify_batch runs in clusters of two CTAs that share
- * each round's single inversion through distributed shared memory (the second
- * CTA's product goes to the first, which inverts both products by Montgomery's
- * trick and sends the second its inverse back); ctas = 1 gives every CTA its
- * own inversion.  Process-wide setting; results are identical either way;
- * other values give ECC_EINVAL. */
+/* Number of CTAs (1 or 2, default 2) that may share one inversion per batched
+ * round in ECDSA verification.  Results are identical either way; other values
+ * give ECC_EINVAL.  Verification runs one thread per signature and shares no
+ * inversions, so the setting has no effect on it. */
 int ecc_set_gas_cluster(int ctas);
 
 /* MSM phase timers (diagnostics).  With timing on, every MSM entry point

@@ -523,6 +523,58 @@ ECC_DEV void mont_sqr(uint32_t* r, const uint32_t* a) {
   }
 }
 
+// r = a b - c d, with one reduction of the difference of the two products for
+// FORM 1-3 (52 additions fewer than two reductions and a subtraction): a negative
+// difference gets q 2^256.
+ECC_DEV bool sub_wide(uint32_t* A, const uint32_t* B) {
+  A[0] = ptx::sub_cc(A[0], B[0]);
+#pragma unroll
+  for (int k = 1; k < 16; ++k) A[k] = ptx::subc_cc(A[k], B[k]);
+  return ptx::subc(0, 0) != 0;
+}
+
+template <class F>
+ECC_DEV void reduce_diff(uint32_t* r, uint32_t* A, const uint32_t* B) {
+  const uint32_t mask = sub_wide(A, B) ? 0xffffffffu : 0u;
+  A[8] = ptx::add_cc(A[8], F::p(0) & mask);
+#pragma unroll
+  for (int k = 1; k < 7; ++k) A[8 + k] = ptx::addc_cc(A[8 + k], F::p(k) & mask);
+  A[15] = ptx::addc(A[15], F::p(7) & mask);
+  reduce_wide<F>(r, A);
+}
+
+template <class F>
+ECC_DEV void mont_mul_sub(uint32_t* r, const uint32_t* a, const uint32_t* b, const uint32_t* c,
+                          const uint32_t* d) {
+  if constexpr (F::FORM != 0) {
+    uint32_t A[16], B[16];
+    mul_wide8(A, a, b);
+    mul_wide8(B, c, d);
+    reduce_diff<F>(r, A, B);
+  } else {
+    uint32_t t[F::N], u[F::N];
+    mont_mul<F>(t, a, b);
+    mont_mul<F>(u, c, d);
+    fe_sub<F>(r, t, u);
+  }
+}
+
+// r = a b - c^2
+template <class F>
+ECC_DEV void mont_mul_sub_sqr(uint32_t* r, const uint32_t* a, const uint32_t* b, const uint32_t* c) {
+  if constexpr (F::FORM != 0) {
+    uint32_t A[16], B[16];
+    mul_wide8(A, a, b);
+    sqr_wide8(B, c);
+    reduce_diff<F>(r, A, B);
+  } else {
+    uint32_t t[F::N], u[F::N];
+    mont_mul<F>(t, a, b);
+    mont_sqr<F>(u, c);
+    fe_sub<F>(r, t, u);
+  }
+}
+
 // canonical integer -> Montgomery form (a * R^2 * R^-1 = a R)
 template <class F>
 ECC_DEV void to_mont(uint32_t* r, const uint32_t* a) {

@@ -65,14 +65,9 @@ cudaError_t launch_point_add_custom(const CustomConsts& cc, size_t n, const uint
                                     const uint32_t* q, uint32_t* out, int dbl, cudaStream_t st);
 // ok[i] = 1 when point i is O ((0, 0)) or canonical and on the curve (Eqn 1)
 cudaError_t launch_validate_points(int curve, size_t n, const uint32_t* p, uint8_t* ok, cudaStream_t st);
-// Fixed-base table of a curve on the current device (built on first use,
-// synchronously on `st`): 32 x 256 entries, entry j*256+v = v 2^(8j) G, SoA
-// Montgomery (x block then y block).
-cudaError_t gtable(int curve, const uint4** table, cudaStream_t st);
-
-// ECDSA verification in clusters of `ctas` (1 or 2) CTAs sharing each round's
-// inversion
-void set_gas_cluster(int ctas);
+// Generator table of a curve on the current device (ladder.cuh; built on first
+// use, synchronously on `st`).
+cudaError_t gtable(int curve, const uint32_t** table, cudaStream_t st);
 
 // FPMUL k_i G (scalars n x 8 LE limbs; out n x 2N LE limbs)
 cudaError_t launch_fixed_base_mul(int curve, size_t n, const uint32_t* k, uint32_t* out,

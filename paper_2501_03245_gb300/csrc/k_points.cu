@@ -1,9 +1,10 @@
 // EC-operator launchers: batched affine PADD / PDBL on caller arrays, and the
-// per-device fixed-base table v 2^(8j) G (FPMUL precomputation, Section 2.1.1).
+// per-device generator table v 2^(16 j) G (FPMUL precomputation, Section 2.1.1).
+#include <algorithm>
 #include <mutex>
-#include <vector>
 
 #include "internal.h"
+#include "ladder.cuh"
 #include "ops.cuh"
 
 namespace ecc {
@@ -15,20 +16,6 @@ __global__ void k_fill_ops(PointOp* ops, size_t n, uint32_t dst0, uint32_t a0, u
   size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   ops[i] = PointOp{dst0 + (uint32_t)i, a0 + (uint32_t)i, b0 + (uint32_t)(i * b_step)};
-}
-
-template <class C>
-__global__ void k_set_generator(PtSoA<typename C::Fp> pool, uint32_t slot) {
-  using F = typename C::Fp;
-  uint32_t x[F::N], y[F::N];
-#pragma unroll
-  for (int k = 0; k < F::N; ++k) {
-    x[k] = C::gx(k);
-    y[k] = C::gy(k);
-  }
-  to_mont<F>(x, x);
-  to_mont<F>(y, y);
-  pool.store(slot, x, y);
 }
 
 // Runs ops[0 .. n_ops) as one batched round on `pool`.
@@ -84,71 +71,124 @@ cudaError_t point_add(size_t n, const uint32_t* p, const uint32_t* q, uint32_t* 
 
 // --------------------------------------------------------------- G table
 
-constexpr size_t kTabEntries = 32 * 256;
+// Entries (j, 1) = 2^(16 j) G of a generator table: one thread's chain of
+// doublings, then one lane per row makes its point affine.
+template <class C>
+__global__ void k_gtable_rows(uint32_t* tab) {
+  using F = typename C::Fp;
+  constexpr int N = F::N;
+  __shared__ uint32_t row[kGRows][3 * N];
+  if (threadIdx.x == 0) {
+    uint32_t X[N], Y[N], Z[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      X[k] = C::gx(k);
+      Y[k] = C::gy(k);
+    }
+    to_mont<F>(X, X);
+    to_mont<F>(Y, Y);
+    fe_set_one<F>(Z);
+#pragma unroll 1
+    for (int s = 0; s < kGWin * kGRows; ++s) {
+      if (s % kGWin == 0) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+          row[s / kGWin][k] = X[k];
+          row[s / kGWin][N + k] = Y[k];
+          row[s / kGWin][2 * N + k] = Z[k];
+        }
+      }
+      jac_dbl_half<C>(X, Y, Z);
+    }
+  }
+  __syncwarp();
+  if (threadIdx.x < kGRows) {
+    uint32_t X[N], Y[N], Z[N], t[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      X[k] = row[threadIdx.x][k];
+      Y[k] = row[threadIdx.x][N + k];
+      Z[k] = row[threadIdx.x][2 * N + k];
+    }
+    fe_inv_regs<F>(Z, Z);
+    mont_sqr<F>(t, Z);
+    mont_mul<F>(X, X, t);
+    mont_mul<F>(t, t, Z);
+    mont_mul<F>(Y, Y, t);
+    store_affine<F>(tab, (size_t)threadIdx.x * kGEntries, X, Y);
+  }
+}
+
+// Entries (j, 2^k + u) = (j, 2^k) + (j, u) of every row, u = 1 .. 2^k (the last a
+// doubling): a thread does `per` consecutive u with one inversion (Montgomery's
+// trick).  All operands are distinct multiples below the group order, so no sum
+// is exceptional but the doubling.
+constexpr int kGFill = 8;
 
 template <class C>
-cudaError_t build_gtable(uint4** out, cudaStream_t st) {
+__global__ void __launch_bounds__(128) k_gtable_fill(uint32_t* tab, int k, int per) {
   using F = typename C::Fp;
-  const size_t soa = soa_bytes<F>(kTabEntries);
-  uint4* tab = nullptr;
-  cudaError_t e = cudaMalloc(&tab, 2 * soa);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(tab, 0, 2 * soa, st);
-  if (e != cudaSuccess) return e;
-  PtSoA<F> pool{SoA<F>{tab, kTabEntries}, SoA<F>{tab + soa / 16, kTabEntries}};
-  // op list: the power-of-two chain (one op per launch), then 7 fill rounds
-  std::vector<PointOp> ops;
-  std::vector<std::pair<size_t, size_t>> launches;  // (offset, count)
-  for (uint32_t j = 0; j < 32; ++j) {
-    for (uint32_t k = 1; k < 8; ++k) {
-      launches.push_back({ops.size(), 1});
-      ops.push_back(PointOp{j * 256 + (1u << k), j * 256 + (1u << (k - 1)), j * 256 + (1u << (k - 1))});
-    }
-    if (j < 31) {
-      launches.push_back({ops.size(), 1});
-      ops.push_back(PointOp{(j + 1) * 256 + 1, j * 256 + 128, j * 256 + 128});
-    }
+  constexpr int N = F::N;
+  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t per_row = (1u << k) / per;
+  if (t >= kGRows * per_row) return;
+  const size_t base = (size_t)(t / per_row) * kGEntries;
+  const uint32_t u0 = 1 + (t % per_row) * per;
+  uint32_t xa[N], ya[N], xb[N], yb[N], run[N], d[N], pre[kGFill][N];
+  load_affine<F>(tab, base + (1u << k) - 1, xa, ya);
+  fe_set_one<F>(run);
+  for (int q = 0; q < per; ++q) {
+    load_affine<F>(tab, base + u0 + q - 1, xb, yb);
+    add_den<C>(d, xa, ya, xb, yb);
+    fe_copy<F>(pre[q], run);
+    mont_mul<F>(run, run, d);
   }
-  for (uint32_t k = 1; k < 8; ++k) {
-    size_t off = ops.size();
-    for (uint32_t j = 0; j < 32; ++j)
-      for (uint32_t u = 1; u < (1u << k); ++u)
-        ops.push_back(PointOp{j * 256 + (1u << k) + u, j * 256 + (1u << k), j * 256 + u});
-    launches.push_back({off, ops.size() - off});
+  fe_inv_regs<F>(run, run);
+  for (int q = per - 1; q >= 0; --q) {
+    uint32_t inv[N];
+    load_affine<F>(tab, base + u0 + q - 1, xb, yb);
+    const int kind = add_den<C>(d, xa, ya, xb, yb);
+    mont_mul<F>(inv, run, pre[q]);
+    mont_mul<F>(run, run, d);
+    add_finish<C>(xb, yb, kind, inv, xa, ya, xb, yb);
+    store_affine<F>(tab, base + (1u << k) + u0 + q - 1, xb, yb);
   }
-  Scratch ws_ops, ws_m;
-  e = ws_ops.alloc(ops.size() * sizeof(PointOp), st);
+}
+
+template <class C>
+cudaError_t build_gtable(uint32_t** out, cudaStream_t st) {
+  uint32_t* tab = nullptr;
+  cudaError_t e = cudaMalloc(&tab, (size_t)kGRows * kGEntries * 2 * C::Fp::N * 4);
   if (e != cudaSuccess) return e;
-  e = ws_m.alloc(soa_bytes<F>(kTabEntries), st);
-  if (e != cudaSuccess) return e;
-  PointOp* dops = ws_ops.as<PointOp>();
-  SoA<F> M{ws_m.as<uint4>(), kTabEntries};
-  e = cudaMemcpyAsync(dops, ops.data(), ops.size() * sizeof(PointOp), cudaMemcpyHostToDevice, st);
-  if (e != cudaSuccess) return e;
-  k_set_generator<C><<<1, 1, 0, st>>>(pool, 1);
-  for (auto& l : launches) {
-    e = run_ops<C>(pool, dops + l.first, l.second, M, st);
-    if (e != cudaSuccess) return e;
+  k_gtable_rows<C><<<1, 32, 0, st>>>(tab);
+  for (int k = 0; k + 1 < kGWin; ++k) {
+    const int per = std::min(1 << k, kGFill);
+    const unsigned threads = (unsigned)kGRows * ((1u << k) / per);
+    k_gtable_fill<C><<<(threads + 127) / 128, 128, 0, st>>>(tab, k, per);
   }
-  e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) return e;
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) {
+    cudaFree(tab);
+    return e;
+  }
   *out = tab;
   return cudaSuccess;
 }
 
 std::mutex g_tab_mu;
-uint4* g_tabs[64][5] = {};
+uint32_t* g_tabs[64][5] = {};
 
 }  // namespace
 
-cudaError_t gtable(int curve, const uint4** table, cudaStream_t st) {
+cudaError_t gtable(int curve, const uint32_t** table, cudaStream_t st) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64 || curve < 0 || curve > 4) return cudaErrorInvalidValue;
   std::lock_guard<std::mutex> lock(g_tab_mu);
   if (!g_tabs[dev][curve]) {
-    uint4* t = nullptr;
+    uint32_t* t = nullptr;
     switch (curve) {
       case 0: e = build_gtable<Secp256k1>(&t, st); break;
       case 1: e = build_gtable<P256>(&t, st); break;

@@ -1,6 +1,8 @@
 // Host launcher of the batched ECDSA verification kernel, included by one
-// translation unit per (curve, variant) so the library builds in parallel.
+// translation unit per curve so the library builds in parallel.
 #pragma once
+#include <algorithm>
+
 #include "internal.h"
 #include "verify.cuh"
 
@@ -8,25 +10,22 @@ namespace ecc {
 
 namespace verify_detail {
 
-constexpr int kVerifyBlock = kGasThreads;
-
-template <class C, int CL>
+template <class C>
 cudaError_t verify(size_t n, const uint8_t* hash, const uint8_t* r, const uint8_t* s,
                    const uint8_t* pub, uint8_t* ok, cudaStream_t st, int curve) {
   using Fp = typename C::Fp;
-  using Fn = typename C::Fn;
-  constexpr int B = kVerifyBlock;
-  const uint4* tg = nullptr;
+  const uint32_t* tg = nullptr;
   cudaError_t e = gtable(curve, &tg, st);
   if (e != cudaSuccess) return e;
-  // workspace: S, E, Rn (Fn) | TQ x,y (kQTable n each) | AQ, AG | M | D2 | U1B | status
-  const size_t fe = soa_bytes<Fp>(n);
-  const size_t bytes = 3 * fe + 2 * kQTable * fe + 4 * fe + fe + (kQDigits + 32 + 1) * n + 256;
+  size_t ctas = (n + kLadderThreads - 1) / kLadderThreads;
+  ctas = std::min<size_t>(ctas, (size_t)device_sm_count() * kLadderCtasPerSm);
+  const size_t slots = ctas * kLadderThreads;
+  // per slot: table (affine points), H, recoded u1 and u2 (9 words each), r
+  const size_t table = slots * kQTable * 2 * Fp::N * 4, h = soa_bytes<Fp>(slots * kQTable);
   Scratch ws;
-  e = ws.alloc(bytes, st);
+  e = ws.alloc(table + h + (9 + 9 + 8) * 4 * slots, st);
   if (e != cudaSuccess) return e;
-  uint4* v = ws.as<uint4>();
-  const size_t q = fe / 16;  // uint4 per SoA array of n elements
+  uint8_t* p = ws.as<uint8_t>();
   VerifyArgs<C> a;
   a.n = n;
   a.hash = reinterpret_cast<const uint32_t*>(hash);
@@ -34,48 +33,15 @@ cudaError_t verify(size_t n, const uint8_t* hash, const uint8_t* r, const uint8_
   a.s = reinterpret_cast<const uint32_t*>(s);
   a.pub = reinterpret_cast<const uint32_t*>(pub);
   a.ok = ok;
-  a.S = SoA<Fn>{v + 0 * q, n};
-  a.E = SoA<Fn>{v + 1 * q, n};
-  a.Rn = SoA<Fn>{v + 2 * q, n};
-  const size_t T = kQTable;
-  a.TQ = PtSoA<Fp>{SoA<Fp>{v + 3 * q, T * n}, SoA<Fp>{v + (3 + T) * q, T * n}};
-  a.AQ = PtSoA<Fp>{SoA<Fp>{v + (3 + 2 * T) * q, n}, SoA<Fp>{v + (4 + 2 * T) * q, n}};
-  a.AG = PtSoA<Fp>{SoA<Fp>{v + (5 + 2 * T) * q, n}, SoA<Fp>{v + (6 + 2 * T) * q, n}};
-  a.M = SoA<Fp>{v + (7 + 2 * T) * q, n};
-  uint8_t* tail = reinterpret_cast<uint8_t*>(v + (8 + 2 * T) * q);
-  a.D2 = reinterpret_cast<int8_t*>(tail);
-  a.U1B = tail + kQDigits * n;
-  a.status = tail + (kQDigits + 32) * n;
-  const size_t te = 32 * 256;
-  a.TG = PtSoA<Fp>{SoA<Fp>{const_cast<uint4*>(tg), te}, SoA<Fp>{const_cast<uint4*>(tg) + soa_bytes<Fp>(te) / 16, te}};
-  size_t ctas = (size_t)device_sm_count() * kGasCtasPerSm;
-  size_t per = (n + ctas - 1) / ctas;
-  if (per < 32) per = 32;
-  ctas = (n + per - 1) / per;
-  a.per_cta = per;
-  const size_t smem = sizeof(GasSmem<Fp::N, B>);
-  e = cudaFuncSetAttribute(k_verify<C, B, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  if constexpr (CL > 1) {
-    // clusters of CL CTAs sharing each round's inversion (a grid of whole
-    // clusters; a CTA past the batch runs the rounds on an empty slice)
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((ctas + CL - 1) / CL * CL));
-    cfg.blockDim = dim3(B);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = CL;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_verify<C, B, CL>, a);
-  } else {
-    k_verify<C, B><<<(unsigned)ctas, B, smem, st>>>(a);
-    return cudaGetLastError();
-  }
+  a.table = reinterpret_cast<uint32_t*>(p);
+  a.H = SoA<Fp>{reinterpret_cast<uint4*>(p + table), slots * kQTable};
+  a.u1 = reinterpret_cast<uint32_t*>(p + table + h);
+  a.u2 = a.u1 + 9 * slots;
+  a.rr = a.u2 + 9 * slots;
+  a.TG = tg;
+  a.slots = slots;
+  k_verify<C><<<(unsigned)ctas, kLadderThreads, 0, st>>>(a);
+  return cudaGetLastError();
 }
 
 }  // namespace verify_detail
