@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_fpmul(Fixe
     }
   }
   uint32_t zi[N], t[N];
-  fe_inv_regs<F>(zi, Z);  // 0 for O, which gives (0, 0)
+  fe_inv_mont<F>(zi, Z);  // 0 for O, which gives (0, 0)
   mont_sqr<F>(t, zi);
   mont_mul<F>(X, X, t);
   mont_mul<F>(t, t, zi);
@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_sign(Fixed
   // 0 < k, d < n: neither result is O.  1 / Z and 1 / Kz from one inversion
   uint32_t zi[N], t[N];
   mont_mul<F>(t, Z, Kz);
-  fe_inv_regs<F>(t, t);
+  fe_inv_mont<F>(t, t);
   mont_mul<F>(zi, t, Kz);
   mont_mul<F>(Kz, t, Z);
   mont_sqr<F>(t, zi);
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_sign(Fixed
   fe_add<Fn>(s, s, w);
   scalar(a.k, v);
   to_mont<Fn>(v, v);
-  fe_inv_regs<Fn>(v, v);
+  fe_inv_mont<Fn>(v, v);
   mont_mul<Fn>(s, v, s);  // (k^-1 R) (e + r d) R^-1
   const bool good = valid && !is_zero256(r) && !is_zero256(s);
   if (!good) {

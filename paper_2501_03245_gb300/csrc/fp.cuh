@@ -624,24 +624,38 @@ __device__ __noinline__ void fe_inv_fermat(uint32_t* r, const uint32_t* a) {
   fe_copy<F>(r, acc);
 }
 
-// r = a^-1 in Montgomery form (a = x R -> r = x^-1 R), a = 0 gives 0, by the
-// divstep inversion of inv.cuh on 30-bit limbs with branch-free single
-// divsteps: (x R)^-1 is computed on the integer, then one Montgomery product
-// with R^3 mod q restores the form.  Out of line: it runs on one thread per
-// batch, where its latency is the serial step of every batched round (GB300,
-// one thread, 256-bit field: 22.8 us, against 27.7 us with batched variable-
-// time divsteps on 30-bit limbs and 32.6 us on 62-bit limbs).
+// a^-1 mod q as an integer, 0 for 0, by the divstep inversion of inv.cuh on 30-bit
+// limbs with branch-free divsteps.  Out of line, operand and result in registers:
+// it is the serial step of every batched round.
 template <class F, bool FLAT = true>
-__device__ __noinline__ void fe_inv_mont(uint32_t* r, const uint32_t* a) {
+__device__ __noinline__ Fe<F> fe_inv_call(Fe<F> a) {
   constexpr int N = F::N;
   constexpr int L = (32 * N + 2 + 29) / 30;
-  uint32_t q[N], x[N], r3[N];
+  uint32_t q[N], x[N];
 #pragma unroll
-  for (int i = 0; i < N; ++i) {
-    q[i] = F::p(i);
-    r3[i] = F::r3(i);
-  }
-  inv_divsteps30<L, FLAT>(x, a, q, N, (uint32_t)F::qinv62() & (uint32_t)kM30);
+  for (int i = 0; i < N; ++i) q[i] = F::p(i);
+  inv_divsteps30<L, N, FLAT>(x, a.v, q, (uint32_t)F::qinv62() & (uint32_t)kM30);
+  fe_copy<F>(a.v, x);
+  return a;
+}
+
+template <class F, bool FLAT = true>
+ECC_DEV void fe_inv_int(uint32_t* r, const uint32_t* a) {
+  Fe<F> x;
+  fe_copy<F>(x.v, a);
+  x = fe_inv_call<F, FLAT>(x);
+  fe_copy<F>(r, x.v);
+}
+
+// r = a^-1 in Montgomery form (a = x R -> r = x^-1 R), a = 0 gives 0: (x R)^-1 on
+// the integer, then one Montgomery product with R^3 mod q restores the form.
+template <class F, bool FLAT = true>
+ECC_DEV void fe_inv_mont(uint32_t* r, const uint32_t* a) {
+  constexpr int N = F::N;
+  uint32_t x[N], r3[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) r3[i] = F::r3(i);
+  fe_inv_int<F, FLAT>(x, a);
   mont_mul<F>(r, x, r3);
 }
 

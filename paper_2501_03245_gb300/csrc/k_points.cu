@@ -110,7 +110,7 @@ __global__ void k_gtable_rows(uint32_t* tab) {
       Y[k] = row[threadIdx.x][N + k];
       Z[k] = row[threadIdx.x][2 * N + k];
     }
-    fe_inv_regs<F>(Z, Z);
+    fe_inv_mont<F>(Z, Z);
     mont_sqr<F>(t, Z);
     mont_mul<F>(X, X, t);
     mont_mul<F>(t, t, Z);
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(128) k_gtable_fill(uint32_t* tab, int k, int p
     fe_copy<F>(pre[q], run);
     mont_mul<F>(run, run, d);
   }
-  fe_inv_regs<F>(run, run);
+  fe_inv_mont<F>(run, run);
   for (int q = per - 1; q >= 0; --q) {
     uint32_t inv[N];
     load_affine<F>(tab, base + u0 + q - 1, xb, yb);

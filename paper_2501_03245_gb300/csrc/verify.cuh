@@ -114,7 +114,7 @@ ECC_DEV bool verify_prep(const VerifyArgs<C>& a, size_t i, size_t slot) {
     store_affine<Fp>(a.table, slot * kQTable, qx, qy);
   }
   to_mont<Fn>(s, s);
-  fe_inv_regs<Fn>(w, s);  // w R
+  fe_inv_mont<Fn>(w, s);  // w R
   // one operand in Montgomery form gives the plain product: (w R) r R^-1 = w r
   uint32_t u[9];
 #pragma unroll
@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_verify(Ver
       } else if (it < kChain + kQDigits) {
         const int w = kChain + kQDigits - 1 - it;
         if (it == kChain) {
-          fe_inv_regs<F>(x, Z);
+          fe_inv_mont<F>(x, Z);
           verify_table_affine<C>(a, slot, x);
           fe_set_zero<F>(Z);
         } else {
