@@ -7,7 +7,7 @@
 // parameter, and copied into shared memory by every CTA before any arithmetic.
 // The traits classes below read them from there, so one compiled copy of the
 // field layer, the per-CTA gather-apply-scatter inversion and the batched
-// PADD / PDBL rounds serves every such curve, and calls on different streams
+// PADD / PDBL kernel serves every such curve, and calls on different streams
 // with different curves do not interfere.  The compiled curves keep their
 // constants in the instruction stream (curves_gen.cuh); this path exists for
 // curves the library was not built with, tiny test curves among them.
@@ -50,48 +50,42 @@ ECC_DEV void custom_enter(const CustomConsts& cc) {
   __syncthreads();
 }
 
-__global__ void k_custom_in(CustomConsts cc, const uint32_t* __restrict__ aos, size_t n,
-                            size_t row_stride, size_t col, SoA<CustomFp> out) {
-  custom_enter(cc);
-  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  uint32_t v[8];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) v[k] = aos[i * row_stride + col + k];
-  to_mont<CustomFp>(v, v);
-  out.store(i, v);
-}
-
-__global__ void k_custom_out(CustomConsts cc, SoA<CustomFp> in, size_t n, uint32_t* __restrict__ aos,
-                             size_t row_stride, size_t col) {
-  custom_enter(cc);
-  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  uint32_t v[8];
-  in.load(i, v);
-  from_mont<CustomFp>(v, v);
-#pragma unroll
-  for (int k = 0; k < 8; ++k) aos[i * row_stride + col + k] = v[k];
-}
-
-__global__ void k_custom_fill(PointOp* ops, size_t n, uint32_t dst0, uint32_t b0) {
-  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  ops[i] = PointOp{dst0 + (uint32_t)i, (uint32_t)i, b0 + (uint32_t)i};
-}
-
-// One batched round of independent point operations (the body of k_point_ops).
-template <int BLOCK>
+template <bool DBL, int BLOCK>
 __global__ void __launch_bounds__(BLOCK, kGasResidentThreads / BLOCK)
-    k_custom_point_ops(CustomConsts cc, PtSoA<CustomFp> pool, const PointOp* ops, size_t n_ops,
-                       SoA<CustomFp> M, size_t per_cta) {
+    k_custom_point_ops(CustomConsts cc, const uint32_t* p, const uint32_t* q, uint32_t* out, SoA<CustomFp> M,
+                       size_t n, int vec) {
   custom_enter(cc);
-  auto& sm = gas_smem<8, BLOCK>();
-  const size_t begin = blockIdx.x * per_cta;
-  size_t end = begin + per_cta < n_ops ? begin + per_cta : n_ops;
-  if (end < begin) end = begin;
-  OpRound<CustomCurve> rd{pool, ops};
-  batch_round<CustomFp, BLOCK>(rd, begin, end, M, sm);
+  point_ops<CustomCurve, DBL, BLOCK>(p, q, out, M, n, vec);
+}
+
+template <bool DBL>
+cudaError_t custom_ops(const CustomConsts& cc, size_t n, const uint32_t* p, const uint32_t* q, uint32_t* out,
+                       cudaStream_t st) {
+  using F = CustomFp;
+  constexpr int B = kGasThreads;
+  const size_t rows = n * 64;
+  const bool cp = shifted_overlap(p, out, rows), cq = !DBL && shifted_overlap(q, out, rows);
+  Scratch ws;
+  cudaError_t e = ws.alloc(soa_bytes<F>(n) + (cp ? rows : 0) + (cq ? rows : 0), st);
+  if (e != cudaSuccess) return e;
+  uint32_t* copy = ws.as<uint32_t>() + soa_bytes<F>(n) / 4;
+  if (cp) {
+    e = cudaMemcpyAsync(copy, p, rows, cudaMemcpyDeviceToDevice, st);
+    if (e != cudaSuccess) return e;
+    p = copy;
+    copy += rows / 4;
+  }
+  if (cq) {
+    e = cudaMemcpyAsync(copy, q, rows, cudaMemcpyDeviceToDevice, st);
+    if (e != cudaSuccess) return e;
+    q = copy;
+  }
+  const size_t smem = sizeof(GasSmem<8, B>);
+  e = cudaFuncSetAttribute(k_custom_point_ops<DBL, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_custom_point_ops<DBL, B><<<row_ctas(n), B, smem, st>>>(cc, p, q, out, SoA<F>{ws.as<uint4>(), n}, n,
+                                                           aligned16(p, DBL ? p : q, out));
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- host side
@@ -176,39 +170,7 @@ int custom_consts(const uint32_t* p, const uint32_t* a, CustomConsts* cc) {
 
 cudaError_t launch_point_add_custom(const CustomConsts& cc, size_t n, const uint32_t* p,
                                     const uint32_t* q, uint32_t* out, int dbl, cudaStream_t st) {
-  using F = CustomFp;
-  constexpr int B = kBlock;
-  const size_t slots = dbl ? 2 * n : 3 * n;
-  Scratch ws;
-  const size_t soa = soa_bytes<F>(slots);
-  cudaError_t e = ws.alloc(2 * soa + soa_bytes<F>(n) + n * sizeof(PointOp) + 64, st);
-  if (e != cudaSuccess) return e;
-  uint4* base = ws.as<uint4>();
-  PtSoA<F> pool{SoA<F>{base, slots}, SoA<F>{base + soa / 16, slots}};
-  SoA<F> M{base + 2 * soa / 16, n};
-  PointOp* ops = reinterpret_cast<PointOp*>(base + (2 * soa + soa_bytes<F>(n)) / 16);
-  const unsigned cb = (unsigned)((n + 255) / 256);
-  k_custom_in<<<cb, 256, 0, st>>>(cc, p, n, 16, 0, pool.x);
-  k_custom_in<<<cb, 256, 0, st>>>(cc, p, n, 16, 8, pool.y);
-  if (!dbl) {
-    k_custom_in<<<cb, 256, 0, st>>>(cc, q, n, 16, 0, pool.x.at(n));
-    k_custom_in<<<cb, 256, 0, st>>>(cc, q, n, 16, 8, pool.y.at(n));
-    k_custom_fill<<<cb, 256, 0, st>>>(ops, n, (uint32_t)(2 * n), (uint32_t)n);
-  } else {
-    k_custom_fill<<<cb, 256, 0, st>>>(ops, n, (uint32_t)n, 0);
-  }
-  size_t ctas = (size_t)device_sm_count() * kGasCtasPerSm;
-  size_t per = (n + ctas - 1) / ctas;
-  if (per < B) per = B;
-  ctas = (n + per - 1) / per;
-  const size_t smem = sizeof(GasSmem<8, B>);
-  e = cudaFuncSetAttribute(k_custom_point_ops<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  k_custom_point_ops<B><<<(unsigned)ctas, B, smem, st>>>(cc, pool, ops, n, M, per);
-  const size_t o = dbl ? n : 2 * n;
-  k_custom_out<<<cb, 256, 0, st>>>(cc, pool.x.at(o), n, out, 16, 0);
-  k_custom_out<<<cb, 256, 0, st>>>(cc, pool.y.at(o), n, out, 16, 8);
-  return cudaGetLastError();
+  return dbl ? custom_ops<true>(cc, n, p, q, out, st) : custom_ops<false>(cc, n, p, q, out, st);
 }
 
 }  // namespace ecc

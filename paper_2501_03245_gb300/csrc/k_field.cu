@@ -40,39 +40,49 @@ cudaError_t noalloc_scratch(void** ptr) {
 template <class F>
 cudaError_t fe_ops(int op, size_t n, const uint32_t* a, const uint32_t* b, uint32_t* out,
                    cudaStream_t st) {
-  const int threads = 256;
+  const int threads = 256, vec = aligned16(a, b, out);
   const unsigned blocks = (unsigned)((n + threads - 1) / threads);
   switch (op) {
-    case 0: k_fe_mul<F><<<blocks, threads, 0, st>>>(a, b, out, n); break;
-    case 1: k_fe_addsub<F><<<blocks, threads, 0, st>>>(a, b, out, n, 0); break;
-    case 2: k_fe_addsub<F><<<blocks, threads, 0, st>>>(a, b, out, n, 1); break;
-    case 3: k_fe_inv_single<F><<<blocks, threads, 0, st>>>(a, out, n); break;
+    case 0: k_fe_mul<F><<<blocks, threads, 0, st>>>(a, b, out, n, vec); break;
+    case 1: k_fe_addsub<F><<<blocks, threads, 0, st>>>(a, b, out, n, 0, vec); break;
+    case 2: k_fe_addsub<F><<<blocks, threads, 0, st>>>(a, b, out, n, 1, vec); break;
+    case 3: {
+      // four resident CTAs of 128 threads per SM; fewer elements than threads
+      // take one inversion each
+      const size_t ctas = std::min<size_t>((n + 127) / 128, (size_t)device_sm_count() * 4);
+      k_fe_inv<F><<<(unsigned)ctas, 128, 0, st>>>(a, out, n, vec);
+      break;
+    }
   }
+  return cudaGetLastError();
+}
+
+// M: prefix products of n elements
+template <class F>
+cudaError_t run_inv_batch(size_t n, const uint32_t* a, uint32_t* out, uint4* M, cudaStream_t st) {
+  constexpr int B = kGasThreads;
+  const size_t smem = sizeof(GasSmem<F::N, B>);
+  cudaError_t e = cudaFuncSetAttribute(k_batch_inverse<F, B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem);
+  if (e != cudaSuccess) return e;
+  k_batch_inverse<F, B><<<row_ctas(n), B, smem, st>>>(a, out, SoA<F>{M, n}, n, aligned16(a, out));
   return cudaGetLastError();
 }
 
 template <class F>
 cudaError_t fe_inv_batch(size_t n, const uint32_t* a, uint32_t* out, cudaStream_t st) {
-  constexpr int B = kBlock;
   Scratch ws;
-  const size_t soa = soa_bytes<F>(n);
-  cudaError_t e = ws.alloc(3 * soa, st);
+  const size_t bytes = soa_bytes<F>(n);
+  const bool copy = shifted_overlap(a, out, bytes);
+  cudaError_t e = ws.alloc((copy ? 2 : 1) * bytes, st);
   if (e != cudaSuccess) return e;
-  SoA<F> in{ws.as<uint4>(), n}, res{ws.as<uint4>() + soa / 16, n}, M{ws.as<uint4>() + 2 * soa / 16, n};
-  const unsigned cb = (unsigned)((n + 255) / 256);
-  k_fe_in<F><<<cb, 256, 0, st>>>(a, n, F::N, 0, in, 1);
-  // one CTA per (SM x 2) slice, at least a full thread row per CTA
-  size_t ctas = (size_t)device_sm_count() * kGasCtasPerSm;
-  size_t per = (n + ctas - 1) / ctas;
-  if (per < B) per = B;
-  ctas = (n + per - 1) / per;
-  const size_t smem = sizeof(GasSmem<F::N, B>);
-  e = cudaFuncSetAttribute(k_batch_inverse<F, B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem);
-  if (e != cudaSuccess) return e;
-  k_batch_inverse<F, B><<<(unsigned)ctas, B, smem, st>>>(in, res, M, n, per);
-  k_fe_out<F><<<cb, 256, 0, st>>>(res, n, out, F::N, 0, 1);
-  return cudaGetLastError();
+  if (copy) {
+    uint32_t* in = ws.as<uint32_t>() + bytes / 4;
+    e = cudaMemcpyAsync(in, a, bytes, cudaMemcpyDeviceToDevice, st);
+    if (e != cudaSuccess) return e;
+    a = in;
+  }
+  return run_inv_batch<F>(n, a, out, ws.as<uint4>(), st);
 }
 
 template <class F>
@@ -99,29 +109,20 @@ __global__ void k_bench_modmul(int iters, uint32_t* sink) {
   sink[t] = acc;
 }
 
-// Batch inversion into caller-free scratch: the same three kernels as
-// fe_inv_batch, with the in / out / prefix arrays carved from the file-scope
-// device array below instead of a stream-ordered allocation.
+// Batch inversion into caller-free scratch: the same kernel as fe_inv_batch, with
+// the prefix products (and a copy of an input that overlaps the output) in the
+// file-scope device array instead of a stream-ordered allocation.
 template <class F>
 cudaError_t fe_inv_batch_noalloc(void* scratch, size_t n, const uint32_t* a, uint32_t* out,
                                  cudaStream_t st) {
-  constexpr int B = kBlock;
-  const size_t soa = soa_bytes<F>(n);
-  uint4* base = static_cast<uint4*>(scratch);
-  SoA<F> in{base, n}, res{base + soa / 16, n}, M{base + 2 * soa / 16, n};
-  const unsigned cb = (unsigned)((n + 255) / 256);
-  k_fe_in<F><<<cb, 256, 0, st>>>(a, n, F::N, 0, in, 1);
-  size_t ctas = (size_t)device_sm_count() * kGasCtasPerSm;
-  size_t per = (n + ctas - 1) / ctas;
-  if (per < B) per = B;
-  ctas = (n + per - 1) / per;
-  const size_t smem = sizeof(GasSmem<F::N, B>);
-  cudaError_t e = cudaFuncSetAttribute(k_batch_inverse<F, B>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  k_batch_inverse<F, B><<<(unsigned)ctas, B, smem, st>>>(in, res, M, n, per);
-  k_fe_out<F><<<cb, 256, 0, st>>>(res, n, out, F::N, 0, 1);
-  return cudaGetLastError();
+  const size_t bytes = soa_bytes<F>(n);
+  if (shifted_overlap(a, out, bytes)) {
+    uint32_t* in = static_cast<uint32_t*>(scratch) + bytes / 4;
+    cudaError_t e = cudaMemcpyAsync(in, a, bytes, cudaMemcpyDeviceToDevice, st);
+    if (e != cudaSuccess) return e;
+    a = in;
+  }
+  return run_inv_batch<F>(n, a, out, static_cast<uint4*>(scratch), st);
 }
 
 // a chain of `iters` dependent inversions per thread: method 0 Fermat, 1 divsteps

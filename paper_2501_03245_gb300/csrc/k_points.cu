@@ -11,62 +11,39 @@ namespace ecc {
 
 namespace {
 
-__global__ void k_fill_ops(PointOp* ops, size_t n, uint32_t dst0, uint32_t a0, uint32_t b0,
-                           uint32_t b_step) {
-  size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  ops[i] = PointOp{dst0 + (uint32_t)i, a0 + (uint32_t)i, b0 + (uint32_t)(i * b_step)};
-}
-
-// Runs ops[0 .. n_ops) as one batched round on `pool`.
-template <class C>
-cudaError_t run_ops(PtSoA<typename C::Fp> pool, const PointOp* ops, size_t n_ops,
-                    SoA<typename C::Fp> M, cudaStream_t st) {
-  constexpr int B = kBlock;
+template <class C, bool DBL>
+cudaError_t point_add(size_t n, const uint32_t* p, const uint32_t* q, uint32_t* out, cudaStream_t st) {
   using F = typename C::Fp;
-  if (n_ops == 0) return cudaSuccess;
-  size_t ctas = (size_t)device_sm_count() * kGasCtasPerSm;
-  size_t per = (n_ops + ctas - 1) / ctas;
-  if (per < B) per = B;
-  ctas = (n_ops + per - 1) / per;
-  const size_t smem = sizeof(GasSmem<F::N, B>);
-  cudaError_t e = cudaFuncSetAttribute(k_point_ops<C, B>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr int N = F::N, B = kGasThreads;
+  const size_t rows = n * 2 * N * 4;
+  const bool cp = shifted_overlap(p, out, rows), cq = !DBL && shifted_overlap(q, out, rows);
+  Scratch ws;
+  cudaError_t e = ws.alloc(soa_bytes<F>(n) + (cp ? rows : 0) + (cq ? rows : 0), st);
   if (e != cudaSuccess) return e;
-  k_point_ops<C, B><<<(unsigned)ctas, B, smem, st>>>(pool, ops, n_ops, M, per);
+  uint32_t* copy = ws.as<uint32_t>() + soa_bytes<F>(n) / 4;
+  if (cp) {
+    e = cudaMemcpyAsync(copy, p, rows, cudaMemcpyDeviceToDevice, st);
+    if (e != cudaSuccess) return e;
+    p = copy;
+    copy += rows / 4;
+  }
+  if (cq) {
+    e = cudaMemcpyAsync(copy, q, rows, cudaMemcpyDeviceToDevice, st);
+    if (e != cudaSuccess) return e;
+    q = copy;
+  }
+  const size_t smem = sizeof(GasSmem<N, B>);
+  e = cudaFuncSetAttribute(k_point_ops<C, DBL, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_point_ops<C, DBL, B><<<row_ctas(n), B, smem, st>>>(p, q, out, SoA<F>{ws.as<uint4>(), n}, n,
+                                                       aligned16(p, DBL ? p : q, out));
   return cudaGetLastError();
 }
 
 template <class C>
 cudaError_t point_add(size_t n, const uint32_t* p, const uint32_t* q, uint32_t* out, int dbl,
                       cudaStream_t st) {
-  using F = typename C::Fp;
-  constexpr int N = F::N;
-  const size_t slots = dbl ? 2 * n : 3 * n;
-  Scratch ws;
-  const size_t soa = soa_bytes<F>(slots);
-  cudaError_t e = ws.alloc(2 * soa + soa_bytes<F>(n) + n * sizeof(PointOp) + 64, st);
-  if (e != cudaSuccess) return e;
-  uint4* base = ws.as<uint4>();
-  PtSoA<F> pool{SoA<F>{base, slots}, SoA<F>{base + soa / 16, slots}};
-  SoA<F> M{base + 2 * soa / 16, n};
-  PointOp* ops = reinterpret_cast<PointOp*>(base + (2 * soa + soa_bytes<F>(n)) / 16);
-  const unsigned cb = (unsigned)((n + 255) / 256);
-  k_fe_in<F><<<cb, 256, 0, st>>>(p, n, 2 * N, 0, pool.x, 1);
-  k_fe_in<F><<<cb, 256, 0, st>>>(p, n, 2 * N, N, pool.y, 1);
-  if (!dbl) {
-    k_fe_in<F><<<cb, 256, 0, st>>>(q, n, 2 * N, 0, pool.x.at(n), 1);
-    k_fe_in<F><<<cb, 256, 0, st>>>(q, n, 2 * N, N, pool.y.at(n), 1);
-    k_fill_ops<<<cb, 256, 0, st>>>(ops, n, (uint32_t)(2 * n), 0, (uint32_t)n, 1);
-  } else {
-    k_fill_ops<<<cb, 256, 0, st>>>(ops, n, (uint32_t)n, 0, 0, 1);
-  }
-  e = run_ops<C>(pool, ops, n, M, st);
-  if (e != cudaSuccess) return e;
-  const size_t o = dbl ? n : 2 * n;
-  k_fe_out<F><<<cb, 256, 0, st>>>(pool.x.at(o), n, out, 2 * N, 0, 1);
-  k_fe_out<F><<<cb, 256, 0, st>>>(pool.y.at(o), n, out, 2 * N, N, 1);
-  return cudaGetLastError();
+  return dbl ? point_add<C, true>(n, p, q, out, st) : point_add<C, false>(n, p, q, out, st);
 }
 
 // --------------------------------------------------------------- G table
