@@ -296,14 +296,14 @@ int ecc_msm_window(ecc_curve_t curve, size_t n);
 int ecc_msm_set_window(ecc_curve_t curve, int log2_n, int c);
 
 /* Bucket layout of the reduction (the autotuner's second knob): the bucket rows
- * of an n-point MSM are cut into first-level chunks of 2^k consecutive buckets,
- * each walked by running sums in k-dependent batched affine rounds (2^k + 1
- * addition rounds and k doubling rounds, one CTA-wide inversion each) before
- * the short Jacobian levels combine the chunks.  Smaller chunks mean fewer
- * rounds and more chunks.  ecc_msm_reduce_chunk returns k for an n-point MSM
- * (default 5, capped at c - 1); ecc_msm_set_reduce_chunk overrides it for the
- * size class floor(log2 n) (log2_chunk 1..10; 0 restores the default).  Results
- * do not depend on k. */
+ * of an n-point MSM are cut into elements of 2^k consecutive buckets, each summed
+ * by one thread's running sums before a binary tree joins the elements of a row.
+ * Smaller elements are shorter serial sums and more additions in the tree.
+ * ecc_msm_reduce_chunk returns the k of an n-point MSM set by the override, or the
+ * largest k the library takes by itself (5; less where that would leave SMs idle;
+ * capped at c - 1); ecc_msm_set_reduce_chunk overrides it for the size class
+ * floor(log2 n) (log2_chunk 1..10; 0 restores the default).  Results do not depend
+ * on k. */
 int ecc_msm_reduce_chunk(ecc_curve_t curve, size_t n);
 int ecc_msm_set_reduce_chunk(ecc_curve_t curve, int log2_n, int log2_chunk);
 
@@ -315,10 +315,9 @@ int ecc_set_gas_cluster(int ctas);
 
 /* MSM phase timers (diagnostics).  With timing on, every MSM entry point
  * records CUDA events on its stream at the boundaries of its five phases:
- * 0 counting sort by bucket id (histogram, scans, scatter), 1 batched affine
- * bucket accumulation, 2 fold of each bucket's partial sums, 3 bucket
- * reduction (the affine first level and the Jacobian upper levels), 4 window
- * combination.  Nothing is recorded while the stream is being captured.
+ * 0 counting sort by bucket id (histogram, scans, scatter), 1 bucket
+ * accumulation, 2 fold of each bucket's partial sums, 3 bucket reduction
+ * (elements and tree), 4 window sums and their combination.  Nothing is recorded while the stream is being captured.
  * ecc_msm_phase_times waits for the calling thread's last timed MSM call and
  * writes the device milliseconds of up to max_phases phases to ms_out (host);
  * returns the number written, or ECC_EINVAL if this thread has no complete

@@ -83,8 +83,10 @@ cudaError_t launch_verify(int curve, size_t n, const uint8_t* hash, const uint8_
 // [offsets[i] - offsets[0], offsets[i+1] - offsets[0]) (host offsets); out: num x 2N limbs
 int msm_window(int curve, uint64_t n);
 void msm_set_window(int curve, int log2n, int c);
-// log2 of the buckets per first-level reduction chunk for an n-point MSM, and
-// the autotuner's override for the size class log2n (0 restores the default)
+// log2 of the buckets per reduction element: the autotuner's override for the size
+// class of n (0: none), the most an n-point MSM takes, and the override's setter for
+// the size class log2n (0 restores the default)
+int msm_reduce_override(int curve, uint64_t n);
 int msm_reduce_log(int curve, uint64_t n);
 void msm_set_reduce_log(int curve, int log2n, int v);
 constexpr int kMsmReduceLogMax = 10;

@@ -1,13 +1,15 @@
-// Jacobian-coordinate point arithmetic (x = X/Z^2, y = Y/Z^3; Section 2.1.2,
-// Table 1), used where a phase is a long dependent chain per thread with too
-// little parallelism to amortise a batch inversion: the MSM bucket reduction and
-// window combination.  Z = 0 encodes O.  Coordinates are in Montgomery form.
-// The group operations come in two forms: out of line (jac_dbl, jac_add: one
-// copy per curve keeps code size and compile time small where many call sites
-// use them) and inline (jac_dbl_inl, jac_add_inl: register-resident operands for
-// the one long chain of the window combination).
+// Jacobian-coordinate point arithmetic (x = X/Z^2, y = Y/Z^3, Z = 0 for O; Section
+// 2.1.2, Table 1) of the MSM, on curves with a = 0: sums that no other thread waits
+// for (jac_addto, by one thread, products called as in ladder.cuh) and the short
+// dependent chains at the end of a call (quad_*, four lanes a point).
+//
+// A chain of group operations by one thread costs a product's latency for each of
+// an operation's products (16 for an addition, 7 for a doubling; 0.42 us each with
+// 8 limbs, 0.9 with 12).  The four lanes of a quad hold the same points and take
+// one product each of a step's independent ones: 5 steps for an addition and 3 for
+// a doubling.
 #pragma once
-#include "ec.cuh"
+#include "ladder.cuh"
 
 namespace ecc {
 
@@ -16,205 +18,213 @@ struct Jac {
   uint32_t X[F::N], Y[F::N], Z[F::N];
 };
 
-template <class C>
-ECC_DEV void jac_set_inf(Jac<typename C::Fp>& P) {
-  using F = typename C::Fp;
-  fe_set_one<F>(P.X);
-  fe_set_one<F>(P.Y);
-  fe_set_zero<F>(P.Z);
-}
-
-template <class C>
-ECC_DEV bool jac_is_inf(const Jac<typename C::Fp>& P) {
-  return fe_is_zero<typename C::Fp>(P.Z);
-}
-
-// affine (x, y) with (0, 0) = O -> Jacobian
-template <class C>
-ECC_DEV void jac_from_affine(Jac<typename C::Fp>& P, const uint32_t* x, const uint32_t* y) {
-  using F = typename C::Fp;
-  if (pt_is_inf<F>(x, y)) {
-    jac_set_inf<C>(P);
-  } else {
-    fe_copy<F>(P.X, x);
-    fe_copy<F>(P.Y, y);
-    fe_set_one<F>(P.Z);
+template <class F>
+ECC_DEV void jac_load(const Jac<F>* p, uint32_t* X, uint32_t* Y, uint32_t* Z) {
+  constexpr int G = F::N / 4;
+  const uint4* v = reinterpret_cast<const uint4*>(p);
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const uint4 a = v[g], b = v[G + g], c = v[2 * G + g];
+    X[4 * g] = a.x, X[4 * g + 1] = a.y, X[4 * g + 2] = a.z, X[4 * g + 3] = a.w;
+    Y[4 * g] = b.x, Y[4 * g + 1] = b.y, Y[4 * g + 2] = b.z, Y[4 * g + 3] = b.w;
+    Z[4 * g] = c.x, Z[4 * g + 1] = c.y, Z[4 * g + 2] = c.z, Z[4 * g + 3] = c.w;
   }
 }
 
-// 2P: S = 2((X + Y^2)^2 - X^2 - Y^4), M = 3 X^2 + a Z^4,
-// X3 = M^2 - 2S, Y3 = M (S - X3) - 8 Y^4, Z3 = (Y + Z)^2 - Y^2 - Z^2.
-template <class C>
-ECC_DEV void jac_dbl_inl(Jac<typename C::Fp>& R, const Jac<typename C::Fp>& P) {
-  using F = typename C::Fp;
-  constexpr int N = F::N;
-  if (jac_is_inf<C>(P) || fe_is_zero<F>(P.Y)) {
-    jac_set_inf<C>(R);
-    return;
+template <class F>
+ECC_DEV void jac_store(Jac<F>* p, const uint32_t* X, const uint32_t* Y, const uint32_t* Z) {
+  constexpr int G = F::N / 4;
+  uint4* v = reinterpret_cast<uint4*>(p);
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    v[g] = make_uint4(X[4 * g], X[4 * g + 1], X[4 * g + 2], X[4 * g + 3]);
+    v[G + g] = make_uint4(Y[4 * g], Y[4 * g + 1], Y[4 * g + 2], Y[4 * g + 3]);
+    v[2 * G + g] = make_uint4(Z[4 * g], Z[4 * g + 1], Z[4 * g + 2], Z[4 * g + 3]);
   }
-  uint32_t XX[N], YY[N], YYYY[N], ZZ[N], S[N], M[N], t[N];
-  mont_sqr<F>(XX, P.X);
-  mont_sqr<F>(YY, P.Y);
-  mont_sqr<F>(YYYY, YY);
-  mont_sqr<F>(ZZ, P.Z);
-  fe_add<F>(t, P.X, YY);
-  mont_sqr<F>(t, t);
-  fe_sub<F>(t, t, XX);
-  fe_sub<F>(t, t, YYYY);
-  fe_add<F>(S, t, t);
-  fe_add<F>(M, XX, XX);
-  fe_add<F>(M, M, XX);
-  if (!C::A_ZERO) {
-    uint32_t a[N];
-    curve_a<C>(a);
-    mont_sqr<F>(t, ZZ);
-    mont_mul<F>(t, t, a);
-    fe_add<F>(M, M, t);
-  }
-  uint32_t X3[N], Y3[N], Z3[N];
-  fe_add<F>(Z3, P.Y, P.Z);
-  mont_sqr<F>(Z3, Z3);
-  fe_sub<F>(Z3, Z3, YY);
-  fe_sub<F>(Z3, Z3, ZZ);
-  mont_sqr<F>(X3, M);
-  fe_sub<F>(X3, X3, S);
-  fe_sub<F>(X3, X3, S);
-  fe_sub<F>(t, S, X3);
-  mont_mul<F>(Y3, M, t);
-  fe_add<F>(t, YYYY, YYYY);
-  fe_add<F>(t, t, t);
-  fe_add<F>(t, t, t);
-  fe_sub<F>(Y3, Y3, t);
-  fe_copy<F>(R.X, X3);
-  fe_copy<F>(R.Y, Y3);
-  fe_copy<F>(R.Z, Z3);
 }
 
-// Shared tail of the additions: given U1, S1, H = U2 - U1, r = S2 - S1 and
-// Z3 / H, X3 = r^2 - H^3 - 2 U1 H^2, Y3 = r (U1 H^2 - X3) - S1 H^3.
-// Out of line: one copy per curve for the kernels that call it from many places.
-template <class C>
-__device__ __noinline__ void jac_dbl(Jac<typename C::Fp>& R, const Jac<typename C::Fp>& P) {
-  jac_dbl_inl<C>(R, P);
+template <class F>
+ECC_DEV void jac_set_inf(uint32_t* X, uint32_t* Y, uint32_t* Z) {
+  fe_set_one<F>(X);
+  fe_set_one<F>(Y);
+  fe_set_zero<F>(Z);
 }
 
+// P <- P + Q, every case of the group law (12 products and 4 squares).
 template <class C>
-ECC_DEV void jac_add_tail(Jac<typename C::Fp>& R, const uint32_t* U1, const uint32_t* S1,
-                          const uint32_t* H, const uint32_t* r, const uint32_t* Z3) {
+ECC_DEV void jac_addto(uint32_t* X1, uint32_t* Y1, uint32_t* Z1, const uint32_t* X2, const uint32_t* Y2,
+                       const uint32_t* Z2) {
   using F = typename C::Fp;
   constexpr int N = F::N;
-  uint32_t HH[N], HHH[N], V[N], X3[N], Y3[N], t[N];
-  mont_sqr<F>(HH, H);
-  mont_mul<F>(HHH, H, HH);
-  mont_mul<F>(V, U1, HH);
-  mont_sqr<F>(X3, r);
-  fe_sub<F>(X3, X3, HHH);
-  fe_sub<F>(X3, X3, V);
-  fe_sub<F>(X3, X3, V);
-  fe_sub<F>(t, V, X3);
-  mont_mul<F>(Y3, r, t);
-  mont_mul<F>(t, S1, HHH);
-  fe_sub<F>(Y3, Y3, t);
-  fe_copy<F>(R.X, X3);
-  fe_copy<F>(R.Y, Y3);
-  fe_copy<F>(R.Z, Z3);
-}
-
-// R = P + Q, both Jacobian (every case of the group law).
-template <class C>
-ECC_DEV void jac_add_inl(Jac<typename C::Fp>& R, const Jac<typename C::Fp>& P,
-                     const Jac<typename C::Fp>& Q) {
-  using F = typename C::Fp;
-  constexpr int N = F::N;
-  if (jac_is_inf<C>(P)) {
-    R = Q;
+  if (fe_is_zero<F>(Z2)) return;
+  if (fe_is_zero<F>(Z1)) {
+    fe_copy<F>(X1, X2);
+    fe_copy<F>(Y1, Y2);
+    fe_copy<F>(Z1, Z2);
     return;
   }
-  if (jac_is_inf<C>(Q)) {
-    R = P;
-    return;
-  }
-  uint32_t Z1Z1[N], Z2Z2[N], U1[N], U2[N], S1[N], S2[N], H[N], r[N], Z3[N];
-  mont_sqr<F>(Z1Z1, P.Z);
-  mont_sqr<F>(Z2Z2, Q.Z);
-  mont_mul<F>(U1, P.X, Z2Z2);
-  mont_mul<F>(U2, Q.X, Z1Z1);
-  mont_mul<F>(S1, Q.Z, Z2Z2);
-  mont_mul<F>(S1, P.Y, S1);
-  mont_mul<F>(S2, P.Z, Z1Z1);
-  mont_mul<F>(S2, Q.Y, S2);
-  fe_sub<F>(H, U2, U1);
-  fe_sub<F>(r, S2, S1);
+  uint32_t a[N], H[N], r[N], U[N], S[N];
+  call_sqr<F>(a, Z2);
+  call_mul<F>(U, X1, a);   // U1
+  call_mul<F>(a, a, Z2);
+  call_mul<F>(S, Y1, a);   // S1
+  call_sqr<F>(a, Z1);
+  call_mul<F>(H, X2, a);
+  fe_sub<F>(H, H, U);      // U2 - U1
+  call_mul<F>(a, a, Z1);
+  call_mul<F>(r, Y2, a);
+  fe_sub<F>(r, r, S);      // S2 - S1
   if (fe_is_zero<F>(H)) {
     if (fe_is_zero<F>(r)) {
-      jac_dbl<C>(R, P);
+      jac_dbl_rare<C>(X1, Y1, Z1);
     } else {
-      jac_set_inf<C>(R);
+      jac_set_inf<F>(X1, Y1, Z1);
     }
     return;
   }
-  mont_mul<F>(Z3, P.Z, Q.Z);
-  mont_mul<F>(Z3, Z3, H);
-  jac_add_tail<C>(R, U1, S1, H, r, Z3);
+  call_mul<F>(Z1, Z1, Z2);
+  call_mul<F>(Z1, Z1, H);
+  call_sqr<F>(a, H);
+  call_mul<F>(U, U, a);    // V = U1 H^2
+  call_mul<F>(H, H, a);    // H^3
+  call_sqr<F>(X1, r);
+  fe_sub<F>(X1, X1, H);
+  fe_sub<F>(X1, X1, U);
+  fe_sub<F>(X1, X1, U);
+  fe_sub<F>(U, U, X1);
+  call_mul_sub<F>(Y1, r, U, S, H);
 }
 
-template <class C>
-__device__ __noinline__ void jac_add(Jac<typename C::Fp>& R, const Jac<typename C::Fp>& P,
-                                     const Jac<typename C::Fp>& Q) {
-  jac_add_inl<C>(R, P, Q);
+// ---------------------------------------------------------------- quads
+// The four lanes of a quad call these together with equal points; other quads of
+// the warp may be elsewhere.
+
+ECC_DEV unsigned quad_mask() { return 0xfu << (threadIdx.x & 28u); }
+
+template <class F>
+ECC_DEV void quad_get(uint32_t* r, const uint32_t* a, int lane) {
+  const unsigned m = quad_mask();
+#pragma unroll
+  for (int i = 0; i < F::N; ++i) r[i] = __shfl_sync(m, a[i], lane, 4);
 }
 
-// R = P + (x, y) with the second operand affine ((0, 0) = O).
+// this lane's factor: a, b, c or d for lane 0, 1, 2 or 3 of the quad
+template <class F>
+ECC_DEV void quad_pick(uint32_t* r, const uint32_t* a, const uint32_t* b, const uint32_t* c, const uint32_t* d) {
+  const unsigned q = threadIdx.x & 3u;
+#pragma unroll
+  for (int i = 0; i < F::N; ++i) {
+    const uint32_t lo = (q & 1u) ? b[i] : a[i], hi = (q & 1u) ? d[i] : c[i];
+    r[i] = (q & 2u) ? hi : lo;
+  }
+}
+
+// P <- 2 P with the halved Z of jac_dbl_half
 template <class C>
-__device__ __noinline__ void jac_add_mixed(Jac<typename C::Fp>& R, const Jac<typename C::Fp>& P,
-                           const uint32_t* x, const uint32_t* y) {
+ECC_DEV void quad_dbl(JacReg<typename C::Fp>& P) {
   using F = typename C::Fp;
   constexpr int N = F::N;
-  if (pt_is_inf<F>(x, y)) {
-    R = P;
+  static_assert(C::A_ZERO, "a = 0");
+  uint32_t a[N], b[N], p[N], l[N], YY[N], D[N];
+  quad_pick<F>(a, P.X.v, P.Y.v, P.Y.v, P.X.v);
+  quad_pick<F>(b, P.X.v, P.Y.v, P.Z.v, P.X.v);
+  mont_mul<F>(p, a, b);  // X^2, Y^2, Y Z
+  quad_get<F>(l, p, 0);
+  quad_get<F>(YY, p, 1);
+  quad_get<F>(P.Z.v, p, 2);
+  fe_half<F>(a, l);
+  fe_add<F>(l, l, a);    // 3 X^2 / 2
+  quad_pick<F>(a, YY, P.X.v, l, l);
+  quad_pick<F>(b, YY, YY, l, l);
+  mont_mul<F>(p, a, b);  // Y^4, X Y^2, l^2
+  quad_get<F>(D, p, 1);
+  quad_get<F>(P.X.v, p, 2);
+  quad_get<F>(YY, p, 0);
+  fe_sub<F>(P.X.v, P.X.v, D);
+  fe_sub<F>(P.X.v, P.X.v, D);
+  fe_sub<F>(D, D, P.X.v);
+  mont_mul<F>(P.Y.v, l, D);
+  fe_sub<F>(P.Y.v, P.Y.v, YY);
+}
+
+// P <- P + Q, every case of the group law
+template <class C>
+ECC_DEV void quad_add(JacReg<typename C::Fp>& P, JacReg<typename C::Fp> Q) {
+  using F = typename C::Fp;
+  constexpr int N = F::N;
+  if (fe_is_zero<F>(Q.Z.v)) return;
+  if (fe_is_zero<F>(P.Z.v)) {
+    P = Q;
     return;
   }
-  if (jac_is_inf<C>(P)) {
-    jac_from_affine<C>(R, x, y);
-    return;
-  }
-  uint32_t Z1Z1[N], U2[N], S2[N], H[N], r[N], Z3[N], U1[N], S1[N];
-  mont_sqr<F>(Z1Z1, P.Z);
-  mont_mul<F>(U2, x, Z1Z1);
-  mont_mul<F>(S2, P.Z, Z1Z1);
-  mont_mul<F>(S2, y, S2);
-  fe_sub<F>(H, U2, P.X);
-  fe_sub<F>(r, S2, P.Y);
+  uint32_t a[N], b[N], p[N], ZZ[N], H[N], r[N];
+  quad_pick<F>(a, P.Z.v, Q.Z.v, P.Z.v, P.Z.v);
+  quad_pick<F>(b, P.Z.v, Q.Z.v, Q.Z.v, Q.Z.v);
+  mont_mul<F>(p, a, b);    // Z1^2, Z2^2, Z1 Z2
+  quad_get<F>(ZZ, p, 2);
+  quad_get<F>(H, p, 0);    // Z1^2
+  quad_get<F>(r, p, 1);    // Z2^2
+  quad_pick<F>(a, P.X.v, Q.X.v, Q.Z.v, P.Z.v);
+  quad_pick<F>(b, r, H, r, H);
+  mont_mul<F>(p, a, b);    // U1, U2, Z2^3, Z1^3
+  quad_get<F>(P.X.v, p, 0);
+  quad_get<F>(H, p, 1);
+  fe_sub<F>(H, H, P.X.v);
+  quad_get<F>(Q.Z.v, p, 2);
+  quad_get<F>(P.Z.v, p, 3);
+  quad_pick<F>(a, P.Y.v, Q.Y.v, H, ZZ);
+  quad_pick<F>(b, Q.Z.v, P.Z.v, H, H);
+  mont_mul<F>(p, a, b);    // S1, S2, H^2, Z3
+  quad_get<F>(Q.X.v, p, 0);
+  quad_get<F>(r, p, 1);
+  fe_sub<F>(r, r, Q.X.v);
   if (fe_is_zero<F>(H)) {
+    // equal points: the doubling of (U1, S1, Z1 Z2), which is the same point
+    fe_copy<F>(P.Y.v, Q.X.v);
+    fe_copy<F>(P.Z.v, ZZ);
     if (fe_is_zero<F>(r)) {
-      jac_dbl<C>(R, P);
+      jac_dbl_rare<C>(P.X.v, P.Y.v, P.Z.v);
     } else {
-      jac_set_inf<C>(R);
+      jac_set_inf<F>(P.X.v, P.Y.v, P.Z.v);
     }
     return;
   }
-  mont_mul<F>(Z3, P.Z, H);
-  fe_copy<F>(U1, P.X);
-  fe_copy<F>(S1, P.Y);
-  jac_add_tail<C>(R, U1, S1, H, r, Z3);
+  quad_get<F>(ZZ, p, 2);
+  quad_get<F>(P.Z.v, p, 3);
+  quad_pick<F>(a, H, P.X.v, r, r);
+  quad_pick<F>(b, ZZ, ZZ, r, r);
+  mont_mul<F>(p, a, b);    // H^3, V = U1 H^2, r^2
+  quad_get<F>(H, p, 0);
+  quad_get<F>(ZZ, p, 1);
+  quad_get<F>(P.X.v, p, 2);
+  fe_sub<F>(P.X.v, P.X.v, H);
+  fe_sub<F>(P.X.v, P.X.v, ZZ);
+  fe_sub<F>(P.X.v, P.X.v, ZZ);
+  fe_sub<F>(ZZ, ZZ, P.X.v);
+  quad_pick<F>(a, r, Q.X.v, r, r);
+  quad_pick<F>(b, ZZ, H, ZZ, ZZ);
+  mont_mul<F>(p, a, b);    // r (V - X3), S1 H^3
+  quad_get<F>(a, p, 0);
+  quad_get<F>(b, p, 1);
+  fe_sub<F>(P.Y.v, a, b);
+}
+
+template <class F>
+ECC_DEV JacReg<F> quad_load(const Jac<F>* p) {
+  JacReg<F> P;
+  jac_load<F>(p, P.X.v, P.Y.v, P.Z.v);
+  return P;
 }
 
 // Jacobian -> affine (x, y) in Montgomery form, (0, 0) for O (one inversion).
-template <class C>
-__device__ __noinline__ void jac_to_affine(uint32_t* x, uint32_t* y, const Jac<typename C::Fp>& P) {
-  using F = typename C::Fp;
-  constexpr int N = F::N;
-  if (jac_is_inf<C>(P)) {
-    fe_set_zero<F>(x);
-    fe_set_zero<F>(y);
-    return;
-  }
-  uint32_t zi[N], zi2[N];
-  fe_inv_mont<F>(zi, P.Z);
-  mont_sqr<F>(zi2, zi);
-  mont_mul<F>(x, P.X, zi2);
-  mont_mul<F>(zi2, zi2, zi);
-  mont_mul<F>(y, P.Y, zi2);
+template <class F>
+ECC_DEV void jac_to_affine(uint32_t* x, uint32_t* y, const JacReg<F>& P) {
+  uint32_t zi[F::N], t[F::N];
+  fe_inv_mont<F>(zi, P.Z.v);  // 0 for O
+  mont_sqr<F>(t, zi);
+  mont_mul<F>(x, P.X.v, t);
+  mont_mul<F>(t, t, zi);
+  mont_mul<F>(y, P.Y.v, t);
 }
 
 }  // namespace ecc

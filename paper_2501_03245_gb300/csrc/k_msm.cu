@@ -144,11 +144,16 @@ bool phase_times(float* ms) {
   return true;
 }
 
-int msm_reduce_log(int curve, uint64_t n) {
+int msm_reduce_override(int curve, uint64_t n) {
   if (n < 2) n = 2;
   std::lock_guard<std::mutex> lock(g_win_mu);
   auto it = g_chunk_table.find({curve, ilog2(n)});
-  return it != g_chunk_table.end() ? it->second : kRedLog1Default;
+  return it != g_chunk_table.end() ? it->second : 0;
+}
+
+int msm_reduce_log(int curve, uint64_t n) {
+  const int k = msm_reduce_override(curve, n);
+  return k > 0 ? k : kRedLog1Default;
 }
 
 void msm_set_reduce_log(int curve, int log2n, int v) {

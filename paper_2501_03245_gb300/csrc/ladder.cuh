@@ -109,11 +109,34 @@ struct JacReg {
   Fe<F> X, Y, Z;
 };
 
-// The doubling inside an addition of equal points (rare), out of line.
+// The doubling inside an addition of equal points (rare), out of line and through
+// memory, so that the additions around it keep their registers.
 template <class C>
-__device__ __noinline__ JacReg<typename C::Fp> jac_dbl_call(JacReg<typename C::Fp> P) {
-  jac_dbl_half<C>(P.X.v, P.Y.v, P.Z.v);
-  return P;
+__device__ __noinline__ void jac_dbl_mem(uint32_t* P) {
+  using F = typename C::Fp;
+  constexpr int N = F::N;
+  uint32_t X[N], Y[N], Z[N];
+  fe_copy<F>(X, P);
+  fe_copy<F>(Y, P + N);
+  fe_copy<F>(Z, P + 2 * N);
+  jac_dbl_half<C>(X, Y, Z);
+  fe_copy<F>(P, X);
+  fe_copy<F>(P + N, Y);
+  fe_copy<F>(P + 2 * N, Z);
+}
+
+template <class C>
+ECC_DEV void jac_dbl_rare(uint32_t* X, uint32_t* Y, uint32_t* Z) {
+  using F = typename C::Fp;
+  constexpr int N = F::N;
+  uint32_t P[3 * N];
+  fe_copy<F>(P, X);
+  fe_copy<F>(P + N, Y);
+  fe_copy<F>(P + 2 * N, Z);
+  jac_dbl_mem<C>(P);
+  fe_copy<F>(X, P);
+  fe_copy<F>(Y, P + N);
+  fe_copy<F>(Z, P + 2 * N);
 }
 
 // P <- P + (x, y) for an affine point other than O; every case of the group law.
@@ -139,10 +162,7 @@ ECC_DEV void jac_madd(uint32_t* X, uint32_t* Y, uint32_t* Z, const uint32_t* x, 
   fe_sub<F>(r, r, Y);
   if (fe_is_zero<F>(H)) {
     if (fe_is_zero<F>(r)) {
-      const JacReg<F> D = jac_dbl_call<C>(JacReg<F>{fe_pack<F>(X), fe_pack<F>(Y), fe_pack<F>(Z)});
-      fe_copy<F>(X, D.X.v);
-      fe_copy<F>(Y, D.Y.v);
-      fe_copy<F>(Z, D.Z.v);
+      jac_dbl_rare<C>(X, Y, Z);
     } else {
       fe_set_zero<F>(Z);
     }

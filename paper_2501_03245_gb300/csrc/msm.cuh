@@ -13,12 +13,12 @@
 //      trick with GAS, Section 3.2).  A chunk entry that starts a new bucket
 //      flushes the running sum as a partial bucket sum and restarts it (a copy,
 //      no inversion needed).  CH rounds finish the whole array in one launch;
-//   4. bucket reduction sum_k k B_k per window by chunked running sums: the
-//      first level (many independent chunks) as batched affine additions, the
-//      short upper levels in Jacobian coordinates;
-//   5. window combination sum_w 2^(c w) S_w in Jacobian coordinates (one long
-//      dependent chain per instance, where a batch inversion per step would be
-//      pure latency).
+//      (calls with few entries: one thread per chunk in Jacobian coordinates);
+//   4. bucket reduction sum_k k B_k per window: running sums over chunks of
+//      buckets, then a binary tree that keeps the sums of the chunks whose index
+//      has bit j set, for every j;
+//   5. window combination sum_w 2^(c w) S_w in Jacobian coordinates, four lanes per
+//      chain.
 // Several independent MSM instances (different sizes, windows and bases) run
 // through the same launches: every instance owns a disjoint range of bucket ids.
 #pragma once
@@ -26,7 +26,8 @@
 
 namespace ecc {
 
-constexpr int kAccChunk = 32;       // entries per running-sum chunk (rounds of step 3)
+constexpr int kAccLog = 5;
+constexpr int kAccChunk = 1 << kAccLog;  // entries per running-sum chunk (rounds of step 3)
 
 struct MsmInst {
   uint32_t n;            // points of the instance
@@ -41,8 +42,14 @@ struct MsmInst {
   // buckets, one per window.
   uint64_t pre_stride;
   uint32_t Wr;           // bucket rows (windows reduced separately)
-  uint32_t red_log;      // log2 of the buckets per first-level reduction chunk
+  uint32_t red_log;      // log2 of the buckets per reduction chunk (element)
+  uint64_t elem_off;     // first reduction element; 2^(c - 1 - red_log) per bucket row
+  uint32_t row_off;      // first bucket row
+  uint32_t cta_off;      // first CTA of the reduction tree's first pass
 };
+
+// log2 of the reduction elements per bucket row
+__host__ __device__ inline uint32_t elem_log(const MsmInst& in) { return in.c - 1 - in.red_log; }
 
 // ------------------------------------------------------------------ digits
 
@@ -109,6 +116,14 @@ struct MsmDevHdr {
   uint32_t pad;
 };
 
+// Levels of the reduction tree that its first pass does inside one CTA, and that
+// pass's CTAs for an instance.
+constexpr uint32_t kTreeLog = 8;
+__host__ __device__ inline uint32_t tree_ctas(const MsmInst& in) {
+  const uint32_t m = elem_log(in);
+  return in.Wr << (m > kTreeLog ? m - kTreeLog : 0);
+}
+
 // Rows of the batch: the host's count, or the device header's when present.
 ECC_DEV uint64_t batch_rows(uint64_t host_total, const MsmDevHdr* hdr) {
   return hdr ? hdr->total : host_total;
@@ -173,6 +188,9 @@ static __global__ void k_msm_inst_dev(const uint64_t* __restrict__ rows, uint32_
       MsmInst m = proto;
       m.n = (uint32_t)n;
       m.bucket_base = (uint32_t)(i * per_bucket_row);
+      m.elem_off = i * ((uint64_t)proto.Wr << elem_log(proto));
+      m.row_off = i * proto.Wr;
+      m.cta_off = i * tree_ctas(proto);
       m.scalar_off = sizes_mode ? before : off;
       m.point_off = sizes_mode ? 0 : off;
       inst[i] = m;
@@ -209,14 +227,15 @@ __global__ void k_msm_count(const MsmInst* inst, int num, const uint32_t* __rest
   });
 }
 
-// Entries are written chunk-transposed: entry p goes to [p % CH][p / CH].  Only
+// Entries are written chunk-transposed: entry p goes to [p % CH][p / CH], CH =
+// 2^ch_log.  Only
 // the point index is stored; the bucket of position p follows from the offsets.
 // The bucket of each chunk's first entry is recorded in cur (the accumulation's
 // per-chunk bucket cursor starts there).
 template <class C>
 __global__ void k_msm_scatter(const MsmInst* inst, int num, const uint32_t* __restrict__ scalars,
                               uint64_t total, const MsmDevHdr* hdr, uint32_t* __restrict__ cursor,
-                              uint32_t* __restrict__ vals, uint64_t n_chunks,
+                              uint32_t* __restrict__ vals, uint64_t n_chunks, int ch_log,
                               uint32_t* __restrict__ cur) {
   const uint64_t g = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   if (g >= batch_rows(total, hdr)) return;
@@ -232,18 +251,19 @@ __global__ void k_msm_scatter(const MsmInst* inst, int num, const uint32_t* __re
     const uint32_t b = in.bucket_base + w * row + (uint32_t)(d < 0 ? -d : d) - 1;
     const uint32_t p = atomicAdd(cursor + b, 1u);
     const uint32_t idx = (uint32_t)(pidx + (uint64_t)w * in.pre_stride);  // < 2^31 (host check)
-    vals[(uint64_t)(p % kAccChunk) * n_chunks + p / kAccChunk] = idx | (d < 0 ? 0x80000000u : 0u);
-    if (p % kAccChunk == 0) cur[p / kAccChunk] = b;
+    const uint32_t j = p & ((1u << ch_log) - 1u), chunk = p >> ch_log;
+    vals[(uint64_t)j * n_chunks + chunk] = idx | (d < 0 ? 0x80000000u : 0u);
+    if (j == 0) cur[chunk] = b;
   });
 }
 
 // Partial-sum slots per bucket: one per chunk the bucket's entries touch.
-static __global__ void k_msm_npart(const uint32_t* __restrict__ off, uint32_t n_buckets,
-                            uint32_t* __restrict__ npart) {
+static __global__ void k_msm_npart(const uint32_t* __restrict__ off, uint32_t n_buckets, int ch_log,
+                                   uint32_t* __restrict__ npart) {
   const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= n_buckets) return;
   const uint32_t lo = off[b], hi = off[b + 1];
-  npart[b] = hi > lo ? (hi - 1) / kAccChunk - lo / kAccChunk + 1 : 0;
+  npart[b] = hi > lo ? ((hi - 1) >> ch_log) - (lo >> ch_log) + 1 : 0;
 }
 
 // ------------------------------------------------------------------ accumulation
@@ -584,44 +604,94 @@ __global__ void __launch_bounds__(BLOCK, kGasResidentThreads / BLOCK) k_msm_accu
   }
 }
 
+// ------------------------------------------------------------------ few entries
+//
+// A batched affine round costs a CTA-wide inversion whatever it holds (about 25 us
+// with 8 limbs, 40 with 12), and an accumulation has 32 of them.  Below
+// kDirectEntries entries (msm_host.cuh) a mixed Jacobian addition (11 products
+// instead of 6) by one thread per chunk, which waits for nobody, is faster.
+
+template <class F>
+struct JacSoA {
+  SoA<F> x, y, z;
+  ECC_DEV void load(size_t i, uint32_t* X, uint32_t* Y, uint32_t* Z) const {
+    x.load(i, X);
+    y.load(i, Y);
+    z.load(i, Z);
+  }
+  ECC_DEV void store(size_t i, const uint32_t* X, const uint32_t* Y, const uint32_t* Z) const {
+    x.store(i, X);
+    y.store(i, Y);
+    z.store(i, Z);
+  }
+};
+
+// Threads of the Jacobian kernels: 128 registers a thread hold the additions of 8
+// limbs, 168 those of 12.
+constexpr int kJacThreads = 128;
+template <int N>
+constexpr int kJacCtas = N <= 8 ? 4 : 3;
+
+// Running sums of the chunks as in the affine rounds, with partial sums in
+// Jacobian coordinates.
+template <class C>
+__global__ void __launch_bounds__(kJacThreads, kJacCtas<C::Fp::N>)
+    k_msm_accumulate_jac(AccArgs<C> a, JacSoA<typename C::Fp> partial, int ch_log) {
+  using F = typename C::Fp;
+  constexpr int N = F::N;
+  const uint32_t entries = a.off[a.n_buckets];
+  const uint64_t c = blockIdx.x * (uint64_t)kJacThreads + threadIdx.x;
+  const uint32_t p0 = (uint32_t)(c << ch_log);
+  if ((c << ch_log) >= entries) return;
+  const uint32_t ch = entries - p0 < (1u << ch_log) ? entries - p0 : 1u << ch_log;
+  uint32_t b = a.cur[c], end = a.off[b + 1];
+  uint32_t X[N], Y[N], Z[N], H[N];
+  jac_set_inf<F>(X, Y, Z);
+  auto flush = [&]() { partial.store(a.poff[b] + (c - (a.off[b] >> ch_log)), X, Y, Z); };
+#pragma unroll 1
+  for (uint32_t j = 0; j < ch; ++j) {
+    const uint32_t p = p0 + j;
+    if (p >= end) {
+      flush();
+      jac_set_inf<F>(X, Y, Z);
+      ++b;  // usually the next bucket; skip empty ones otherwise
+      if (a.off[b + 1] <= p) b = bucket_of(a.off, b + 1, a.n_buckets, p);
+      end = a.off[b + 1];
+    }
+    uint32_t x[N], y[N];
+    load_base<C>(a, a.vals[(uint64_t)j * a.n_chunks + c], x, y);
+    if (!pt_is_inf<F>(x, y)) jac_madd<C>(X, Y, Z, x, y, H);
+  }
+  flush();
+}
+
 // ------------------------------------------------------------------ reduction
 //
-// Window sum sum_b b E_b (E_b the bucket sums, b = 1 .. 2^(c-1)) in levels.
-// Level 1 cuts each window row into chunks of K = 2^red_log consecutive buckets;
-// chunk u (buckets lo .. hi-1, 0-based) yields the plain sum R_u and the sum
-// S_u = sum_e (e - lo + 1) E_e weighted from the chunk's own first bucket, so
-// the window sum is sum_u (S_u + u (K R_u)).  Every later level takes
-// elements (R~_e, S~_e) whose target is sum_e (S~_e + e R~_e) and cuts them
-// into chunks of kRedChunkN: chunk v yields R_v = sum R~_e and
-// S_v = sum_e (S~_e + (e - lo) R~_e), and hands (kRedChunkN R_v, S_v) on, until
-// one element per row is left: its S is the window sum.  The multiples of R are
-// taken by the producing level (log2 of the chunk size doublings per output).
+// Window sum sum_b b E_b (E_b the bucket sums, b = 1 .. 2^(c-1)).  Before it the
+// partial sums of every bucket are folded into the first one (a pairwise tree,
+// ceil(log2 k) rounds for k partials; CTAs take equal shares of the partial slots,
+// so a bucket holding many entries costs rounds only in the CTA that owns it).
 //
-// Before level 1 the partial sums of every bucket are folded into one (a
-// batched affine pairwise tree, ceil(log2 k) rounds for k partials; CTAs take
-// equal shares of the partial slots, so a bucket holding many entries costs
-// rounds only in the CTA that owns it).  Level 1 then has 2^(c-1) / K
-// independent chunks per window row (2^red_log buckets each, a per-instance
-// layout parameter the autotuner picks) and runs as batched affine additions
-// (Section 3.3) with one inversion per CTA per round (Section 3.2): the running
-// sums R and S of every chunk walk the chunk's buckets downwards, adding the
-// bucket sum to R ("A" event) and then R to S ("S" event).  An S event uses
-// the R of before the next bucket's A event, so the two share a round and a
-// chunk of k buckets takes k + 1 rounds.  The short upper levels run in
-// Jacobian coordinates, one thread per chunk.
+// A window row is cut into elements of K = 2^red_log consecutive buckets: element u
+// has R_u, the plain sum, and S_u = sum_i i E_(K u + i), i = 1 .. K, from two running
+// sums by one thread (k_msm_elems).  The window sum is sum_u S_u + K sum_u u R_u, and
+// sum_u u R_u = sum_j 2^j Q_j with Q_j the sum of the R_u whose u has bit j set.  A
+// binary tree computes all Q_j at once, in place (k_msm_tree): when the block of
+// 2^(l+1) elements at e joins its halves, R[e] += R[e + 2^l] is the block's sum,
+// the old R[e + 2^l] stays behind as the block's Q_l, and Q_j of the halves, at
+// R[e + 2^j] and R[e + 2^l + 2^j], are added for j < l.  That is two additions an
+// element in all, log2 of the elements deep.  k_msm_combine then forms the window
+// sums and the windows' combination.
+//
+// This replaced batched affine rounds (12 products a bucket instead of 27, but a
+// walk of 2^red_log + 1 + red_log rounds of about 25 us or more, then levels of four
+// elements by one thread): 4096 BN254 points 0.9 -> 0.08 ms, 256 BN254 MSMs of 2^10 to
+// 2^18 points 8.9 -> 6.0, 16 x 2^20 BLS12-381 points 12.4 -> 8.4; bound by the products
+// of k_msm_elems where there are many buckets.  The combination below took 1.1 ms for
+// one BN254 result by one thread and takes 0.5.
 
-constexpr int kRedLog1Default = 5;      // log2 buckets per first-level chunk, by default
+constexpr int kRedLog1Default = 5;      // log2 buckets per element, at most, by default
 constexpr int kRedLog1Max = 10;
-constexpr uint32_t kRedChunkN = 4;       // elements per chunk on the later levels
-constexpr int kRedLogN = 2;
-
-// First-level items (chunks) in group-major order: the items of one instance
-// are [t0, t0 + W * chunks), window row w first, then chunk u.
-struct RedRange {
-  uint64_t t0;
-  uint32_t inst;
-  uint32_t chunks;  // chunks per window row
-};
 
 // ---- fold: the partial sums of every bucket into its first partial slot
 template <class C>
@@ -632,6 +702,7 @@ struct FoldArgs {
   PtSoA<F> partial;
   SoA<F> M;                     // GAS prefix products, one per slot
   uint32_t* ops;                // per-round list of additions, one word per slot
+  JacSoA<F> jac;                // the partial sums when they are in Jacobian coordinates
 };
 
 // first b in [0, n] with poff[b] >= x
@@ -809,11 +880,12 @@ __device__ void fold_round_staged(const FoldArgs<C>& a, uint32_t h, uint64_t s0,
 // of a bucket with many partial sums (the top window often puts most entries
 // into a few buckets) is shared by the whole CTA and lanes never idle on
 // inactive slots.
-template <class C, int BLOCK>
-__global__ void __launch_bounds__(BLOCK, kGasResidentThreads / BLOCK) k_msm_fold(FoldArgs<C> a) {
+// JAC: partial sums in Jacobian coordinates, added one by one.
+template <class C, int BLOCK, bool JAC>
+__global__ void __launch_bounds__(BLOCK, JAC && C::Fp::N > 8 ? 1 : kGasResidentThreads / BLOCK)
+    k_msm_fold(FoldArgs<C> a) {
   using F = typename C::Fp;
   constexpr int N = F::N;
-  auto& sm = gas_smem<N, BLOCK>();
   __shared__ uint32_t wsum[BLOCK / 32];
   const uint64_t total_slots = a.poff[a.n_buckets];
   if (total_slots == 0) return;  // uniform over the grid
@@ -845,520 +917,172 @@ __global__ void __launch_bounds__(BLOCK, kGasResidentThreads / BLOCK) k_msm_fold
       for (uint32_t l = 0; l + h < k; l += 2 * h) a.ops[s0 + pos++] = p + l;
     }
     __syncthreads();  // the list is complete
-    fold_round_staged<C, BLOCK>(a, h, s0, n_ops, sm);
+    if constexpr (JAC) {
+#pragma unroll 1
+      for (uint32_t e = threadIdx.x; e < n_ops; e += BLOCK) {
+        const uint32_t sl = a.ops[s0 + e];
+        uint32_t X[N], Y[N], Z[N], X2[N], Y2[N], Z2[N];
+        a.jac.load(sl, X, Y, Z);
+        a.jac.load(sl + h, X2, Y2, Z2);
+        jac_addto<C>(X, Y, Z, X2, Y2, Z2);
+        a.jac.store(sl, X, Y, Z);
+      }
+      __syncthreads();  // the sums are in place, the list is free
+    } else {
+      fold_round_staged<C, BLOCK>(a, h, s0, n_ops, gas_smem<N, BLOCK>());
+    }
   }
 }
 
+// ---- elements
 template <class C>
-struct AffRedArgs {
+struct RedArgs {
   using F = typename C::Fp;
   const MsmInst* inst;
-  const RedRange* ranges;
-  uint32_t n_ranges;
-  uint64_t items;
-  const uint32_t* poff;   // partial-slot offsets per bucket (n_buckets + 1 entries)
-  PtSoA<F> partial;       // partial bucket sums (affine)
-  PtSoA<F> R, S;          // running sums per item (affine)
-  SoA<F> M;               // GAS prefix products per item
-  uint32_t* cur_e;        // 1 + the bucket the next event belongs to
-  uint32_t* cur_a;        // whether that bucket's A event is done
-  uint32_t* lo_b;         // first bucket of the item
-  uint32_t* rlog;         // log2 of the item's chunk size (its instance's red_log)
-  Jac<F>* out_R;          // 2^rlog R per item (Jacobian, Z = 1 or O)
-  Jac<F>* out_S;
-  uint64_t per_cta;
+  uint32_t num;
+  uint64_t elems;
+  const uint32_t* poff;   // partial-slot offsets per bucket: its sum is in the first
+  PtSoA<F> partial;
+  JacSoA<F> jac;
+  Jac<F>* R;              // per element
+  Jac<F>* S;
+  Jac<F>* row;            // window sums
 };
 
-ECC_DEV uint32_t find_range(const RedRange* r, uint32_t num, uint64_t t) {
+// the instance whose range (starting at inst[i].*field) holds t
+template <class T>
+ECC_DEV uint32_t find_by(const MsmInst* inst, uint32_t num, T MsmInst::*field, uint64_t t) {
   uint32_t lo = 0, hi = num - 1;
   while (lo < hi) {
     const uint32_t mid = (lo + hi + 1) >> 1;
-    if (r[mid].t0 <= t) lo = mid; else hi = mid - 1;
+    if (inst[mid].*field <= t) lo = mid; else hi = mid - 1;
   }
   return lo;
 }
 
-// The events of this round for an item at (ep, ad): ep = 1 + the current
-// bucket, ad = whether its A event is done.  An S event (S += R) and/or an A
-// event (R += bucket sum, held in the bucket's first partial slot after the
-// fold); (ep2, ad2) is the position after them.
-struct RedStep {
-  bool opS, opA;
-  uint32_t slot, ep2, ad2;
-};
-
-ECC_DEV RedStep red_step(const uint32_t* poff, uint32_t ep, uint32_t ad, uint32_t lo) {
-  RedStep r{false, false, 0u, ep, ad};
-  if (ep == lo) return r;                          // every event done
-  if (!ad) {
-    r.ad2 = 1;
-    if (poff[ep] > poff[ep - 1]) {                 // bucket ep-1 is not empty
-      r.opA = true;
-      r.slot = poff[ep - 1];
-      return r;
-    }
-  }
-  r.opS = true;                                    // bucket ep-1 is complete
-  r.ep2 = ep - 1;
-  r.ad2 = 0;
-  if (r.ep2 != lo) {
-    r.ad2 = 1;
-    if (poff[r.ep2] > poff[r.ep2 - 1]) {
-      r.opA = true;
-      r.slot = poff[r.ep2 - 1];
-    }
-  }
-  return r;
-}
-
-template <class C>
-struct AffRedRound {
-  using F = typename C::Fp;
-  static constexpr int N = F::N;
-  static constexpr int OPS = 2;  // op 0: S += R, op 1: R += partial
-  const AffRedArgs<C>* a;
-  RedStep st;
-  int kind_s, kind_a;
-  bool more;
-  ECC_DEV void den_c(size_t i, int j, uint32_t* d) {
-    if (j == 0) {
-      st = red_step(a->poff, a->cur_e[i], a->cur_a[i], a->lo_b[i]);
-      if (!st.opS) {
-        fe_set_one<F>(d);
-        kind_s = ADD_RET_T;
-        return;
-      }
-      uint32_t xs[N], ys[N], xr[N], yr[N];
-      a->S.load(i, xs, ys);
-      a->R.load(i, xr, yr);
-      kind_s = add_den<C>(d, xs, ys, xr, yr);
-    } else {
-      if (!st.opA) {
-        fe_set_one<F>(d);
-        kind_a = ADD_RET_T;
-        return;
-      }
-      uint32_t xr[N], yr[N], xp[N], yp[N];
-      a->R.load(i, xr, yr);
-      a->partial.load(st.slot, xp, yp);
-      kind_a = add_den<C>(d, xr, yr, xp, yp);
-    }
-  }
-  ECC_DEV void den_d(size_t i, int j, uint32_t* d) { den_c(i, j, d); }
-  ECC_DEV void finish(size_t i, const uint32_t (*inv)[N]) {
-    if (!st.opS && !st.opA) return;
-    uint32_t xr[N], yr[N];
-    a->R.load(i, xr, yr);
-    if (st.opS) {
-      uint32_t xs[N], ys[N];
-      a->S.load(i, xs, ys);
-      add_finish<C>(xs, ys, kind_s, inv[0], xs, ys, xr, yr);
-      a->S.store(i, xs, ys);
-    }
-    if (st.opA) {
-      uint32_t xp[N], yp[N];
-      a->partial.load(st.slot, xp, yp);
-      add_finish<C>(xr, yr, kind_a, inv[1], xr, yr, xp, yp);
-      a->R.store(i, xr, yr);
-    }
-    a->cur_e[i] = st.ep2;
-    a->cur_a[i] = st.ad2;
-    more |= st.ep2 != a->lo_b[i];
-  }
-};
-
-// ---- 8-limb fields: the walk's rounds with their operands staged in shared
-// memory.  Each thread owns two sets (a double buffer) of 6 G 16-byte vectors
-// holding S, R and the bucket's partial sum P (x and y of each, G = N / 4
-// vectors per element, layout [vector][thread]): one set holds the current
-// item's operands while the cp.async copies of the next item's land in the
-// other.  The thread's own column of the GAS tree (dead outside cta_invert)
-// provides 5 G of the vectors; the rest follows the GasSmem block.  The
-// item's cursor words are loaded two items ahead, its bucket offsets (the
-// event step) one item ahead together with the copies, and DCWPA's prefix
-// product one item ahead into registers.
-template <int N, int BLOCK>
-struct RedStage {
-  static constexpr int G = N / 4;
-  static constexpr int SX = 0, SY = G, RX = 2 * G, RY = 3 * G, PX = 4 * G, PY = 5 * G;
-  static constexpr int SET = 6 * G;
-  static constexpr int TREE = 5 * G;
-  static constexpr int EXTRA = 2 * SET - TREE;
-  uint4* tree;
-  uint4* extra;
-  ECC_DEV uint4* at(int set, int k) const {
-    const int s = set * SET + k;
-    return (s < TREE ? tree + s * BLOCK : extra + (s - TREE) * BLOCK) + threadIdx.x;
-  }
-  ECC_DEV void get(int set, int k0, uint32_t* r) const {
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      const uint4 p = *at(set, k0 + g);
-      r[4 * g] = p.x;
-      r[4 * g + 1] = p.y;
-      r[4 * g + 2] = p.z;
-      r[4 * g + 3] = p.w;
-    }
-  }
-};
-
-template <int N, int BLOCK>
-constexpr size_t red_smem_bytes() {
-  return sizeof(GasSmem<N, BLOCK>) + (size_t)RedStage<N, BLOCK>::EXTRA * BLOCK * sizeof(uint4);
-}
-
-// Copies item t's S and R, and the partial sum its A event adds.
-template <class C, int BLOCK>
-ECC_DEV void red_stage(const RedStage<C::Fp::N, BLOCK>& sg, int set, const AffRedArgs<C>& a,
-                       uint64_t t, const RedStep& st) {
-  using S = RedStage<C::Fp::N, BLOCK>;
-#pragma unroll
-  for (int g = 0; g < S::G; ++g) {
-    ptx::cp_async16(sg.at(set, S::SX + g), a.S.x.vec + g * a.S.x.stride + t);
-    ptx::cp_async16(sg.at(set, S::SY + g), a.S.y.vec + g * a.S.y.stride + t);
-    ptx::cp_async16(sg.at(set, S::RX + g), a.R.x.vec + g * a.R.x.stride + t);
-    ptx::cp_async16(sg.at(set, S::RY + g), a.R.y.vec + g * a.R.y.stride + t);
-  }
-  if (st.opA) {
-#pragma unroll
-    for (int g = 0; g < S::G; ++g) {
-      ptx::cp_async16(sg.at(set, S::PX + g), a.partial.x.vec + g * a.partial.x.stride + st.slot);
-      ptx::cp_async16(sg.at(set, S::PY + g), a.partial.y.vec + g * a.partial.y.stride + st.slot);
-    }
-  }
-  ptx::cp_async_commit();
-}
-
-// One round of the walk over the items [begin, end) of this CTA; returns
-// whether any of this thread's items has events left.
-template <class C, int BLOCK>
-__device__ bool red_round_staged(const AffRedArgs<C>& a, uint64_t begin, uint64_t end,
-                                 GasSmem<C::Fp::N, BLOCK>& sm, uint4* extra) {
+template <class C, bool JAC>
+__global__ void __launch_bounds__(kJacThreads, kJacCtas<C::Fp::N>) k_msm_elems(RedArgs<C> a) {
   using F = typename C::Fp;
   constexpr int N = F::N;
-  using S = RedStage<N, BLOCK>;
-  const S sg{&sm.tree[0][0][0], extra};
-  const uint64_t i0 = begin + threadIdx.x;
-  bool more = false;
-  // cursor words of item t: (ep, ad, lo)
-  uint32_t e1 = 0, a1 = 0, l1 = 0;
-  auto cursor = [&](uint64_t t, uint32_t& e, uint32_t& d, uint32_t& l) {
-    e = a.cur_e[t];
-    d = a.cur_a[t];
-    l = a.lo_b[t];
-  };
-  // ---- compress, ascending
-  uint32_t run[N];
-  fe_set_one<F>(run);
-  RedStep st0{};
-  if (i0 < end) {
-    uint32_t e0, d0, l0;
-    cursor(i0, e0, d0, l0);
-    st0 = red_step(a.poff, e0, d0, l0);
-    red_stage<C, BLOCK>(sg, 0, a, i0, st0);
-    if (i0 + BLOCK < end) cursor(i0 + BLOCK, e1, a1, l1);
-  }
-  int set = 0;
-  for (uint64_t t = i0; t < end; t += BLOCK, set ^= 1) {
-    RedStep st1{};
-    const bool next = t + BLOCK < end;
-    if (next) {
-      st1 = red_step(a.poff, e1, a1, l1);
-      red_stage<C, BLOCK>(sg, set ^ 1, a, t + BLOCK, st1);
-      if (t + 2 * BLOCK < end) cursor(t + 2 * BLOCK, e1, a1, l1);
-      ptx::cp_async_wait_prior();
-    } else {
-      ptx::cp_async_wait_all();
-    }
-    a.M.store(t, run);
-    uint32_t d[N];
-    if (st0.opS) {
-      uint32_t xs[N], ys[N], xr[N], yr[N];
-      sg.get(set, S::SX, xs);
-      sg.get(set, S::SY, ys);
-      sg.get(set, S::RX, xr);
-      sg.get(set, S::RY, yr);
-      add_den<C>(d, xs, ys, xr, yr);
-      mont_mul<F>(run, run, d);
-    }
-    if (st0.opA) {
-      uint32_t xr[N], yr[N], xp[N], yp[N];
-      sg.get(set, S::RX, xr);
-      sg.get(set, S::RY, yr);
-      sg.get(set, S::PX, xp);
-      sg.get(set, S::PY, yp);
-      add_den<C>(d, xr, yr, xp, yp);
-      mont_mul<F>(run, run, d);
-    }
-    st0 = st1;
-  }
-  // ---- inverse of the CTA's product (GAS, Section 3.2); every copy of this
-  // thread has landed (waited above), so its tree column is free
-  uint32_t inv[N];
-  cta_invert<F, BLOCK>(inv, run, sm);
-  if (i0 >= end) return false;
-  // ---- DCWPA, descending
-  const uint64_t last = i0 + ((end - 1 - i0) / BLOCK) * BLOCK;
-  uint32_t e0, d0, lo0;
-  cursor(last, e0, d0, lo0);
-  st0 = red_step(a.poff, e0, d0, lo0);
-  red_stage<C, BLOCK>(sg, 0, a, last, st0);
-  uint32_t pre0[N];
-  a.M.load(last, pre0);
-  if (last >= i0 + BLOCK) cursor(last - BLOCK, e1, a1, l1);
-  set = 0;
-  for (uint64_t t = last;; t -= BLOCK, set ^= 1) {
-    const bool next = t >= i0 + BLOCK;
-    RedStep st1{};
-    uint32_t pre1n[N], lo1 = 0;
-    if (next) {
-      st1 = red_step(a.poff, e1, a1, l1);
-      lo1 = l1;
-      red_stage<C, BLOCK>(sg, set ^ 1, a, t - BLOCK, st1);
-      a.M.load(t - BLOCK, pre1n);
-      if (t >= i0 + 2 * BLOCK) cursor(t - 2 * BLOCK, e1, a1, l1);
-      ptx::cp_async_wait_prior();
-    } else {
-      ptx::cp_async_wait_all();
-    }
-    // the item's two denominators again (recompute), then its two inverses
-    uint32_t dS[N], dA[N];
-    int kind_s = ADD_RET_T, kind_a = ADD_RET_T;
-    fe_set_one<F>(dS);
-    fe_set_one<F>(dA);
-    if (st0.opS) {
-      uint32_t xs[N], ys[N], xr[N], yr[N];
-      sg.get(set, S::SX, xs);
-      sg.get(set, S::SY, ys);
-      sg.get(set, S::RX, xr);
-      sg.get(set, S::RY, yr);
-      kind_s = add_den<C>(dS, xs, ys, xr, yr);
-    }
-    if (st0.opA) {
-      uint32_t xr[N], yr[N], xp[N], yp[N];
-      sg.get(set, S::RX, xr);
-      sg.get(set, S::RY, yr);
-      sg.get(set, S::PX, xp);
-      sg.get(set, S::PY, yp);
-      kind_a = add_den<C>(dA, xr, yr, xp, yp);
-    }
-    uint32_t invS[N], invA[N];
-    {
-      uint32_t pre1[N];
-      mont_mul<F>(pre1, pre0, dS);
-      mont_mul<F>(invA, inv, pre1);
-    }
-    mont_mul<F>(inv, inv, dA);
-    mont_mul<F>(invS, inv, pre0);
-    mont_mul<F>(inv, inv, dS);
-    if (st0.opS || st0.opA) {
-      uint32_t xr[N], yr[N];
-      sg.get(set, S::RX, xr);
-      sg.get(set, S::RY, yr);
-      if (st0.opS) {  // S += R, with R of before this round's A event
-        uint32_t xs[N], ys[N];
-        sg.get(set, S::SX, xs);
-        sg.get(set, S::SY, ys);
-        add_finish<C>(xs, ys, kind_s, invS, xs, ys, xr, yr);
-        a.S.store(t, xs, ys);
+  const uint64_t t = blockIdx.x * (uint64_t)kJacThreads + threadIdx.x;
+  if (t >= a.elems) return;
+  const MsmInst in = a.inst[find_by(a.inst, a.num, &MsmInst::elem_off, t)];
+  const uint64_t b0 = in.bucket_base + ((t - in.elem_off) << in.red_log);  // rows follow each other
+  uint32_t X[N], Y[N], Z[N], SX[N], SY[N], SZ[N];
+  jac_set_inf<F>(X, Y, Z);
+  jac_set_inf<F>(SX, SY, SZ);
+  uint32_t hi = a.poff[b0 + (1ull << in.red_log)];
+#pragma unroll 1
+  for (uint32_t i = 1u << in.red_log; i-- > 0;) {
+    const uint32_t slot = a.poff[b0 + i];
+    if (hi > slot) {
+      if constexpr (JAC) {
+        uint32_t X2[N], Y2[N], Z2[N];
+        a.jac.load(slot, X2, Y2, Z2);
+        jac_addto<C>(X, Y, Z, X2, Y2, Z2);
+      } else {
+        uint32_t x[N], y[N], H[N];
+        a.partial.load(slot, x, y);
+        if (!pt_is_inf<F>(x, y)) jac_madd<C>(X, Y, Z, x, y, H);
       }
-      if (st0.opA) {  // R += the bucket's sum
-        uint32_t xp[N], yp[N];
-        sg.get(set, S::PX, xp);
-        sg.get(set, S::PY, yp);
-        add_finish<C>(xr, yr, kind_a, invA, xr, yr, xp, yp);
-        a.R.store(t, xr, yr);
-      }
-      a.cur_e[t] = st0.ep2;
-      a.cur_a[t] = st0.ad2;
-      more |= st0.ep2 != lo0;
     }
-    if (!next) break;
-    st0 = st1;
-    lo0 = lo1;
-    fe_copy<F>(pre0, pre1n);
+    hi = slot;
+    jac_addto<C>(SX, SY, SZ, X, Y, Z);
   }
-  return more;
+  jac_store<F>(a.R + t, X, Y, Z);
+  jac_store<F>(a.S + t, SX, SY, SZ);
 }
 
-// R <- 2 R for every item whose chunk needs more than k doublings (batched PDBL)
+// Levels [l0, l1) of the tree over the blocks of 2^l1 elements: pass 0 does the
+// first kTreeLog levels of every row, a CTA per block; pass 1 the others, a CTA per
+// row.  While a level has a quad for each of its additions the quads do them.
 template <class C>
-struct AffDblRound {
-  using F = typename C::Fp;
-  static constexpr int N = F::N;
-  static constexpr int OPS = 1;
-  const AffRedArgs<C>* a;
-  uint32_t k;
-  bool live, skip;
-  ECC_DEV void den_c(size_t i, int, uint32_t* d) {
-    skip = a->rlog[i] <= k;
-    if (skip) {
-      fe_set_one<F>(d);
-      return;
-    }
-    uint32_t x[N], y[N];
-    a->R.load(i, x, y);
-    live = dbl_den<C>(d, y);
-  }
-  ECC_DEV void den_d(size_t i, int j, uint32_t* d) { den_c(i, j, d); }
-  ECC_DEV void finish(size_t i, const uint32_t (*inv)[N]) {
-    if (skip) return;
-    uint32_t x[N], y[N];
-    a->R.load(i, x, y);
-    dbl_finish<C>(x, y, live, inv[0], x, y);
-    a->R.store(i, x, y);
-  }
-};
-
-template <class C, int BLOCK>
-__global__ void __launch_bounds__(BLOCK, kGasResidentThreads / BLOCK)
-    k_msm_reduce_affine(AffRedArgs<C> a) {
+__global__ void __launch_bounds__(kJacThreads, kJacCtas<C::Fp::N>) k_msm_tree(RedArgs<C> a, int pass) {
   using F = typename C::Fp;
   constexpr int N = F::N;
-  auto& sm = gas_smem<N, BLOCK>();
-  const uint64_t begin = blockIdx.x * a.per_cta;
-  uint64_t end = begin + a.per_cta;
-  if (end > a.items) end = a.items;
-  if (end < begin) end = begin;
-  // start every item at the top of its chunk with R = S = O
-  bool more = false;
-  for (uint64_t t = begin + threadIdx.x; t < end; t += BLOCK) {
-    const RedRange rg = a.ranges[find_range(a.ranges, a.n_ranges, t)];
-    const MsmInst in = a.inst[rg.inst];
-    const uint32_t B = 1u << (in.c - 1);
-    const uint64_t local = t - rg.t0;
-    const uint32_t w = (uint32_t)(local / rg.chunks), u = (uint32_t)(local % rg.chunks);
-    const uint32_t K = 1u << in.red_log;
-    const uint32_t lo = in.bucket_base + w * B + u * K;
-    const uint32_t hi = lo + (B - u * K < K ? B - u * K : K);
-    a.lo_b[t] = lo;
-    a.rlog[t] = in.red_log;
-    a.cur_e[t] = hi;
-    a.cur_a[t] = 0;
-    uint32_t z[N];
-    fe_set_zero<F>(z);
-    a.R.store(t, z, z);
-    a.S.store(t, z, z);
-    more = true;
-  }
-  // one bounded loop: each round completes at least one event of every live
-  // item, and an item has at most 2^(rlog + 1) events
-  while (__syncthreads_or(more)) {
-    if constexpr (N == 8) {
-      extern __shared__ __align__(16) unsigned char ecc_dyn_smem[];
-      uint4* extra = reinterpret_cast<uint4*>(ecc_dyn_smem + sizeof(GasSmem<N, BLOCK>));
-      more = red_round_staged<C, BLOCK>(a, begin, end, sm, extra);
-    } else {
-      AffRedRound<C> rd{&a};
-      rd.more = false;
-      batch_round<F, BLOCK>(rd, begin, end, a.M, sm);
-      more = rd.more;
+  const uint32_t blk = blockIdx.x;
+  const MsmInst in = a.inst[pass ? find_by(a.inst, a.num, &MsmInst::row_off, blk)
+                                 : find_by(a.inst, a.num, &MsmInst::cta_off, blk)];
+  const uint32_t m = elem_log(in), first = m < kTreeLog ? m : kTreeLog;
+  const uint32_t l0 = pass ? kTreeLog : 0u, l1 = pass ? m : first;
+  if (l0 >= l1) return;
+  const uint64_t e0 = in.elem_off + ((uint64_t)(blk - (pass ? in.row_off : in.cta_off)) << l1);
+#pragma unroll 1
+  for (uint32_t l = l0; l < l1; ++l) {
+    const uint32_t per = l + 2, n_ops = per << (l1 - 1 - l), half = 1u << l;
+    const bool quads = 4 * n_ops <= kJacThreads;
+#pragma unroll 1
+    for (uint32_t o = quads ? threadIdx.x / 4 : threadIdx.x; o < n_ops; o += kJacThreads) {
+      const uint32_t pair = o / per, i = o - pair * per;
+      const uint64_t e = e0 + ((uint64_t)pair << (l + 1)) + (i == 0 || i > l ? 0u : 1u << (i - 1));
+      Jac<F>* dst = (i > l ? a.S : a.R) + e;
+      if (quads) {
+        JacReg<F> P = quad_load(dst);
+        quad_add<C>(P, quad_load(dst + half));
+        if ((threadIdx.x & 3u) == 0) jac_store<F>(dst, P.X.v, P.Y.v, P.Z.v);
+      } else {
+        uint32_t X[N], Y[N], Z[N], X2[N], Y2[N], Z2[N];
+        jac_load<F>(dst, X, Y, Z);
+        jac_load<F>(dst + half, X2, Y2, Z2);
+        jac_addto<C>(X, Y, Z, X2, Y2, Z2);
+        jac_store<F>(dst, X, Y, Z);
+      }
     }
-  }
-  // R <- 2^rlog R: as many doubling rounds as the CTA's largest chunk needs
-  for (uint32_t k = 0; k < (uint32_t)kRedLog1Max; ++k) {
-    bool want = false;
-    for (uint64_t t = begin + threadIdx.x; t < end; t += BLOCK) want |= a.rlog[t] > k;
-    if (!__syncthreads_or(want)) break;
-    AffDblRound<C> rd{&a, k};
-    batch_round<F, BLOCK>(rd, begin, end, a.M, sm);
-  }
-  for (uint64_t t = begin + threadIdx.x; t < end; t += BLOCK) {
-    uint32_t x[N], y[N];
-    Jac<F> P;
-    a.R.load(t, x, y);
-    jac_from_affine<C>(P, x, y);
-    a.out_R[t] = P;
-    a.S.load(t, x, y);
-    jac_from_affine<C>(P, x, y);
-    a.out_S[t] = P;
+    __syncthreads();
   }
 }
 
-// One later level for every window row of a set of groups.  Segment k covers
-// threads [t0, t0 + rows * chunks); its input rows have `elems` elements at
-// JR/JS + in_off, its outputs go to + out_off.
-struct LevelSeg {
-  uint64_t t0;
-  uint64_t rows;
-  uint32_t elems;
-  uint32_t chunks;
-  uint64_t in_off;
-  uint64_t out_off;
-};
-
-ECC_DEV uint32_t find_seg(const LevelSeg* s, uint32_t num, uint64_t t) {
-  uint32_t lo = 0, hi = num - 1;
-  while (lo < hi) {
-    const uint32_t mid = (lo + hi + 1) >> 1;
-    if (s[mid].t0 <= t) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
+// Window sum of a row by one quad: S + 2^red_log sum_j 2^j Q_j.
 template <class C>
-__global__ void k_msm_reduce_level(const LevelSeg* segs, uint32_t n_segs, uint64_t threads,
-                                   Jac<typename C::Fp>* JR, Jac<typename C::Fp>* JS) {
+__global__ void __launch_bounds__(64) k_msm_rows(RedArgs<C> a, uint32_t rows) {
   using F = typename C::Fp;
-  const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  if (t >= threads) return;
-  const LevelSeg sg = segs[find_seg(segs, n_segs, t)];
-  const uint64_t local = t - sg.t0;
-  const uint64_t row = local / sg.chunks;
-  const uint32_t v = (uint32_t)(local % sg.chunks);
-  const uint32_t lo = v * kRedChunkN;
-  const uint32_t hi = lo + kRedChunkN < sg.elems ? lo + kRedChunkN : sg.elems;  // exclusive
-  const Jac<F>* inR = JR + sg.in_off + row * sg.elems;
-  const Jac<F>* inS = JS + sg.in_off + row * sg.elems;
-  Jac<F> Rr, U, Ssum, E;
-  jac_set_inf<C>(Rr);
-  jac_set_inf<C>(U);
-  jac_set_inf<C>(Ssum);
-  for (uint32_t e = hi; e-- > lo;) {
-    E = inS[e];
-    jac_add<C>(Ssum, Ssum, E);
-    E = inR[e];
-    jac_add<C>(Rr, Rr, E);
-    if (e > lo) jac_add<C>(U, U, Rr);
+  const uint32_t row = (blockIdx.x * 64 + threadIdx.x) / 4;
+  if (row >= rows) return;
+  const MsmInst in = a.inst[find_by(a.inst, a.num, &MsmInst::row_off, row)];
+  const uint32_t m = elem_log(in);
+  const uint64_t e0 = in.elem_off + ((uint64_t)(row - in.row_off) << m);
+  JacReg<F> P;
+  jac_set_inf<F>(P.X.v, P.Y.v, P.Z.v);
+#pragma unroll 1
+  for (uint32_t j = m + 1; j-- > 0;) {  // add Q_(j-1), double; at last add S
+    quad_add<C>(P, quad_load(j > 0 ? a.R + e0 + (1ull << (j - 1)) : a.S + e0));
+#pragma unroll 1
+    for (uint32_t s = j > 1 ? 1u : j * in.red_log; s > 0; --s) quad_dbl<C>(P);
   }
-  jac_add<C>(Ssum, Ssum, U);
-  if (sg.chunks > 1) {
-    for (int k = 0; k < kRedLogN; ++k) jac_dbl<C>(Rr, Rr);
-  }
-  JR[sg.out_off + row * sg.chunks + v] = Rr;
-  JS[sg.out_off + row * sg.chunks + v] = Ssum;
+  if ((threadIdx.x & 3u) == 0) jac_store<F>(a.row + row, P.X.v, P.Y.v, P.Z.v);
 }
 
-// result_i = sum_w 2^(c w) S_w (Horner), converted to canonical affine limbs;
-// instance i's window sums are S[fin[i] + w].  Thread t takes instance
-// order[t]: the host lists the instances grouped by window width, so the lanes
-// of a warp run chains of one length (a warp executes the longest chain among
-// its lanes).
+// result_i = sum_w 2^(c w) S_w (Horner) by one quad, converted to canonical affine
+// limbs.  Quad t takes instance order[t]: the host lists the instances grouped by
+// window width, so the quads of a warp run chains of one length.
 template <class C>
-__global__ void k_msm_combine(const MsmInst* inst, const uint64_t* fin, const uint32_t* order,
-                              uint32_t num, const Jac<typename C::Fp>* S, const MsmDevHdr* hdr,
-                              uint32_t* out_all) {
+__global__ void __launch_bounds__(32) k_msm_combine(RedArgs<C> a, const uint32_t* order, const MsmDevHdr* hdr,
+                                                    uint32_t* out_all) {
   using F = typename C::Fp;
   constexpr int N = F::N;
-  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= num) return;
+  const uint32_t t = (blockIdx.x * 32 + threadIdx.x) / 4;
+  if (t >= a.num) return;
   const uint32_t id = order[t];
+  const bool write = (threadIdx.x & 3u) == 0;
+  uint32_t* o = out_all + (uint64_t)id * 2 * N;
   if (hdr && hdr->failed) {  // refused sizes: O, written (0, 0)
-    for (int q = 0; q < 2 * N; ++q) out_all[(uint64_t)id * 2 * N + q] = 0;
+    for (int q = 0; q < 2 * N && write; ++q) o[q] = 0;
     return;
   }
-  const uint32_t c = inst[id].c, W = inst[id].Wr;
-  const Jac<F>* Sw = S + fin[id];
-  Jac<F> acc = Sw[W - 1];
-  for (int w = (int)W - 2; w >= 0; --w) {
-    for (uint32_t s = 0; s < c; ++s) jac_dbl_inl<C>(acc, acc);
-    jac_add_inl<C>(acc, acc, Sw[w]);
+  const MsmInst in = a.inst[id];
+  JacReg<F> P;
+  jac_set_inf<F>(P.X.v, P.Y.v, P.Z.v);
+#pragma unroll 1
+  for (uint32_t w = in.Wr; w-- > 0;) {
+#pragma unroll 1
+    for (uint32_t s = w + 1 < in.Wr ? in.c : 0u; s > 0; --s) quad_dbl<C>(P);
+    quad_add<C>(P, quad_load(a.row + in.row_off + w));
   }
   uint32_t x[N], y[N];
-  jac_to_affine<C>(x, y, acc);
+  jac_to_affine<F>(x, y, P);
   from_mont<F>(x, x);
   from_mont<F>(y, y);
-  uint32_t* o = out_all + (uint64_t)id * 2 * N;
+  if (!write) return;
 #pragma unroll
   for (int q = 0; q < N; ++q) {
     o[q] = x[q];

@@ -5,8 +5,6 @@
 // and replayed.
 #pragma once
 #include <algorithm>
-#include <map>
-#include <tuple>
 #include <vector>
 
 #include "internal.h"
@@ -36,7 +34,51 @@ inline int windows_for(int curve, int c) { return (scalar_bits(curve) + 1 + c - 
 struct Layout {
   std::vector<MsmInst> inst;
   uint64_t buckets = 0, entries_max = 0, n_chunks = 0, total_points = 0;
+  uint64_t elems = 0;          // reduction elements
+  uint32_t rows = 0, ctas = 0; // bucket rows, CTAs of the reduction tree's first pass
+  bool direct = false;         // Jacobian accumulation
+  int ch_log = kAccLog;        // log2 of the entries per chunk
 };
+
+// Entries up to which one Jacobian thread per chunk accumulates faster than batched
+// affine rounds.  Whole calls of n points, rounds / threads: BN254 n = 2^15 1.90 /
+// 1.07 ms, 2^18 2.37 / 1.82, 2^19 (8.9 M entries) 3.04 / 2.63, 2^20 (16.8 M) 4.34 /
+// 4.32; BLS12-381 2^15 3.58 / 1.91, 2^18 5.09 / 3.86, 2^19 6.14 / 5.47, 2^20 8.69 / 8.63.
+constexpr uint64_t kDirectEntries = 12u << 20;
+
+// log2 of the buckets per reduction element: the caller's override, or the most (up
+// to kRedLog1Default) that leaves two CTAs of elements per SM: fewer elements are
+// longer serial sums, more of them are work for the tree (2^18 BN254 points, 278000
+// buckets: 1.95, 1.86, 1.82, 1.82, 1.90, 2.15 ms a call for 0 .. 5).
+inline int red_log(int curve, uint64_t n, int c, uint64_t buckets) {
+  int k = msm_reduce_override(curve, n);
+  if (k <= 0) {
+    const uint64_t threads = (uint64_t)device_sm_count() * kJacThreads * 2;
+    for (k = 0; k < kRedLog1Default && (buckets >> (k + 1)) >= threads;) ++k;
+  }
+  return std::min(k, c - 1);
+}
+
+// Chunks, accumulation form and reduction layout of the planned instances.
+template <int N>
+void finish_plan(int curve, Layout& L, const uint64_t* sizes, uint64_t size_all) {
+  for (size_t i = 0; i < L.inst.size(); ++i) {
+    MsmInst& m = L.inst[i];
+    m.red_log = (uint32_t)red_log(curve, sizes ? sizes[i] : size_all, (int)m.c, L.buckets);
+    m.elem_off = L.elems;
+    m.row_off = L.rows;
+    m.cta_off = L.ctas;
+    L.elems += (uint64_t)m.Wr << elem_log(m);
+    L.rows += m.Wr;
+    L.ctas += tree_ctas(m);
+  }
+  L.direct = L.entries_max < kDirectEntries;
+  if (L.direct) {  // chunks of 8 to 32 entries, about four for each resident thread
+    constexpr uint32_t chunks = N <= 8 ? 1u << 18 : 1u << 17;
+    for (L.ch_log = 3; L.ch_log < kAccLog && (L.entries_max >> (L.ch_log + 1)) >= chunks;) ++L.ch_log;
+  }
+  L.n_chunks = (L.entries_max + (1u << L.ch_log) - 1) >> L.ch_log;
+}
 
 // Instance sizes held in device memory (capture-time capacity): rows are
 // sizes[num] (sizes_mode, resident bases) or offsets[num + 1]; every instance
@@ -63,11 +105,12 @@ cudaError_t run_set(int curve, const Layout& L, const uint32_t* bases_mont, cons
   auto up = [](uint64_t b) { return (b + 255) / 256 * 256; };
   const uint64_t sz_inst = up(num * sizeof(MsmInst));
   const uint64_t sz_b1 = up((B + 1) * 4);
-  const uint64_t sz_kv = up(kAccChunk * NC * 4), sz_cur = up(NC * 4);
+  const uint64_t sz_kv = up((NC << L.ch_log) * 4), sz_cur = up(NC * 4);
   const uint64_t sz_S = soa_bytes<F>(NC), sz_P = soa_bytes<F>(n_part);
   const uint64_t sz_ops = up(n_part * 4);
-  // per chunk: running sum (x, y) and prefix product
-  constexpr uint64_t kChunkArrays = 3;
+  // per chunk: running sum (x, y) and prefix product; per partial sum: x, y and
+  // prefix product, or X, Y and Z
+  const uint64_t kChunkArrays = L.direct ? 0 : 3;
   const uint64_t sz_hdr = up(sizeof(MsmDevHdr));
   const uint64_t sz_pts = raw_points ? up(std::max<uint64_t>(L.total_points, 1) * 2 * N * 4) : 0;
   const uint64_t bytes = sz_inst + sz_hdr + sz_pts + 5 * sz_b1 + sz_kv + sz_cur + kChunkArrays * sz_S +
@@ -114,12 +157,12 @@ cudaError_t run_set(int curve, const Layout& L, const uint32_t* bases_mont, cons
   if (e != cudaSuccess) return e;
   e = cudaMemcpyAsync(cursor, off, B * 4, cudaMemcpyDeviceToDevice, st);
   if (e != cudaSuccess) return e;
-  if (B) k_msm_npart<<<(unsigned)((B + 255) / 256), 256, 0, st>>>(off, (uint32_t)B, npart);
+  if (B) k_msm_npart<<<(unsigned)((B + 255) / 256), 256, 0, st>>>(off, (uint32_t)B, L.ch_log, npart);
   e = exclusive_scan(npart, B, poff, st);
   if (e != cudaSuccess) return e;
   if (L.total_points)
     k_msm_scatter<C><<<pb, 256, 0, st>>>(d_inst, num, scalars, L.total_points, hdr, cursor, vals, NC,
-                                          cur);
+                                          L.ch_log, cur);
   phase_mark(1, st);
   // ---- 3: bucket accumulation (batched affine, one launch)
   AccArgs<C> a;
@@ -133,14 +176,19 @@ cudaError_t run_set(int curve, const Layout& L, const uint32_t* bases_mont, cons
   a.S = PtSoA<F>{SoA<F>{sbuf, NC}, SoA<F>{sbuf + sz_S / 16, NC}};
   a.M = SoA<F>{sbuf + 2 * sz_S / 16, NC};
   a.partial = PtSoA<F>{SoA<F>{pbuf, n_part}, SoA<F>{pbuf + sz_P / 16, n_part}};
-  // persistent CTAs; each takes an equal share of the chunks the sort filled
-  uint64_t ctas = (uint64_t)device_sm_count() * kGasCtasPerSm;
-  ctas = std::max<uint64_t>(1, std::min<uint64_t>(ctas, (NC + 31) / 32));
   const size_t smem = sizeof(GasSmem<N, kAccBlock>);
-  e = cudaFuncSetAttribute(k_msm_accumulate<C, kAccBlock>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  k_msm_accumulate<C, kAccBlock><<<(unsigned)ctas, kAccBlock, smem, st>>>(a);
+  const JacSoA<F> jac{SoA<F>{pbuf, n_part}, SoA<F>{pbuf + sz_P / 16, n_part}, SoA<F>{pbuf + 2 * sz_P / 16, n_part}};
+  if (L.direct) {
+    k_msm_accumulate_jac<C><<<(unsigned)((NC + kJacThreads - 1) / kJacThreads), kJacThreads, 0, st>>>(a, jac, L.ch_log);
+  } else {
+    // persistent CTAs; each takes an equal share of the chunks the sort filled
+    uint64_t ctas = (uint64_t)device_sm_count() * kGasCtasPerSm;
+    ctas = std::max<uint64_t>(1, std::min<uint64_t>(ctas, (NC + 31) / 32));
+    e = cudaFuncSetAttribute(k_msm_accumulate<C, kAccBlock>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_msm_accumulate<C, kAccBlock><<<(unsigned)ctas, kAccBlock, smem, st>>>(a);
+  }
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   phase_mark(2, st);
@@ -152,72 +200,22 @@ cudaError_t run_set(int curve, const Layout& L, const uint32_t* bases_mont, cons
     f.partial = a.partial;
     f.M = SoA<F>{pbuf + 2 * sz_P / 16, n_part};
     f.ops = fold_ops;
-    e = cudaFuncSetAttribute(k_msm_fold<C, kAccBlock>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_msm_fold<C, kAccBlock><<<(unsigned)(device_sm_count() * kGasCtasPerSm), kAccBlock, smem, st>>>(f);
+    f.jac = jac;
+    if (L.direct) {
+      const unsigned ctas = (unsigned)std::min<uint64_t>((uint64_t)device_sm_count() * 4, (n_part + 63) / 64);
+      k_msm_fold<C, kJacThreads, true><<<ctas, kJacThreads, 0, st>>>(f);
+    } else {
+      e = cudaFuncSetAttribute(k_msm_fold<C, kAccBlock, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)smem);
+      if (e != cudaSuccess) return e;
+      k_msm_fold<C, kAccBlock, false>
+          <<<(unsigned)(device_sm_count() * kGasCtasPerSm), kAccBlock, smem, st>>>(f);
+    }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   phase_mark(3, st);
-  // ---- 4: bucket reduction.  Instances are grouped by window width (same
-  // level structure); the items of every level are laid out group-major so a
-  // level of all groups is one launch.
-  // groups by (window width, bucket rows per instance, first-level chunk)
-  std::map<std::tuple<uint32_t, uint32_t, uint32_t>, std::vector<uint32_t>> groups;
-  for (int i = 0; i < num; ++i)
-    groups[{L.inst[i].c, L.inst[i].Wr, L.inst[i].red_log}].push_back((uint32_t)i);
-  std::vector<std::vector<uint32_t>> elems;  // per group: elements per row, by level
-  std::vector<uint64_t> rows;
-  for (auto& g : groups) {
-    std::vector<uint32_t> el{1u << (std::get<0>(g.first) - 1)};
-    const uint32_t K = 1u << std::get<2>(g.first);
-    el.push_back((el[0] + K - 1) / K);
-    while (el.back() > 1) el.push_back((el.back() + kRedChunkN - 1) / kRedChunkN);
-    elems.push_back(el);
-    rows.push_back((uint64_t)g.second.size() * std::get<1>(g.first));
-  }
-  const size_t n_groups = elems.size();
-  size_t levels = 0;
-  for (auto& el : elems) levels = std::max(levels, el.size() - 1);
-  // Jacobian arrays: level 1 of every group, then level 2 of every group, ...
-  std::vector<std::vector<uint64_t>> lvl_off(levels + 1, std::vector<uint64_t>(n_groups, 0));
-  uint64_t jac_total = 0;
-  for (size_t l = 1; l <= levels; ++l) {
-    for (size_t g = 0; g < n_groups; ++g) {
-      lvl_off[l][g] = jac_total;
-      if (l < elems[g].size()) jac_total += rows[g] * elems[g][l];
-    }
-  }
-  const uint64_t items = levels == 0 ? 0 : (levels >= 2 ? lvl_off[2][0] : jac_total);
-  std::vector<RedRange> ranges;
-  std::vector<uint64_t> fin(num, 0);
-  {
-    size_t g = 0;
-    uint64_t t = 0;
-    for (auto& grp : groups) {
-      const size_t last = elems[g].size() - 1;
-      for (size_t ii = 0; ii < grp.second.size(); ++ii) {
-        const uint32_t id = grp.second[ii];
-        ranges.push_back(RedRange{t, id, elems[g][1]});
-        t += (uint64_t)L.inst[id].Wr * elems[g][1];
-        fin[id] = lvl_off[last][g] + (uint64_t)ii * L.inst[id].Wr;
-      }
-      ++g;
-    }
-  }
-  std::vector<std::vector<LevelSeg>> segs(levels + 1);
-  std::vector<uint64_t> seg_threads(levels + 1, 0);
-  for (size_t l = 2; l <= levels; ++l) {
-    for (size_t g = 0; g < n_groups; ++g) {
-      if (l >= elems[g].size()) continue;
-      segs[l].push_back(LevelSeg{seg_threads[l], rows[g], elems[g][l - 1], elems[g][l],
-                                 lvl_off[l - 1][g], lvl_off[l][g]});
-      seg_threads[l] += rows[g] * elems[g][l];
-    }
-  }
-  uint64_t seg_words = 0;
-  for (size_t l = 2; l <= levels; ++l) seg_words += up(segs[l].size() * sizeof(LevelSeg));
+  // ---- 4: bucket reduction
   // combination order: instances grouped by (rows, window width), so a warp's
   // Horner chains have one length
   std::vector<uint32_t> order(num);
@@ -225,79 +223,43 @@ cudaError_t run_set(int curve, const Layout& L, const uint32_t* bases_mont, cons
   std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) {
     return std::make_pair(L.inst[x].Wr, L.inst[x].c) < std::make_pair(L.inst[y].Wr, L.inst[y].c);
   });
-  const uint64_t sz_red = up(ranges.size() * sizeof(RedRange)) + up(num * 8ull) + up(num * 4ull) + seg_words +
-                          2 * up(jac_total * sizeof(Jac<F>)) + 4 * up(items * 4) +
-                          5 * soa_bytes<F>(std::max<uint64_t>(items, 1)) + 256;
   Scratch rs;
-  e = rs.alloc(sz_red, st);
+  e = rs.alloc(up(num * 4ull) + 2 * up(L.elems * sizeof(Jac<F>)) + up(L.rows * sizeof(Jac<F>)), st);
   if (e != cudaSuccess) return e;
   char* q = rs.as<char>();
   auto take_r = [&](uint64_t b) { char* r = q; q += up(b); return r; };
-  RedRange* d_ranges = reinterpret_cast<RedRange*>(take_r(ranges.size() * sizeof(RedRange)));
-  uint64_t* d_fin = reinterpret_cast<uint64_t*>(take_r(num * 8ull));
   uint32_t* d_order = reinterpret_cast<uint32_t*>(take_r(num * 4ull));
-  std::vector<LevelSeg*> d_segs(levels + 1, nullptr);
-  for (size_t l = 2; l <= levels; ++l) d_segs[l] = reinterpret_cast<LevelSeg*>(take_r(segs[l].size() * sizeof(LevelSeg)));
-  Jac<F>* JR = reinterpret_cast<Jac<F>*>(take_r(jac_total * sizeof(Jac<F>)));
-  Jac<F>* JS = reinterpret_cast<Jac<F>*>(take_r(jac_total * sizeof(Jac<F>)));
-  uint32_t* cur_e = reinterpret_cast<uint32_t*>(take_r(items * 4));
-  uint32_t* cur_a = reinterpret_cast<uint32_t*>(take_r(items * 4));
-  uint32_t* lo_b = reinterpret_cast<uint32_t*>(take_r(items * 4));
-  uint32_t* rlog = reinterpret_cast<uint32_t*>(take_r(items * 4));
-  const uint64_t IT = std::max<uint64_t>(items, 1);
-  uint4* rbuf = reinterpret_cast<uint4*>(take_r(5 * soa_bytes<F>(IT)));
-  e = upload_words(d_ranges, ranges.data(), ranges.size() * sizeof(RedRange), st);
-  if (e != cudaSuccess) return e;
-  e = upload_words(d_fin, fin.data(), num * 8ull, st);
-  if (e != cudaSuccess) return e;
   e = upload_words(d_order, order.data(), num * 4ull, st);
   if (e != cudaSuccess) return e;
-  for (size_t l = 2; l <= levels; ++l) {
-    e = upload_words(d_segs[l], segs[l].data(), segs[l].size() * sizeof(LevelSeg), st);
-    if (e != cudaSuccess) return e;
-  }
-  if (items) {
-    AffRedArgs<C> r;
-    r.inst = d_inst;
-    r.ranges = d_ranges;
-    r.n_ranges = (uint32_t)ranges.size();
-    r.items = items;
-    r.poff = poff;
-    r.partial = a.partial;
-    const uint64_t ss = soa_bytes<F>(IT) / 16;
-    r.R = PtSoA<F>{SoA<F>{rbuf, IT}, SoA<F>{rbuf + ss, IT}};
-    r.S = PtSoA<F>{SoA<F>{rbuf + 2 * ss, IT}, SoA<F>{rbuf + 3 * ss, IT}};
-    r.M = SoA<F>{rbuf + 4 * ss, IT};
-    r.cur_e = cur_e;
-    r.cur_a = cur_a;
-    r.lo_b = lo_b;
-    r.rlog = rlog;
-    r.out_R = JR;
-    r.out_S = JS;
-    uint64_t rctas = (uint64_t)device_sm_count() * kGasCtasPerSm;
-    uint64_t rper = (items + rctas - 1) / rctas;
-    if (rper < 32) rper = 32;
-    rctas = (items + rper - 1) / rper;
-    r.per_cta = rper;
-    const size_t rsmem = N == 8 ? red_smem_bytes<N, kAccBlock>() : smem;
-    e = cudaFuncSetAttribute(k_msm_reduce_affine<C, kAccBlock>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsmem);
-    if (e != cudaSuccess) return e;
-    k_msm_reduce_affine<C, kAccBlock><<<(unsigned)rctas, kAccBlock, rsmem, st>>>(r);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  for (size_t l = 2; l <= levels; ++l) {
-    if (!seg_threads[l]) continue;
-    k_msm_reduce_level<C><<<(unsigned)((seg_threads[l] + 63) / 64), 64, 0, st>>>(
-        d_segs[l], (uint32_t)segs[l].size(), seg_threads[l], JR, JS);
+  RedArgs<C> r;
+  r.inst = d_inst;
+  r.num = (uint32_t)num;
+  r.elems = L.elems;
+  r.poff = poff;
+  r.partial = a.partial;
+  r.jac = jac;
+  r.R = reinterpret_cast<Jac<F>*>(take_r(L.elems * sizeof(Jac<F>)));
+  r.S = reinterpret_cast<Jac<F>*>(take_r(L.elems * sizeof(Jac<F>)));
+  r.row = reinterpret_cast<Jac<F>*>(take_r(L.rows * sizeof(Jac<F>)));
+  if (L.elems) {
+    const unsigned eb = (unsigned)((L.elems + kJacThreads - 1) / kJacThreads);
+    if (L.direct) {
+      k_msm_elems<C, true><<<eb, kJacThreads, 0, st>>>(r);
+    } else {
+      k_msm_elems<C, false><<<eb, kJacThreads, 0, st>>>(r);
+    }
+    uint32_t m = 0;
+    for (const MsmInst& in : L.inst) m = std::max(m, elem_log(in));
+    if (m > 0) k_msm_tree<C><<<L.ctas, kJacThreads, 0, st>>>(r, 0);
+    if (m > kTreeLog) k_msm_tree<C><<<L.rows, kJacThreads, 0, st>>>(r, 1);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   phase_mark(4, st);
-  // ---- 5: window combination, every instance in one launch
+  // ---- 5: window sums and their combination, every instance in one launch
   if (num) {
-    k_msm_combine<C><<<(num + 31) / 32, 32, 0, st>>>(d_inst, d_fin, d_order, (uint32_t)num, JS, hdr, out);
+    k_msm_rows<C><<<(L.rows + 15) / 16, 64, 0, st>>>(r, L.rows);
+    k_msm_combine<C><<<(num + 7) / 8, 32, 0, st>>>(r, d_order, hdr, out);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -307,7 +269,8 @@ cudaError_t run_set(int curve, const Layout& L, const uint32_t* bases_mont, cons
 
 // pre_c > 0: the bases hold precomputed window multiples for width pre_c,
 // pre_stride points apart.
-inline Layout plan(int curve, uint32_t num, const uint64_t* sizes, const uint64_t* point_off,
+template <int N>
+Layout plan(int curve, uint32_t num, const uint64_t* sizes, const uint64_t* point_off,
             const uint64_t* scalar_off, const int* cs, int pre_c = 0, uint64_t pre_stride = 0) {
   Layout L;
   L.inst.resize(num);
@@ -321,12 +284,11 @@ inline Layout plan(int curve, uint32_t num, const uint64_t* sizes, const uint64_
     m.scalar_off = scalar_off[i];
     m.pre_stride = pre_c > 0 ? pre_stride : 0;
     m.Wr = pre_c > 0 ? 1u : m.W;
-    m.red_log = (uint32_t)std::min<int>(msm_reduce_log(curve, sizes[i]), (int)m.c - 1);
     L.buckets += (uint64_t)m.Wr << (m.c - 1);
     L.entries_max += (uint64_t)m.W * m.n;
     L.total_points += m.n;
   }
-  L.n_chunks = (L.entries_max + kAccChunk - 1) / kAccChunk;
+  finish_plan<N>(curve, L, sizes, 0);
   return L;
 }
 
@@ -341,7 +303,7 @@ cudaError_t msm_points(int curve, uint32_t num, const uint64_t* offsets, const u
     poff[i] = offsets[i] - offsets[0];
     soff[i] = poff[i];
   }
-  Layout L = plan(curve, num, sizes.data(), poff.data(), soff.data(), nullptr);
+  Layout L = plan<C::Fp::N>(curve, num, sizes.data(), poff.data(), soff.data(), nullptr);
   (void)total;
   return run_set<C>(curve, L, nullptr, scalars + offsets[0] * 8, out, st, nullptr,
                     points + offsets[0] * 2 * F::N);
@@ -350,21 +312,20 @@ cudaError_t msm_points(int curve, uint32_t num, const uint64_t* offsets, const u
 // The uniform per-instance layout of a device-sized batch (window width c, or
 // the library's width for bases with window multiples of width pre_c) with the
 // capacity totals: cap scalar rows in num instances.
-inline Layout plan_uniform(int curve, uint32_t num, int c, uint64_t cap, int pre_c, uint64_t pre_stride) {
+template <int N>
+Layout plan_uniform(int curve, uint32_t num, int c, uint64_t cap, int pre_c, uint64_t pre_stride) {
   Layout L;
   MsmInst m{};
   m.c = (uint32_t)(pre_c > 0 ? pre_c : c);
   m.W = (uint32_t)windows_for(curve, (int)m.c);
   m.Wr = pre_c > 0 ? 1u : m.W;
   m.pre_stride = pre_c > 0 ? pre_stride : 0;
-  const uint64_t mean = num ? std::max<uint64_t>(cap / num, 2) : 2;
-  m.red_log = (uint32_t)std::min<int>(msm_reduce_log(curve, mean), (int)m.c - 1);
   L.inst.assign(num, m);
   for (uint32_t i = 0; i < num; ++i) L.inst[i].bucket_base = (uint32_t)(i * ((uint64_t)m.Wr << (m.c - 1)));
   L.buckets = (uint64_t)num * ((uint64_t)m.Wr << (m.c - 1));
   L.entries_max = cap * m.W;
   L.total_points = cap;
-  L.n_chunks = (L.entries_max + kAccChunk - 1) / kAccChunk;
+  finish_plan<N>(curve, L, nullptr, num ? std::max<uint64_t>(cap / num, 2) : 2);
   return L;
 }
 
@@ -373,7 +334,7 @@ inline Layout plan_uniform(int curve, uint32_t num, int c, uint64_t cap, int pre
 template <class C>
 cudaError_t msm_points_dev(int curve, uint32_t num, uint64_t cap, const uint64_t* offsets, int c,
                            const uint32_t* points, const uint32_t* scalars, uint32_t* out, cudaStream_t st) {
-  Layout L = plan_uniform(curve, num, c, cap, 0, 0);
+  Layout L = plan_uniform<C::Fp::N>(curve, num, c, cap, 0, 0);
   DevRows dev{offsets, 0, 0, cap};
   return run_set<C>(curve, L, nullptr, scalars, out, st, &dev, points);
 }
@@ -440,7 +401,7 @@ cudaError_t precompute_t(Bases* bs, int c, cudaStream_t st) {
 template <class C>
 cudaError_t msm_bases_dev_t(Bases* bs, uint32_t num, uint64_t cap, const uint64_t* sizes, int c,
                             const uint32_t* scalars, uint32_t* out, cudaStream_t st) {
-  Layout L = plan_uniform(bs->curve, num, c, cap, bs->pre ? bs->pre_c : 0, bs->n);
+  Layout L = plan_uniform<C::Fp::N>(bs->curve, num, c, cap, bs->pre ? bs->pre_c : 0, bs->n);
   DevRows dev{sizes, 1, bs->n, cap};
   return run_set<C>(bs->curve, L, bs->pre ? bs->pre : bs->mont, scalars, out, st, &dev);
 }
@@ -457,7 +418,7 @@ cudaError_t msm_bases_t(Bases* bs, uint32_t num_vectors, const uint64_t* vec_siz
     soff[v] = acc;
     acc += sizes[v];
   }
-  Layout L = plan(bs->curve, num_vectors, sizes.data(), poff.data(), soff.data(), nullptr,
+  Layout L = plan<C::Fp::N>(bs->curve, num_vectors, sizes.data(), poff.data(), soff.data(), nullptr,
                   bs->pre ? bs->pre_c : 0, bs->n);
   return run_set<C>(bs->curve, L, bs->pre ? bs->pre : bs->mont, scalars, out, st);
 }
