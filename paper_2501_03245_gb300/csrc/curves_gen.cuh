@@ -102,6 +102,29 @@ struct Secp256k1 {
     switch (i) { case 0: return 0xd0364141u; case 1: return 0xbfd25e8cu; case 2: return 0xaf48a03bu; case 3: return 0xbaaedce6u; case 4: return 0xfffffffeu; case 5: return 0xffffffffu; case 6: return 0xffffffffu; case 7: return 0xffffffffu; default: return 0u; }
   }
   static constexpr int SCALAR_BITS = 256;
+  static constexpr bool GLV = true;
+  static constexpr int GLV_BITS = 128;  // |k1|, |k2| < 2^GLV_BITS
+  ECC_DEV static constexpr uint32_t glv_beta(int i) {
+    switch (i) { case 0: return 0x8e6afa40u; case 1: return 0x3ec693d6u; case 2: return 0xed0a766au; case 3: return 0x630fb68au; case 4: return 0x53cbcb16u; case 5: return 0x919bb861u; case 6: return 0x9a83f8efu; case 7: return 0x851695d4u; default: return 0u; }
+  }
+  ECC_DEV static constexpr uint32_t glv_g1(int i) {
+    switch (i) { case 0: return 0x0fddd146u; case 1: return 0x5fbc92c1u; case 2: return 0x9d44cfd9u; case 3: return 0x57c1108du; case 4: return 0xa8e2f3f6u; case 5: return 0x14ca50f7u; case 6: return 0x00000001u; default: return 0u; }
+  }
+  ECC_DEV static constexpr uint32_t glv_g2(int i) {
+    switch (i) { case 0: return 0x71e8ca80u; case 1: return 0x3daa8a14u; case 2: return 0x9284eb15u; case 3: return 0xe86c90e4u; case 4: return 0xa7d46bcdu; case 5: return 0x3086d221u; case 6: return 0x00000000u; default: return 0u; }
+  }
+  ECC_DEV static constexpr uint32_t glv_a1(int i) {
+    switch (i) { case 0: return 0xf5401b3du; case 1: return 0x90ab8056u; case 2: return 0xfef177d7u; case 3: return 0x1bbc8129u; case 4: return 0xffffffffu; default: return 0u; }
+  }
+  ECC_DEV static constexpr uint32_t glv_a2(int i) {
+    switch (i) { case 0: return 0x6d7b14ebu; case 1: return 0x17936f1bu; case 2: return 0x582b9432u; case 3: return 0xcf792ddeu; case 4: return 0xffffffffu; default: return 0u; }
+  }
+  ECC_DEV static constexpr uint32_t glv_b1(int i) {
+    switch (i) { case 0: return 0x9284eb15u; case 1: return 0xe86c90e4u; case 2: return 0xa7d46bcdu; case 3: return 0x3086d221u; case 4: return 0x00000000u; default: return 0u; }
+  }
+  ECC_DEV static constexpr uint32_t glv_b2(int i) {
+    switch (i) { case 0: return 0x62bb3028u; case 1: return 0xa83eef72u; case 2: return 0x571d0c09u; case 3: return 0xeb35af08u; case 4: return 0xfffffffeu; default: return 0u; }
+  }
 };
 
 struct P256Fp {
@@ -178,6 +201,7 @@ struct P256 {
     switch (i) { case 0: return 0xfc632551u; case 1: return 0xf3b9cac2u; case 2: return 0xa7179e84u; case 3: return 0xbce6faadu; case 4: return 0xffffffffu; case 5: return 0xffffffffu; case 6: return 0x00000000u; case 7: return 0xffffffffu; default: return 0u; }
   }
   static constexpr int SCALAR_BITS = 256;
+  static constexpr bool GLV = false;
 };
 
 struct BN254Fp {
@@ -250,6 +274,29 @@ struct BN254 {
     switch (i) { case 0: return 0xf0000001u; case 1: return 0x43e1f593u; case 2: return 0x79b97091u; case 3: return 0x2833e848u; case 4: return 0x8181585du; case 5: return 0xb85045b6u; case 6: return 0xe131a029u; case 7: return 0x30644e72u; default: return 0u; }
   }
   static constexpr int SCALAR_BITS = 254;
+  static constexpr bool GLV = true;
+  static constexpr int GLV_BITS = 126;  // |k1|, |k2| < 2^GLV_BITS
+  ECC_DEV static constexpr uint32_t glv_beta(int i) {
+    switch (i) { case 0: return 0xd782e155u; case 1: return 0x71930c11u; case 2: return 0xffbe3323u; case 3: return 0xa6bb947cu; case 4: return 0xd4741444u; case 5: return 0xaa303344u; case 6: return 0x26594943u; case 7: return 0x2c3b3f0du; default: return 0u; }
+  }
+  ECC_DEV static constexpr uint32_t glv_g1(int i) {
+    switch (i) { case 0: return 0x773a6ef3u; case 1: return 0x6eb9c714u; case 2: return 0xc7e0b3d7u; case 3: return 0xd91d232eu; case 4: return 0x00000002u; case 5: return 0x00000000u; case 6: return 0x00000000u; default: return 0u; }
+  }
+  ECC_DEV static constexpr uint32_t glv_g2(int i) {
+    switch (i) { case 0: return 0x5eaa26dau; case 1: return 0xa5e38cfbu; case 2: return 0x391eb18du; case 3: return 0x7a7bd9d4u; case 4: return 0xa773d2cfu; case 5: return 0x4ccef014u; case 6: return 0x00000002u; default: return 0u; }
+  }
+  ECC_DEV static constexpr uint32_t glv_a1(int i) {
+    switch (i) { case 0: return 0x6b2dec1du; case 1: return 0x762cda97u; case 2: return 0xffffffffu; case 3: return 0xffffffffu; case 4: return 0xffffffffu; default: return 0u; }
+  }
+  ECC_DEV static constexpr uint32_t glv_a2(int i) {
+    switch (i) { case 0: return 0xeddedaf5u; case 1: return 0xf41b1eabu; case 2: return 0x1147a602u; case 3: return 0x90b27db7u; case 4: return 0xffffffffu; default: return 0u; }
+  }
+  ECC_DEV static constexpr uint32_t glv_b1(int i) {
+    switch (i) { case 0: return 0x7d4f1128u; case 1: return 0x8211bbebu; case 2: return 0xeeb859fcu; case 3: return 0x6f4d8248u; case 4: return 0x00000000u; default: return 0u; }
+  }
+  ECC_DEV static constexpr uint32_t glv_b2(int i) {
+    switch (i) { case 0: return 0x6b2dec1du; case 1: return 0x762cda97u; case 2: return 0xffffffffu; case 3: return 0xffffffffu; case 4: return 0xffffffffu; default: return 0u; }
+  }
 };
 
 struct BLS12_381Fp {
@@ -322,6 +369,7 @@ struct BLS12_381 {
     switch (i) { case 0: return 0x00000001u; case 1: return 0xffffffffu; case 2: return 0xfffe5bfeu; case 3: return 0x53bda402u; case 4: return 0x09a1d805u; case 5: return 0x3339d808u; case 6: return 0x299d7d48u; case 7: return 0x73eda753u; default: return 0u; }
   }
   static constexpr int SCALAR_BITS = 255;
+  static constexpr bool GLV = false;
 };
 
 struct SM2Fp {
@@ -398,6 +446,7 @@ struct SM2 {
     switch (i) { case 0: return 0x39d54123u; case 1: return 0x53bbf409u; case 2: return 0x21c6052bu; case 3: return 0x7203df6bu; case 4: return 0xffffffffu; case 5: return 0xffffffffu; case 6: return 0xffffffffu; case 7: return 0xfffffffeu; default: return 0u; }
   }
   static constexpr int SCALAR_BITS = 256;
+  static constexpr bool GLV = false;
 };
 
 }  // namespace ecc

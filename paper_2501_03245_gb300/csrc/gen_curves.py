@@ -94,6 +94,75 @@ def field(name, q):
     return s, n, R
 
 
+# The endomorphism (x, y) -> (beta x, y) of the curves with a = 0 multiplies the points
+# of a group of prime order by lambda, beta and lambda cube roots of unity mod p and mod
+# n (Gallant, Lambert and Vanstone, "Faster point multiplication on elliptic curves with
+# efficient endomorphisms", CRYPTO 2001).  Only for groups that are the whole curve
+# (cofactor 1), where every point on the curve is such a point.
+GLV = ("Secp256k1", "BN254")
+GLV_SHIFT = 320
+
+
+def cube_root(q):
+    g = 2
+    while pow(g, (q - 1) // 3, q) == 1:
+        g += 1
+    return pow(g, (q - 1) // 3, q)
+
+
+def times(k, x, y, p):
+    """k (x, y) on y^2 = x^3 + b, affine; k > 0 below the order."""
+    rx = None
+    for bit in bin(k)[2:]:
+        if rx is not None:
+            m = 3 * rx * rx * pow(2 * ry, -1, p) % p
+            nx = (m * m - 2 * rx) % p
+            rx, ry = nx, (m * (rx - nx) - ry) % p
+        if bit == "1":
+            if rx is None:
+                rx, ry = x, y
+            else:
+                m = (ry - y) * pow(rx - x, -1, p) % p
+                nx = (m * m - rx - x) % p
+                rx, ry = nx, (m * (x - nx) - y) % p
+    return rx, ry
+
+
+def glv(p, n, gx, gy, R, N):
+    """Constants that write k as k1 + k2 lambda with short k1, k2: with a basis (a1, b1),
+    (a2, b2) of the lattice of a + b lambda = 0 mod n, c1 = round(b2 k / n), c2 =
+    round(-b1 k / n), k1 = k - c1 a1 - c2 a2, k2 = -c1 b1 - c2 b2.  c_i comes from k times
+    g_i = 2^320 |b| / n; the signs are in the other factors (mod 2^160)."""
+    lam, beta = cube_root(n), cube_root(p)
+    lx, ly = times(lam, gx, gy, p)
+    assert ly == gy
+    if lx != beta * gx % p:
+        beta = beta * beta % p
+    assert lx == beta * gx % p
+    # half-extended Euclid on (n, lambda): the remainders around sqrt(n)
+    rows, (r0, t0), (r1, t1) = [], (n, 0), (lam, 1)
+    while r1:
+        rows.append((r1, -t1))
+        q = r0 // r1
+        (r0, t0), (r1, t1) = (r1, t1), (r0 - q * r1, t0 - q * t1)
+    i = next(j for j, (r, _) in enumerate(rows) if r * r < n)
+    (a1, b1), (a2, b2) = sorted(rows[i - 1:i + 2], key=lambda v: v[0] ** 2 + v[1] ** 2)[:2]
+    if a1 * b2 - a2 * b1 < 0:
+        (a1, b1), (a2, b2) = (a2, b2), (a1, b1)
+    assert a1 * b2 - a2 * b1 == n and (a1 + b1 * lam) % n == 0 and (a2 + b2 * lam) % n == 0
+    bits = max(abs(a1) + abs(a2), abs(b1) + abs(b2)) // 2 + 1
+    s1, s2 = (1 if b2 > 0 else -1), (1 if -b1 > 0 else -1)
+    g = [((abs(v) << GLV_SHIFT) + n // 2) // n for v in (b2, b1)]
+    assert max(g) < 1 << 224
+    m = 1 << 160
+    s = "  static constexpr bool GLV = true;\n"
+    s += f"  static constexpr int GLV_BITS = {bits.bit_length()};  // |k1|, |k2| < 2^GLV_BITS\n"
+    s += arr("glv_beta", beta * R % p, N) + arr("glv_g1", g[0], 7) + arr("glv_g2", g[1], 7)
+    s += arr("glv_a1", -s1 * a1 % m, 5) + arr("glv_a2", -s2 * a2 % m, 5)
+    s += arr("glv_b1", -s1 * b1 % m, 5) + arr("glv_b2", -s2 * b2 % m, 5)
+    return s
+
+
 def main():
     out = ["// Generated by gen_curves.py; do not edit.\n#pragma once\n#include <cstdint>\n",
            "#ifndef ECC_DEV\n#define ECC_DEV __device__ __forceinline__\n#endif\n\n",
@@ -111,6 +180,7 @@ def main():
         s += arr("gx", gx, N) + arr("gy", gy, N)
         s += arr("n", n, 8)
         s += f"  static constexpr int SCALAR_BITS = {n.bit_length()};\n"
+        s += glv(p, n, gx, gy, R, N) if name in GLV else "  static constexpr bool GLV = false;\n"
         s += "};\n\n"
         out.append(s)
     out.append("}  // namespace ecc\n")

@@ -9,7 +9,9 @@
 //     inversion.  An addition leaves Z_k = Z_(k-1) H_k, so 1 / Z_(k-1) is
 //     H_k / Z_k and the chain of H replaces Montgomery's prefix products;
 //   * u2 Q: signed kQW-bit fixed windows, most significant first: 255 doublings
-//     and at most 52 additions of affine table points;
+//     and at most 52 additions of affine table points.  secp256k1 splits u2 = k1 +
+//     k2 lambda (glv.cuh): 125 doublings and the same additions, those of k2 with
+//     beta x in the place of x (one triple 0.71 -> 0.55 ms);
 //   * u1 G: 16 additions from the generator's table onto the same accumulator
 //     (the digits of u1 need no doublings);
 //   * x_R mod n == r without an inversion: X = r Z^2 or X = (r + n) Z^2.
@@ -19,6 +21,7 @@
 // the scalars live in a small workspace that stays in L2 (80 MB for a full GPU),
 // whatever the batch size.
 #pragma once
+#include "glv.cuh"
 #include "ladder.cuh"
 
 namespace ecc {
@@ -35,7 +38,7 @@ struct VerifyArgs {
   uint32_t* table;       // kQTable affine points per slot
   SoA<Fp> H;             // Z ratios of the table's chain, kQTable per slot
   uint32_t* u1;          // recoded u1: word k of a slot at [k * slots + slot], 9 words
-  uint32_t* u2;          // recoded u2, likewise
+  uint32_t* u2;          // recoded u2, likewise: 9 words, or 5 of each half (sign in the top bit)
   uint32_t* rr;          // r, likewise, 8 words
   const uint32_t* TG;    // generator table (ladder.cuh)
   size_t slots;          // threads of the launch
@@ -45,19 +48,28 @@ struct VerifyArgs {
 // digit the digits are the windows minus 2^(kQW-1), in [-16, 15], no carries.
 constexpr int kQW = 5;
 constexpr int kQTable = 1 << (kQW - 1);
-constexpr int kQDigits = (256 + kQW - 1) / kQW;
-// the top window has room for u + offset: u < 2^256 <= 2^(kQW kQDigits - 4)
-static_assert(kQW * kQDigits >= 260 && kQW * kQDigits <= 288, "recoded scalar fits nine words");
 
-// word k of sum_i 2^(kQW - 1) 2^(kQW i), i < kQDigits
-ECC_DEV constexpr uint32_t q_offset(int k) {
-  uint32_t w = 0;
-  for (int i = 0; i < kQDigits; ++i) {
-    const int bit = kQW * i + kQW - 1;
-    if (bit >> 5 == k) w |= 1u << (bit & 31);
+// The windows of u2, or of both halves of a split u2 (word k of half h at row 5 h + k).
+template <class C>
+struct QWindows {
+  static constexpr int HALVES = C::GLV ? 2 : 1;
+  static constexpr int BITS = C::GLV ? 128 : 256;
+  static constexpr int DIGITS = (BITS + kQW - 1) / kQW;  // of a half
+  static constexpr int WORDS = C::GLV ? 5 : 9;
+  static constexpr int STEPS = HALVES * DIGITS;
+  // the top window has room for u + offset: u < 2^BITS <= 2^(kQW DIGITS - 2)
+  static_assert(kQW * DIGITS >= BITS + 2 && kQW * DIGITS < 32 * WORDS, "recoded scalar and sign fit the words");
+
+  // word k of sum_i 2^(kQW - 1) 2^(kQW i), i < DIGITS
+  ECC_DEV static constexpr uint32_t offset(int k) {
+    uint32_t w = 0;
+    for (int i = 0; i < DIGITS; ++i) {
+      const int bit = kQW * i + kQW - 1;
+      if (bit >> 5 == k) w |= 1u << (bit & 31);
+    }
+    return w;
   }
-  return w;
-}
+};
 
 template <class C>
 ECC_DEV bool on_curve_mont(const uint32_t* x, const uint32_t* y) {
@@ -120,12 +132,26 @@ ECC_DEV bool verify_prep(const VerifyArgs<C>& a, size_t i, size_t slot) {
 #pragma unroll
   for (int k = 0; k < 8; ++k) a.rr[k * a.slots + slot] = r[k];
   mont_mul<Fn>(u, w, r);
-  u[0] = ptx::add_cc(u[0], q_offset(0));
+  using QWin = QWindows<C>;
+  // v + offset in every window, row0 its first row
+  auto recode = [&](uint32_t* v, bool neg, int row0) {
+    v[0] = ptx::add_cc(v[0], QWin::offset(0));
 #pragma unroll
-  for (int k = 1; k < 8; ++k) u[k] = ptx::addc_cc(u[k], q_offset(k));
-  u[8] = ptx::addc(q_offset(8), 0);
+    for (int k = 1; k < QWin::WORDS - 1; ++k) v[k] = ptx::addc_cc(v[k], QWin::offset(k));
+    v[QWin::WORDS - 1] = ptx::addc(QWin::offset(QWin::WORDS - 1), 0);
+    if (neg) v[QWin::WORDS - 1] |= 0x80000000u;
 #pragma unroll
-  for (int k = 0; k < 9; ++k) a.u2[k * a.slots + slot] = u[k];
+    for (int k = 0; k < QWin::WORDS; ++k) a.u2[(row0 + k) * a.slots + slot] = v[k];
+  };
+  if constexpr (C::GLV) {
+    uint32_t m1[5], m2[5];
+    bool n1, n2;
+    glv_split<C>(u, m1, n1, m2, n2);
+    recode(m1, n1, 0);
+    recode(m2, n2, 5);
+  } else {
+    recode(u, false, 0);
+  }
   uint32_t e[8];
   load_be256(e, a.hash + 8 * i);
   if (!lt256(e, nn)) sub256(e, e, nn);  // e < 2^256 < 2n
@@ -164,6 +190,7 @@ __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_verify(Ver
   using F = typename C::Fp;
   constexpr int N = F::N;
   static_assert(N == 8 && C::Fn::N == 8, "256-bit curves");
+  using QWin = QWindows<C>;
   const size_t slot = blockIdx.x * (size_t)kLadderThreads + threadIdx.x;
   // threads past the batch repeat its last item (the barriers need every thread)
 #pragma unroll 1
@@ -180,21 +207,24 @@ __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_verify(Ver
     store_affine<F>(a.table, slot * kQTable + 1, X, Y);
     constexpr int kChain = kQTable - 2;
 #pragma unroll 1
-    for (int it = 0; it < kChain + kQDigits + kGRows; ++it) {
+    for (int it = 0; it < kChain + QWin::STEPS + kGRows; ++it) {
       int d;
       const uint32_t* src;
       size_t row;
+      bool phi = false;  // the point's image under the endomorphism
       if (it < kChain) {
         d = 1;
         src = a.table;
         row = slot * kQTable;
-      } else if (it < kChain + kQDigits) {
-        const int w = kChain + kQDigits - 1 - it;
-        if (it == kChain) {
+      } else if (it < kChain + QWin::STEPS) {
+        const int step = it - kChain;
+        const int half = QWin::HALVES == 2 ? step & 1 : 0;
+        const int w = QWin::DIGITS - 1 - step / QWin::HALVES;
+        if (step == 0) {
           fe_inv_mont<F>(x, Z);
           verify_table_affine<C>(a, slot, x);
           fe_set_zero<F>(Z);
-        } else {
+        } else if (half == 0) {
 #pragma unroll 1
           for (int k = 0; k < kQW; ++k) {
             __syncthreads();
@@ -202,13 +232,18 @@ __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_verify(Ver
           }
         }
         const int bit = kQW * w, wd = bit >> 5, sh = bit & 31;
-        uint32_t v = a.u2[wd * a.slots + slot] >> sh;
-        if (sh > 32 - kQW) v |= a.u2[(wd + 1) * a.slots + slot] << (32 - sh);
+        const uint32_t* u2 = a.u2 + 5 * half * a.slots + slot;
+        uint32_t v = u2[wd * a.slots] >> sh;
+        if (sh > 32 - kQW) v |= u2[(wd + 1) * a.slots] << (32 - sh);
         d = (int)(v & (2 * kQTable - 1)) - kQTable;
         src = a.table;
         row = slot * kQTable + (d < 0 ? -d : d) - 1;
+        if constexpr (C::GLV) {
+          if (u2[4 * a.slots] >> 31) d = -d;
+          phi = half != 0;
+        }
       } else {
-        const int j = it - kChain - kQDigits;
+        const int j = it - kChain - QWin::STEPS;
         const uint32_t c = a.u1[8 * a.slots + slot];
         d = comb_digit(a.u1[(j >> 1) * a.slots + slot], c & 1u, j);
         src = a.TG;
@@ -219,6 +254,14 @@ __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_verify(Ver
       if (d != 0) {
         load_affine<F>(src, row, x, y);
         if (d < 0) fe_neg<F>(y, y);
+        if constexpr (C::GLV) {
+          if (phi) {
+            uint32_t beta[N];
+#pragma unroll
+            for (int k = 0; k < N; ++k) beta[k] = C::glv_beta(k);
+            call_mul<F>(x, x, beta);
+          }
+        }
         jac_madd<C>(X, Y, Z, x, y, H);
       }
       if (it < kChain) {

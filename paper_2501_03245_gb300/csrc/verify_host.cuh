@@ -20,10 +20,11 @@ cudaError_t verify(size_t n, const uint8_t* hash, const uint8_t* r, const uint8_
   size_t ctas = (n + kLadderThreads - 1) / kLadderThreads;
   ctas = std::min<size_t>(ctas, (size_t)device_sm_count() * kLadderCtasPerSm);
   const size_t slots = ctas * kLadderThreads;
-  // per slot: table (affine points), H, recoded u1 and u2 (9 words each), r
+  // per slot: table (affine points), H, recoded u1 (9 words) and u2, r
+  constexpr size_t kU2 = QWindows<C>::HALVES * QWindows<C>::WORDS;
   const size_t table = slots * kQTable * 2 * Fp::N * 4, h = soa_bytes<Fp>(slots * kQTable);
   Scratch ws;
-  e = ws.alloc(table + h + (9 + 9 + 8) * 4 * slots, st);
+  e = ws.alloc(table + h + (9 + kU2 + 8) * 4 * slots, st);
   if (e != cudaSuccess) return e;
   uint8_t* p = ws.as<uint8_t>();
   VerifyArgs<C> a;
@@ -37,7 +38,7 @@ cudaError_t verify(size_t n, const uint8_t* hash, const uint8_t* r, const uint8_
   a.H = SoA<Fp>{reinterpret_cast<uint4*>(p + table), slots * kQTable};
   a.u1 = reinterpret_cast<uint32_t*>(p + table + h);
   a.u2 = a.u1 + 9 * slots;
-  a.rr = a.u2 + 9 * slots;
+  a.rr = a.u2 + kU2 * slots;
   a.TG = tg;
   a.slots = slots;
   k_verify<C><<<(unsigned)ctas, kLadderThreads, 0, st>>>(a);
