@@ -457,7 +457,7 @@ int ecc_msm(ecc_curve_t curve, size_t n, const uint32_t* points, const uint32_t*
 }
 
 static bool msm_dev_sizes_ok(int curve, size_t num, size_t max_points, int c, int pre_c) {
-  const int w = pre_c > 0 ? pre_c : (c > 0 ? c : msm_window(curve, num ? std::max<size_t>(max_points / num, 2) : 2));
+  const int w = pre_c > 0 ? pre_c : (c > 0 ? c : msm_admitted_window(curve, num ? std::max<size_t>(max_points / num, 2) : 2));
   const uint64_t W = (uint64_t)((curve == ECC_BN254 ? 254 : 255) + 1 + w - 1) / w;
   const uint64_t rows = pre_c > 0 ? 1 : W;
   return (uint64_t)max_points * W < kMsmMaxDigits && (uint64_t)num * (rows << (w - 1)) < kMsmMaxDigits;

@@ -81,7 +81,10 @@ cudaError_t launch_verify(int curve, size_t n, const uint8_t* hash, const uint8_
 
 // MSM: `num` instances, instance i = points / scalars rows
 // [offsets[i] - offsets[0], offsets[i+1] - offsets[0]) (host offsets); out: num x 2N limbs
-int msm_window(int curve, uint64_t n);
+// window width of an n-point MSM in a batch of num; the width by which a size is
+// admitted (the same when the caller set one)
+int msm_window(int curve, uint64_t n, uint64_t num = 1);
+int msm_admitted_window(int curve, uint64_t n);
 void msm_set_window(int curve, int log2n, int c);
 // log2 of the buckets per reduction element: the autotuner's override for the size
 // class of n (0: none), the most an n-point MSM takes, and the override's setter for

@@ -20,7 +20,7 @@ cudaError_t msm_bases_bn254(void* bases, uint32_t num_vectors, const uint64_t* s
 cudaError_t msm_bases_bls12_381(void* bases, uint32_t num_vectors, const uint64_t* sizes,
                                 const uint32_t* scalars,
                                 uint32_t* out, cudaStream_t st);
-cudaError_t points_to_mont(int curve, const uint32_t* in, uint64_t n, uint32_t* out,
+cudaError_t points_to_mont(int curve, const uint32_t* in, uint64_t n, uint32_t* out, uint64_t phi,
                            cudaStream_t st);
 cudaError_t bases_precompute_bn254(void* bases, int c, cudaStream_t st);
 cudaError_t msm_points_dev_bn254(uint32_t num, uint64_t cap, const uint64_t* offsets, int c,
@@ -41,10 +41,34 @@ std::mutex g_win_mu;
 std::map<std::pair<int, int>, int> g_window_table;  // (curve, floor(log2 n)) -> c
 std::map<std::pair<int, int>, int> g_chunk_table;   // (curve, floor(log2 n)) -> red_log
 
-// Cost model: one batched addition (6 modmul) per (point, window) digit plus the
-// bucket reduction, about two and a half batched additions per bucket (the walk's
-// A and S events and the fold's share).
-int model_window(int curve, uint64_t n) {
+// Cost model, in products: 6 per (point, window) digit and 15 per bucket (of the
+// affine form; the Jacobian form's 11 and 27 or more are in the same proportion);
+// 100 (about 5 ns) for every digit in its way when the top window has only `top` bits
+// and its points share 2^top buckets; and for a single call the latency of its tail,
+// two steps of the reduction for each bit of c and one of the combination for each
+// window (8 and 2.8 us with 8 limbs), which the instances of a batch share.
+int model_window(int curve, uint64_t n, uint64_t num) {
+  const bool split = curve == 2;
+  const int bits = split ? BN254::GLV_BITS : msm_detail::scalar_bits(curve);
+  int best = 4;
+  double best_cost = 1e300;
+  for (int c = 4; c <= 20; ++c) {
+    const double W = (bits + 1 + c - 1) / c, digits = (double)n * W * (split ? 2 : 1);
+    const int top = bits - c * ((int)W - 1);
+    double cost = digits * 6.0 + W * (double)(1u << (c - 1)) * 15.0;
+    cost += digits / W / (double)(1u << std::max(top, 0)) * 100.0;
+    cost += (150e3 * c + 59e3 * W) / (double)std::max<uint64_t>(num, 1);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = c;
+    }
+  }
+  return best;
+}
+
+// The width by which sizes are admitted: whole scalars, 6 products per digit and 15
+// per bucket.
+int admitted_model(int curve, uint64_t n) {
   int best = 4;
   double best_cost = 1e300;
   for (int c = 4; c <= 20; ++c) {
@@ -69,14 +93,27 @@ int ilog2(uint64_t n) {
 
 }  // namespace
 
-int msm_window(int curve, uint64_t n) {
+namespace {
+
+// the caller's width for the size class of n (0: none)
+int window_override(int curve, uint64_t n) {
+  std::lock_guard<std::mutex> lock(g_win_mu);
+  auto it = g_window_table.find({curve, ilog2(n)});
+  return it != g_window_table.end() ? it->second : 0;
+}
+
+}  // namespace
+
+int msm_window(int curve, uint64_t n, uint64_t num) {
   if (n < 2) n = 2;
-  {
-    std::lock_guard<std::mutex> lock(g_win_mu);
-    auto it = g_window_table.find({curve, ilog2(n)});
-    if (it != g_window_table.end()) return it->second;
-  }
-  return model_window(curve, n);
+  const int c = window_override(curve, n);
+  return c > 0 ? c : model_window(curve, n, num);
+}
+
+int msm_admitted_window(int curve, uint64_t n) {
+  if (n < 2) n = 2;
+  const int c = window_override(curve, n);
+  return c > 0 ? c : admitted_model(curve, n);
 }
 
 void msm_set_window(int curve, int log2n, int c) {
@@ -168,7 +205,6 @@ void msm_set_reduce_log(int curve, int log2n, int v) {
 cudaError_t launch_msm_dev(int curve, uint32_t num, uint64_t cap, const uint64_t* offsets, int c,
                            const uint32_t* points, const uint32_t* scalars, uint32_t* out,
                            cudaStream_t st) {
-  if (c <= 0) c = msm_window(curve, num ? std::max<uint64_t>(cap / num, 2) : 2);
   switch (curve) {
     case 2: return msm_points_dev_bn254(num, cap, offsets, c, points, scalars, out, st);
     case 3: return msm_points_dev_bls12_381(num, cap, offsets, c, points, scalars, out, st);
@@ -179,7 +215,6 @@ cudaError_t launch_msm_dev(int curve, uint32_t num, uint64_t cap, const uint64_t
 cudaError_t launch_msm_bases_dev(void* handle, uint32_t num, uint64_t cap, const uint64_t* sizes, int c,
                                  const uint32_t* scalars, uint32_t* out, cudaStream_t st) {
   const int curve = bases_curve(handle);
-  if (c <= 0) c = msm_window(curve, num ? std::max<uint64_t>(cap / num, 2) : 2);
   switch (curve) {
     case 2: return msm_bases_dev_bn254(handle, num, cap, sizes, c, scalars, out, st);
     case 3: return msm_bases_dev_bls12_381(handle, num, cap, sizes, c, scalars, out, st);
@@ -201,14 +236,21 @@ cudaError_t bases_create(int curve, uint64_t n, const uint32_t* points, void** h
   if (curve != 2 && curve != 3) return cudaErrorNotSupported;
   const int N = curve == 3 ? 12 : 8;
   uint32_t* m = nullptr;
-  cudaError_t e = cudaMalloc(&m, std::max<uint64_t>(n, 1) * 2 * N * 4);
+  // BN254: the points' images beside them (glv.cuh), where there is room
+  uint64_t phi = curve == 2 ? n : 0;
+  cudaError_t e = cudaMalloc(&m, std::max<uint64_t>(phi + n, 1) * 2 * N * 4);
+  if (e == cudaErrorMemoryAllocation && phi) {
+    cudaGetLastError();
+    phi = 0;
+    e = cudaMalloc(&m, n * 2 * N * 4);
+  }
   if (e != cudaSuccess) return e;
-  if (n) e = points_to_mont(curve, points, n, m, st);
+  if (n) e = points_to_mont(curve, points, n, m, phi, st);
   if (e != cudaSuccess) {
     cudaFree(m);
     return e;
   }
-  *handle = new msm_detail::Bases{curve, n, m};
+  *handle = new msm_detail::Bases{curve, n, m, phi};
   return cudaSuccess;
 }
 
@@ -233,7 +275,7 @@ void msm_counts(int curve, uint64_t num, const uint64_t* sizes, uint64_t size_al
   uint64_t d = 0, b = 0;
   for (uint64_t i = 0; i < num; ++i) {
     const uint64_t n = sizes ? sizes[i] : size_all;
-    const int c = pre_c > 0 ? pre_c : msm_window(curve, n);
+    const int c = pre_c > 0 ? pre_c : msm_admitted_window(curve, n);
     const uint64_t W = (uint64_t)msm_detail::windows_for(curve, c);
     d += W * n;
     b += (pre_c > 0 ? 1 : W) << (c - 1);

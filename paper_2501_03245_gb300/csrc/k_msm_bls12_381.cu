@@ -18,7 +18,7 @@ cudaError_t msm_bases_bls12_381(void* bases, uint32_t num_vectors, const uint64_
 
 cudaError_t points_to_mont_bls12_381(const uint32_t* in, uint64_t n, uint32_t* out,
                                      cudaStream_t st) {
-  k_points_to_mont<BLS12_381><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(in, n, nullptr, out);
+  k_points_to_mont<BLS12_381><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(in, n, nullptr, out, 0);
   return cudaGetLastError();
 }
 

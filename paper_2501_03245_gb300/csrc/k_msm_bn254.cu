@@ -19,11 +19,11 @@ cudaError_t msm_bases_bn254(void* bases, uint32_t num_vectors, const uint64_t* s
                                      out, st);
 }
 
-cudaError_t points_to_mont(int curve, const uint32_t* in, uint64_t n, uint32_t* out,
+cudaError_t points_to_mont(int curve, const uint32_t* in, uint64_t n, uint32_t* out, uint64_t phi,
                            cudaStream_t st) {
   const unsigned b = (unsigned)((n + 255) / 256);
   if (curve == 2) {
-    k_points_to_mont<BN254><<<b, 256, 0, st>>>(in, n, nullptr, out);
+    k_points_to_mont<BN254><<<b, 256, 0, st>>>(in, n, nullptr, out, phi);
     return cudaGetLastError();
   }
   return points_to_mont_bls12_381(in, n, out, st);

@@ -3,7 +3,9 @@
 // The paper's text has no MSM section; the method is the standard bucket
 // method built from the paper's primitives:
 //   1. digits: scalar k_i (reduced mod r) in signed c-bit windows
-//      d_w in [-2^(c-1) + 1, 2^(c-1)], W = ceil((bits(r) + 1) / c) windows;
+//      d_w in [-2^(c-1) + 1, 2^(c-1)], W = ceil((bits(r) + 1) / c) windows, or of
+//      both halves of a split scalar (glv.cuh), half as many windows of twice the
+//      points: as many additions, half the buckets and half the doublings at the end;
 //   2. counting (one-digit radix) sort of the (bucket id, point) pairs by bucket
 //      id: histogram with atomics, exclusive scan, scatter with atomic cursors;
 //   3. bucket accumulation with batched affine additions (Section 3.3): the
@@ -22,6 +24,7 @@
 // Several independent MSM instances (different sizes, windows and bases) run
 // through the same launches: every instance owns a disjoint range of bucket ids.
 #pragma once
+#include "glv.cuh"
 #include "jac.cuh"
 
 namespace ecc {
@@ -46,6 +49,9 @@ struct MsmInst {
   uint64_t elem_off;     // first reduction element; 2^(c - 1 - red_log) per bucket row
   uint32_t row_off;      // first bucket row
   uint32_t cta_off;      // first CTA of the reduction tree's first pass
+  // Split scalars: the image of the point at index i under the endomorphism is at
+  // i + phi, and both halves' digits of a window go to its buckets.  0: not split.
+  uint64_t phi;
 };
 
 // log2 of the reduction elements per bucket row
@@ -71,32 +77,46 @@ ECC_DEV void scalar_mod_r(uint32_t* k) {
   }
 }
 
-// bits [pos, pos + c) of k (c <= 24)
-ECC_DEV uint32_t scalar_bits(const uint32_t* k, int pos, int c) {
-  const int w = pos >> 5, s = pos & 31;
-  if (w >= 8) return 0;
-  uint64_t v = k[w];
-  if (w + 1 < 8) v |= (uint64_t)k[w + 1] << 32;
-  return (uint32_t)(v >> s) & ((1u << c) - 1u);
+// Calls fn(w, d) for every window with signed digit d != 0 of the K-word k, or of -k.
+// The words shift down by a window at a time, which keeps them in registers.
+template <int K, class Fn>
+ECC_DEV void for_each_digit(const uint32_t* src, bool neg, int c, int W, Fn fn) {
+  uint32_t k[K + 1], carry = 0;
+#pragma unroll
+  for (int q = 0; q < K; ++q) k[q] = src[q];
+  k[K] = 0;
+  const uint32_t half = 1u << (c - 1);
+#pragma unroll 1
+  for (int w = 0; w < W; ++w) {
+    const uint32_t v = (k[0] & ((1u << c) - 1u)) + carry;
+#pragma unroll
+    for (int q = 0; q < K; ++q) k[q] = __funnelshift_r(k[q], k[q + 1], c);
+    carry = v > half ? 1u : 0u;
+    const int d = carry ? (int)v - (int)(1u << c) : (int)v;
+    if (d != 0) fn(w, neg ? -d : d);
+  }
 }
 
-// Calls fn(w, d) for every window with signed digit d != 0.
-template <class Fn>
-ECC_DEV void for_each_digit(const uint32_t* k, int c, int W, Fn fn) {
-  uint32_t carry = 0;
-  const uint32_t half = 1u << (c - 1);
-  for (int w = 0; w < W; ++w) {
-    uint32_t v = scalar_bits(k, w * c, c) + carry;
-    int d;
-    if (v > half) {
-      d = (int)v - (int)(1u << c);
-      carry = 1;
-    } else {
-      d = (int)v;
-      carry = 0;
+// Calls fn(w, d, shift) for the nonzero digits of the scalar at `src` of instance
+// `in`: bucket row w, and the point at `shift` from the scalar's own.
+template <class C, class Fn>
+ECC_DEV void for_each_entry(const MsmInst& in, const uint32_t* __restrict__ src, Fn fn) {
+  uint32_t k[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) k[q] = src[q];
+  scalar_mod_r<C>(k);
+  if constexpr (C::GLV) {
+    if (in.phi) {
+      uint32_t m[2][5];
+      bool neg[2];
+      glv_split<C>(k, m[0], neg[0], m[1], neg[1]);
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        for_each_digit<4>(m[h], neg[h], in.c, in.W, [&](int w, int d) { fn(w, d, h ? in.phi : 0ull); });
+      return;
     }
-    if (d != 0) fn(w, d);
   }
+  for_each_digit<8>(k, false, in.c, in.W, [&](int w, int d) { fn(w, d, (uint64_t)w * in.pre_stride); });
 }
 
 ECC_DEV int find_inst(const MsmInst* inst, int num, uint64_t g) {
@@ -215,15 +235,9 @@ __global__ void k_msm_count(const MsmInst* inst, int num, const uint32_t* __rest
   const uint64_t g = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   if (g >= batch_rows(total, hdr)) return;
   const MsmInst in = inst[find_inst(inst, num, g)];
-  uint32_t k[8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q) k[q] = scalars[8 * g + q];
-  scalar_mod_r<C>(k);
-  const uint32_t half = 1u << (in.c - 1);
-  const uint32_t row = in.pre_stride ? 0u : half;
-  for_each_digit(k, in.c, in.W, [&](int w, int d) {
-    const uint32_t b = in.bucket_base + w * row + (uint32_t)(d < 0 ? -d : d) - 1;
-    atomicAdd(count + b, 1u);
+  const uint32_t row = in.pre_stride ? 0u : 1u << (in.c - 1);
+  for_each_entry<C>(in, scalars + 8 * g, [&](int w, int d, uint64_t) {
+    atomicAdd(count + in.bucket_base + w * row + (uint32_t)(d < 0 ? -d : d) - 1, 1u);
   });
 }
 
@@ -240,17 +254,12 @@ __global__ void k_msm_scatter(const MsmInst* inst, int num, const uint32_t* __re
   const uint64_t g = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   if (g >= batch_rows(total, hdr)) return;
   const MsmInst in = inst[find_inst(inst, num, g)];
-  uint32_t k[8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q) k[q] = scalars[8 * g + q];
-  scalar_mod_r<C>(k);
-  const uint32_t half = 1u << (in.c - 1);
-  const uint32_t row = in.pre_stride ? 0u : half;
+  const uint32_t row = in.pre_stride ? 0u : 1u << (in.c - 1);
   const uint64_t pidx = in.point_off + (g - in.scalar_off);
-  for_each_digit(k, in.c, in.W, [&](int w, int d) {
+  for_each_entry<C>(in, scalars + 8 * g, [&](int w, int d, uint64_t shift) {
     const uint32_t b = in.bucket_base + w * row + (uint32_t)(d < 0 ? -d : d) - 1;
     const uint32_t p = atomicAdd(cursor + b, 1u);
-    const uint32_t idx = (uint32_t)(pidx + (uint64_t)w * in.pre_stride);  // < 2^31 (host check)
+    const uint32_t idx = (uint32_t)(pidx + shift);  // < 2^31 (host check)
     const uint32_t j = p & ((1u << ch_log) - 1u), chunk = p >> ch_log;
     vals[(uint64_t)j * n_chunks + chunk] = idx | (d < 0 ? 0x80000000u : 0u);
     if (j == 0) cur[chunk] = b;
@@ -1090,10 +1099,11 @@ __global__ void __launch_bounds__(32) k_msm_combine(RedArgs<C> a, const uint32_t
   }
 }
 
-// canonical AoS points -> Montgomery AoS points (gather layout of the bases)
+// canonical AoS points -> Montgomery AoS points (gather layout of the bases), and
+// with phi > 0 their images (beta x, y) at rows phi, phi + 1, ..
 template <class C>
 __global__ void k_points_to_mont(const uint32_t* __restrict__ in, uint64_t n, const MsmDevHdr* hdr,
-                                 uint32_t* __restrict__ out) {
+                                 uint32_t* __restrict__ out, uint64_t phi) {
   using F = typename C::Fp;
   constexpr int N = F::N;
   const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
@@ -1106,10 +1116,15 @@ __global__ void k_points_to_mont(const uint32_t* __restrict__ in, uint64_t n, co
   }
   to_mont<F>(x, x);
   to_mont<F>(y, y);
+  store_affine<F>(out, i, x, y);
+  if constexpr (C::GLV) {
+    if (phi) {
+      uint32_t beta[N];
 #pragma unroll
-  for (int q = 0; q < N; ++q) {
-    out[2 * N * i + q] = x[q];
-    out[2 * N * i + N + q] = y[q];
+      for (int q = 0; q < N; ++q) beta[q] = C::glv_beta(q);
+      mont_mul<F>(x, x, beta);
+      store_affine<F>(out, phi + i, x, y);
+    }
   }
 }
 

@@ -31,11 +31,22 @@ inline int scalar_bits(int curve) {
 
 inline int windows_for(int curve, int c) { return (scalar_bits(curve) + 1 + c - 1) / c; }
 
+// Windows of the halves of a split scalar (below 2^GLV_BITS in magnitude).
+template <class C>
+int half_windows(int c) {
+  if constexpr (C::GLV) {
+    static_assert(C::GLV_BITS < 128, "magnitudes and their top carry fit four words");
+    return (C::GLV_BITS + 1 + c - 1) / c;
+  }
+  return 0;
+}
+
 struct Layout {
   std::vector<MsmInst> inst;
   uint64_t buckets = 0, entries_max = 0, n_chunks = 0, total_points = 0;
   uint64_t elems = 0;          // reduction elements
   uint32_t rows = 0, ctas = 0; // bucket rows, CTAs of the reduction tree's first pass
+  uint64_t phi = 0;            // split scalars: rows between the points and their images
   bool direct = false;         // Jacobian accumulation
   int ch_log = kAccLog;        // log2 of the entries per chunk
 };
@@ -112,7 +123,7 @@ cudaError_t run_set(int curve, const Layout& L, const uint32_t* bases_mont, cons
   // prefix product, or X, Y and Z
   const uint64_t kChunkArrays = L.direct ? 0 : 3;
   const uint64_t sz_hdr = up(sizeof(MsmDevHdr));
-  const uint64_t sz_pts = raw_points ? up(std::max<uint64_t>(L.total_points, 1) * 2 * N * 4) : 0;
+  const uint64_t sz_pts = raw_points ? up(std::max<uint64_t>(L.phi + L.total_points, 1) * 2 * N * 4) : 0;
   const uint64_t bytes = sz_inst + sz_hdr + sz_pts + 5 * sz_b1 + sz_kv + sz_cur + kChunkArrays * sz_S +
                          3 * sz_P + sz_ops + 256;
   Scratch ws;
@@ -143,7 +154,7 @@ cudaError_t run_set(int curve, const Layout& L, const uint32_t* bases_mont, cons
   if (e != cudaSuccess) return e;
   if (raw_points && L.total_points) {
     k_points_to_mont<C><<<(unsigned)((L.total_points + 255) / 256), 256, 0, st>>>(raw_points, L.total_points,
-                                                                                 hdr, pts_mont);
+                                                                                 hdr, pts_mont, L.phi);
     bases_mont = pts_mont;
   }
   phase_mark(0, st);
@@ -268,27 +279,33 @@ cudaError_t run_set(int curve, const Layout& L, const uint32_t* bases_mont, cons
 }
 
 // pre_c > 0: the bases hold precomputed window multiples for width pre_c,
-// pre_stride points apart.
-template <int N>
+// pre_stride points apart.  phi > 0: the points' images are phi rows after them, and
+// scalars are split.  A batch whose digits, buckets or rows do not fit their 31-bit
+// indices that way is planned as its size was admitted (msm_counts).
+template <class C>
 Layout plan(int curve, uint32_t num, const uint64_t* sizes, const uint64_t* point_off,
-            const uint64_t* scalar_off, const int* cs, int pre_c = 0, uint64_t pre_stride = 0) {
+            const uint64_t* scalar_off, int pre_c, uint64_t pre_stride, uint64_t phi, bool admitted = false) {
   Layout L;
   L.inst.resize(num);
+  L.phi = phi;
   for (uint32_t i = 0; i < num; ++i) {
     MsmInst& m = L.inst[i];
     m.n = (uint32_t)sizes[i];
-    m.c = (uint32_t)(pre_c > 0 ? pre_c : cs && cs[i] > 0 ? cs[i] : msm_window(curve, sizes[i]));
-    m.W = (uint32_t)windows_for(curve, (int)m.c);
+    m.c = (uint32_t)(pre_c > 0 ? pre_c : admitted ? msm_admitted_window(curve, sizes[i]) : msm_window(curve, sizes[i], num));
+    m.W = (uint32_t)(phi ? half_windows<C>((int)m.c) : windows_for(curve, (int)m.c));
     m.bucket_base = (uint32_t)L.buckets;
     m.point_off = point_off[i];
     m.scalar_off = scalar_off[i];
     m.pre_stride = pre_c > 0 ? pre_stride : 0;
+    m.phi = phi;
     m.Wr = pre_c > 0 ? 1u : m.W;
     L.buckets += (uint64_t)m.Wr << (m.c - 1);
-    L.entries_max += (uint64_t)m.W * m.n;
+    L.entries_max += (uint64_t)m.W * m.n * (phi ? 2 : 1);
     L.total_points += m.n;
+    if (!admitted && (L.entries_max >= kMsmMaxDigits || L.buckets >= kMsmMaxDigits || 2 * phi >= kMsmMaxDigits))
+      return plan<C>(curve, num, sizes, point_off, scalar_off, pre_c, pre_stride, 0, true);
   }
-  finish_plan<N>(curve, L, sizes, 0);
+  finish_plan<C::Fp::N>(curve, L, sizes, 0);
   return L;
 }
 
@@ -297,35 +314,50 @@ cudaError_t msm_points(int curve, uint32_t num, const uint64_t* offsets, const u
                        const uint32_t* scalars, uint32_t* out, cudaStream_t st) {
   using F = typename C::Fp;
   const uint64_t total = offsets[num] - offsets[0];
-  std::vector<uint64_t> sizes(num), poff(num), soff(num);
+  std::vector<uint64_t> sizes(num), poff(num);
   for (uint32_t i = 0; i < num; ++i) {
     sizes[i] = offsets[i + 1] - offsets[i];
     poff[i] = offsets[i] - offsets[0];
-    soff[i] = poff[i];
   }
-  Layout L = plan<C::Fp::N>(curve, num, sizes.data(), poff.data(), soff.data(), nullptr);
-  (void)total;
-  return run_set<C>(curve, L, nullptr, scalars + offsets[0] * 8, out, st, nullptr,
-                    points + offsets[0] * 2 * F::N);
+  auto run = [&](uint64_t phi) {
+    const Layout L = plan<C>(curve, num, sizes.data(), poff.data(), poff.data(), 0, 0, phi);
+    return run_set<C>(curve, L, nullptr, scalars + offsets[0] * 8, out, st, nullptr, points + offsets[0] * 2 * F::N);
+  };
+  cudaError_t e = run(C::GLV ? total : 0);
+  if (C::GLV && e == cudaErrorMemoryAllocation) {  // without the images' workspace
+    cudaGetLastError();
+    e = run(0);
+  }
+  return e;
 }
 
 // The uniform per-instance layout of a device-sized batch (window width c, or
 // the library's width for bases with window multiples of width pre_c) with the
-// capacity totals: cap scalar rows in num instances.
-template <int N>
-Layout plan_uniform(int curve, uint32_t num, int c, uint64_t cap, int pre_c, uint64_t pre_stride) {
+// capacity totals: cap scalar rows in num instances.  phi and the indices as in plan;
+// c = 0: the library's width for the mean size.
+template <class C>
+Layout plan_uniform(int curve, uint32_t num, int c, uint64_t cap, int pre_c, uint64_t pre_stride, uint64_t phi) {
   Layout L;
   MsmInst m{};
+  if (pre_c <= 0 && c <= 0) {
+    const uint64_t mean = num ? std::max<uint64_t>(cap / num, 2) : 2;
+    c = msm_window(curve, mean, num);
+    const uint64_t W = (uint64_t)windows_for(curve, c);
+    if (W * cap >= kMsmMaxDigits || (num * W) << (c - 1) >= kMsmMaxDigits) c = msm_admitted_window(curve, mean);
+  }
   m.c = (uint32_t)(pre_c > 0 ? pre_c : c);
-  m.W = (uint32_t)windows_for(curve, (int)m.c);
+  if (phi && ((uint64_t)half_windows<C>((int)m.c) * cap * 2 >= kMsmMaxDigits || 2 * phi >= kMsmMaxDigits)) phi = 0;
+  m.W = (uint32_t)(phi ? half_windows<C>((int)m.c) : windows_for(curve, (int)m.c));
   m.Wr = pre_c > 0 ? 1u : m.W;
   m.pre_stride = pre_c > 0 ? pre_stride : 0;
+  m.phi = phi;
+  L.phi = phi;
   L.inst.assign(num, m);
   for (uint32_t i = 0; i < num; ++i) L.inst[i].bucket_base = (uint32_t)(i * ((uint64_t)m.Wr << (m.c - 1)));
   L.buckets = (uint64_t)num * ((uint64_t)m.Wr << (m.c - 1));
-  L.entries_max = cap * m.W;
+  L.entries_max = cap * m.W * (phi ? 2 : 1);
   L.total_points = cap;
-  finish_plan<N>(curve, L, nullptr, num ? std::max<uint64_t>(cap / num, 2) : 2);
+  finish_plan<C::Fp::N>(curve, L, nullptr, num ? std::max<uint64_t>(cap / num, 2) : 2);
   return L;
 }
 
@@ -334,9 +366,16 @@ Layout plan_uniform(int curve, uint32_t num, int c, uint64_t cap, int pre_c, uin
 template <class C>
 cudaError_t msm_points_dev(int curve, uint32_t num, uint64_t cap, const uint64_t* offsets, int c,
                            const uint32_t* points, const uint32_t* scalars, uint32_t* out, cudaStream_t st) {
-  Layout L = plan_uniform<C::Fp::N>(curve, num, c, cap, 0, 0);
   DevRows dev{offsets, 0, 0, cap};
-  return run_set<C>(curve, L, nullptr, scalars, out, st, &dev, points);
+  auto run = [&](uint64_t phi) {
+    return run_set<C>(curve, plan_uniform<C>(curve, num, c, cap, 0, 0, phi), nullptr, scalars, out, st, &dev, points);
+  };
+  cudaError_t e = run(C::GLV ? cap : 0);
+  if (C::GLV && e == cudaErrorMemoryAllocation) {  // without the images' workspace
+    cudaGetLastError();
+    e = run(0);
+  }
+  return e;
 }
 
 
@@ -344,6 +383,7 @@ struct Bases {
   int curve;
   uint64_t n;
   uint32_t* mont;          // AoS Montgomery affine, owned
+  uint64_t phi = 0;        // rows to the points' images under the endomorphism (0: none)
   uint32_t* pre = nullptr; // window multiples (window-major, window 0 = mont copy), owned
   int pre_c = 0;           // window width of pre (0: none)
 };
@@ -401,7 +441,7 @@ cudaError_t precompute_t(Bases* bs, int c, cudaStream_t st) {
 template <class C>
 cudaError_t msm_bases_dev_t(Bases* bs, uint32_t num, uint64_t cap, const uint64_t* sizes, int c,
                             const uint32_t* scalars, uint32_t* out, cudaStream_t st) {
-  Layout L = plan_uniform<C::Fp::N>(bs->curve, num, c, cap, bs->pre ? bs->pre_c : 0, bs->n);
+  Layout L = plan_uniform<C>(bs->curve, num, c, cap, bs->pre ? bs->pre_c : 0, bs->n, bs->pre ? 0 : bs->phi);
   DevRows dev{sizes, 1, bs->n, cap};
   return run_set<C>(bs->curve, L, bs->pre ? bs->pre : bs->mont, scalars, out, st, &dev);
 }
@@ -418,8 +458,8 @@ cudaError_t msm_bases_t(Bases* bs, uint32_t num_vectors, const uint64_t* vec_siz
     soff[v] = acc;
     acc += sizes[v];
   }
-  Layout L = plan<C::Fp::N>(bs->curve, num_vectors, sizes.data(), poff.data(), soff.data(), nullptr,
-                  bs->pre ? bs->pre_c : 0, bs->n);
+  Layout L = plan<C>(bs->curve, num_vectors, sizes.data(), poff.data(), soff.data(), bs->pre ? bs->pre_c : 0, bs->n,
+                     bs->pre ? 0 : bs->phi);
   return run_set<C>(bs->curve, L, bs->pre ? bs->pre : bs->mont, scalars, out, st);
 }
 
