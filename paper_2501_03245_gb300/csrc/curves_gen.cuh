@@ -12,6 +12,7 @@ struct Secp256k1Fp {
   static constexpr int BITS = 256;
   static constexpr uint32_t QINV = 0xd2253531u;
   static constexpr int FORM = 2;
+  static constexpr bool SQR_ROWS = false;
   static constexpr uint64_t QINV62 = 0x27c7f6e22ddacacfull;  // q^-1 mod 2^62
   ECC_DEV static constexpr uint32_t qinv() { return QINV; }
   ECC_DEV static constexpr uint64_t qinv62() { return QINV62; }
@@ -37,6 +38,7 @@ struct Secp256k1FpMont {
   static constexpr int BITS = 256;
   static constexpr uint32_t QINV = 0xd2253531u;
   static constexpr int FORM = 0;
+  static constexpr bool SQR_ROWS = false;
   static constexpr uint64_t QINV62 = 0x27c7f6e22ddacacfull;  // q^-1 mod 2^62
   ECC_DEV static constexpr uint32_t qinv() { return QINV; }
   ECC_DEV static constexpr uint64_t qinv62() { return QINV62; }
@@ -62,6 +64,7 @@ struct Secp256k1Fn {
   static constexpr int BITS = 256;
   static constexpr uint32_t QINV = 0x5588b13fu;
   static constexpr int FORM = 0;
+  static constexpr bool SQR_ROWS = false;
   static constexpr uint64_t QINV62 = 0x34f20099aa774ec1ull;  // q^-1 mod 2^62
   ECC_DEV static constexpr uint32_t qinv() { return QINV; }
   ECC_DEV static constexpr uint64_t qinv62() { return QINV62; }
@@ -132,6 +135,7 @@ struct P256Fp {
   static constexpr int BITS = 256;
   static constexpr uint32_t QINV = 0x00000001u;
   static constexpr int FORM = 1;
+  static constexpr bool SQR_ROWS = false;
   static constexpr uint64_t QINV62 = 0x3fffffffffffffffull;  // q^-1 mod 2^62
   ECC_DEV static constexpr uint32_t qinv() { return QINV; }
   ECC_DEV static constexpr uint64_t qinv62() { return QINV62; }
@@ -161,6 +165,7 @@ struct P256Fn {
   static constexpr int BITS = 256;
   static constexpr uint32_t QINV = 0xee00bc4fu;
   static constexpr int FORM = 0;
+  static constexpr bool SQR_ROWS = false;
   static constexpr uint64_t QINV62 = 0x332e375511ff43b1ull;  // q^-1 mod 2^62
   ECC_DEV static constexpr uint32_t qinv() { return QINV; }
   ECC_DEV static constexpr uint64_t qinv62() { return QINV62; }
@@ -209,6 +214,7 @@ struct BN254Fp {
   static constexpr int BITS = 254;
   static constexpr uint32_t QINV = 0xe4866389u;
   static constexpr int FORM = 0;
+  static constexpr bool SQR_ROWS = true;
   static constexpr uint64_t QINV62 = 0x382df87d1b799c77ull;  // q^-1 mod 2^62
   ECC_DEV static constexpr uint32_t qinv() { return QINV; }
   ECC_DEV static constexpr uint64_t qinv62() { return QINV62; }
@@ -234,6 +240,7 @@ struct BN254Fn {
   static constexpr int BITS = 254;
   static constexpr uint32_t QINV = 0xefffffffu;
   static constexpr int FORM = 0;
+  static constexpr bool SQR_ROWS = true;
   static constexpr uint64_t QINV62 = 0x3d1e0a6c10000001ull;  // q^-1 mod 2^62
   ECC_DEV static constexpr uint32_t qinv() { return QINV; }
   ECC_DEV static constexpr uint64_t qinv62() { return QINV62; }
@@ -304,6 +311,7 @@ struct BLS12_381Fp {
   static constexpr int BITS = 381;
   static constexpr uint32_t QINV = 0xfffcfffdu;
   static constexpr int FORM = 0;
+  static constexpr bool SQR_ROWS = true;
   static constexpr uint64_t QINV62 = 0x360c000300030003ull;  // q^-1 mod 2^62
   ECC_DEV static constexpr uint32_t qinv() { return QINV; }
   ECC_DEV static constexpr uint64_t qinv62() { return QINV62; }
@@ -329,6 +337,7 @@ struct BLS12_381Fn {
   static constexpr int BITS = 255;
   static constexpr uint32_t QINV = 0xffffffffu;
   static constexpr int FORM = 0;
+  static constexpr bool SQR_ROWS = true;
   static constexpr uint64_t QINV62 = 0x0000000100000001ull;  // q^-1 mod 2^62
   ECC_DEV static constexpr uint32_t qinv() { return QINV; }
   ECC_DEV static constexpr uint64_t qinv62() { return QINV62; }
@@ -377,6 +386,7 @@ struct SM2Fp {
   static constexpr int BITS = 256;
   static constexpr uint32_t QINV = 0x00000001u;
   static constexpr int FORM = 3;
+  static constexpr bool SQR_ROWS = false;
   static constexpr uint64_t QINV62 = 0x3fffffffffffffffull;  // q^-1 mod 2^62
   ECC_DEV static constexpr uint32_t qinv() { return QINV; }
   ECC_DEV static constexpr uint64_t qinv62() { return QINV62; }
@@ -406,6 +416,7 @@ struct SM2Fn {
   static constexpr int BITS = 256;
   static constexpr uint32_t QINV = 0x72350975u;
   static constexpr int FORM = 0;
+  static constexpr bool SQR_ROWS = false;
   static constexpr uint64_t QINV62 = 0x0d8061778dcaf68bull;  // q^-1 mod 2^62
   ECC_DEV static constexpr uint32_t qinv() { return QINV; }
   ECC_DEV static constexpr uint64_t qinv62() { return QINV62; }

@@ -512,20 +512,175 @@ ECC_DEV void mont_mul(uint32_t* r, const uint32_t* a, const uint32_t* b) {
   fe_sub_once<F>(r, t);
 }
 
+// r = a^2 R^-1 mod q for q < 2^(32 N - 1), rows as in mont_mul: row i adds only
+// a_i^2 and 2 a_i a_j, j > i, so it has N - i products and its lowest word is i; the
+// reduction row of word 0 can go first.  N (N + 1) / 2 + N^2 + N multiply-adds (108 of
+// 136 with 8 limbs, 234 of 300 with 12) in as many registers as mont_mul.
+template <class F>
+ECC_DEV void mont_sqr_rows(uint32_t* r, const uint32_t* a) {
+  constexpr int N = F::N;
+  uint32_t c[N + 1], d[N + 1], a2[N];  // a2: limbs of 2 a
+#pragma unroll
+  for (int i = 0; i < N + 1; ++i) c[i] = d[i] = 0;
+#pragma unroll
+  for (int i = 1; i < N; ++i) a2[i] = __funnelshift_l(a[i - 1], a[i], 1);
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    // the row's factor of a_i at word j >= i: 2 (a >> 32 (i + 1)) has no bit of a_i
+    auto f = [&](int j) { return j == i ? a[i] : j == i + 1 ? a[j] << 1 : a2[j]; };
+    auto row = [&]() {
+      const int o = i | 1, e = (i + 1) & ~1;  // first odd and even word
+#pragma unroll
+      for (int j = o; j < N; j += 2) {
+        d[j - 1] = j == o ? ptx::mad_lo_cc(f(j), a[i], d[j - 1]) : ptx::madc_lo_cc(f(j), a[i], d[j - 1]);
+        d[j] = ptx::madc_hi_cc(f(j), a[i], d[j]);
+      }
+      d[N] = ptx::addc(d[N], 0);
+      if (e < N) {
+#pragma unroll
+        for (int j = e; j < N; j += 2) {
+          c[j] = j == e ? ptx::mad_lo_cc(f(j), a[i], c[j]) : ptx::madc_lo_cc(f(j), a[i], c[j]);
+          c[j + 1] = ptx::madc_hi_cc(f(j), a[i], c[j + 1]);
+        }
+        c[N] = ptx::addc(c[N], 0);
+      }
+    };
+    uint32_t u;
+    if (i == 0) {
+      row();
+      u = c[0] * F::qinv();
+      d[0] = ptx::mad_lo_cc(u, F::p(1), d[0]);
+    } else {  // T /= 2^32; the carry of d0 + c1 enters the odd reduction chain
+      const uint32_t nc0 = ptx::add_cc(d[0], c[1]);
+#pragma unroll
+      for (int k = 0; k < N - 1; ++k) {
+        const uint32_t t = d[k + 1];
+        d[k] = c[k + 2];
+        c[k + 1] = t;
+      }
+      c[N] = d[N];
+      c[0] = nc0;
+      d[N - 1] = 0;
+      d[N] = 0;
+      u = nc0 * F::qinv();
+      d[0] = ptx::madc_lo_cc(u, F::p(1), d[0]);
+    }
+    d[1] = ptx::madc_hi_cc(u, F::p(1), d[1]);
+#pragma unroll
+    for (int j = 3; j < N; j += 2) {
+      d[j - 1] = ptx::madc_lo_cc(u, F::p(j), d[j - 1]);
+      d[j] = ptx::madc_hi_cc(u, F::p(j), d[j]);
+    }
+    d[N] = ptx::addc(d[N], 0);
+    c[0] = ptx::mad_lo_cc(u, F::p(0), c[0]);
+    c[1] = ptx::madc_hi_cc(u, F::p(0), c[1]);
+#pragma unroll
+    for (int j = 2; j < N; j += 2) {
+      c[j] = ptx::madc_lo_cc(u, F::p(j), c[j]);
+      c[j + 1] = ptx::madc_hi_cc(u, F::p(j), c[j + 1]);
+    }
+    c[N] = ptx::addc(c[N], 0);
+    if (i > 0) row();
+  }
+  uint32_t t[N + 1];
+  t[0] = ptx::add_cc(d[0], c[1]);
+#pragma unroll
+  for (int k = 1; k < N; ++k) t[k] = ptx::addc_cc(d[k], c[k + 1]);
+  t[N] = ptx::addc(d[N], 0);
+  fe_sub_once<F>(r, t);
+}
+
+// r = (a b + x y) R^-1 mod q for q < R / 4 with one reduction (2 N^2 + N^2 + N
+// multiply-adds instead of 4 N^2 + 2 N): the sum is below 2 q R / 4 + q R, so one
+// subtraction is enough.
+template <class F>
+ECC_DEV void mont_mul2(uint32_t* r, const uint32_t* a, const uint32_t* b, const uint32_t* x, const uint32_t* y) {
+  constexpr int N = F::N;
+  static_assert(F::BITS <= 32 * N - 2, "room for the sum");
+  uint32_t c[N + 1], d[N + 1];
+#pragma unroll
+  for (int i = 0; i < N + 1; ++i) c[i] = d[i] = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    if (i == 0) {
+      d[0] = ptx::mad_lo_cc(a[1], b[0], d[0]);
+    } else {
+      const uint32_t nc0 = ptx::add_cc(d[0], c[1]);
+#pragma unroll
+      for (int k = 0; k < N - 1; ++k) {
+        const uint32_t t = d[k + 1];
+        d[k] = c[k + 2];
+        c[k + 1] = t;
+      }
+      c[N] = d[N];
+      c[0] = nc0;
+      d[N - 1] = 0;
+      d[N] = 0;
+      d[0] = ptx::madc_lo_cc(a[1], b[i], d[0]);
+    }
+    d[1] = ptx::madc_hi_cc(a[1], b[i], d[1]);
+#pragma unroll
+    for (int j = 3; j < N; j += 2) {
+      d[j - 1] = ptx::madc_lo_cc(a[j], b[i], d[j - 1]);
+      d[j] = ptx::madc_hi_cc(a[j], b[i], d[j]);
+    }
+    d[N] = ptx::addc(d[N], 0);
+#pragma unroll
+    for (int j = 1; j < N; j += 2) {
+      d[j - 1] = j == 1 ? ptx::mad_lo_cc(x[j], y[i], d[j - 1]) : ptx::madc_lo_cc(x[j], y[i], d[j - 1]);
+      d[j] = ptx::madc_hi_cc(x[j], y[i], d[j]);
+    }
+    d[N] = ptx::addc(d[N], 0);
+#pragma unroll
+    for (int j = 0; j < N; j += 2) {
+      c[j] = j == 0 ? ptx::mad_lo_cc(a[j], b[i], c[j]) : ptx::madc_lo_cc(a[j], b[i], c[j]);
+      c[j + 1] = ptx::madc_hi_cc(a[j], b[i], c[j + 1]);
+    }
+    c[N] = ptx::addc(c[N], 0);
+#pragma unroll
+    for (int j = 0; j < N; j += 2) {
+      c[j] = j == 0 ? ptx::mad_lo_cc(x[j], y[i], c[j]) : ptx::madc_lo_cc(x[j], y[i], c[j]);
+      c[j + 1] = ptx::madc_hi_cc(x[j], y[i], c[j + 1]);
+    }
+    c[N] = ptx::addc(c[N], 0);
+    const uint32_t u = c[0] * F::qinv();
+#pragma unroll
+    for (int j = 0; j < N; j += 2) {
+      c[j] = j == 0 ? ptx::mad_lo_cc(u, F::p(j), c[j]) : ptx::madc_lo_cc(u, F::p(j), c[j]);
+      c[j + 1] = ptx::madc_hi_cc(u, F::p(j), c[j + 1]);
+    }
+    c[N] = ptx::addc(c[N], 0);
+#pragma unroll
+    for (int j = 1; j < N; j += 2) {
+      d[j - 1] = j == 1 ? ptx::mad_lo_cc(u, F::p(j), d[j - 1]) : ptx::madc_lo_cc(u, F::p(j), d[j - 1]);
+      d[j] = ptx::madc_hi_cc(u, F::p(j), d[j]);
+    }
+    d[N] = ptx::addc(d[N], 0);
+  }
+  uint32_t t[N + 1];
+  t[0] = ptx::add_cc(d[0], c[1]);
+#pragma unroll
+  for (int k = 1; k < N; ++k) t[k] = ptx::addc_cc(d[k], c[k + 1]);
+  t[N] = ptx::addc(d[N], 0);
+  fe_sub_once<F>(r, t);
+}
+
 template <class F>
 ECC_DEV void mont_sqr(uint32_t* r, const uint32_t* a) {
   if constexpr (F::FORM != 0) {
     uint32_t T[16];
     sqr_wide8(T, a);
     reduce_wide<F>(r, T);
+  } else if constexpr (F::SQR_ROWS) {
+    mont_sqr_rows<F>(r, a);
   } else {
     mont_mul<F>(r, a, a);
   }
 }
 
-// r = a b - c d, with one reduction of the difference of the two products for
-// FORM 1-3 (52 additions fewer than two reductions and a subtraction): a negative
-// difference gets q 2^256.
+// r = a b - c d with one reduction: of the difference of the two products for FORM
+// 1-3 (52 additions fewer than two reductions and a subtraction; a negative
+// difference gets q 2^256), of a b + (q - c) d for the others.
 ECC_DEV bool sub_wide(uint32_t* A, const uint32_t* B) {
   A[0] = ptx::sub_cc(A[0], B[0]);
 #pragma unroll
@@ -552,10 +707,9 @@ ECC_DEV void mont_mul_sub(uint32_t* r, const uint32_t* a, const uint32_t* b, con
     mul_wide8(B, c, d);
     reduce_diff<F>(r, A, B);
   } else {
-    uint32_t t[F::N], u[F::N];
-    mont_mul<F>(t, a, b);
-    mont_mul<F>(u, c, d);
-    fe_sub<F>(r, t, u);
+    uint32_t t[F::N];
+    fe_neg<F>(t, c);
+    mont_mul2<F>(r, a, b, t, d);
   }
 }
 
@@ -568,10 +722,9 @@ ECC_DEV void mont_mul_sub_sqr(uint32_t* r, const uint32_t* a, const uint32_t* b,
     sqr_wide8(B, c);
     reduce_diff<F>(r, A, B);
   } else {
-    uint32_t t[F::N], u[F::N];
-    mont_mul<F>(t, a, b);
-    mont_sqr<F>(u, c);
-    fe_sub<F>(r, t, u);
+    uint32_t t[F::N];
+    fe_neg<F>(t, c);
+    mont_mul2<F>(r, a, b, t, c);
   }
 }
 

@@ -75,6 +75,7 @@ def traits(name, q, form):
     s += f"  static constexpr int BITS = {q.bit_length()};\n"
     s += f"  static constexpr uint32_t QINV = 0x{qinv:08x}u;\n"
     s += f"  static constexpr int FORM = {form};\n"
+    s += f"  static constexpr bool SQR_ROWS = {'true' if q.bit_length() < 32 * n else 'false'};\n"
     s += f"  static constexpr uint64_t QINV62 = 0x{pow(q, -1, 1 << 62):016x}ull;  // q^-1 mod 2^62\n"
     s += "  ECC_DEV static constexpr uint32_t qinv() { return QINV; }\n"
     s += "  ECC_DEV static constexpr uint64_t qinv62() { return QINV62; }\n"

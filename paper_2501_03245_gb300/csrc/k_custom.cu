@@ -25,6 +25,7 @@ __shared__ CustomConsts g_custom;
 struct CustomFp {
   static constexpr int N = 8;
   static constexpr int FORM = 0;
+  static constexpr bool SQR_ROWS = false;  // p may have 256 bits
   ECC_DEV static uint32_t qinv() { return g_custom.qinv; }
   ECC_DEV static uint64_t qinv62() { return g_custom.qinv62; }
   ECC_DEV static uint32_t p(int i) { return g_custom.p[i]; }
