@@ -5,9 +5,7 @@
 //
 // A chain of group operations by one thread costs a product's latency for each of
 // an operation's products (16 for an addition, 7 for a doubling; 0.42 us each with
-// 8 limbs, 0.9 with 12).  The four lanes of a quad hold the same points and take
-// one product each of a step's independent ones: 5 steps for an addition and 3 for
-// a doubling.
+// 8 limbs, 0.9 with 12); a quad (ladder.cuh) takes 5 steps and 3.
 #pragma once
 #include "ladder.cuh"
 
@@ -95,59 +93,7 @@ ECC_DEV void jac_addto(uint32_t* X1, uint32_t* Y1, uint32_t* Z1, const uint32_t*
   call_mul_sub<F>(Y1, r, U, S, H);
 }
 
-// ---------------------------------------------------------------- quads
-// The four lanes of a quad call these together with equal points; other quads of
-// the warp may be elsewhere.
-
-ECC_DEV unsigned quad_mask() { return 0xfu << (threadIdx.x & 28u); }
-
-template <class F>
-ECC_DEV void quad_get(uint32_t* r, const uint32_t* a, int lane) {
-  const unsigned m = quad_mask();
-#pragma unroll
-  for (int i = 0; i < F::N; ++i) r[i] = __shfl_sync(m, a[i], lane, 4);
-}
-
-// this lane's factor: a, b, c or d for lane 0, 1, 2 or 3 of the quad
-template <class F>
-ECC_DEV void quad_pick(uint32_t* r, const uint32_t* a, const uint32_t* b, const uint32_t* c, const uint32_t* d) {
-  const unsigned q = threadIdx.x & 3u;
-#pragma unroll
-  for (int i = 0; i < F::N; ++i) {
-    const uint32_t lo = (q & 1u) ? b[i] : a[i], hi = (q & 1u) ? d[i] : c[i];
-    r[i] = (q & 2u) ? hi : lo;
-  }
-}
-
-// P <- 2 P with the halved Z of jac_dbl_half
-template <class C>
-ECC_DEV void quad_dbl(JacReg<typename C::Fp>& P) {
-  using F = typename C::Fp;
-  constexpr int N = F::N;
-  static_assert(C::A_ZERO, "a = 0");
-  uint32_t a[N], b[N], p[N], l[N], YY[N], D[N];
-  quad_pick<F>(a, P.X.v, P.Y.v, P.Y.v, P.X.v);
-  quad_pick<F>(b, P.X.v, P.Y.v, P.Z.v, P.X.v);
-  mont_mul<F>(p, a, b);  // X^2, Y^2, Y Z
-  quad_get<F>(l, p, 0);
-  quad_get<F>(YY, p, 1);
-  quad_get<F>(P.Z.v, p, 2);
-  fe_half<F>(a, l);
-  fe_add<F>(l, l, a);    // 3 X^2 / 2
-  quad_pick<F>(a, YY, P.X.v, l, l);
-  quad_pick<F>(b, YY, YY, l, l);
-  mont_mul<F>(p, a, b);  // Y^4, X Y^2, l^2
-  quad_get<F>(D, p, 1);
-  quad_get<F>(P.X.v, p, 2);
-  quad_get<F>(YY, p, 0);
-  fe_sub<F>(P.X.v, P.X.v, D);
-  fe_sub<F>(P.X.v, P.X.v, D);
-  fe_sub<F>(D, D, P.X.v);
-  mont_mul<F>(P.Y.v, l, D);
-  fe_sub<F>(P.Y.v, P.Y.v, YY);
-}
-
-// P <- P + Q, every case of the group law
+// P <- P + Q by a quad, every case of the group law
 template <class C>
 ECC_DEV void quad_add(JacReg<typename C::Fp>& P, JacReg<typename C::Fp> Q) {
   using F = typename C::Fp;

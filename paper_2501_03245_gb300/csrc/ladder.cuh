@@ -181,6 +181,135 @@ ECC_DEV void jac_madd(uint32_t* X, uint32_t* Y, uint32_t* Z, const uint32_t* x, 
   call_mul_sub<F>(Y, r, V, Y, t);
 }
 
+// ---------------------------------------------------------------- quads
+// A group operation by the four lanes of a quad, for chains with too few of them to
+// fill the GPU: the lanes hold the same points and take one product each of a
+// step's independent ones, so a doubling costs 3 (a = 0) or 4 products' latency and
+// an addition of an affine point 5, instead of 7, 8 and 11, plus the exchange of the
+// products.  The four lanes call these together with equal operands; other quads of
+// the warp may be elsewhere.
+
+ECC_DEV unsigned quad_mask() { return 0xfu << (threadIdx.x & 28u); }
+
+template <class F>
+ECC_DEV void quad_get(uint32_t* r, const uint32_t* a, int lane) {
+  const unsigned m = quad_mask();
+#pragma unroll
+  for (int i = 0; i < F::N; ++i) r[i] = __shfl_sync(m, a[i], lane, 4);
+}
+
+// this lane's factor: a, b, c or d for lane 0, 1, 2 or 3 of the quad
+template <class F>
+ECC_DEV void quad_pick(uint32_t* r, const uint32_t* a, const uint32_t* b, const uint32_t* c, const uint32_t* d) {
+  const unsigned q = threadIdx.x & 3u;
+#pragma unroll
+  for (int i = 0; i < F::N; ++i) {
+    const uint32_t lo = (q & 1u) ? b[i] : a[i], hi = (q & 1u) ? d[i] : c[i];
+    r[i] = (q & 2u) ? hi : lo;
+  }
+}
+
+// P <- 2 P, the formulas of jac_dbl_half
+template <class C>
+ECC_DEV void quad_dbl(JacReg<typename C::Fp>& P) {
+  using F = typename C::Fp;
+  constexpr int N = F::N;
+  uint32_t a[N], b[N], p[N], l[N], YY[N], D[N];
+  if constexpr (C::A_ZERO) {
+    quad_pick<F>(a, P.X.v, P.Y.v, P.Y.v, P.X.v);
+    quad_pick<F>(b, P.X.v, P.Y.v, P.Z.v, P.X.v);
+    mont_mul<F>(p, a, b);  // X^2, Y^2, Y Z
+    quad_get<F>(l, p, 0);
+    quad_get<F>(YY, p, 1);
+    quad_get<F>(P.Z.v, p, 2);
+    fe_half<F>(a, l);
+    fe_add<F>(l, l, a);    // 3 X^2 / 2
+    quad_pick<F>(a, YY, P.X.v, l, l);
+    quad_pick<F>(b, YY, YY, l, l);
+    mont_mul<F>(p, a, b);  // Y^4, X Y^2, l^2
+  } else {
+    quad_pick<F>(a, P.Z.v, P.Y.v, P.Y.v, P.Z.v);
+    quad_pick<F>(b, P.Z.v, P.Y.v, P.Z.v, P.Z.v);
+    mont_mul<F>(p, a, b);  // Z^2, Y^2, Y Z
+    quad_get<F>(l, p, 0);
+    quad_get<F>(YY, p, 1);
+    quad_get<F>(P.Z.v, p, 2);
+    fe_add<F>(D, P.X.v, l);
+    fe_sub<F>(l, P.X.v, l);
+    quad_pick<F>(a, YY, P.X.v, l, l);
+    quad_pick<F>(b, YY, YY, D, D);
+    mont_mul<F>(p, a, b);  // Y^4, X Y^2, X^2 - Z^4
+    quad_get<F>(l, p, 2);
+    fe_half<F>(a, l);
+    fe_add<F>(l, l, a);
+    mont_mul<F>(a, l, l);  // l^2, in every lane; p keeps the other products
+  }
+  quad_get<F>(YY, p, 0);
+  quad_get<F>(D, p, 1);
+  if constexpr (C::A_ZERO) {
+    quad_get<F>(P.X.v, p, 2);
+  } else {
+    fe_copy<F>(P.X.v, a);
+  }
+  fe_sub<F>(P.X.v, P.X.v, D);
+  fe_sub<F>(P.X.v, P.X.v, D);
+  fe_sub<F>(D, D, P.X.v);
+  mont_mul<F>(P.Y.v, l, D);
+  fe_sub<F>(P.Y.v, P.Y.v, YY);
+}
+
+// jac_madd by a quad
+template <class C>
+ECC_DEV void quad_madd(JacReg<typename C::Fp>& P, const uint32_t* x, const uint32_t* y, uint32_t* H) {
+  using F = typename C::Fp;
+  constexpr int N = F::N;
+  if (fe_is_zero<F>(P.Z.v)) {
+    fe_copy<F>(P.X.v, x);
+    fe_copy<F>(P.Y.v, y);
+    fe_set_one<F>(P.Z.v);
+    return;
+  }
+  uint32_t a[N], b[N], p[N], t[N], r[N], V[N];
+  quad_pick<F>(a, P.Z.v, y, P.Z.v, y);
+  mont_mul<F>(p, a, P.Z.v);  // Z^2, y Z
+  quad_get<F>(t, p, 0);
+  quad_get<F>(r, p, 1);
+  quad_pick<F>(a, x, r, x, r);
+  mont_mul<F>(p, a, t);      // x Z^2, y Z^3
+  quad_get<F>(H, p, 0);
+  fe_sub<F>(H, H, P.X.v);
+  quad_get<F>(r, p, 1);
+  fe_sub<F>(r, r, P.Y.v);
+  if (fe_is_zero<F>(H)) {
+    if (fe_is_zero<F>(r)) {
+      jac_dbl_rare<C>(P.X.v, P.Y.v, P.Z.v);
+    } else {
+      fe_set_zero<F>(P.Z.v);
+    }
+    return;
+  }
+  quad_pick<F>(a, H, P.Z.v, r, H);
+  quad_pick<F>(b, H, H, r, H);
+  mont_mul<F>(p, a, b);      // H^2, Z H, r^2
+  quad_get<F>(t, p, 0);
+  quad_get<F>(P.Z.v, p, 1);
+  quad_get<F>(V, p, 2);
+  quad_pick<F>(a, P.X.v, H, P.X.v, H);
+  mont_mul<F>(p, a, t);      // X H^2, H^3
+  quad_get<F>(t, p, 1);
+  fe_sub<F>(P.X.v, V, t);
+  quad_get<F>(V, p, 0);
+  fe_sub<F>(P.X.v, P.X.v, V);
+  fe_sub<F>(P.X.v, P.X.v, V);
+  fe_sub<F>(V, V, P.X.v);
+  quad_pick<F>(a, r, P.Y.v, r, P.Y.v);
+  quad_pick<F>(b, V, t, V, t);
+  mont_mul<F>(p, a, b);      // r (V - X3), Y H^3
+  quad_get<F>(a, p, 0);
+  quad_get<F>(b, p, 1);
+  fe_sub<F>(P.Y.v, a, b);
+}
+
 // ---------------------------------------------------------------- fixed base
 // Table of a generator: entry (j, v) = v 2^(16 j) G for v = 1 .. 2^15, j < 16, as
 // affine Montgomery points (x limbs, y limbs; row j 2^15 + v - 1).  With signed

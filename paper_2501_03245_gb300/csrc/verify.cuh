@@ -11,7 +11,7 @@
 //   * u2 Q: signed kQW-bit fixed windows, most significant first: 255 doublings
 //     and at most 52 additions of affine table points.  secp256k1 splits u2 = k1 +
 //     k2 lambda (glv.cuh): 125 doublings and the same additions, those of k2 with
-//     beta x in the place of x (one triple 0.71 -> 0.55 ms);
+//     beta x in the place of x (30000 triples 0.89 -> 0.80 ms, one by a thread 0.71 -> 0.55);
 //   * u1 G: 16 additions from the generator's table onto the same accumulator
 //     (the digits of u1 need no doublings);
 //   * x_R mod n == r without an inversion: X = r Z^2 or X = (r + n) Z^2.
@@ -166,43 +166,71 @@ ECC_DEV bool verify_prep(const VerifyArgs<C>& a, size_t i, size_t slot) {
 
 // The chain's points (X_k, Y_k) and H_k, k = 2 .. kQTable, become affine in
 // place; zi = 1 / Z of the last one.
-template <class C>
+template <class C, bool QUAD>
 ECC_DEV void verify_table_affine(const VerifyArgs<C>& a, size_t slot, uint32_t* zi) {
   using F = typename C::Fp;
   constexpr int N = F::N;
 #pragma unroll 1
   for (int k = kQTable; k >= 2; --k) {
-    uint32_t x[N], y[N], t[N];
+    uint32_t x[N], y[N], t[N], h[N];
     const size_t row = slot * kQTable + k - 1;
     load_affine<F>(a.table, row, x, y);
-    call_sqr<F>(t, zi);
-    call_mul<F>(x, x, t);
-    call_mul<F>(t, t, zi);
-    call_mul<F>(y, y, t);
+    a.H.load((size_t)(k - 1) * a.slots + slot, h);
+    if constexpr (QUAD) {
+      uint32_t u[N], p[N];
+      quad_pick<F>(u, zi, h, zi, h);
+      mont_mul<F>(p, u, zi);  // zi^2, zi h
+      quad_get<F>(t, p, 0);
+      quad_pick<F>(u, x, zi, x, zi);
+      quad_get<F>(zi, p, 1);
+      mont_mul<F>(p, u, t);   // x zi^2, zi^3
+      quad_get<F>(x, p, 0);
+      quad_get<F>(t, p, 1);
+      mont_mul<F>(y, y, t);
+    } else {
+      call_sqr<F>(t, zi);
+      call_mul<F>(x, x, t);
+      call_mul<F>(t, t, zi);
+      call_mul<F>(y, y, t);
+      call_mul<F>(zi, zi, h);
+    }
     store_affine<F>(a.table, row, x, y);
-    a.H.load((size_t)(k - 1) * a.slots + slot, t);
-    call_mul<F>(zi, zi, t);
   }
 }
 
-template <class C>
+// QUAD: four lanes per item, each doing all of it but the products of the group
+// operations, which they share; what they store they store alike.
+template <class C, bool QUAD>
 __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_verify(VerifyArgs<C> a) {
   using F = typename C::Fp;
   constexpr int N = F::N;
   static_assert(N == 8 && C::Fn::N == 8, "256-bit curves");
   using QWin = QWindows<C>;
-  const size_t slot = blockIdx.x * (size_t)kLadderThreads + threadIdx.x;
+  constexpr int kItems = kLadderThreads / (QUAD ? 4 : 1);  // of a CTA
+  const size_t own = QUAD ? threadIdx.x / 4 : threadIdx.x;
+  const size_t slot = blockIdx.x * (size_t)kItems + own;
   // threads past the batch repeat its last item (the barriers need every thread)
 #pragma unroll 1
-  for (size_t i0 = blockIdx.x * (size_t)kLadderThreads; i0 < a.n; i0 += a.slots) {
-    const bool mine = i0 + threadIdx.x < a.n;
-    const size_t i = mine ? i0 + threadIdx.x : a.n - 1;
+  for (size_t i0 = blockIdx.x * (size_t)kItems; i0 < a.n; i0 += a.slots) {
+    const bool mine = i0 + own < a.n;
+    const size_t i = mine ? i0 + own : a.n - 1;
     const bool valid = verify_prep<C>(a, i, slot);
-    uint32_t X[N], Y[N], Z[N], H[N], x[N], y[N];
+    JacReg<F> P;
+    uint32_t* const X = P.X.v;
+    uint32_t* const Y = P.Y.v;
+    uint32_t* const Z = P.Z.v;
+    uint32_t H[N], x[N], y[N];
+    auto dbl = [&]() {
+      if constexpr (QUAD) {
+        quad_dbl<C>(P);
+      } else {
+        jac_dbl_half<C>(X, Y, Z);
+      }
+    };
     // table chain: 2Q by doubling (Z = y_Q), then + Q up to kQTable Q
     load_affine<F>(a.table, slot * kQTable, X, Y);
     fe_set_one<F>(Z);
-    jac_dbl_half<C>(X, Y, Z);
+    dbl();
     a.H.store(a.slots + slot, Z);
     store_affine<F>(a.table, slot * kQTable + 1, X, Y);
     constexpr int kChain = kQTable - 2;
@@ -222,13 +250,13 @@ __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_verify(Ver
         const int w = QWin::DIGITS - 1 - step / QWin::HALVES;
         if (step == 0) {
           fe_inv_mont<F>(x, Z);
-          verify_table_affine<C>(a, slot, x);
+          verify_table_affine<C, QUAD>(a, slot, x);
           fe_set_zero<F>(Z);
         } else if (half == 0) {
 #pragma unroll 1
           for (int k = 0; k < kQW; ++k) {
             __syncthreads();
-            jac_dbl_half<C>(X, Y, Z);
+            dbl();
           }
         }
         const int bit = kQW * w, wd = bit >> 5, sh = bit & 31;
@@ -262,7 +290,11 @@ __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_verify(Ver
             call_mul<F>(x, x, beta);
           }
         }
-        jac_madd<C>(X, Y, Z, x, y, H);
+        if constexpr (QUAD) {
+          quad_madd<C>(P, x, y, H);
+        } else {
+          jac_madd<C>(X, Y, Z, x, y, H);
+        }
       }
       if (it < kChain) {
         a.H.store((size_t)(it + 2) * a.slots + slot, H);

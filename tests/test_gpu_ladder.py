@@ -86,3 +86,24 @@ def test_verify_sizes(gpu_lib, n):
     gpu_lib.ecc_verify_batch(1, n, *(to_cuda(np.ascontiguousarray(a[idx])) for a in (e, r, s, pub)), ok)
     torch.cuda.synchronize()
     assert np.array_equal(from_cuda(ok), (idx % 3 != 0).astype(np.uint8))
+
+
+@pytest.mark.parametrize("cid", [0, 1, 4])
+def test_quads_and_threads_agree(gpu_lib, cid):
+    """The largest batch that four lanes verify an item of, and one more, with the edge
+    digits and colliding points in the rows of both."""
+    import torch
+
+    n = curves.BY_ID[cid].n
+    us = [1, 16, 17, n - 1, n - 17, n // 2]
+    dus = [(d, u1, u2) for d in (1, n - 1, 16) for u2 in us for u1 in (0, 1, 0x8000, u2 * d % n, -u2 * d % n)]
+    e, r, s, pub = triples(cid, dus)
+    r[1::7, 31] ^= 1
+    want = cpp_oracle.verify(cid, e, r, s, pub)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for m in (1, 31, 33, 64 * sms, 64 * sms + 1):
+        idx = np.arange(m) * 11 % len(e)
+        ok = torch.full((m,), 7, dtype=torch.uint8, device="cuda")
+        gpu_lib.ecc_verify_batch(cid, m, *(to_cuda(np.ascontiguousarray(a[idx])) for a in (e, r, s, pub)), ok)
+        torch.cuda.synchronize()
+        assert np.array_equal(from_cuda(ok), want[idx]), m
