@@ -2,7 +2,9 @@
 // batched ECDSA signing (Section 5.2: one modinv plus one FPMUL), one thread per
 // item (ladder.cuh): k G is 16 additions of entries of the generator's table,
 // then one inversion makes the result affine.  A signature does k G and d G one
-// after the other through the same loop and inverts both Z together.
+// after the other through the same loop and inverts both Z together.  Small batches
+// (QUAD) take the four lanes of a quad per item, which do all of it alike but the
+// products of the additions.
 #pragma once
 #include "ladder.cuh"
 
@@ -32,9 +34,9 @@ ECC_DEV void scalar_mod_n(uint32_t* k) {
 }
 
 // P += digit j of the recoded scalar kr (9 words) times 2^(16 j) G
-template <class C>
-ECC_DEV void comb_add(const uint32_t* TG, uint32_t word, uint32_t carry, bool neg, int j, uint32_t* X,
-                      uint32_t* Y, uint32_t* Z) {
+template <class C, bool QUAD>
+ECC_DEV void comb_add(const uint32_t* TG, uint32_t word, uint32_t carry, bool neg, int j,
+                      JacReg<typename C::Fp>& P) {
   using F = typename C::Fp;
   constexpr int N = F::N;
   const int d = comb_digit(word, carry, j);
@@ -42,29 +44,45 @@ ECC_DEV void comb_add(const uint32_t* TG, uint32_t word, uint32_t carry, bool ne
   uint32_t x[N], y[N], H[N];
   load_affine<F>(TG, (size_t)j * kGEntries + (d < 0 ? -d : d) - 1, x, y);
   if ((d < 0) != neg) fe_neg<F>(y, y);
-  jac_madd<C>(X, Y, Z, x, y, H);
+  if constexpr (QUAD) {
+    quad_madd<C>(P, x, y, H);
+  } else {
+    jac_madd<C>(P.X.v, P.Y.v, P.Z.v, x, y, H);
+  }
 }
 
-template <class C>
-__global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_fpmul(FixedArgs<C> a) {
+// This thread's item: its number and whether it writes the results.  Threads past the
+// batch repeat its last item (the barriers need every thread).
+template <bool QUAD>
+ECC_DEV size_t comb_item(size_t n, bool& writes) {
+  const size_t t = blockIdx.x * (size_t)kLadderThreads + threadIdx.x, g = QUAD ? t / 4 : t;
+  writes = g < n && (!QUAD || (t & 3) == 0);
+  return g < n ? g : n - 1;
+}
+
+template <class C, bool QUAD>
+__global__ void __launch_bounds__(kLadderThreads, QUAD ? 2 : kLadderCtasPerSm) k_fpmul(FixedArgs<C> a) {
   using F = typename C::Fp;
   constexpr int N = F::N;
-  // threads past the batch repeat its last item (the barriers need every thread)
-  const size_t g = blockIdx.x * (size_t)kLadderThreads + threadIdx.x, i = g < a.n ? g : a.n - 1;
+  bool writes;
+  const size_t i = comb_item<QUAD>(a.n, writes);
   uint32_t k[9];
 #pragma unroll
   for (int q = 0; q < 8; ++q) k[q] = a.k[8 * i + q];
   scalar_mod_n<C>(k);
   bool neg;
   comb_recode<C>(k, neg);
-  uint32_t X[N], Y[N], Z[N];
+  JacReg<F> P;
+  uint32_t* const X = P.X.v;
+  uint32_t* const Y = P.Y.v;
+  uint32_t* const Z = P.Z.v;
   fe_set_zero<F>(X);
   fe_set_zero<F>(Y);
   fe_set_zero<F>(Z);
 #pragma unroll 1
   for (int j = 0; j < kGRows; ++j) {
     __syncthreads();
-    comb_add<C>(a.TG, k[0], k[8], neg, j, X, Y, Z);
+    comb_add<C, QUAD>(a.TG, k[0], k[8], neg, j, P);
     if (j & 1) {  // next word
 #pragma unroll
       for (int q = 0; q < 7; ++q) k[q] = k[q + 1];
@@ -78,7 +96,8 @@ __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_fpmul(Fixe
   mont_mul<F>(Y, Y, t);
   from_mont<F>(X, X);
   from_mont<F>(Y, Y);
-  if (g >= a.n) return;
+  if constexpr (QUAD) __syncwarp();  // the scalar may be in the output's buffer
+  if (!writes) return;
 #pragma unroll
   for (int q = 0; q < N; ++q) {
     a.out_pt[2 * N * i + q] = X[q];
@@ -87,13 +106,14 @@ __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_fpmul(Fixe
 }
 
 // r = x(k G) mod n, s = k^-1 (e + r d) mod n and the public key d G.
-template <class C>
-__global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_sign(FixedArgs<C> a) {
+template <class C, bool QUAD>
+__global__ void __launch_bounds__(kLadderThreads, QUAD ? 2 : kLadderCtasPerSm) k_sign(FixedArgs<C> a) {
   using F = typename C::Fp;
   using Fn = typename C::Fn;
   constexpr int N = F::N;
   static_assert(N == 8 && Fn::N == 8, "256-bit curves");
-  const size_t g = blockIdx.x * (size_t)kLadderThreads + threadIdx.x, i = g < a.n ? g : a.n - 1;
+  bool writes;
+  const size_t i = comb_item<QUAD>(a.n, writes);
   uint32_t nn[8], kr[9];
 #pragma unroll
   for (int q = 0; q < 8; ++q) nn[q] = C::n(q);
@@ -110,7 +130,11 @@ __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_sign(Fixed
 #pragma unroll
     for (int q = 0; q < 8; ++q) v[q] = valid ? v[q] : (q == 0 ? 1u : 0u);
   };
-  uint32_t X[N], Y[N], Z[N], Kx[N], Kz[N];
+  JacReg<F> P;
+  uint32_t* const X = P.X.v;
+  uint32_t* const Y = P.Y.v;
+  uint32_t* const Z = P.Z.v;
+  uint32_t Kx[N], Kz[N];
   bool neg = false;
 #pragma unroll 1
   for (int j = 0; j < 2 * kGRows; ++j) {  // k G, then d G
@@ -124,7 +148,7 @@ __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_sign(Fixed
       fe_set_zero<F>(Z);
     }
     __syncthreads();
-    comb_add<C>(a.TG, kr[0], kr[8], neg, j & (kGRows - 1), X, Y, Z);
+    comb_add<C, QUAD>(a.TG, kr[0], kr[8], neg, j & (kGRows - 1), P);
     if (j & 1) {
 #pragma unroll
       for (int q = 0; q < 7; ++q) kr[q] = kr[q + 1];
@@ -163,7 +187,8 @@ __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_sign(Fixed
     fe_set_zero<Fn>(s);
   }
   // every input of this item has been read: an output may be an input's buffer
-  if (g >= a.n) return;
+  if constexpr (QUAD) __syncwarp();
+  if (!writes) return;
   store_be256(a.out_r + 8 * i, r);
   store_be256(a.out_s + 8 * i, s);
   store_be256(a.out_pub + 16 * i, X);

@@ -6,7 +6,9 @@ namespace ecc {
 
 namespace {
 
-unsigned ladder_ctas(size_t n) { return (unsigned)((n + kLadderThreads - 1) / kLadderThreads); }
+unsigned ladder_ctas(size_t threads) { return (unsigned)((threads + kLadderThreads - 1) / kLadderThreads); }
+
+bool use_quads(size_t n) { return n <= (size_t)device_sm_count() * kQuadItemsPerSm; }
 
 template <class C>
 cudaError_t fpmul(int curve, size_t n, const uint32_t* k, uint32_t* out, cudaStream_t st) {
@@ -16,7 +18,11 @@ cudaError_t fpmul(int curve, size_t n, const uint32_t* k, uint32_t* out, cudaStr
   a.n = n;
   a.k = k;
   a.out_pt = out;
-  k_fpmul<C><<<ladder_ctas(n), kLadderThreads, 0, st>>>(a);
+  if (use_quads(n)) {
+    k_fpmul<C, true><<<ladder_ctas(4 * n), kLadderThreads, 0, st>>>(a);
+  } else {
+    k_fpmul<C, false><<<ladder_ctas(n), kLadderThreads, 0, st>>>(a);
+  }
   return cudaGetLastError();
 }
 
@@ -33,7 +39,11 @@ cudaError_t sign(int curve, size_t n, const uint32_t* d, const uint32_t* h, cons
   a.out_r = r;
   a.out_s = s;
   a.out_pub = pub;
-  k_sign<C><<<ladder_ctas(n), kLadderThreads, 0, st>>>(a);
+  if (use_quads(n)) {
+    k_sign<C, true><<<ladder_ctas(4 * n), kLadderThreads, 0, st>>>(a);
+  } else {
+    k_sign<C, false><<<ladder_ctas(n), kLadderThreads, 0, st>>>(a);
+  }
   return cudaGetLastError();
 }
 

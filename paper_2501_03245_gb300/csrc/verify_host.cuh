@@ -10,12 +10,6 @@ namespace ecc {
 
 namespace verify_detail {
 
-// Items up to which four lanes verify one (verify.cuh): two CTAs of quads per SM, on
-// which their warps' products do not wait for each other yet.  secp256k1 by threads /
-// quads: 1 triple 0.55 / 0.37 ms, 4096 0.56 / 0.38, 9000 0.57 / 0.52; P-256 0.89 / 0.58, 0.89 /
-// 0.58, 0.89 / 0.83.
-constexpr size_t kQuadItemsPerSm = 64;
-
 template <class C>
 cudaError_t verify(size_t n, const uint8_t* hash, const uint8_t* r, const uint8_t* s,
                    const uint8_t* pub, uint8_t* ok, cudaStream_t st, int curve) {

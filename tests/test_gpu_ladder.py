@@ -107,3 +107,38 @@ def test_quads_and_threads_agree(gpu_lib, cid):
         gpu_lib.ecc_verify_batch(cid, m, *(to_cuda(np.ascontiguousarray(a[idx])) for a in (e, r, s, pub)), ok)
         torch.cuda.synchronize()
         assert np.array_equal(from_cuda(ok), want[idx]), m
+
+
+@pytest.mark.parametrize("cid", [0, 1, 2, 3, 4])
+def test_fpmul_and_sign_by_quads_and_threads(gpu_lib, cid):
+    """k G at the largest batch of quads, one more and the first sizes of a CTA, with the
+    edge digits in every batch; signatures with the same nonces, their r is x(k G)."""
+    import torch
+
+    C = curves.BY_ID[cid]
+    ks = [k for k in edge_scalars(C.n) if 0 < k < C.n]
+    want = [ec.encode(ec.mul(C, k, C.G)) for k in ks]
+    wx, wy = (np.array([synth.ints_to_limbs([w[i]], C.limbs)[0] for w in want]) for i in (0, 1))
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for m in (1, 31, 33, 64 * sms, 64 * sms + 1):
+        idx = np.arange(m) * 7 % len(ks)
+        limbs = synth.ints_to_limbs(ks, 8)[idx]
+        out = torch.zeros((m, 2 * C.limbs), dtype=torch.int32, device="cuda")
+        gpu_lib.ecc_fixed_base_mul(cid, m, to_cuda(limbs), out)
+        got = from_cuda(out).view(np.uint32)
+        assert np.array_equal(got[:, :C.limbs], wx[idx]) and np.array_equal(got[:, C.limbs:], wy[idx]), m
+        if cid not in (0, 1, 4):
+            continue
+        k = to_cuda(np.ascontiguousarray(synth.limbs_to_be32(limbs)))
+        e = k.flip(0).contiguous()
+        d = k.clone()
+        r, pub = torch.zeros_like(k), torch.zeros((m, 64), dtype=torch.uint8, device="cuda")
+        s = d  # over the private keys' own buffer
+        gpu_lib.ecc_sign_batch(cid, m, d, e, k, r, s, pub)
+        assert np.array_equal(from_cuda(pub)[:, :32], synth.limbs_to_be32(wx[idx]))
+        rows = range(min(m, len(ks)))
+        for i in rows:
+            kk, h = ks[idx[i]], ks[idx[m - 1 - i]]
+            rr = want[idx[i]][0] % C.n
+            assert int.from_bytes(bytes(from_cuda(r[i])), "big") == rr
+            assert int.from_bytes(bytes(from_cuda(s[i])), "big") == pow(kk, -1, C.n) * (h + rr * kk) % C.n
