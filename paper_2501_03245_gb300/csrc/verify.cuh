@@ -22,7 +22,7 @@
 // whatever the batch size.
 #pragma once
 #include "glv.cuh"
-#include "ladder.cuh"
+#include "jac.cuh"
 
 namespace ecc {
 
@@ -177,6 +177,7 @@ ECC_DEV void verify_table_affine(const VerifyArgs<C>& a, size_t slot, uint32_t* 
     load_affine<F>(a.table, row, x, y);
     a.H.load((size_t)(k - 1) * a.slots + slot, h);
     if constexpr (QUAD) {
+      __syncwarp();  // every lane of the item has its operands before one stores the row
       uint32_t u[N], p[N];
       quad_pick<F>(u, zi, h, zi, h);
       mont_mul<F>(p, u, zi);  // zi^2, zi h
@@ -198,16 +199,22 @@ ECC_DEV void verify_table_affine(const VerifyArgs<C>& a, size_t slot, uint32_t* 
   }
 }
 
-// QUAD: four lanes per item, each doing all of it but the products of the group
-// operations, which they share; what they store they store alike.
-template <class C, bool QUAD>
-__global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_verify(VerifyArgs<C> a) {
+// LANES = 4: four lanes per item, each doing all of it but the products of the group
+// operations, which they share; what they store they store alike.  LANES = 8: two
+// such quads per item, which sum one part of u1 G + u2 Q each (the halves of a split
+// u2 and of u1's rows, or u2 Q and u1 G) and add the two at the end.
+template <class C, int LANES>
+__global__ void __launch_bounds__(kLadderThreads, LANES > 1 ? 2 : kLadderCtasPerSm) k_verify(VerifyArgs<C> a) {
   using F = typename C::Fp;
   constexpr int N = F::N;
   static_assert(N == 8 && C::Fn::N == 8, "256-bit curves");
   using QWin = QWindows<C>;
-  constexpr int kItems = kLadderThreads / (QUAD ? 4 : 1);  // of a CTA
-  const size_t own = QUAD ? threadIdx.x / 4 : threadIdx.x;
+  constexpr bool QUAD = LANES > 1, PAIR = LANES == 8;
+  constexpr int kSteps = PAIR ? QWin::DIGITS : QWin::STEPS;          // additions of table points
+  constexpr int kRows = !PAIR ? kGRows : C::GLV ? kGRows / 2 : 0;  // further additions of G's
+  const bool second = PAIR && (threadIdx.x & 4u);                  // the item's second quad
+  constexpr int kItems = kLadderThreads / LANES;  // of a CTA
+  const size_t own = threadIdx.x / LANES;
   const size_t slot = blockIdx.x * (size_t)kItems + own;
   // threads past the batch repeat its last item (the barriers need every thread)
 #pragma unroll 1
@@ -235,48 +242,59 @@ __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_verify(Ver
     store_affine<F>(a.table, slot * kQTable + 1, X, Y);
     constexpr int kChain = kQTable - 2;
 #pragma unroll 1
-    for (int it = 0; it < kChain + QWin::STEPS + kGRows; ++it) {
+    for (int it = 0; it < kChain + kSteps + kRows; ++it) {
       int d;
       const uint32_t* src;
       size_t row;
       bool phi = false;  // the point's image under the endomorphism
-      if (it < kChain) {
-        d = 1;
-        src = a.table;
-        row = slot * kQTable;
-      } else if (it < kChain + QWin::STEPS) {
-        const int step = it - kChain;
-        const int half = QWin::HALVES == 2 ? step & 1 : 0;
-        const int w = QWin::DIGITS - 1 - step / QWin::HALVES;
-        if (step == 0) {
-          fe_inv_mont<F>(x, Z);
-          verify_table_affine<C, QUAD>(a, slot, x);
-          fe_set_zero<F>(Z);
-        } else if (half == 0) {
-#pragma unroll 1
-          for (int k = 0; k < kQW; ++k) {
-            __syncthreads();
-            dbl();
-          }
-        }
-        const int bit = kQW * w, wd = bit >> 5, sh = bit & 31;
-        const uint32_t* u2 = a.u2 + 5 * half * a.slots + slot;
-        uint32_t v = u2[wd * a.slots] >> sh;
-        if (sh > 32 - kQW) v |= u2[(wd + 1) * a.slots] << (32 - sh);
-        d = (int)(v & (2 * kQTable - 1)) - kQTable;
-        src = a.table;
-        row = slot * kQTable + (d < 0 ? -d : d) - 1;
-        if constexpr (C::GLV) {
-          if (u2[4 * a.slots] >> 31) d = -d;
-          phi = half != 0;
-        }
-      } else {
-        const int j = it - kChain - QWin::STEPS;
+      auto g_row = [&](int j) {
         const uint32_t c = a.u1[8 * a.slots + slot];
         d = comb_digit(a.u1[(j >> 1) * a.slots + slot], c & 1u, j);
         src = a.TG;
         row = (size_t)j * kGEntries + (d < 0 ? -d : d) - 1;
         if (c & 2u) d = -d;
+      };
+      if (it < kChain) {
+        d = 1;
+        src = a.table;
+        row = slot * kQTable;
+      } else if (it < kChain + kSteps) {
+        const int step = it - kChain;
+        // the quads of a pair have a half of a split scalar each, else they take turns
+        const int half = !C::GLV ? 0 : PAIR ? (int)second : step & 1;
+        const int w = QWin::DIGITS - 1 - (PAIR ? step : step / QWin::HALVES);
+        const bool only_g = PAIR && !C::GLV && second;
+        if (step == 0) {
+          fe_inv_mont<F>(x, Z);
+          verify_table_affine<C, QUAD>(a, slot, x);
+          fe_set_zero<F>(Z);
+        } else if (PAIR || half == 0) {
+#pragma unroll 1
+          for (int k = 0; k < kQW; ++k) {
+            __syncthreads();
+            if (!only_g) dbl();
+          }
+        }
+        if (only_g) {
+          d = 0;
+          src = a.TG;
+          row = 0;
+          if (step < kGRows) g_row(step);
+        } else {
+          const int bit = kQW * w, wd = bit >> 5, sh = bit & 31;
+          const uint32_t* u2 = a.u2 + 5 * half * a.slots + slot;
+          uint32_t v = u2[wd * a.slots] >> sh;
+          if (sh > 32 - kQW) v |= u2[(wd + 1) * a.slots] << (32 - sh);
+          d = (int)(v & (2 * kQTable - 1)) - kQTable;
+          src = a.table;
+          row = slot * kQTable + (d < 0 ? -d : d) - 1;
+          if constexpr (C::GLV) {
+            if (u2[4 * a.slots] >> 31) d = -d;
+            phi = half != 0;
+          }
+        }
+      } else {
+        g_row(it - kChain - kSteps + (second ? kRows : 0));
       }
       __syncthreads();
       if (d != 0) {
@@ -301,6 +319,17 @@ __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_verify(Ver
         store_affine<F>(a.table, slot * kQTable + it + 2, X, Y);
       }
     }
+    if constexpr (PAIR) {  // the other quad's part
+      __syncwarp();
+      JacReg<F> Q;
+#pragma unroll
+      for (int k = 0; k < N; ++k) {
+        Q.X.v[k] = __shfl_xor_sync(0xffffffffu, X[k], 4);
+        Q.Y.v[k] = __shfl_xor_sync(0xffffffffu, Y[k], 4);
+        Q.Z.v[k] = __shfl_xor_sync(0xffffffffu, Z[k], 4);
+      }
+      quad_add<C>(P, Q);
+    }
     // R != O and x_R mod n == r, i.e. X = r Z^2 or (r + n < p) X = (r + n) Z^2
     uint32_t r[8], t[8], zz[8], pp[8];
 #pragma unroll
@@ -322,6 +351,7 @@ __global__ void __launch_bounds__(kLadderThreads, kLadderCtasPerSm) k_verify(Ver
     }
     ok = ok && valid && !fe_is_zero<F>(Z);
     if (mine) a.ok[i] = ok ? 1 : 0;
+    if constexpr (QUAD) __syncwarp();  // the slot is free
   }
 }
 

@@ -90,8 +90,8 @@ def test_verify_sizes(gpu_lib, n):
 
 @pytest.mark.parametrize("cid", [0, 1, 4])
 def test_quads_and_threads_agree(gpu_lib, cid):
-    """The largest batch that four lanes verify an item of, and one more, with the edge
-    digits and colliding points in the rows of both."""
+    """The largest batches that eight and four lanes verify an item of, and one more, with
+    the edge digits and colliding points in the rows of all."""
     import torch
 
     n = curves.BY_ID[cid].n
@@ -101,7 +101,7 @@ def test_quads_and_threads_agree(gpu_lib, cid):
     r[1::7, 31] ^= 1
     want = cpp_oracle.verify(cid, e, r, s, pub)
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    for m in (1, 31, 33, 64 * sms, 64 * sms + 1):
+    for m in (1, 15, 17, 33, 16 * sms, 16 * sms + 1, 64 * sms, 64 * sms + 1):
         idx = np.arange(m) * 11 % len(e)
         ok = torch.full((m,), 7, dtype=torch.uint8, device="cuda")
         gpu_lib.ecc_verify_batch(cid, m, *(to_cuda(np.ascontiguousarray(a[idx])) for a in (e, r, s, pub)), ok)
