@@ -324,11 +324,12 @@ ECC_DEV Trans30 divsteps30(int32_t& delta, uint32_t f, uint32_t g) {
 // The adds of a multiple of 0 or +-1 are multiply-adds, which run on another
 // pipe than the logic beside them: one thread's chain is bound by the pipes'
 // two cycles an instruction, and the step has 13 of them against 24 with the
-// four entries apart and selects.  One inversion on GB300: 16.8 us for 8 limbs and
-// 28.8 for 12, against 22.8 and 39.0; a full warp takes no longer than one lane.
+// four entries apart and selects.  One inversion on GB300: 13.4 us for 8 limbs and
+// 23.3 for 12, against 22.8 and 39.0 (unrolled by 5 14.5 and 25.0; with the products of
+// the updates as separate multiplications and additions 16.8 and 28.8); a full warp
+// takes no longer than one lane.
 ECC_DEV void divsteps15(int32_t& zeta, uint32_t& f, uint32_t& g, uint32_t& P, uint32_t& Q) {
-  // unrolled by 5: the code shares the instruction cache with the kernel's rounds
-#pragma unroll 5
+#pragma unroll
   for (int i = 0; i < 15; ++i) {
     const uint32_t odd = g & 1u;
     const uint32_t t = g & ((uint32_t)zeta >> 31);  // swaps
@@ -366,26 +367,15 @@ ECC_DEV Trans30 divsteps30_flat(int32_t& zeta, uint32_t f, uint32_t g) {
                  q[1] * v[0] + r[1] * r[0]};
 }
 
-ECC_DEV int64_t mul32w(int32_t a, int32_t b) { return (int64_t)a * (int64_t)b; }
-
-// (f, g) <- T (f, g) / 2^30 (exact)
-template <int L>
-ECC_DEV void update_fg30(int32_t* f, int32_t* g, const Trans30& t) {
-  int64_t cf = mul32w(t.u, f[0]) + mul32w(t.v, g[0]);
-  int64_t cg = mul32w(t.q, f[0]) + mul32w(t.r, g[0]);
-  cf >>= 30;
-  cg >>= 30;
-#pragma unroll
-  for (int i = 1; i < L; ++i) {
-    cf += mul32w(t.u, f[i]) + mul32w(t.v, g[i]);
-    cg += mul32w(t.q, f[i]) + mul32w(t.r, g[i]);
-    f[i - 1] = (int32_t)cf & kM30;
-    g[i - 1] = (int32_t)cg & kM30;
-    cf >>= 30;
-    cg >>= 30;
-  }
-  f[L - 1] = (int32_t)cf;
-  g[L - 1] = (int32_t)cg;
+// c + a b, one multiply-add
+ECC_DEV int64_t mad32w(int32_t a, int32_t b, int64_t c) {
+#ifdef __CUDA_ARCH__
+  int64_t r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+#else
+  return c + (int64_t)a * (int64_t)b;
+#endif
 }
 
 template <int L>
@@ -425,35 +415,52 @@ ECC_DEV void s30_normalise(int32_t* a, const int32_t* q) {
   while (s30_ge<L>(a, q)) s30_add_mul<L>(a, q, -1);
 }
 
-// (d, e) <- T (d, e) / 2^30 mod q for d, e in (-2q, q), results in (-2q, q);
-// qinv30 = q^-1 mod 2^30.  A negative input is first raised by q, folded into
-// the multiple of q that is added anyway: with d, e in (-q, q) and |u| + |v|,
-// |q| + |r| <= 2^30, T (d, e) + m q with m in [0, 2^30) lies in
-// (-2^31 q, 2^30 q), so the exact quotient lies in (-2q, q) and no
-// normalisation is needed until the end.
+// (f, g) <- T (f, g) / 2^30 (exact) and (d, e) <- T (d, e) / 2^30 mod q for d, e in
+// (-2q, q), results in (-2q, q); qinv30 = q^-1 mod 2^30.  A negative d or e is first
+// raised by q, folded into the multiple of q that is added anyway: with d, e in
+// (-q, q) and |u| + |v|, |q| + |r| <= 2^30, T (d, e) + m q with m in [0, 2^30) lies in
+// (-2^31 q, 2^30 q), so the exact quotient lies in (-2q, q) and no normalisation is
+// needed until the end.  The four carry chains run side by side.
 template <int L>
-ECC_DEV void update_de30(int32_t* d, int32_t* e, const Trans30& t, const int32_t* q, uint32_t qinv30) {
+ECC_DEV void update30(int32_t* f, int32_t* g, int32_t* d, int32_t* e, const Trans30& t, const int32_t* q,
+                      uint32_t qinv30) {
   const int32_t sd = d[L - 1] >> 31, se = e[L - 1] >> 31;  // -1 when negative
   int32_t md = (t.u & sd) + (t.v & se);
   int32_t me = (t.q & sd) + (t.r & se);
-  int64_t cd = mul32w(t.u, d[0]) + mul32w(t.v, e[0]);
-  int64_t ce = mul32w(t.q, d[0]) + mul32w(t.r, e[0]);
+  int64_t cd = mad32w(t.v, e[0], 0), ce = mad32w(t.r, e[0], 0);
+  int64_t cf = mad32w(t.v, g[0], 0), cg = mad32w(t.r, g[0], 0);
+  cd = mad32w(t.u, d[0], cd);
+  ce = mad32w(t.q, d[0], ce);
+  cf = mad32w(t.u, f[0], cf) >> 30;
+  cg = mad32w(t.q, f[0], cg) >> 30;
   // subtract from m what makes the low 30 bits of T (d, e) + m q vanish
   md -= (int32_t)((qinv30 * (uint32_t)cd + (uint32_t)md) & (uint32_t)kM30);
   me -= (int32_t)((qinv30 * (uint32_t)ce + (uint32_t)me) & (uint32_t)kM30);
-  cd += mul32w(md, q[0]);
-  ce += mul32w(me, q[0]);
-  cd >>= 30;
-  ce >>= 30;
+  cd = mad32w(md, q[0], cd) >> 30;
+  ce = mad32w(me, q[0], ce) >> 30;
 #pragma unroll
   for (int i = 1; i < L; ++i) {
-    cd += mul32w(t.u, d[i]) + mul32w(t.v, e[i]) + mul32w(md, q[i]);
-    ce += mul32w(t.q, d[i]) + mul32w(t.r, e[i]) + mul32w(me, q[i]);
+    cd = mad32w(md, q[i], cd);
+    ce = mad32w(me, q[i], ce);
+    cf = mad32w(t.v, g[i], cf);
+    cg = mad32w(t.r, g[i], cg);
+    cd = mad32w(t.v, e[i], cd);
+    ce = mad32w(t.r, e[i], ce);
+    cf = mad32w(t.u, f[i], cf);
+    cg = mad32w(t.q, f[i], cg);
+    cd = mad32w(t.u, d[i], cd);
+    ce = mad32w(t.q, d[i], ce);
+    f[i - 1] = (int32_t)cf & kM30;
+    g[i - 1] = (int32_t)cg & kM30;
     d[i - 1] = (int32_t)cd & kM30;
     e[i - 1] = (int32_t)ce & kM30;
+    cf >>= 30;
+    cg >>= 30;
     cd >>= 30;
     ce >>= 30;
   }
+  f[L - 1] = (int32_t)cf;
+  g[L - 1] = (int32_t)cg;
   d[L - 1] = (int32_t)cd;
   e[L - 1] = (int32_t)ce;
 }
@@ -506,8 +513,7 @@ ECC_DEV void inv_divsteps30(uint32_t* out, const uint32_t* x, const uint32_t* q3
   for (int it = 0; it < 128; ++it) {  // 30 * 128 divsteps bound any 1024-bit modulus
     const uint32_t fl = (uint32_t)f[0] | ((uint32_t)f[1] << 30), gl = (uint32_t)g[0] | ((uint32_t)g[1] << 30);
     const Trans30 t = FLAT ? divsteps30_flat(delta, fl, gl) : divsteps30(delta, fl, gl);
-    update_fg30<L>(f, g, t);
-    update_de30<L>(d, e, t, q, qinv30);
+    update30<L>(f, g, d, e, t, q, qinv30);
     if (s30_is_zero<L>(g)) break;
   }
   // f = +-1: x^-1 = f d, d in (-2q, q); q - d lies in (0, 3q)
