@@ -290,8 +290,11 @@ int ecc_set_allocator(ecc_alloc_fn alloc, ecc_free_fn release, void* ctx);
 int ecc_validate_points(ecc_curve_t curve, size_t n, const uint32_t* points, uint8_t* ok_out,
                         void* stream);
 
-/* Window width used for an n-point MSM, and the autotuner's override for the
- * size class floor(log2 n) (c = 0 restores the cost-model default). */
+/* Window width of an n-point MSM, and the autotuner's override for the size class
+ * floor(log2 n) (c = 0 restores the default).  The default is the width of least work
+ * by the textbook's count, by which sizes are admitted; without an override a call may
+ * use another one (for split scalars and a single call's latency).  Results do not
+ * depend on it. */
 int ecc_msm_window(ecc_curve_t curve, size_t n);
 int ecc_msm_set_window(ecc_curve_t curve, int log2_n, int c);
 

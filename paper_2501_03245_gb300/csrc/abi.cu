@@ -659,7 +659,7 @@ int ecc_bases_destroy(void* handle) {
 
 int ecc_msm_window(ecc_curve_t curve, size_t n) {
   if (!valid_curve(curve)) return fail(ECC_EINVAL, "ecc_msm_window: unknown curve %d", (int)curve);
-  return msm_window(curve, n);
+  return msm_admitted_window(curve, n);
 }
 
 int ecc_msm_set_window(ecc_curve_t curve, int log2_n, int c) {
