@@ -211,9 +211,10 @@ def gen_inputs(ecc, synth, torch, n, seed, curve=CURVE_P256):
 # DRAM traffic of one k_verify launch over 2^20 P-256 triples (dram__bytes_read.sum +
 # dram__bytes_write.sum, from one ncu capture), valid only for the kernel sources
 # it was taken on: the digest of those sources must match, else it is null.
-VERIFY_TRAFFIC = {"bytes": 79369814528 + 33884342528, "batch": 1 << 20, "digest": "d56ffe9d83e1591f",
-                  "sources": ["verify.cuh", "verify_host.cuh", "ladder.cuh", "ec.cuh", "fp.cuh", "inv.cuh",
-                              "ptx.cuh", "curves_gen.cuh", "internal.h", "k_verify_p256.cu", "k_verify.cu"]}
+VERIFY_TRAFFIC = {"bytes": 1495312640 + 1494215680, "batch": 1 << 20, "digest": "cde39205b1615b10",
+                  "sources": ["verify.cuh", "verify_host.cuh", "ladder.cuh", "jac.cuh", "glv.cuh", "ec.cuh", "fp.cuh",
+                              "inv.cuh", "ptx.cuh", "curves_gen.cuh", "internal.h", "k_verify_p256.cu",
+                              "k_verify.cu"]}
 
 
 def verify_traffic(n):
@@ -396,7 +397,7 @@ def bench_sm2(ecc, costmodel, synth, torch, peak, rank, n, steps, world=1, clk=N
             "paper": {"value": PAPER_SM2_VERIFY_A100, "hardware": "NVIDIA A100 40 GB",
                       "source": "Table 4"},
             "ratio_to_paper": value / world / PAPER_SM2_VERIFY_A100,
-            "roofline": {"bound": "alu", "kernel": "k_verify<SM2>", "achieved": alg / t / 1e12,
+            "roofline": {"bound": "alu", "kernel": "k_verify<SM2, 1>", "achieved": alg / t / 1e12,
                          "peak": peak / 1e12, "unit": "T IMAD.WIDE/s", "frac": alg / t / peak}}
 
 
@@ -509,10 +510,10 @@ def bench_k1(ecc, costmodel, synth, torch, peak, rank, world=1, clk=None, reps=2
             "timed_calls": reps, "valid_signatures": int(ok.sum().item()), "clocks": clk.summary("secp256k1"),
             "plain": {"value": job_rate(plain_n, t1, world), "unit": "verifies/s",
                       "form": f"one triple per launch, first {plain_n} triples"},
-            "roofline": {"bound": "alu", "kernel": "k_verify<Secp256k1>", "achieved": alg / t / 1e12,
+            "roofline": {"bound": "alu", "kernel": "k_verify<Secp256k1, 4>", "achieved": alg / t / 1e12,
                          "peak": peak / 1e12, "unit": "T IMAD.WIDE/s", "frac": alg / t / peak,
-                         "note": "4096 triples fill 16 of 304 resident CTAs: latency, not the pipe, "
-                                 "bounds this size"}}
+                         "note": "4096 triples by four lanes each are 128 of 608 resident CTAs: latency, "
+                                 "not the pipe, bounds this size"}}
 
 
 # The paper's ECDSA signing and fixed-point multiplication throughputs on its
@@ -551,12 +552,12 @@ def bench_sign_fpmul(ecc, costmodel, synth, torch, peak, rank, n, world=1, clk=N
             "sign": {"value": job_rate(n, t_sign, world), "unit": "signs/s", "ms_per_step": t_sign * 1e3,
                      "paper": {"value": PAPER_SM2_SIGN_A100, "hardware": "NVIDIA A100 40 GB",
                                "source": "Table 4"},
-                     "roofline": {"bound": "alu", "kernel": "k_fixed_base<SM2> (signing mode)", "achieved": a_sign / t_sign / 1e12,
+                     "roofline": {"bound": "alu", "kernel": "k_sign<SM2>", "achieved": a_sign / t_sign / 1e12,
                                   "peak": peak / 1e12, "unit": "T IMAD.WIDE/s", "frac": a_sign / t_sign / peak}},
             "fpmul": {"value": job_rate(n, t_fp, world), "unit": "kG/s", "ms_per_step": t_fp * 1e3,
                       "paper": {"value": PAPER_SM2_FPMUL_A100, "hardware": "NVIDIA A100 40 GB",
                                 "source": "Table 5"},
-                      "roofline": {"bound": "alu", "kernel": "k_fixed_base<SM2> (FPMUL mode)", "achieved": a_fp / t_fp / 1e12,
+                      "roofline": {"bound": "alu", "kernel": "k_fpmul<SM2>", "achieved": a_fp / t_fp / 1e12,
                                    "peak": peak / 1e12, "unit": "T IMAD.WIDE/s", "frac": a_fp / t_fp / peak}}}
 
 
@@ -564,8 +565,7 @@ def verify_config(n):
     """The verification workload's config, shared by both arms."""
     shape = "2^20" if n == N_VERIFY else str(n)
     return {"workload": f"ECDSA verify, NIST P-256, {shape} seeded triples per GPU, 1/16 corrupted",
-            "curve": "P-256", "batch": n, "l2": "working set > L2 (inputs 160 MiB + "
-            "per-item state ~0.8 GiB per step)"}
+            "curve": "P-256", "batch": n, "l2": "inputs larger than L2 (160 MiB per step)"}
 
 
 def run_reference(args):
@@ -706,10 +706,11 @@ def run_ours(args):
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "u32",
         "data": "synthetic",
         "config": verify_config(n), "valid_signatures": n_valid,
-        "roofline": {"bound": "alu", "kernel": "k_verify<P256, 256, 2>", "achieved": achieved / 1e12,
+        "roofline": {"bound": "alu", "kernel": "k_verify<P256, 1>", "achieved": achieved / 1e12,
                      "peak": peak / 1e12, "unit": "T IMAD.WIDE/s", "frac": achieved / peak,
                      "traffic": verify_traffic(n), "traffic_unit": "DRAM bytes per launch",
-                     "basis": f"{costmodel.verify_modmul()} modmul x 136 wide mul-adds per verify; "
+                     "basis": f"{costmodel.verify_modmul()} modmul x 136 wide mul-adds per verify (textbook: "
+                              "products by the shape of the prime need 64, so the fraction can pass 1); "
                               "peak = measured mad.lo/madc.hi pair rate (ecc_bench_imad, same run)"},
         "plain": {"value": plain, "unit": "verifies/s", "form": "one verification per launch"},
         "e2e": {"value": e2e_value, "unit": "verifies/s",
