@@ -72,3 +72,43 @@ def test_heavy_buckets(gpu_lib, cid):
     _check(gpu_lib, cid, [a[0] if i & 1 else C.n - a[0] for i in range(n)], [k] * n)
     _check(gpu_lib, cid, a, [0] * (n - 1) + [k])
     _check(gpu_lib, cid, a, [(C.n - 1 if i & 1 else 1) for i in range(n)])
+
+
+def test_split_scalars_fall_back_when_the_workspace_is_refused(gpu_lib):
+    """An allocator that refuses the first request (the split form's, with the points'
+    images): the call answers alike without them, from host and device offsets."""
+    import torch
+
+    C = curves.BY_ID[2]
+    n = 5000
+    a, k = _ints(C.n, n, 11), _ints(C.n, n, 12)
+    pts, sc = _points(gpu_lib, 2, a), to_cuda(synth.ints_to_limbs(k, 8))
+    want = ec.mul(C, sum(x * y for x, y in zip(a, k)) % C.n, C.G)
+    offs = torch.tensor([0, n], dtype=torch.int64, device="cuda")
+    for dev in (False, True):
+        sizes, held = [], {}
+
+        def alloc(nbytes, stream):
+            sizes.append(nbytes)
+            if len(sizes) == 1:
+                return 0
+            t = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+            held[t.data_ptr()] = t
+            return t.data_ptr()
+
+        def release(ptr, stream):
+            torch.cuda.synchronize()
+            held.pop(ptr)
+
+        out = torch.zeros((1, 2 * C.limbs), dtype=torch.int32, device="cuda")
+        gpu_lib.ecc_set_allocator(alloc, release)
+        try:
+            if dev:
+                gpu_lib.ecc_msm_ragged_dev(2, 1, n, offs, pts, sc, out, 0)
+            else:
+                gpu_lib.ecc_msm(2, n, pts, sc, out)
+            torch.cuda.synchronize()
+        finally:
+            gpu_lib.ecc_set_allocator(None, None)
+        assert len(sizes) > 1 and not held
+        assert limbs_to_points(C, from_cuda(out).view(np.uint32))[0] == want, dev
