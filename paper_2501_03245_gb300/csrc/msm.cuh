@@ -1027,7 +1027,9 @@ __global__ void __launch_bounds__(kJacThreads, kJacCtas<C::Fp::N>) k_msm_tree(Re
       Jac<F>* dst = (i > l ? a.S : a.R) + e;
       if (quads) {
         JacReg<F> P = quad_load(dst);
-        quad_add<C>(P, quad_load(dst + half));
+        const JacReg<F> Q = quad_load(dst + half);
+        __syncwarp(quad_mask());  // all four have dst before one stores it: O + Q exchanges nothing
+        quad_add<C>(P, Q);
         if ((threadIdx.x & 3u) == 0) jac_store<F>(dst, P.X.v, P.Y.v, P.Z.v);
       } else {
         uint32_t X[N], Y[N], Z[N], X2[N], Y2[N], Z2[N];
