@@ -32,6 +32,9 @@
  *     the point at infinity O is written (0, 0), which is on none of the
  *     supported curves (b != 0).
  *   - Pointers must be 4-byte aligned.
+ *   - ecc_fp_* (but ecc_fp_mul, _add, _sub and _inv only row for row), ecc_point_*,
+ *     ecc_fixed_base_mul, ecc_sign_batch and ecc_verify_batch may write their
+ *     results over their inputs' memory, in place or shifted.
  */
 #ifndef GECC_H
 #define GECC_H

@@ -30,6 +30,13 @@ struct Scratch {
   }
 };
 
+// Whether two arrays share memory.
+inline bool overlap(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
+  const char* x = static_cast<const char*>(a);
+  const char* y = static_cast<const char*>(b);
+  return x < y + b_bytes && y < x + a_bytes;
+}
+
 int device_sm_count();
 std::string cuda_msg(cudaError_t e);
 

@@ -8,6 +8,20 @@ namespace {
 
 unsigned ladder_ctas(size_t threads) { return (unsigned)((threads + kLadderThreads - 1) / kLadderThreads); }
 
+// Copies the `rows` inputs of n rows of 32 bytes that are named in `in` into ws and points
+// them there.  An item's rows are read by its own thread, while other items' results
+// are written already: an output may be an input's buffer row for row, not otherwise.
+cudaError_t keep_rows(Scratch& ws, size_t n, const uint32_t** in[], size_t rows, cudaStream_t st) {
+  if (rows == 0) return cudaSuccess;
+  cudaError_t e = ws.alloc(rows * n * 32, st);
+  for (size_t j = 0; j < rows && e == cudaSuccess; ++j) {
+    uint32_t* copy = ws.as<uint32_t>() + j * n * 8;
+    e = cudaMemcpyAsync(copy, *in[j], n * 32, cudaMemcpyDeviceToDevice, st);
+    *in[j] = copy;
+  }
+  return e;
+}
+
 bool use_quads(size_t n) { return n <= (size_t)device_sm_count() * kQuadItemsPerSm; }
 
 template <class C>
@@ -18,6 +32,10 @@ cudaError_t fpmul(int curve, size_t n, const uint32_t* k, uint32_t* out, cudaStr
   a.n = n;
   a.k = k;
   a.out_pt = out;
+  Scratch ws;
+  const uint32_t** in[] = {&a.k};
+  e = keep_rows(ws, n, in, overlap(k, n * 32, out, n * 2 * C::Fp::N * 4) ? 1 : 0, st);
+  if (e != cudaSuccess) return e;
   if (use_quads(n)) {
     k_fpmul<C, true><<<ladder_ctas(4 * n), kLadderThreads, 0, st>>>(a);
   } else {
@@ -39,6 +57,15 @@ cudaError_t sign(int curve, size_t n, const uint32_t* d, const uint32_t* h, cons
   a.out_r = r;
   a.out_s = s;
   a.out_pub = pub;
+  Scratch ws;
+  const uint32_t** in[3];
+  size_t rows = 0;
+  for (const uint32_t** p : {&a.k, &a.d, &a.e}) {
+    auto hit = [&](const uint32_t* out) { return out != *p && overlap(*p, n * 32, out, n * 32); };
+    if (hit(r) || hit(s) || overlap(*p, n * 32, pub, n * 64)) in[rows++] = p;
+  }
+  e = keep_rows(ws, n, in, rows, st);
+  if (e != cudaSuccess) return e;
   if (use_quads(n)) {
     k_sign<C, true><<<ladder_ctas(4 * n), kLadderThreads, 0, st>>>(a);
   } else {

@@ -326,9 +326,7 @@ inline unsigned row_ctas(size_t n) {
 // Whether out's rows overlap in's without being the same rows: then a row may be
 // written before another thread reads it, and the input is copied first.
 inline bool shifted_overlap(const void* in, const void* out, size_t bytes) {
-  const char* a = static_cast<const char*>(in);
-  const char* o = static_cast<const char*>(out);
-  return a != o && a < o + bytes && o < a + bytes;
+  return in != out && overlap(in, bytes, out, bytes);
 }
 
 }  // namespace ecc

@@ -31,16 +31,31 @@ cudaError_t verify(size_t n, const uint8_t* hash, const uint8_t* r, const uint8_
   // per slot: table (affine points), H, recoded u1 (9 words) and u2, r
   constexpr size_t kU2 = QWindows<C>::HALVES * QWindows<C>::WORDS;
   const size_t table = slots * kQTable * 2 * Fp::N * 4, h = soa_bytes<Fp>(slots * kQTable);
+  const size_t work = table + h + (9 + kU2 + 8) * 4 * slots;
+  // an input that the results overlap is copied: an item's result is written while other
+  // items are still to be read
+  const uint8_t* in[4] = {hash, r, s, pub};
+  const size_t row[4] = {32, 32, 32, 64};
+  size_t copies = 0;
+  for (int j = 0; j < 4; ++j) copies += overlap(in[j], row[j] * n, ok, n) ? row[j] * n : 0;
   Scratch ws;
-  e = ws.alloc(table + h + (9 + kU2 + 8) * 4 * slots, st);
+  e = ws.alloc(work + copies, st);
   if (e != cudaSuccess) return e;
   uint8_t* p = ws.as<uint8_t>();
+  uint8_t* copy = p + work;
+  for (int j = 0; j < 4; ++j) {
+    if (!overlap(in[j], row[j] * n, ok, n)) continue;
+    e = cudaMemcpyAsync(copy, in[j], row[j] * n, cudaMemcpyDeviceToDevice, st);
+    if (e != cudaSuccess) return e;
+    in[j] = copy;
+    copy += row[j] * n;
+  }
   VerifyArgs<C> a;
   a.n = n;
-  a.hash = reinterpret_cast<const uint32_t*>(hash);
-  a.r = reinterpret_cast<const uint32_t*>(r);
-  a.s = reinterpret_cast<const uint32_t*>(s);
-  a.pub = reinterpret_cast<const uint32_t*>(pub);
+  a.hash = reinterpret_cast<const uint32_t*>(in[0]);
+  a.r = reinterpret_cast<const uint32_t*>(in[1]);
+  a.s = reinterpret_cast<const uint32_t*>(in[2]);
+  a.pub = reinterpret_cast<const uint32_t*>(in[3]);
   a.ok = ok;
   a.table = reinterpret_cast<uint32_t*>(p);
   a.H = SoA<Fp>{reinterpret_cast<uint4*>(p + table), slots * kQTable};
