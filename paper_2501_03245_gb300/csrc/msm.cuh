@@ -678,8 +678,8 @@ __global__ void __launch_bounds__(kJacThreads, kJacCtas<C::Fp::N>)
 //
 // Window sum sum_b b E_b (E_b the bucket sums, b = 1 .. 2^(c-1)).  Before it the
 // partial sums of every bucket are folded into the first one (a pairwise tree,
-// ceil(log2 k) rounds for k partials; CTAs take equal shares of the partial slots,
-// so a bucket holding many entries costs rounds only in the CTA that owns it).
+// ceil(log2 k) rounds for k partials; CTAs take equal shares of the partial slots and
+// buckets, so a bucket holding many entries costs rounds only in the CTA that owns it).
 //
 // A window row is cut into elements of K = 2^red_log consecutive buckets: element u
 // has R_u, the plain sum, and S_u = sum_i i E_(K u + i), i = 1 .. K, from two running
@@ -714,12 +714,22 @@ struct FoldArgs {
   JacSoA<F> jac;                // the partial sums when they are in Jacobian coordinates
 };
 
-// first b in [0, n] with poff[b] >= x
-ECC_DEV uint32_t lower_bound_u32(const uint32_t* v, uint32_t n, uint64_t x) {
+// Buckets are shared out among the fold's CTAs by kFoldSlot for each partial slot before
+// them and one for each bucket.  By slots alone one CTA gets all empty buckets between
+// two full ones and walks them in every round: 4 vectors of 4096 zeros and ones on a
+// table of 22-bit windows 33 ms, now 0.2; 65536 BN254 points with 20-bit windows, whose
+// top window fills 2^6 of 2^19 buckets, 8.1 ms, now 0.5.  By slots and buckets alike a top
+// window of many partial sums comes to too few CTAs (2^20 points, 24 bits: 0.65, 1.33 ms).
+constexpr uint64_t kFoldSlot = 8;
+
+ECC_DEV uint64_t fold_key(const uint32_t* poff, uint32_t b) { return kFoldSlot * poff[b] + b; }
+
+// first b in [0, n] with fold_key(b) >= x
+ECC_DEV uint32_t fold_bound(const uint32_t* poff, uint32_t n, uint64_t x) {
   uint32_t lo = 0, hi = n;
   while (lo < hi) {
-    const uint32_t mid = (lo + hi) >> 1;
-    if (v[mid] < x) lo = mid + 1; else hi = mid;
+    const uint32_t mid = lo + ((hi - lo) >> 1);
+    if (fold_key(poff, mid) < x) lo = mid + 1; else hi = mid;
   }
   return lo;
 }
@@ -898,12 +908,12 @@ __global__ void __launch_bounds__(BLOCK, JAC && C::Fp::N > 8 ? 1 : kGasResidentT
   __shared__ uint32_t wsum[BLOCK / 32];
   const uint64_t total_slots = a.poff[a.n_buckets];
   if (total_slots == 0) return;  // uniform over the grid
-  // this CTA owns the buckets whose first slot lies in its equal share
-  const uint64_t share = (total_slots + gridDim.x - 1) / gridDim.x;
-  const uint32_t b0 = lower_bound_u32(a.poff, a.n_buckets, blockIdx.x * share);
+  // this CTA owns the buckets that begin in its equal share
+  const uint64_t share = (fold_key(a.poff, a.n_buckets) + gridDim.x - 1) / gridDim.x;
+  const uint32_t b0 = fold_bound(a.poff, a.n_buckets, blockIdx.x * share);
   const uint32_t b1 = blockIdx.x + 1 == gridDim.x
                           ? a.n_buckets
-                          : lower_bound_u32(a.poff, a.n_buckets, (blockIdx.x + 1) * share);
+                          : fold_bound(a.poff, a.n_buckets, (blockIdx.x + 1) * share);
   const uint64_t s0 = a.poff[b0];
   uint32_t kmax = 0;
   for (uint32_t b = b0 + threadIdx.x; b < b1; b += BLOCK) {

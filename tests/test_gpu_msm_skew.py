@@ -1,0 +1,81 @@
+"""MSMs whose entries fall into few buckets (scalars of zeros and ones, a nearly empty top
+window): the closed form, and no CTA of the fold is left to walk the empty buckets."""
+import numpy as np
+import pytest
+
+from oracle import curves, ec
+from paper_2501_03245_gb300 import synth
+from tests.helpers import from_cuda, limbs_to_points, to_cuda
+
+pytestmark = pytest.mark.gpu
+
+
+def _multiples(n):
+    a = np.zeros((n, 8), np.uint32)
+    a[:, 0] = np.arange(1, n + 1)
+    return a
+
+
+def _fold_ms(lib, call):
+    best = None
+    for _ in range(4):
+        call()
+        t = lib.ecc_msm_phase_times()["fold"]
+        best = t if best is None else min(best, t)
+    return best
+
+
+@pytest.mark.parametrize("cid", [2, 3])
+def test_zeros_and_ones_on_a_window_table(gpu_lib, cid):
+    """4 vectors cost no more than 4 times one, and a millisecond; by slots alone the empty
+    buckets between the vectors' first ones went to one CTA each (8 ms against 0.1)."""
+    import torch
+
+    C, n, V = curves.BY_ID[cid], 4096, 4
+    a = _multiples(n)
+    pts = torch.empty((n, 2 * C.limbs), dtype=torch.int32, device="cuda")
+    gpu_lib.ecc_fixed_base_mul(cid, n, to_cuda(a), pts)
+    k = np.zeros((V * n, 8), np.uint32)
+    k[:, 0] = np.random.default_rng(cid).integers(0, 2, V * n)
+    kd = to_cuda(k)
+    out = torch.zeros((V, 2 * C.limbs), dtype=torch.int32, device="cuda")
+    h = gpu_lib.ecc_bases_create(cid, n, pts)
+    try:
+        gpu_lib.ecc_bases_precompute(h, 20)
+        gpu_lib.ecc_set_phase_timing(1)
+        one = _fold_ms(gpu_lib, lambda: gpu_lib.ecc_msm_bases(h, 1, kd[:n], out[:1]))
+        four = _fold_ms(gpu_lib, lambda: gpu_lib.ecc_msm_bases(h, V, kd, out))
+    finally:
+        gpu_lib.ecc_set_phase_timing(0)
+        torch.cuda.synchronize()
+        gpu_lib.ecc_bases_destroy(h)
+    got = limbs_to_points(C, from_cuda(out).view(np.uint32))
+    for v in range(V):
+        total = int((a[:, 0].astype(np.int64) * k[v * n:(v + 1) * n, 0]).sum())
+        assert got[v] == ec.mul(C, total % C.n, C.G), v
+    assert four < 4 * one + 1.0, (one, four)
+
+
+@pytest.mark.parametrize("cid", [2, 3])
+def test_nearly_empty_top_window(gpu_lib, cid):
+    """Uniform scalars and 20-bit windows: few values of the top window hold a row's
+    entries, the rest of its buckets are empty."""
+    import torch
+
+    C, n = curves.BY_ID[cid], 1 << 16
+    a = _multiples(n)
+    pts = torch.empty((n, 2 * C.limbs), dtype=torch.int32, device="cuda")
+    gpu_lib.ecc_fixed_base_mul(cid, n, to_cuda(a), pts)
+    k = synth.uniform_limbs(91, 1, n, C.n)
+    kd = to_cuda(k.view(np.int32))
+    out = torch.zeros((1, 2 * C.limbs), dtype=torch.int32, device="cuda")
+    gpu_lib.ecc_msm_set_window(cid, 16, 20)
+    try:
+        gpu_lib.ecc_set_phase_timing(1)
+        t = _fold_ms(gpu_lib, lambda: gpu_lib.ecc_msm(cid, n, pts, kd, out))
+    finally:
+        gpu_lib.ecc_set_phase_timing(0)
+        gpu_lib.ecc_msm_set_window(cid, 16, 0)
+    total = sum(int(x) * y for x, y in zip(a[:, 0], synth.limbs_to_ints(k)))
+    assert limbs_to_points(C, from_cuda(out).view(np.uint32))[0] == ec.mul(C, total % C.n, C.G)
+    assert t < 2.0, t  # 8.1 (BN254) and 3.0 ms (BLS12-381) by slots alone, 0.5 and 0.8 now
