@@ -79,3 +79,42 @@ def test_nearly_empty_top_window(gpu_lib, cid):
     total = sum(int(x) * y for x, y in zip(a[:, 0], synth.limbs_to_ints(k)))
     assert limbs_to_points(C, from_cuda(out).view(np.uint32))[0] == ec.mul(C, total % C.n, C.G)
     assert t < 2.0, t  # 8.1 (BN254) and 3.0 ms (BLS12-381) by slots alone, 0.5 and 0.8 now
+
+
+def test_batches_of_tiny_msms(gpu_lib):
+    """16384 BLS12-381 MSMs of 0 to 4 points: every one right, and no slower than with the
+    4-bit windows that are too wide for them (16 buckets a row for 4 entries)."""
+    import torch
+
+    cid, C, num = 3, curves.BLS12_381, 16384
+    sizes = np.arange(num) % 5
+    offs = np.concatenate([[0], np.cumsum(sizes)]).astype(np.uint64)
+    n = int(offs[-1])
+    pts = torch.empty((n, 2 * C.limbs), dtype=torch.int32, device="cuda")
+    gpu_lib.ecc_fixed_base_mul(cid, n, to_cuda(_multiples(n)), pts)
+    k = synth.uniform_limbs(92, 1, n, C.n)
+    kd, ks = to_cuda(k.view(np.int32)), synth.limbs_to_ints(k)
+    totals = [sum((i + 1) * ks[i] for i in range(int(a), int(b))) % C.n for a, b in zip(offs[:-1], offs[1:])]
+    want = torch.empty((num, 2 * C.limbs), dtype=torch.int32, device="cuda")
+    gpu_lib.ecc_fixed_base_mul(cid, num, to_cuda(synth.ints_to_limbs(totals, 8).view(np.int32)), want)
+
+    def run():
+        out = torch.zeros_like(want)
+        ms = []
+        for _ in range(4):
+            gpu_lib.ecc_msm_ragged(cid, num, offs, pts, kd, out)
+            ms.append(sum(gpu_lib.ecc_msm_phase_times().values()))
+        assert torch.equal(out, want)
+        return min(ms)
+
+    try:
+        gpu_lib.ecc_set_phase_timing(1)
+        own = run()
+        for lg in (1, 2):
+            gpu_lib.ecc_msm_set_window(cid, lg, 4)
+        wide = run()
+    finally:
+        gpu_lib.ecc_set_phase_timing(0)
+        for lg in (1, 2):
+            gpu_lib.ecc_msm_set_window(cid, lg, 0)
+    assert own < 0.9 * wide, (own, wide)
