@@ -70,12 +70,15 @@ inline int red_log(int curve, uint64_t n, int c, uint64_t buckets) {
   return std::min(k, c - 1);
 }
 
-// Chunks, accumulation form and reduction layout of the planned instances.
+// Chunks, accumulation form and reduction layout of the planned instances.  lean: the
+// longest chunks and elements, which take the least workspace.
 template <int N>
-void finish_plan(int curve, Layout& L, const uint64_t* sizes, uint64_t size_all) {
+void finish_plan(int curve, Layout& L, const uint64_t* sizes, uint64_t size_all, bool lean) {
   for (size_t i = 0; i < L.inst.size(); ++i) {
     MsmInst& m = L.inst[i];
-    m.red_log = (uint32_t)red_log(curve, sizes ? sizes[i] : size_all, (int)m.c, L.buckets);
+    const uint64_t n = sizes ? sizes[i] : size_all;
+    m.red_log = (uint32_t)(lean ? std::min(msm_reduce_log(curve, n), (int)m.c - 1)
+                                : red_log(curve, n, (int)m.c, L.buckets));
     m.elem_off = L.elems;
     m.row_off = L.rows;
     m.cta_off = L.ctas;
@@ -84,7 +87,7 @@ void finish_plan(int curve, Layout& L, const uint64_t* sizes, uint64_t size_all)
     L.ctas += tree_ctas(m);
   }
   L.direct = L.entries_max < kDirectEntries;
-  if (L.direct) {  // chunks of 8 to 32 entries, about four for each resident thread
+  if (L.direct && !lean) {  // chunks of 8 to 32 entries, about four for each resident thread
     constexpr uint32_t chunks = N <= 8 ? 1u << 18 : 1u << 17;
     for (L.ch_log = 3; L.ch_log < kAccLog && (L.entries_max >> (L.ch_log + 1)) >= chunks;) ++L.ch_log;
   }
@@ -280,18 +283,20 @@ cudaError_t run_set(int curve, const Layout& L, const uint32_t* bases_mont, cons
 
 // pre_c > 0: the bases hold precomputed window multiples for width pre_c,
 // pre_stride points apart.  phi > 0: the points' images are phi rows after them, and
-// scalars are split.  A batch whose digits, buckets or rows do not fit their 31-bit
-// indices that way is planned as its size was admitted (msm_counts).
+// scalars are split.  lean: the plan of least workspace, with whole scalars and the widths
+// by which sizes are admitted (msm_counts): also that of a batch whose digits, buckets or
+// rows would not fit their 31-bit indices.
 template <class C>
 Layout plan(int curve, uint32_t num, const uint64_t* sizes, const uint64_t* point_off,
-            const uint64_t* scalar_off, int pre_c, uint64_t pre_stride, uint64_t phi, bool admitted = false) {
+            const uint64_t* scalar_off, int pre_c, uint64_t pre_stride, uint64_t phi, bool lean) {
   Layout L;
+  if (lean) phi = 0;
   L.inst.resize(num);
   L.phi = phi;
   for (uint32_t i = 0; i < num; ++i) {
     MsmInst& m = L.inst[i];
     m.n = (uint32_t)sizes[i];
-    m.c = (uint32_t)(pre_c > 0 ? pre_c : admitted ? msm_admitted_window(curve, sizes[i]) : msm_window(curve, sizes[i], num));
+    m.c = (uint32_t)(pre_c > 0 ? pre_c : lean ? msm_admitted_window(curve, sizes[i]) : msm_window(curve, sizes[i], num));
     m.W = (uint32_t)(phi ? half_windows<C>((int)m.c) : windows_for(curve, (int)m.c));
     m.bucket_base = (uint32_t)L.buckets;
     m.point_off = point_off[i];
@@ -302,11 +307,24 @@ Layout plan(int curve, uint32_t num, const uint64_t* sizes, const uint64_t* poin
     L.buckets += (uint64_t)m.Wr << (m.c - 1);
     L.entries_max += (uint64_t)m.W * m.n * (phi ? 2 : 1);
     L.total_points += m.n;
-    if (!admitted && (L.entries_max >= kMsmMaxDigits || L.buckets >= kMsmMaxDigits || 2 * phi >= kMsmMaxDigits))
+    if (!lean && (L.entries_max >= kMsmMaxDigits || L.buckets >= kMsmMaxDigits || 2 * phi >= kMsmMaxDigits))
       return plan<C>(curve, num, sizes, point_off, scalar_off, pre_c, pre_stride, 0, true);
   }
-  finish_plan<C::Fp::N>(curve, L, sizes, 0);
+  finish_plan<C::Fp::N>(curve, L, sizes, 0, lean);
   return L;
+}
+
+// run(false), or, where its workspace is refused, run(true) with the lean plan: chunks of 8
+// entries, short elements, wider windows and the points' images take up to 3 times (and a
+// few MB for the smallest calls) the workspace that the call needs.
+template <class Run>
+cudaError_t run_or_lean(Run run) {
+  cudaError_t e = run(false);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    e = run(true);
+  }
+  return e;
 }
 
 template <class C>
@@ -319,29 +337,25 @@ cudaError_t msm_points(int curve, uint32_t num, const uint64_t* offsets, const u
     sizes[i] = offsets[i + 1] - offsets[i];
     poff[i] = offsets[i] - offsets[0];
   }
-  auto run = [&](uint64_t phi) {
-    const Layout L = plan<C>(curve, num, sizes.data(), poff.data(), poff.data(), 0, 0, phi);
+  return run_or_lean([&](bool lean) {
+    const Layout L = plan<C>(curve, num, sizes.data(), poff.data(), poff.data(), 0, 0, C::GLV ? total : 0, lean);
     return run_set<C>(curve, L, nullptr, scalars + offsets[0] * 8, out, st, nullptr, points + offsets[0] * 2 * F::N);
-  };
-  cudaError_t e = run(C::GLV ? total : 0);
-  if (C::GLV && e == cudaErrorMemoryAllocation) {  // without the images' workspace
-    cudaGetLastError();
-    e = run(0);
-  }
-  return e;
+  });
 }
 
 // The uniform per-instance layout of a device-sized batch (window width c, or
 // the library's width for bases with window multiples of width pre_c) with the
-// capacity totals: cap scalar rows in num instances.  phi and the indices as in plan;
-// c = 0: the library's width for the mean size.
+// capacity totals: cap scalar rows in num instances.  phi, lean and the indices as in
+// plan; c = 0: the library's width for the mean size.
 template <class C>
-Layout plan_uniform(int curve, uint32_t num, int c, uint64_t cap, int pre_c, uint64_t pre_stride, uint64_t phi) {
+Layout plan_uniform(int curve, uint32_t num, int c, uint64_t cap, int pre_c, uint64_t pre_stride, uint64_t phi,
+                    bool lean) {
   Layout L;
   MsmInst m{};
+  if (lean) phi = 0;
   if (pre_c <= 0 && c <= 0) {
     const uint64_t mean = num ? std::max<uint64_t>(cap / num, 2) : 2;
-    c = msm_window(curve, mean, num);
+    c = lean ? msm_admitted_window(curve, mean) : msm_window(curve, mean, num);
     const uint64_t W = (uint64_t)windows_for(curve, c);
     if (W * cap >= kMsmMaxDigits || (num * W) << (c - 1) >= kMsmMaxDigits) c = msm_admitted_window(curve, mean);
   }
@@ -357,7 +371,7 @@ Layout plan_uniform(int curve, uint32_t num, int c, uint64_t cap, int pre_c, uin
   L.buckets = (uint64_t)num * ((uint64_t)m.Wr << (m.c - 1));
   L.entries_max = cap * m.W * (phi ? 2 : 1);
   L.total_points = cap;
-  finish_plan<C::Fp::N>(curve, L, nullptr, num ? std::max<uint64_t>(cap / num, 2) : 2);
+  finish_plan<C::Fp::N>(curve, L, nullptr, num ? std::max<uint64_t>(cap / num, 2) : 2, lean);
   return L;
 }
 
@@ -367,17 +381,11 @@ template <class C>
 cudaError_t msm_points_dev(int curve, uint32_t num, uint64_t cap, const uint64_t* offsets, int c,
                            const uint32_t* points, const uint32_t* scalars, uint32_t* out, cudaStream_t st) {
   DevRows dev{offsets, 0, 0, cap};
-  auto run = [&](uint64_t phi) {
-    return run_set<C>(curve, plan_uniform<C>(curve, num, c, cap, 0, 0, phi), nullptr, scalars, out, st, &dev, points);
-  };
-  cudaError_t e = run(C::GLV ? cap : 0);
-  if (C::GLV && e == cudaErrorMemoryAllocation) {  // without the images' workspace
-    cudaGetLastError();
-    e = run(0);
-  }
-  return e;
+  return run_or_lean([&](bool lean) {
+    const Layout L = plan_uniform<C>(curve, num, c, cap, 0, 0, C::GLV ? cap : 0, lean);
+    return run_set<C>(curve, L, nullptr, scalars, out, st, &dev, points);
+  });
 }
-
 
 struct Bases {
   int curve;
@@ -441,9 +449,12 @@ cudaError_t precompute_t(Bases* bs, int c, cudaStream_t st) {
 template <class C>
 cudaError_t msm_bases_dev_t(Bases* bs, uint32_t num, uint64_t cap, const uint64_t* sizes, int c,
                             const uint32_t* scalars, uint32_t* out, cudaStream_t st) {
-  Layout L = plan_uniform<C>(bs->curve, num, c, cap, bs->pre ? bs->pre_c : 0, bs->n, bs->pre ? 0 : bs->phi);
   DevRows dev{sizes, 1, bs->n, cap};
-  return run_set<C>(bs->curve, L, bs->pre ? bs->pre : bs->mont, scalars, out, st, &dev);
+  return run_or_lean([&](bool lean) {
+    const Layout L =
+        plan_uniform<C>(bs->curve, num, c, cap, bs->pre ? bs->pre_c : 0, bs->n, bs->pre ? 0 : bs->phi, lean);
+    return run_set<C>(bs->curve, L, bs->pre ? bs->pre : bs->mont, scalars, out, st, &dev);
+  });
 }
 
 template <class C>
@@ -458,9 +469,11 @@ cudaError_t msm_bases_t(Bases* bs, uint32_t num_vectors, const uint64_t* vec_siz
     soff[v] = acc;
     acc += sizes[v];
   }
-  Layout L = plan<C>(bs->curve, num_vectors, sizes.data(), poff.data(), soff.data(), bs->pre ? bs->pre_c : 0, bs->n,
-                     bs->pre ? 0 : bs->phi);
-  return run_set<C>(bs->curve, L, bs->pre ? bs->pre : bs->mont, scalars, out, st);
+  return run_or_lean([&](bool lean) {
+    const Layout L = plan<C>(bs->curve, num_vectors, sizes.data(), poff.data(), soff.data(), bs->pre ? bs->pre_c : 0,
+                             bs->n, bs->pre ? 0 : bs->phi, lean);
+    return run_set<C>(bs->curve, L, bs->pre ? bs->pre : bs->mont, scalars, out, st);
+  });
 }
 
 }  // namespace msm_detail
