@@ -27,20 +27,26 @@ cudaError_t verify(size_t n, const uint8_t* hash, const uint8_t* r, const uint8_
   const size_t items = kLadderThreads / lanes;
   size_t ctas = (n + items - 1) / items;
   ctas = std::min<size_t>(ctas, (size_t)device_sm_count() * kLadderCtasPerSm);
-  const size_t slots = ctas * items;
-  // per slot: table (affine points), H, recoded u1 (9 words) and u2, r
-  constexpr size_t kU2 = QWindows<C>::HALVES * QWindows<C>::WORDS;
-  const size_t table = slots * kQTable * 2 * Fp::N * 4, h = soa_bytes<Fp>(slots * kQTable);
-  const size_t work = table + h + (9 + kU2 + 8) * 4 * slots;
   // an input that the results overlap is copied: an item's result is written while other
   // items are still to be read
   const uint8_t* in[4] = {hash, r, s, pub};
   const size_t row[4] = {32, 32, 32, 64};
   size_t copies = 0;
   for (int j = 0; j < 4; ++j) copies += overlap(in[j], row[j] * n, ok, n) ? row[j] * n : 0;
+  // per slot: table (affine points), H, recoded u1 (9 words) and u2, r: 1640 or 1644 bytes
+  constexpr size_t kU2 = QWindows<C>::HALVES * QWindows<C>::WORDS;
+  size_t slots, table, h, work;
   Scratch ws;
-  e = ws.alloc(work + copies, st);
-  if (e != cudaSuccess) return e;
+  for (;; ctas = (ctas + 1) / 2) {  // half the CTAs, with more items each, where it is refused
+    slots = ctas * items;
+    table = slots * kQTable * 2 * Fp::N * 4;
+    h = soa_bytes<Fp>(slots * kQTable);
+    work = table + h + (9 + kU2 + 8) * 4 * slots;
+    e = ws.alloc(work + copies, st);
+    if (e == cudaSuccess) break;
+    if (e != cudaErrorMemoryAllocation || ctas == 1) return e;
+    cudaGetLastError();
+  }
   uint8_t* p = ws.as<uint8_t>();
   uint8_t* copy = p + work;
   for (int j = 0; j < 4; ++j) {

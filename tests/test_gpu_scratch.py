@@ -128,3 +128,25 @@ def test_ragged(gpu_lib, cid, num, per, budget):
         torch.cuda.synchronize()
     assert not arena.held
     _check(C, out, totals)
+
+
+@pytest.mark.parametrize("cid", [0, 1])
+@pytest.mark.parametrize("n,budget", [(33, 45301), (1000, 1365256), (9728, 13278976), (30000, 40950256),
+                                      (77825, 106231381), (9728, 100000), (77825, 2000000)])
+def test_verify(gpu_lib, cid, n, budget):
+    """Fewer items at once, by eight, four and one lanes: as with the full workspace."""
+    import torch
+
+    C = curves.BY_ID[cid]
+    d, e, k = (to_cuda(np.ascontiguousarray(synth.limbs_to_be32(synth.uniform_limbs(3 + i, 1, n, C.n, lo=1))))
+               for i in range(3))
+    r, s = torch.empty_like(d), torch.empty_like(d)
+    pub = torch.empty((n, 64), dtype=torch.uint8, device="cuda")
+    gpu_lib.ecc_sign_batch(cid, n, d, e, k, r, s, pub)
+    s[::7, 3] ^= 16
+    ok = torch.full((n,), 7, dtype=torch.uint8, device="cuda")
+    with Arena(gpu_lib, budget) as arena:
+        gpu_lib.ecc_verify_batch(cid, n, e, r, s, pub, ok)
+        torch.cuda.synchronize()
+    assert arena.refused and not arena.held
+    assert np.array_equal(from_cuda(ok), (np.arange(n) % 7 != 0).astype(np.uint8))
