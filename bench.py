@@ -405,9 +405,10 @@ def bench_ragged(ecc, costmodel, synth, torch, peak, rank, world=1, clk=None, re
     """BN254 ragged batch: 256 MSMs with log-uniform sizes 2^10..2^18, all in one
     launch sequence captured once in a CUDA graph and replayed, against one
     launch sequence per MSM.  Window widths are autotuned per size class, then
-    a common width shift and the reduction's bucket layout on this batch.  The
-    algorithmic work is the sum of every instance's Pippenger count at the
-    window width the library picks for its size."""
+    a common width shift and the reduction's bucket layout on this batch; what
+    does not beat the library's own plan is not installed.  The algorithmic work
+    is the sum of every instance's Pippenger count at the width reported for its
+    size."""
     from paper_2501_03245_gb300 import autotune
 
     clk = clk or _NoClock()

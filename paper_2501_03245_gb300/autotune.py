@@ -1,20 +1,23 @@
 """Measured window-width autotuner for MSM size classes.
 
 For every size class floor(log2 n) the tuner times ``ecc_msm`` on seeded
-synthetic inputs for the cost model's window width and its neighbours, keeps the
-fastest, installs it with ``ecc_msm_set_window`` and can persist the table as
-JSON (keyed by GPU name and curve) so a later process reloads it instead of
-measuring again.  Inputs are made on the device by the library itself
-(``ecc_fixed_base_mul`` for the bases), so tuning needs no CPU arithmetic.
+synthetic inputs as the library plans it by itself and with the textbook's window
+width and its neighbours, keeps the fastest, installs a faster width with
+``ecc_msm_set_window`` and can persist the table as JSON (keyed by GPU name, curve
+and kernels) so a later process reloads it instead of measuring again.  Inputs are
+made on the device by the library itself (``ecc_fixed_base_mul`` for the bases), so
+tuning needs no CPU arithmetic.
 ``tune_precomputed`` picks the width of a resident base set's window-multiple
 table; ``tune_batch`` tunes, on a caller's ragged batch itself, the knobs its
-instances share (a common width shift, the first-level reduction chunk, one
-width step per group of classes).
+instances share (a common width shift, the buckets per reduction element, one
+width step per group of classes).  No tuner leaves a call slower than the library's
+own plan.
 """
 import json
 import os
 
 from . import ecc, synth
+from .ecc import msm_own_plan
 
 
 def _curve_order(curve):
@@ -93,14 +96,23 @@ def tune_precomputed(handle, vectors, scalars, torch, candidates, reps=3):
     return best, times
 
 
-def tune(curve, log2_sizes, torch, spread=2, seed=0x6ECC7777, cache=None, vectors=1):
-    """Returns {log2_n: c} and installs it in the library.  With vectors > 1
+# Part of a saved table's key: raised when the kernels or plans that it was measured on
+# change, so that an older table is measured again.
+_TABLE = 2
+
+
+def _table_key(torch, curve, vectors):
+    return f"{torch.cuda.get_device_name()}|{curve}|{vectors}|{_TABLE}"
+
+
+def tune(curve, log2_sizes, torch, spread=2, seed=0x6ECC7777, cache=None, vectors=1, min_gain=0.005):
+    """Returns {log2_n: c} and installs it in the library; c = 0 where no forced width
+    beats the library's own plan by more than min_gain.  With vectors > 1
     every candidate is timed on the resident-bases form with that many scalar
     vectors per call (the best window grows with the vectors sharing a call)."""
-    key = None
     table = {}
     if cache and os.path.exists(cache):
-        key = f"{torch.cuda.get_device_name()}|{curve}|{vectors}"
+        key = _table_key(torch, curve, vectors)
         saved = json.load(open(cache)).get(key, {})
         table = {int(k): int(v) for k, v in saved.items()}
     missing = [l for l in log2_sizes if l not in table]
@@ -113,20 +125,19 @@ def tune(curve, log2_sizes, torch, spread=2, seed=0x6ECC7777, cache=None, vector
             n = 1 << l
             ecc.ecc_msm_set_window(curve, l, 0)
             c0 = ecc.ecc_msm_window(curve, n)
-            best = None
-            for c in range(max(2, c0 - spread), min(20, c0 + spread) + 1):
+            times = {}
+            for c in [0, *range(max(2, c0 - spread), min(20, c0 + spread) + 1)]:
                 ecc.ecc_msm_set_window(curve, l, c)
                 if vectors > 1:
-                    t = time_msm_bases(curve, bases, scalars[:n * vectors].contiguous(), n, vectors, torch)
+                    times[c] = time_msm_bases(curve, bases, scalars[:n * vectors].contiguous(), n, vectors, torch)
                 else:
-                    t = time_msm(curve, bases, scalars, n, torch)
-                if best is None or t < best[0]:
-                    best = (t, c)
-            table[l] = best[1]
+                    times[c] = time_msm(curve, bases, scalars, n, torch)
+            best = min(times, key=times.get)
+            table[l] = best if times[best] < times[0] * (1 - min_gain) else 0
     for l, c in table.items():
         ecc.ecc_msm_set_window(curve, l, c)
     if cache:
-        key = key or f"{torch.cuda.get_device_name()}|{curve}|{vectors}"
+        key = _table_key(torch, curve, vectors)
         data = json.load(open(cache)) if os.path.exists(cache) else {}
         data[key] = {str(k): v for k, v in sorted(table.items())}
         with open(cache, "w") as f:
@@ -138,18 +149,18 @@ def tune_batch(curve, log2_sizes, run, torch, shifts=(-1, 0, 1), chunks=(3, 4, 5
     """Tunes the knobs that one ragged launch sequence shares across its
     instances on the batch itself: run() makes the caller's ecc_msm_ragged call.
 
-    The first-level reduction of all instances runs in one launch whose round
-    count is set by the largest chunk in it, so a per-class chunk choice made
-    on batches of one size does not transfer to a mix; likewise the window
-    widths of the classes interact through the shared launches.  So, starting
-    from the per-class widths already installed (tune), every width is shifted
-    by the same s (each in [2, 20]) for each s in shifts, then one chunk 2^k
-    (capped at c - 1 per class) is set for every class for each k in chunks;
-    each candidate is timed as reps calls of run(), the fastest is installed.
-    Last, each group of classes that share a width tries that width - 1 and
-    + 1 on the batch (the others fixed); a change stays when it is faster by
-    more than min_gain.  Returns {"shift": s, "chunk_log2": k, "widths":
-    {log2_n: c}, "ms": {...}}."""
+    All instances share one set of launches, so what is best for a class alone does
+    not transfer to a mix.  First the batch is timed as the library plans it, without
+    overrides.  Then, starting from the widths reported for the classes (those that
+    tune installed), every width is shifted by the same s (each in [2, 20]) for each
+    s in shifts, and one element of 2^k buckets (capped at c - 1 per class) is set for
+    every class for each k in chunks; each candidate is timed as reps calls of run(),
+    and the fastest goes on.  Last, each group of classes that share a width tries
+    that width - 1 and + 1 on the batch (the others fixed); a change stays when it is
+    faster by more than min_gain.  The result is installed, or, where the library's
+    own plan was faster, every override of the classes is removed.  Returns {"own":
+    whether it was, "shift": s, "chunk_log2": k, "widths": {log2_n: c}, "ms": {...}};
+    shift and chunk_log2 are None for the library's own plan."""
     base = {l: ecc.ecc_msm_window(curve, 1 << l) for l in log2_sizes}
 
     def timed():
@@ -172,7 +183,9 @@ def tune_batch(curve, log2_sizes, run, torch, shifts=(-1, 0, 1), chunks=(3, 4, 5
             c = ecc.ecc_msm_window(curve, 1 << l)
             ecc.ecc_msm_set_reduce_chunk(curve, l, max(1, min(k, c - 1)))
 
-    ms = {}
+    msm_own_plan(curve, log2_sizes)
+    own = timed()
+    ms = {"own plan": own}
     set_chunk(chunks[len(chunks) // 2])
     for s in shifts:
         set_shift(s)
@@ -203,6 +216,9 @@ def tune_batch(curve, log2_sizes, run, torch, shifts=(-1, 0, 1), chunks=(3, 4, 5
             for l in ls:
                 ecc.ecc_msm_set_window(curve, l, c)
             set_chunk(chunk)
+    if own < best:
+        msm_own_plan(curve, log2_sizes)
+        shift = chunk = None
     widths = {l: ecc.ecc_msm_window(curve, 1 << l) for l in log2_sizes}
-    return {"shift": shift, "chunk_log2": chunk, "widths": widths,
+    return {"own": own < best, "shift": shift, "chunk_log2": chunk, "widths": widths,
             "ms": {k: round(v, 3) for k, v in ms.items()}}

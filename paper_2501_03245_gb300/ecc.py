@@ -341,6 +341,13 @@ def ecc_msm_phase_times():
     return {MSM_PHASES[i]: float(buf[i]) for i in range(k)}
 
 
+def msm_own_plan(curve, log2_sizes):
+    """Removes the overrides of the size classes: their calls plan by themselves again."""
+    for l in log2_sizes:
+        ecc_msm_set_window(curve, l, 0)
+        ecc_msm_set_reduce_chunk(curve, l, 0)
+
+
 def ecc_bench_imad(threads, iters, sink, stream=None):
     return _check(load().ecc_bench_imad(threads, iters, _ptr(sink), _stream(stream)))
 
