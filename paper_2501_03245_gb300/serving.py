@@ -24,7 +24,8 @@ resident, the server reads the free device memory (cudaMemGetInfo) and keeps a
 reserve; the rest is the workspace budget.  Each kind's workspace is measured
 from the library itself: a calibration round of two sizes runs with a counting
 workspace allocator installed (ecc_set_allocator), giving bytes = fixed + per
-item.  A round is admitted only while the workspaces of the rounds in flight
+item; a verification takes no more than the largest round it can be given (the
+library holds only the items the GPU works on at once), which is measured too.  A round is admitted only while the workspaces of the rounds in flight
 plus its own fit the budget; a request larger than the whole budget is
 refused.
 
@@ -184,22 +185,23 @@ class Server:
             live["now"] -= sizes_of.pop(p, 0)
             torch.cuda.caching_allocator_delete(p)
 
+        def peak_of(kind, n):
+            live["peak"] = live["now"] = 0
+            rnd = self._launch(kind, [Request(-1, kind, n, 0.0, 0)])
+            rnd["event"].synchronize()
+            return live["peak"]
+
         model = {}
         ecc.ecc_set_allocator(alloc, release)
         try:
             v2 = min(4096, self.e.shape[0])
             m2 = min(1 << 15, self.n_bases, self.scalars.shape[0])
             for kind, (n1, n2) in (("verify", (max(1, v2 // 16), v2)), ("msm", (max(1, m2 // 8), m2))):
-                peaks = []
-                for n in (n1, n2):
-                    live["peak"] = live["now"] = 0
-                    q = Request(-1, kind, n, 0.0, 0)
-                    rnd = self._launch(kind, [q])
-                    rnd["event"].synchronize()
-                    peaks.append(live["peak"])
+                peaks = [peak_of(kind, n) for n in (n1, n2)]
                 per = max(0.0, (peaks[1] - peaks[0]) / (n2 - n1))
                 fixed = max(0.0, peaks[0] - per * n1)
                 model[kind] = (fixed, per)
+            self.verify_top = peak_of("verify", max(1, min(self.max_verify_round, self.e.shape[0])))
         finally:
             ecc.ecc_set_allocator(None, None)
         return model
@@ -207,7 +209,10 @@ class Server:
     def cost(self, kind, items):
         """Workspace bytes of a round of `items` items of `kind` (with 25% slack)."""
         fixed, per = self.model[kind]
-        return int(1.25 * (fixed + per * items)) + (1 << 20)
+        need = fixed + per * items
+        if kind == "verify":
+            need = min(need, self.verify_top)
+        return int(1.25 * need) + (1 << 20)
 
     # -------------------------------------------------------------- rounds
     def _launch(self, kind, batch):
