@@ -111,7 +111,7 @@ int ecc_fp_inv_batch(ecc_curve_t curve, int field, size_t n, const uint32_t* a, 
  * device-wide synchronisation cudaMalloc implies, or a host library without an
  * allocator of its own.  It calls no cudaMalloc, cudaFree or allocating library
  * routine: its scratch is a fixed device array inside the library, sized for
- * n <= 65536 elements of any field (9 MiB, held by every GPU that loads the
+ * n <= 65536 elements of any field (6 MiB, held by every GPU that loads the
  * library until the process exits); larger n returns ECC_EINVAL.
  *   - a, out: DEVICE memory only (host buffers would need a staging
  *     allocation: ECC_EINVAL); same layout and results as ecc_fp_inv_batch.

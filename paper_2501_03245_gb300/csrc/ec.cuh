@@ -37,7 +37,6 @@ struct SoA {
       vec[g * stride + i] = make_uint4(r[4 * g + 0], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
     }
   }
-  __host__ __device__ __forceinline__ SoA at(size_t offset) const { return SoA{vec + offset, stride}; }
 };
 
 template <class F>
@@ -304,32 +303,21 @@ __device__ void cta_invert(uint32_t* out, const uint32_t* in, GasSmem<F::N, BLOC
 // --------------------------------------------------------------------------
 // One batched round over the items [begin, end) owned by this CTA (Montgomery's
 // trick with the DCWPA step, Section 3.3).  R provides
-//   OPS                       denominators per item,
-//   den_c(i, j, d)            denominator j of item i, loading only what it needs
-//                             (compress step: e.g. only x for PADD),
-//   den_d(i, j, d)            the same value in the DCWPA step, where R may keep
-//                             the loaded operands for finish,
-//   finish(i, inv)            complete item i given inv[j] = 1 / den_j.
+//   den(i, d)        the denominator of item i,
+//   finish(i, inv)   complete item i given inv = 1 / den.
 // Compress stores only the running product before each item in M (the
-// intermediate array of Section 3.3); DCWPA recomputes the item's denominators
-// and, for OPS > 1, the partial products inside the item (find-then-recompute,
-// Section 3.4) instead of storing them.
+// intermediate array of Section 3.3); DCWPA computes the denominators again.
 template <class F, int BLOCK, class R>
 __device__ void batch_round(R& rd, size_t begin, size_t end, const SoA<F>& M,
                             GasSmem<F::N, BLOCK>& sm) {
   constexpr int N = F::N;
-  constexpr int OPS = R::OPS;
-  uint32_t run[N];
+  uint32_t run[N], d[N];
   fe_set_one<F>(run);
   const size_t i0 = begin + threadIdx.x;
   for (size_t i = i0; i < end; i += BLOCK) {
     M.store(i, run);
-#pragma unroll
-    for (int j = 0; j < OPS; ++j) {
-      uint32_t d[N];
-      rd.den_c(i, j, d);
-      mont_mul<F>(run, run, d);
-    }
+    rd.den(i, d);
+    mont_mul<F>(run, run, d);
   }
   uint32_t inv[N];
   cta_invert<F, BLOCK>(inv, run, sm);
@@ -337,19 +325,12 @@ __device__ void batch_round(R& rd, size_t begin, size_t end, const SoA<F>& M,
     const size_t last = i0 + ((end - 1 - i0) / BLOCK) * BLOCK;
     for (size_t i = last + BLOCK; i > i0;) {
       i -= BLOCK;
-      uint32_t pre[OPS][N], dd[OPS][N], invs[OPS][N];
-      M.load(i, pre[0]);
-#pragma unroll
-      for (int j = 0; j < OPS; ++j) {
-        rd.den_d(i, j, dd[j]);
-        if (j + 1 < OPS) mont_mul<F>(pre[j + 1], pre[j], dd[j]);
-      }
-#pragma unroll
-      for (int j = OPS - 1; j >= 0; --j) {
-        mont_mul<F>(invs[j], inv, pre[j]);
-        mont_mul<F>(inv, inv, dd[j]);
-      }
-      rd.finish(i, invs);
+      uint32_t mine[N];
+      M.load(i, mine);
+      rd.den(i, d);
+      mont_mul<F>(mine, inv, mine);
+      mont_mul<F>(inv, inv, d);
+      rd.finish(i, mine);
     }
   }
 }

@@ -78,21 +78,6 @@ ECC_DEV bool fe_eq(const uint32_t* a, const uint32_t* b) {
   return acc == 0;
 }
 
-template <class F>
-ECC_DEV bool fe_is_one(const uint32_t* a) {
-  uint32_t acc = 0;
-#pragma unroll
-  for (int i = 0; i < F::N; ++i) acc |= a[i] ^ F::one(i);
-  return acc == 0;
-}
-
-// r = cond ? a : b
-template <class F>
-ECC_DEV void fe_select(uint32_t* r, bool cond, const uint32_t* a, const uint32_t* b) {
-#pragma unroll
-  for (int i = 0; i < F::N; ++i) r[i] = cond ? a[i] : b[i];
-}
-
 // a < q as plain integers (used to validate canonical inputs)
 template <class F>
 ECC_DEV bool fe_lt_modulus(const uint32_t* a) {

@@ -7,11 +7,11 @@
 
 namespace ecc {
 
-// Fixed device scratch of the allocation-free batch inversion: the input,
-// output and prefix-product arrays of up to kNoAllocMaxElems elements of the
-// widest field (12 limbs).  Every GPU that loads the library holds it
-// (3 x 65536 x 48 B = 9 MiB) until the process exits.
-static __device__ __align__(256) uint32_t g_noalloc_scratch[3 * kNoAllocMaxElems * 12];
+// Fixed device scratch of the allocation-free batch inversion: the prefix products
+// and a copy of the input (where the output overlaps it) of up to kNoAllocMaxElems
+// elements of the widest field (12 limbs).  Every GPU that loads the library holds it
+// (2 x 65536 x 48 B = 6 MiB) until the process exits.
+static __device__ __align__(256) uint32_t g_noalloc_scratch[2 * kNoAllocMaxElems * 12];
 
 namespace {
 

@@ -15,23 +15,9 @@ template <class C, bool DBL>
 cudaError_t point_add(size_t n, const uint32_t* p, const uint32_t* q, uint32_t* out, cudaStream_t st) {
   using F = typename C::Fp;
   constexpr int N = F::N, B = kGasThreads;
-  const size_t rows = n * 2 * N * 4;
-  const bool cp = shifted_overlap(p, out, rows), cq = !DBL && shifted_overlap(q, out, rows);
   Scratch ws;
-  cudaError_t e = ws.alloc(soa_bytes<F>(n) + (cp ? rows : 0) + (cq ? rows : 0), st);
+  cudaError_t e = point_scratch<F>(ws, n, p, DBL ? nullptr : &q, out, st);
   if (e != cudaSuccess) return e;
-  uint32_t* copy = ws.as<uint32_t>() + soa_bytes<F>(n) / 4;
-  if (cp) {
-    e = cudaMemcpyAsync(copy, p, rows, cudaMemcpyDeviceToDevice, st);
-    if (e != cudaSuccess) return e;
-    p = copy;
-    copy += rows / 4;
-  }
-  if (cq) {
-    e = cudaMemcpyAsync(copy, q, rows, cudaMemcpyDeviceToDevice, st);
-    if (e != cudaSuccess) return e;
-    q = copy;
-  }
   const size_t smem = sizeof(GasSmem<N, B>);
   e = cudaFuncSetAttribute(k_point_ops<C, DBL, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

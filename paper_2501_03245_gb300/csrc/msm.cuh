@@ -1156,51 +1156,22 @@ struct ShiftArgs {
 };
 
 template <class C>
-ECC_DEV void aos_load(const uint32_t* base, uint64_t i, uint32_t* x, uint32_t* y) {
-  constexpr int N = C::Fp::N;
-  const uint4* p = reinterpret_cast<const uint4*>(base + i * 2 * N);
-#pragma unroll
-  for (int g = 0; g < N / 4; ++g) {
-    const uint4 t = p[g];
-    x[4 * g] = t.x; x[4 * g + 1] = t.y; x[4 * g + 2] = t.z; x[4 * g + 3] = t.w;
-  }
-#pragma unroll
-  for (int g = 0; g < N / 4; ++g) {
-    const uint4 t = p[N / 4 + g];
-    y[4 * g] = t.x; y[4 * g + 1] = t.y; y[4 * g + 2] = t.z; y[4 * g + 3] = t.w;
-  }
-}
-
-template <class C>
-ECC_DEV void aos_store(uint32_t* base, uint64_t i, const uint32_t* x, const uint32_t* y) {
-  constexpr int N = C::Fp::N;
-  uint4* p = reinterpret_cast<uint4*>(base + i * 2 * N);
-#pragma unroll
-  for (int g = 0; g < N / 4; ++g) p[g] = make_uint4(x[4 * g], x[4 * g + 1], x[4 * g + 2], x[4 * g + 3]);
-#pragma unroll
-  for (int g = 0; g < N / 4; ++g)
-    p[N / 4 + g] = make_uint4(y[4 * g], y[4 * g + 1], y[4 * g + 2], y[4 * g + 3]);
-}
-
-template <class C>
 struct ShiftRound {
   using F = typename C::Fp;
   static constexpr int N = F::N;
-  static constexpr int OPS = 1;
   const uint32_t* src;
   uint32_t* dst;
   bool live;
-  ECC_DEV void den_c(size_t i, int, uint32_t* d) {
+  ECC_DEV void den(size_t i, uint32_t* d) {
     uint32_t x[N], y[N];
-    aos_load<C>(src, i, x, y);
+    load_affine<F>(src, i, x, y);
     live = dbl_den<C>(d, y);
   }
-  ECC_DEV void den_d(size_t i, int j, uint32_t* d) { den_c(i, j, d); }
-  ECC_DEV void finish(size_t i, const uint32_t (*inv)[N]) {
+  ECC_DEV void finish(size_t i, const uint32_t* inv) {
     uint32_t x[N], y[N];
-    aos_load<C>(src, i, x, y);
-    dbl_finish<C>(x, y, live, inv[0], x, y);
-    aos_store<C>(dst, i, x, y);
+    load_affine<F>(src, i, x, y);
+    dbl_finish<C>(x, y, live, inv, x, y);
+    store_affine<F>(dst, i, x, y);
   }
 };
 

@@ -329,4 +329,24 @@ inline bool shifted_overlap(const void* in, const void* out, size_t bytes) {
   return in != out && overlap(in, bytes, out, bytes);
 }
 
+// Scratch of a point operation over n rows: prefix products, then copies of the inputs
+// that the output overlaps other than row for row (q null: none).
+template <class F>
+cudaError_t point_scratch(Scratch& ws, size_t n, const uint32_t*& p, const uint32_t** q, const uint32_t* out,
+                          cudaStream_t st) {
+  const size_t rows = n * 2 * F::N * 4;
+  const bool cp = shifted_overlap(p, out, rows), cq = q && shifted_overlap(*q, out, rows);
+  cudaError_t e = ws.alloc(soa_bytes<F>(n) + (cp ? rows : 0) + (cq ? rows : 0), st);
+  if (e != cudaSuccess) return e;
+  uint32_t* copy = ws.as<uint32_t>() + soa_bytes<F>(n) / 4;
+  auto take = [&](const uint32_t*& in) {
+    e = cudaMemcpyAsync(copy, in, rows, cudaMemcpyDeviceToDevice, st);
+    in = copy;
+    copy += rows / 4;
+  };
+  if (cp) take(p);
+  if (cq && e == cudaSuccess) take(*q);
+  return e;
+}
+
 }  // namespace ecc
