@@ -22,10 +22,11 @@ requests that arrive while a round is running join a later one.
 Admission by device memory.  At start-up, after the bases, tables and rings are
 resident, the server reads the free device memory (cudaMemGetInfo) and keeps a
 reserve; the rest is the workspace budget.  Each kind's workspace is measured
-from the library itself: a calibration round of two sizes runs with a counting
+from the library itself: calibration rounds of two sizes run with a counting
 workspace allocator installed (ecc_set_allocator), giving bytes = fixed + per
-item; a verification takes no more than the largest round it can be given (the
-library holds only the items the GPU works on at once), which is measured too.  A round is admitted only while the workspaces of the rounds in flight
+item.  Larger calls take less an item (a verification holds only the items the GPU
+works on at once, an MSM takes longer chunks), so the largest single call is
+measured too, and what it took bounds the charge of smaller ones.  A round is admitted only while the workspaces of the rounds in flight
 plus its own fit the budget; a request larger than the whole budget is
 refused.
 
@@ -191,7 +192,7 @@ class Server:
             rnd["event"].synchronize()
             return live["peak"]
 
-        model = {}
+        model, self.top = {}, {}
         ecc.ecc_set_allocator(alloc, release)
         try:
             v2 = min(4096, self.e.shape[0])
@@ -201,7 +202,11 @@ class Server:
                 per = max(0.0, (peaks[1] - peaks[0]) / (n2 - n1))
                 fixed = max(0.0, peaks[0] - per * n1)
                 model[kind] = (fixed, per)
-            self.verify_top = peak_of("verify", max(1, min(self.max_verify_round, self.e.shape[0])))
+                n3 = {"verify": min(self.max_verify_round, self.e.shape[0]),
+                      "msm": min(self.max_msm_round_points, self.n_bases, self.scalars.shape[0])}[kind]
+                n3 = max(n3, n2)
+                top = peak_of(kind, n3) if n3 > n2 else peaks[1]
+                self.top[kind] = (n3, top, max(0.0, (top - peaks[1]) / (n3 - n2)) if n3 > n2 else per)
         finally:
             ecc.ecc_set_allocator(None, None)
         return model
@@ -209,9 +214,8 @@ class Server:
     def cost(self, kind, items):
         """Workspace bytes of a round of `items` items of `kind` (with 25% slack)."""
         fixed, per = self.model[kind]
-        need = fixed + per * items
-        if kind == "verify":
-            need = min(need, self.verify_top)
+        n3, top, slope = self.top[kind]
+        need = min(fixed + per * items, top + slope * max(0, items - n3))
         return int(1.25 * need) + (1 << 20)
 
     # -------------------------------------------------------------- rounds
