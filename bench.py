@@ -211,7 +211,7 @@ def gen_inputs(ecc, synth, torch, n, seed, curve=CURVE_P256):
 # DRAM traffic of one k_verify launch over 2^20 P-256 triples (dram__bytes_read.sum +
 # dram__bytes_write.sum, from one ncu capture), valid only for the kernel sources
 # it was taken on: the digest of those sources must match, else it is null.
-VERIFY_TRAFFIC = {"bytes": 1495312640 + 1494215680, "batch": 1 << 20, "digest": "cde39205b1615b10",
+VERIFY_TRAFFIC = {"bytes": 1494313216 + 1496545792, "batch": 1 << 20, "digest": "3925ef7a01be7fbe",
                   "sources": ["verify.cuh", "verify_host.cuh", "ladder.cuh", "jac.cuh", "glv.cuh", "ec.cuh", "fp.cuh",
                               "inv.cuh", "ptx.cuh", "curves_gen.cuh", "internal.h", "k_verify_p256.cu",
                               "k_verify.cu"]}
@@ -379,7 +379,7 @@ PAPER_SM2_VERIFY_A100 = 4372853.0
 def bench_sm2(ecc, costmodel, synth, torch, peak, rank, n, steps, world=1, clk=None):
     """ECDSA verification on the SM2 curve, the paper's curve: 2^20 triples with
     the same recipe as the P-256 line (1/16 corrupted), inputs resident.  The
-    schedule and the limb count are the P-256 kernel's, so is the work basis."""
+    schedule and the products are the P-256 kernel's, so is the work basis."""
     curve = ecc.ECC_SM2
     e, r, s, pub = gen_inputs(ecc, synth, torch, n, synth.SEED_BASE + 5 + 1000 * rank, curve)
     ok = torch.zeros(n, dtype=torch.uint8, device="cuda")
@@ -390,7 +390,7 @@ def bench_sm2(ecc, costmodel, synth, torch, peak, rank, n, steps, world=1, clk=N
     t = _event_time(torch, lambda: ecc.ecc_verify_batch(curve, n, e, r, s, pub, ok), max(steps, 5))
     clk.end("sm2")
     value = job_rate(n, t, world)
-    alg = costmodel.verify_imad() * n
+    alg = costmodel.ladder_verify_imad("SM2") * n
     return {"workload": "ECDSA verify, SM2, 2^20 seeded triples, 1/16 corrupted", "value": value,
             "unit": "verifies/s", "ms_per_step": t * 1e3, "valid_signatures": int(ok.sum().item()),
             "timed_calls": max(steps, 5), "clocks": clk.summary("sm2"),
@@ -505,7 +505,7 @@ def bench_k1(ecc, costmodel, synth, torch, peak, rank, world=1, clk=None, reps=2
     ok1 = torch.zeros(1, dtype=torch.uint8, device="cuda")
     t1 = _event_time(torch, lambda: [ecc.ecc_verify_batch(curve, 1, e[i:i + 1], r[i:i + 1], s[i:i + 1],
                                                           pub[i:i + 1], ok1) for i in range(plain_n)], 1)
-    alg = costmodel.verify_imad() * n
+    alg = costmodel.ladder_verify_imad("secp256k1") * n
     return {"workload": "ECDSA verify, secp256k1, 4096 seeded triples, 1/8 corrupted",
             "value": job_rate(n, t, world), "unit": "verifies/s", "ms_per_step": t * 1e3,
             "timed_calls": reps, "valid_signatures": int(ok.sum().item()), "clocks": clk.summary("secp256k1"),
@@ -544,9 +544,8 @@ def bench_sign_fpmul(ecc, costmodel, synth, torch, peak, rank, n, world=1, clk=N
     t_sign = _event_time(torch, lambda: ecc.ecc_sign_batch(curve, n, d, e, k, r, s, pub), reps)
     t_fp = _event_time(torch, lambda: ecc.ecc_fixed_base_mul(curve, n, kl, pts), reps)
     clk.end("sign_fpmul")
-    m8 = costmodel.imad_per_modmul(8)
-    a_sign = costmodel.sign_modmul() * m8 * n
-    a_fp = costmodel.fpmul_modmul() * m8 * n
+    a_sign = costmodel.ladder_sign_imad("SM2") * n
+    a_fp = costmodel.ladder_fpmul_imad("SM2") * n
     shape = "2^20" if n == 1 << 20 else str(n)
     return {"workload": f"ECDSA sign and FPMUL, SM2, {shape} items each", "timed_calls": reps,
             "clocks": clk.summary("sign_fpmul"),
@@ -698,7 +697,7 @@ def run_ours(args):
         cpu_baseline = cpu_baseline_verify(e.cpu().numpy(), r.cpu().numpy(), s.cpu().numpy(),
                                            pub.cpu().numpy(), 16384)
     peak = imad_peak(ecc, torch, sms)
-    alg = costmodel.verify_imad() * n
+    alg = costmodel.ladder_verify_imad("P-256") * n
     launch_s = statistics.median(per_launch)
     achieved = alg / launch_s
     line = {
@@ -710,9 +709,9 @@ def run_ours(args):
         "roofline": {"bound": "alu", "kernel": "k_verify<P256, 1>", "achieved": achieved / 1e12,
                      "peak": peak / 1e12, "unit": "T IMAD.WIDE/s", "frac": achieved / peak,
                      "traffic": verify_traffic(n), "traffic_unit": "DRAM bytes per launch",
-                     "basis": f"{costmodel.verify_modmul()} modmul x 136 wide mul-adds per verify (textbook: "
-                              "products by the shape of the prime need 64, so the fraction can pass 1); "
-                              "peak = measured mad.lo/madc.hi pair rate (ecc_bench_imad, same run)"},
+                     "basis": f"{costmodel.ladder_verify_imad('P-256'):.0f} wide mul-adds per verify in the kernel's "
+                              "products, without its inversions; peak = measured mad.lo/madc.hi pair rate "
+                              "(ecc_bench_imad, same run)"},
         "plain": {"value": plain, "unit": "verifies/s", "form": "one verification per launch"},
         "e2e": {"value": e2e_value, "unit": "verifies/s",
                 "h2d_bytes_per_step": 160 * n, "d2h_bytes_per_step": n, "bit_equal": e2e_ok},

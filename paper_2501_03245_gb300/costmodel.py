@@ -1,7 +1,7 @@
-"""Algorithmic work counts used for the roofline (no GPU code, no arithmetic of
-the method itself -- only operation counts).
+"""Work counts used for the roofline (no GPU code, no arithmetic of the method itself
+-- only operation counts).
 
-Basis (fixed, whatever reduction a kernel uses):
+The textbook's basis (fixed, whatever reduction or formulas a kernel uses):
   * one modmul or modsqr of an m-limb field costs 2 m^2 + m 32-bit wide
     multiply-adds (m^2 for the product, m^2 + m for the Montgomery reduction;
     Section 4.1: 136 for m = 8);
@@ -10,6 +10,10 @@ Basis (fixed, whatever reduction a kernel uses):
     (Section 2.2.1), so a batched PADD costs 6 and a batched PDBL 7 modmul
     (Section 3.1: "6N modmul" for N PADDs).  The per-batch modinv and the
     gather tree are overhead, not counted.
+
+A scalar multiplication in registers has other formulas and products by the shape of
+the prime, so its share of the multiply-add pipe follows from what it executes
+(``ladder_*_imad``): the wide multiply-adds of its products, without the inversions'.
 """
 
 # Table 1 (affine column) and Section 2.2.1
@@ -74,6 +78,49 @@ def sign_modmul():
     """Algorithmic modmul per ECDSA signature: k G and the public key d G share
     the 32 comb rounds (two additions per round), then s = k^-1 (e + r d)."""
     return 2 * G_COMB_ADDS * BATCH_PADD_MODMUL + SIGN_SCALAR_MODMUL
+
+
+# Wide multiply-adds of one (product, square) modulo the primes with a form of their own
+# and modulo the group orders (fp.cuh)
+LADDER_PRODUCT_IMAD = {"P-256": (64, 36), "SM2": (64, 36), "secp256k1": (73, 45)}
+ORDER_PRODUCT_IMAD = 136
+
+
+def _ladder_point_imad(curve):
+    """(doubling, addition of an affine point) in Jacobian coordinates (ladder.cuh)."""
+    mul, sqr = LADDER_PRODUCT_IMAD[curve]
+    return (3 if curve == "secp256k1" else 4) * mul + 4 * sqr, 8 * mul + 3 * sqr
+
+
+def ladder_verify_imad(curve):
+    """Wide multiply-adds of the products of one verification (verify.cuh): a table of 16
+    multiples, 52 signed 5-bit windows (of both halves on secp256k1) of which one in
+    32 is zero, 16 rows of the generator's table; the first addition is a copy."""
+    mul, sqr = LADDER_PRODUCT_IMAD[curve]
+    dbl, add = _ladder_point_imad(curve)
+    split = curve == "secp256k1"
+    digits = 52 * 31 / 32
+    n = (1 + (125 if split else 255)) * dbl + (14 + digits - 1 + 16) * add
+    n += 15 * (4 * mul + sqr) + mul               # the table made affine, and its inverse's form
+    n += digits / 2 * mul if split else 0         # beta x for the second half
+    n += 2 * mul + 3 * sqr                        # on the curve (y^2, x^2, x^3) and r Z^2
+    n += 0 if split else 3 * mul                  # x, y and r into Montgomery form
+    return n + 4 * ORDER_PRODUCT_IMAD             # s into it, its inverse's form, u1, u2
+
+
+def ladder_fpmul_imad(curve):
+    """Wide multiply-adds of the products of one k G: 16 additions, the first a copy,
+    and the result made affine and plain."""
+    mul, sqr = LADDER_PRODUCT_IMAD[curve]
+    return 15 * _ladder_point_imad(curve)[1] + 4 * mul + sqr + (0 if curve == "secp256k1" else 2 * mul)
+
+
+def ladder_sign_imad(curve):
+    """Wide multiply-adds of the products of one signature with its public key: k G and
+    d G, both Z from one inverse, and s = k^-1 (e + r d)."""
+    mul, sqr = LADDER_PRODUCT_IMAD[curve]
+    affine = 4 * mul + 3 * mul + sqr + mul + sqr + (0 if curve == "secp256k1" else 3 * mul)
+    return 30 * _ladder_point_imad(curve)[1] + affine + 5 * ORDER_PRODUCT_IMAD
 
 
 def break_even_batch(inv_over_mul=100):

@@ -1,12 +1,13 @@
 // Single modular inversion by Bernstein-Yang divsteps ("safegcd", Bernstein and
-// Yang, "Fast constant-time gcd computation and modular inversion", TCHES 2019),
-// variable-time form: the inputs of a batch inversion are public here.
+// Yang, "Fast constant-time gcd computation and modular inversion", TCHES 2019).
 //
-// The paper discusses Fermat (x^(q-2)) versus extended-Euclid inversion and
-// notes the latter is ~3x faster but branchy (Section 2.2); in the GAS batch
-// inversion only one thread per batch runs it (Section 3.2), so branches cost
-// nothing, while its short dependent chain shortens the serial "apply" step that
-// the whole CTA waits for.
+// The paper discusses Fermat (x^(q-2)) versus extended-Euclid inversion and notes
+// the latter is ~3x faster but branchy (Section 2.2).  Every kernel runs the form
+// without branches at the end of this file (30-bit limbs, divsteps30_flat), because
+// the lanes of a warp invert different values: the 32 group products of a CTA
+// (cta_invert, Section 3.2), or each item's own Z at the ends of a scalar
+// multiplication.  The forms with branches (62-bit limbs, and 30-bit ones) serve the
+// inversion probe, which compares them.
 //
 // State: f, g, d, e as signed integers in L limbs of 62 bits (least significant
 // first, every limb but the top in [0, 2^62), top limb signed).  Start f = q,
@@ -317,9 +318,10 @@ ECC_DEV Trans30 divsteps30(int32_t& delta, uint32_t f, uint32_t g) {
 // Fifteen divsteps one at a time without branches, with both columns of the
 // matrix in one word: P = u + 2^16 v and Q = q + 2^16 r as integers mod 2^32
 // (the steps are linear, so carries between the halves cancel).  zeta =
-// -(delta + 1/2) with delta counted in halves from 1/2 (the variant that needs
-// at most 590 divsteps for 256 bits instead of 741), negative when an odd g
-// swaps: then (f, g) <- (g, (g - f) / 2), else g <- (g + (g odd) f) / 2.
+// -(delta + 1/2) with delta counted in halves from 1/2, negative when an odd g swaps
+// (Pieter Wuille's "half-delta" variant of the divsteps, libsecp256k1's safegcd
+// notes and the safegcd-bounds proof: at most 590 of them for 256 bits instead of
+// 741): then (f, g) <- (g, (g - f) / 2), else g <- (g + (g odd) f) / 2.
 //
 // The adds of a multiple of 0 or +-1 are multiply-adds, which run on another
 // pipe than the logic beside them: one thread's chain is bound by the pipes'

@@ -694,10 +694,11 @@ __global__ void __launch_bounds__(kJacThreads, kJacCtas<C::Fp::N>)
 //
 // This replaced batched affine rounds (12 products a bucket instead of 27, but a
 // walk of 2^red_log + 1 + red_log rounds of about 25 us or more, then levels of four
-// elements by one thread): 4096 BN254 points 0.9 -> 0.08 ms, 256 BN254 MSMs of 2^10 to
-// 2^18 points 8.9 -> 6.0, 16 x 2^20 BLS12-381 points 12.4 -> 8.4; bound by the products
+// elements by one thread): 4096 BN254 points 0.9 -> 0.06 ms, 256 BN254 MSMs of 2^10 to
+// 2^18 points 8.9 -> 5.3, 16 x 2^20 BLS12-381 points 12.4 -> 7.6; bound by the products
 // of k_msm_elems where there are many buckets.  The combination below took 1.1 ms for
-// one BN254 result by one thread and takes 0.5.
+// one BN254 result by one thread and takes 0.28 (half the doublings, by a quad); for
+// 65536 results of whole scalars it takes as long either way.
 
 constexpr int kRedLog1Default = 5;      // log2 buckets per element, at most, by default
 constexpr int kRedLog1Max = 10;
