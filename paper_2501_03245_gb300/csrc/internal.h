@@ -92,6 +92,26 @@ cudaError_t launch_verify(int curve, size_t n, const uint8_t* hash, const uint8_
 // admitted (the same when the caller set one)
 int msm_window(int curve, uint64_t n, uint64_t num = 1);
 int msm_admitted_window(int curve, uint64_t n);
+// A function of an instance's size, remembered within a call: batches of many
+// instances repeat their sizes, and a width costs a lookup and a search of the model.
+template <class T>
+class BySize {
+ public:
+  template <class Fn>
+  T get(uint64_t n, Fn fn) {
+    Slot& s = slot_[(n * 0x9E3779B97F4A7C15ull) >> 56];
+    if (!s.set || s.n != n) s = Slot{true, n, fn()};
+    return s.value;
+  }
+
+ private:
+  struct Slot {
+    bool set = false;
+    uint64_t n = 0;
+    T value{};
+  };
+  Slot slot_[256];
+};
 void msm_set_window(int curve, int log2n, int c);
 // log2 of the buckets per reduction element: the autotuner's override for the size
 // class of n (0: none), the most an n-point MSM takes, and the override's setter for

@@ -61,24 +61,25 @@ constexpr uint64_t kDirectEntries = 12u << 20;
 // to kRedLog1Default) that leaves two CTAs of elements per SM: fewer elements are
 // longer serial sums, more of them are work for the tree (2^18 BN254 points, 278000
 // buckets: 1.95, 1.86, 1.82, 1.82, 1.90, 2.15 ms a call for 0 .. 5).
-inline int red_log(int curve, uint64_t n, int c, uint64_t buckets) {
+inline int red_log(int curve, uint64_t n, uint64_t buckets) {
   int k = msm_reduce_override(curve, n);
   if (k <= 0) {
     const uint64_t threads = (uint64_t)device_sm_count() * kJacThreads * 2;
     for (k = 0; k < kRedLog1Default && (buckets >> (k + 1)) >= threads;) ++k;
   }
-  return std::min(k, c - 1);
+  return k;
 }
 
 // Chunks, accumulation form and reduction layout of the planned instances.  lean: the
 // longest chunks and elements, which take the least workspace.
 template <int N>
 void finish_plan(int curve, Layout& L, const uint64_t* sizes, uint64_t size_all, bool lean) {
+  BySize<int> log;
   for (size_t i = 0; i < L.inst.size(); ++i) {
     MsmInst& m = L.inst[i];
     const uint64_t n = sizes ? sizes[i] : size_all;
-    m.red_log = (uint32_t)(lean ? std::min(msm_reduce_log(curve, n), (int)m.c - 1)
-                                : red_log(curve, n, (int)m.c, L.buckets));
+    const int k = log.get(n, [&] { return lean ? msm_reduce_log(curve, n) : red_log(curve, n, L.buckets); });
+    m.red_log = (uint32_t)std::min(k, (int)m.c - 1);
     m.elem_off = L.elems;
     m.row_off = L.rows;
     m.cta_off = L.ctas;
@@ -293,10 +294,13 @@ Layout plan(int curve, uint32_t num, const uint64_t* sizes, const uint64_t* poin
   if (lean) phi = 0;
   L.inst.resize(num);
   L.phi = phi;
+  BySize<int> width;
   for (uint32_t i = 0; i < num; ++i) {
     MsmInst& m = L.inst[i];
     m.n = (uint32_t)sizes[i];
-    m.c = (uint32_t)(pre_c > 0 ? pre_c : lean ? msm_admitted_window(curve, sizes[i]) : msm_window(curve, sizes[i], num));
+    m.c = (uint32_t)(pre_c > 0 ? pre_c : width.get(sizes[i], [&] {
+      return lean ? msm_admitted_window(curve, sizes[i]) : msm_window(curve, sizes[i], num);
+    }));
     m.W = (uint32_t)(phi ? half_windows<C>((int)m.c) : windows_for(curve, (int)m.c));
     m.bucket_base = (uint32_t)L.buckets;
     m.point_off = point_off[i];
