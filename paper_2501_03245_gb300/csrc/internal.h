@@ -88,10 +88,14 @@ cudaError_t launch_verify(int curve, size_t n, const uint8_t* hash, const uint8_
 
 // MSM: `num` instances, instance i = points / scalars rows
 // [offsets[i] - offsets[0], offsets[i+1] - offsets[0]) (host offsets); out: num x 2N limbs
-// window width of an n-point MSM in a batch of num; the width by which a size is
-// admitted (the same when the caller set one)
-int msm_window(int curve, uint64_t n, uint64_t num = 1);
+// window width of an n-point MSM in a batch of num, with split scalars or whole ones;
+// the width by which a size is admitted (the same when the caller set one)
+int msm_window(int curve, uint64_t n, uint64_t num, bool split);
 int msm_admitted_window(int curve, uint64_t n);
+// Modelled products that an n-point BN254 MSM in a batch of num saves by splitting its
+// scalars (c > 0: at that width); never negative up to 2^21 points without a set width.
+double msm_split_gain(uint64_t n, uint64_t num, int c);
+
 // A function of an instance's size, remembered within a call: batches of many
 // instances repeat their sizes, and a width costs a lookup and a search of the model.
 template <class T>

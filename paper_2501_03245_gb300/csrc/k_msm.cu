@@ -49,8 +49,7 @@ std::map<std::pair<int, int>, int> g_chunk_table;   // (curve, floor(log2 n)) ->
 // window (8 and 2.8 us with 8 limbs), which the instances of a batch share.  Batches of
 // tiny MSMs are all buckets: 65536 BLS12-381 MSMs of 4 points take 38 ms with 2 bits and
 // 58 with 4, 262144 of one point 100 and 161.
-int model_window(int curve, uint64_t n, uint64_t num) {
-  const bool split = curve == 2;
+int model_window(int curve, uint64_t n, uint64_t num, bool split) {
   const int bits = split ? BN254::GLV_BITS : msm_detail::scalar_bits(curve);
   int best = 2;
   double best_cost = 1e300;
@@ -65,6 +64,31 @@ int model_window(int curve, uint64_t n, uint64_t num) {
       best = c;
     }
   }
+  return best;
+}
+
+// The same for the choice between split and whole scalars of an n-point BN254 MSM, from
+// the phase times of both forms at 2^16 to 2^25 points and 13 to 20 bits: 20 a bucket; a
+// tenth more for a digit of a split scalar past 2^21 points, where the points and their
+// images no longer share the L2; for a digit of the top window what its bucket's x
+// entries wait for each other in the sort, at most 12 (5 of a whole scalar: half as many
+// meet); the doublings of the combination.
+constexpr uint64_t kSplitPoints = 1u << 21;
+
+double form_cost(uint64_t n, uint64_t num, int c, bool split) {
+  const int bits = split ? BN254::GLV_BITS : BN254::SCALAR_BITS;
+  const double W = (bits + 1 + c - 1) / c, top_digits = (double)n * (split ? 2 : 1);
+  const int top = bits - c * ((int)W - 1);
+  const double x = top_digits / (double)(1u << std::max(top, 0));
+  double cost = top_digits * W * (split && n > kSplitPoints ? 6.6 : 6.0) + W * (double)(1u << (c - 1)) * 20.0;
+  cost += top_digits * (split ? std::min(12.0, x / 128) : std::min(5.0, x / 256));
+  return cost + (150e3 * c + 59e3 * W + 41.5e3 * bits) / (double)std::max<uint64_t>(num, 1);
+}
+
+int whole_window(uint64_t n, uint64_t num) {
+  int best = 2;
+  for (int c = 3; c <= 20; ++c)
+    if (form_cost(n, num, c, false) < form_cost(n, num, best, false)) best = c;
   return best;
 }
 
@@ -106,10 +130,20 @@ int window_override(int curve, uint64_t n) {
 
 }  // namespace
 
-int msm_window(int curve, uint64_t n, uint64_t num) {
+int msm_window(int curve, uint64_t n, uint64_t num, bool split) {
   if (n < 2) n = 2;
   const int c = window_override(curve, n);
-  return c > 0 ? c : model_window(curve, n, num);
+  if (c > 0) return c;
+  return curve == 2 && !split ? whole_window(n, num) : model_window(curve, n, num, split);
+}
+
+double msm_split_gain(uint64_t n, uint64_t num, int c) {
+  if (n < 2) n = 2;
+  if (c <= 0) c = window_override(2, n);
+  if (c > 0) return form_cost(n, num, c, false) - form_cost(n, num, c, true);
+  const double gain = form_cost(n, num, whole_window(n, num), false) -
+                      form_cost(n, num, model_window(2, n, num, true), true);
+  return n <= kSplitPoints ? std::max(gain, 0.0) : gain;
 }
 
 int msm_admitted_window(int curve, uint64_t n) {

@@ -291,7 +291,13 @@ template <class C>
 Layout plan(int curve, uint32_t num, const uint64_t* sizes, const uint64_t* point_off,
             const uint64_t* scalar_off, int pre_c, uint64_t pre_stride, uint64_t phi, bool lean) {
   Layout L;
-  if (lean) phi = 0;
+  if (phi) {  // split where that is the better half of the work
+    BySize<double> gain;
+    double sum = 0;
+    for (uint32_t i = 0; i < num && !lean; ++i)
+      sum += gain.get(sizes[i], [&] { return msm_split_gain(sizes[i], num, 0); });
+    if (lean || sum < 0) phi = 0;
+  }
   L.inst.resize(num);
   L.phi = phi;
   BySize<int> width;
@@ -299,7 +305,7 @@ Layout plan(int curve, uint32_t num, const uint64_t* sizes, const uint64_t* poin
     MsmInst& m = L.inst[i];
     m.n = (uint32_t)sizes[i];
     m.c = (uint32_t)(pre_c > 0 ? pre_c : width.get(sizes[i], [&] {
-      return lean ? msm_admitted_window(curve, sizes[i]) : msm_window(curve, sizes[i], num);
+      return lean ? msm_admitted_window(curve, sizes[i]) : msm_window(curve, sizes[i], num, phi > 0);
     }));
     m.W = (uint32_t)(phi ? half_windows<C>((int)m.c) : windows_for(curve, (int)m.c));
     m.bucket_base = (uint32_t)L.buckets;
@@ -356,10 +362,10 @@ Layout plan_uniform(int curve, uint32_t num, int c, uint64_t cap, int pre_c, uin
                     bool lean) {
   Layout L;
   MsmInst m{};
-  if (lean) phi = 0;
+  const uint64_t mean = num ? std::max<uint64_t>(cap / num, 2) : 2;
+  if (phi && (lean || msm_split_gain(mean, num, c) < 0)) phi = 0;
   if (pre_c <= 0 && c <= 0) {
-    const uint64_t mean = num ? std::max<uint64_t>(cap / num, 2) : 2;
-    c = lean ? msm_admitted_window(curve, mean) : msm_window(curve, mean, num);
+    c = lean ? msm_admitted_window(curve, mean) : msm_window(curve, mean, num, phi > 0);
     const uint64_t W = (uint64_t)windows_for(curve, c);
     if (W * cap >= kMsmMaxDigits || (num * W) << (c - 1) >= kMsmMaxDigits) c = msm_admitted_window(curve, mean);
   }
@@ -375,7 +381,7 @@ Layout plan_uniform(int curve, uint32_t num, int c, uint64_t cap, int pre_c, uin
   L.buckets = (uint64_t)num * ((uint64_t)m.Wr << (m.c - 1));
   L.entries_max = cap * m.W * (phi ? 2 : 1);
   L.total_points = cap;
-  finish_plan<C::Fp::N>(curve, L, nullptr, num ? std::max<uint64_t>(cap / num, 2) : 2, lean);
+  finish_plan<C::Fp::N>(curve, L, nullptr, mean, lean);
   return L;
 }
 

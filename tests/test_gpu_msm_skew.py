@@ -118,3 +118,42 @@ def test_batches_of_tiny_msms(gpu_lib):
         for lg in (1, 2):
             gpu_lib.ecc_msm_set_window(cid, lg, 0)
     assert own < 0.9 * wide, (own, wide)
+
+
+def test_split_or_whole_scalars(gpu_lib):
+    """BN254 on each side of the size up to which scalars are split, and with 18-bit windows,
+    whose halves' top window holds only a carry: right either way, and no slower at 18
+    bits than the halves were (19 ms for 2^22 points against 12 with 19 bits)."""
+    import torch
+
+    cid, C, n_max = 2, curves.BN254, 1 << 22
+    a = _multiples(n_max)
+    pts = torch.empty((n_max, 2 * C.limbs), dtype=torch.int32, device="cuda")
+    gpu_lib.ecc_fixed_base_mul(cid, n_max, to_cuda(a), pts)
+    k = synth.uniform_limbs(93, 1, n_max, C.n)
+    kd = to_cuda(k.view(np.int32))
+    out = torch.zeros((1, 2 * C.limbs), dtype=torch.int32, device="cuda")
+
+    def run(n, c):
+        gpu_lib.ecc_msm_set_window(cid, n.bit_length() - 1, c)
+        ms = []
+        for _ in range(4):
+            gpu_lib.ecc_msm(cid, n, pts[:n], kd[:n], out)
+            ms.append(sum(gpu_lib.ecc_msm_phase_times().values()))
+        gpu_lib.ecc_msm_set_window(cid, n.bit_length() - 1, 0)
+        total = 0
+        for j in range(8):  # 16-bit halves of the limbs: every partial sum fits 64 bits
+            for h in (0, 16):
+                v = (k[:n, j] >> h & 0xFFFF).astype(np.int64)
+                total += int((v * a[:n, 0].astype(np.int64)).sum()) << (32 * j + h)
+        assert limbs_to_points(C, from_cuda(out).view(np.uint32))[0] == ec.mul(C, total % C.n, C.G), (n, c)
+        return min(ms)
+
+    try:
+        gpu_lib.ecc_set_phase_timing(1)
+        for n, c in ((1 << 21, 0), ((1 << 21) + 1, 0), (1 << 18, 18), (1 << 18, 16), (n_max, 0)):
+            run(n, c)
+        t18, t19 = run(n_max, 18), run(n_max, 19)
+    finally:
+        gpu_lib.ecc_set_phase_timing(0)
+    assert t18 < 1.35 * t19, (t18, t19)
