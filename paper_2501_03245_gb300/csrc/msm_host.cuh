@@ -406,25 +406,6 @@ struct Bases {
   int pre_c = 0;           // window width of pre (0: none)
 };
 
-// Gives back the points' images, which calls on a window table do not read.
-template <class C>
-cudaError_t drop_images(Bases* bs, cudaStream_t st) {
-  const size_t bytes = bs->n * 2 * C::Fp::N * 4;
-  uint32_t* mont = nullptr;
-  cudaError_t e = cudaMalloc(&mont, bytes);
-  if (e != cudaSuccess) return e;
-  e = cudaMemcpyAsync(mont, bs->mont, bytes, cudaMemcpyDeviceToDevice, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) {
-    cudaFree(mont);
-    return e;
-  }
-  cudaFree(bs->mont);
-  bs->mont = mont;
-  bs->phi = 0;
-  return cudaSuccess;
-}
-
 // Fills bs->pre with 2^(c w) P_i for w < W (W windows of width c).
 template <class C>
 cudaError_t precompute_t(Bases* bs, int c, cudaStream_t st) {
@@ -434,13 +415,7 @@ cudaError_t precompute_t(Bases* bs, int c, cudaStream_t st) {
   const uint64_t n = bs->n;
   if ((uint64_t)W * n >= (1ull << 31)) return cudaErrorInvalidValue;  // 31-bit point indices
   uint32_t* pre = nullptr;
-  const size_t bytes = std::max<uint64_t>(W * n, 1) * 2 * N * 4;
-  cudaError_t e = cudaMalloc(&pre, bytes);
-  if (e == cudaErrorMemoryAllocation && bs->phi) {  // in the images' place
-    cudaGetLastError();
-    e = drop_images<C>(bs, st);
-    if (e == cudaSuccess) e = cudaMalloc(&pre, bytes);
-  }
+  cudaError_t e = cudaMalloc(&pre, std::max<uint64_t>(W * n, 1) * 2 * N * 4);
   if (e != cudaSuccess) return e;
   if (n) e = cudaMemcpyAsync(pre, bs->mont, n * 2 * N * 4, cudaMemcpyDeviceToDevice, st);
   if (e == cudaSuccess && n && W > 1) {
@@ -475,7 +450,6 @@ cudaError_t precompute_t(Bases* bs, int c, cudaStream_t st) {
   if (bs->pre) cudaFree(bs->pre);
   bs->pre = pre;
   bs->pre_c = c;
-  if (bs->phi && drop_images<C>(bs, st) != cudaSuccess) cudaGetLastError();  // kept where there is no room to move
   return cudaSuccess;
 }
 

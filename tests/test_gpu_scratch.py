@@ -150,37 +150,3 @@ def test_verify(gpu_lib, cid, n, budget):
         torch.cuda.synchronize()
     assert arena.refused and not arena.held
     assert np.array_equal(from_cuda(ok), (np.arange(n) % 7 != 0).astype(np.uint8))
-
-
-def test_window_table_gives_the_images_back(gpu_lib):
-    """A BN254 handle with a window table holds the points and the table, not the points'
-    images; it answers as before and takes another table."""
-    import torch
-
-    cid, C, n = 2, curves.BN254, 1 << 20
-    pts = _points(gpu_lib, cid, n)
-    k = np.zeros((n, 8), np.uint32)
-    k[:, 0] = np.arange(n) % 5
-    k[:, 7] = np.arange(n) % 3 << 20
-    kd = to_cuda(k)
-    total = int((np.arange(1, n + 1) * k[:, 0].astype(np.int64)).sum())
-    total += int((np.arange(1, n + 1) * (np.arange(n) % 3)).sum()) << (224 + 20)
-    out = torch.zeros((1, 16), dtype=torch.int32, device="cuda")
-    for turn in range(2):  # the first turn fills the stream-ordered pool
-        torch.cuda.synchronize()
-        free = torch.cuda.mem_get_info()[0]
-        h = gpu_lib.ecc_bases_create(cid, n, pts)
-        try:
-            gpu_lib.ecc_msm_bases(h, 1, kd, out)
-            _check(C, out, [total])
-            for c in (20, 16):
-                gpu_lib.ecc_bases_precompute(h, c)
-                gpu_lib.ecc_msm_bases(h, 1, kd, out.zero_())
-                torch.cuda.synchronize()
-                _check(C, out, [total])
-                held = free - torch.cuda.mem_get_info()[0]
-                table = (254 + c) // c * n * 64
-                if turn == 1:
-                    assert held < n * 64 + table + (32 << 20), (c, held, table)
-        finally:
-            gpu_lib.ecc_bases_destroy(h)
