@@ -225,8 +225,11 @@ int ecc_msm_ragged_dev(ecc_curve_t curve, size_t num, size_t max_points, const u
 
 /* Resident bases: convert n points once into the library's device layout
  * (owned by the handle until ecc_bases_destroy), then run MSMs of many scalar
- * vectors against them.  ecc_msm_bases: scalars = num_vectors x n x 8 limbs,
- * out = num_vectors points; all vectors run through the same launches. */
+ * vectors against them.  A handle holds 96 bytes a point on BLS12-381 and 128 on BN254,
+ * 64 of them the points' images under the curve's endomorphism, which are left out
+ * where a window table would not fit the free memory beside them.  ecc_msm_bases:
+ * scalars = num_vectors x n x 8 limbs, out = num_vectors points; all vectors run
+ * through the same launches. */
 int ecc_bases_create(ecc_curve_t curve, size_t n, const uint32_t* points, void** handle,
                      void* stream);
 int ecc_msm_bases(void* handle, size_t num_vectors, const uint32_t* scalars, uint32_t* out,

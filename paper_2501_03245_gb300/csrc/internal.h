@@ -128,6 +128,11 @@ cudaError_t launch_msm(int curve, uint32_t num, const uint64_t* offsets, const u
                        const uint32_t* scalars, uint32_t* out, cudaStream_t st);
 cudaError_t bases_create(int curve, uint64_t n, const uint32_t* points, void** handle,
                          cudaStream_t st);
+// Whether a handle keeps the images of its n BN254 points (64 bytes a point, as long as
+// the handle lives: graphs recorded on it may read them): where the points, the images
+// and a table of 8-bit window multiples, 32 windows, fit the free memory, so that the
+// images are not in the way of ecc_bases_precompute.
+inline bool images_fit(uint64_t n, uint64_t free_bytes) { return n <= free_bytes / 64 / (1 + 1 + 32); }
 cudaError_t bases_destroy(void* handle);
 cudaError_t bases_precompute(void* handle, int c, cudaStream_t st);
 int bases_window(void* handle);

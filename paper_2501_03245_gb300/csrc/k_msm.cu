@@ -274,11 +274,16 @@ cudaError_t bases_create(int curve, uint64_t n, const uint32_t* points, void** h
   uint32_t* m = nullptr;
   // BN254: the points' images beside them (glv.cuh), where there is room
   uint64_t phi = curve == 2 ? n : 0;
+  size_t room = 0, all = 0;
+  if (phi && (cudaMemGetInfo(&room, &all) != cudaSuccess || !images_fit(n, room))) {
+    cudaGetLastError();
+    phi = 0;
+  }
   cudaError_t e = cudaMalloc(&m, std::max<uint64_t>(phi + n, 1) * 2 * N * 4);
   if (e == cudaErrorMemoryAllocation && phi) {
     cudaGetLastError();
     phi = 0;
-    e = cudaMalloc(&m, n * 2 * N * 4);
+    e = cudaMalloc(&m, std::max<uint64_t>(n, 1) * 2 * N * 4);
   }
   if (e != cudaSuccess) return e;
   if (n) e = points_to_mont(curve, points, n, m, phi, st);

@@ -150,3 +150,37 @@ def test_verify(gpu_lib, cid, n, budget):
         torch.cuda.synchronize()
     assert arena.refused and not arena.held
     assert np.array_equal(from_cuda(ok), (np.arange(n) % 7 != 0).astype(np.uint8))
+
+
+@pytest.mark.parametrize("cid", [2, 3])
+def test_graph_recorded_before_a_window_table(gpu_lib, cid):
+    """A call recorded on a handle replays on new scalars after the handle got a window
+    table: what it reads stays where it was."""
+    import torch
+
+    C, n = curves.BY_ID[cid], 3000
+    ks = [_scalars(C, n, s) for s in (20, 21)]
+    out = torch.zeros((1, 2 * C.limbs), dtype=torch.int32, device="cuda")
+    h = gpu_lib.ecc_bases_create(cid, n, _points(gpu_lib, cid, n))
+    try:
+        kd = ks[0][0].clone()
+        s = torch.cuda.Stream()
+        s.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(s):
+            gpu_lib.ecc_msm_bases(h, 1, kd, out, s)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            gpu_lib.ecc_msm_bases(h, 1, kd, out, s)
+        gpu_lib.ecc_bases_precompute(h, 12)
+        kd.copy_(ks[1][0])
+        out.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        _check(C, out, [sum((i + 1) * x for i, x in enumerate(ks[1][1]))])
+        gpu_lib.ecc_msm_bases(h, 1, ks[0][0], out.zero_())
+        _check(C, out, [sum((i + 1) * x for i, x in enumerate(ks[0][1]))])
+        del g
+    finally:
+        torch.cuda.synchronize()
+        gpu_lib.ecc_bases_destroy(h)
